@@ -86,8 +86,10 @@ typedef struct {
   const double *cl_fid;
   const double *N;
   int32_t precision;             /* qml_precision */
-  int32_t nslices;               /* bf16 slices per operand for QML_SPLIT_BF16
-                                    (0 = library default) */
+  int32_t nslices;               /* operand precision for QML_SPLIT_BF16 in units
+                                    of 6 bits, carried in 8-bit bf16 digits: at
+                                    least 6 nslices bits up to 54 (0 = library
+                                    default, 48 bits; 9 and 10 = 55 bits) */
   /* Native multipole binning (Sect. 2.4), read by qml_fisher only: 0 = one
    * bin per multipole; else nbins bins per spectrum with HOST edges
    * bin_edges[0] = lmin < bin_edges[1] < ... < bin_edges[nbins] = lmax + 1,
@@ -347,8 +349,8 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *   batch_streams   worker streams of pix_loglike_batch (default 4, 1..16)
  *   batch_graphs    1 (default) / 0: pix_loglike_batch replays each worker's
  *                   per-item kernel sequence as a captured CUDA graph
- *   ozaki_stages    3 (default) / 2: depth of the split kernel's TMA ring
- *                   (stages of 64 KB; always 2 for more than 8 digits)
+ *   ozaki_stages    4 (default) / 3 / 2: depth of the split kernel's ring of
+ *                   operand stages (48 or 56 KB each)
  *   ozaki_pairs     1 (default) / 0: the split kernel runs in clusters of two
  *                   CTAs on pairs of tile rows that share their B digit tiles
  *                   (loaded once from L2, multicast to both) / one CTA per

@@ -378,43 +378,61 @@ void build_C(Call &c, const Staged &s, const Dims &d, double *Y, double *C) {
 // K = kNBS.
 constexpr int64_t kNBS = 512;
 
+// One digit buffer of the split products (oz_digits_bytes large), taken from
+// a caller's workspace or allocated on first use and grown as needed.
+struct DigitBuf {
+  void *p = nullptr;
+  size_t bytes = 0;
+};
+
 struct Split {
   Call *c;
-  int nslices;
+  int S;  // digits per operand (oz_split_digits, kOzF64Digits)
   // SMs the split kernel leaves free (for float64 work on a second stream)
   int reserve_sms = 0;
-  void *ws = nullptr;
-  size_t ws_bytes = 0;
+  DigitBuf buf[3];
   double *tinv = nullptr;  // (kNBS/2)^2 scratch of the block-inverse doubling
   // the doubling scratch, allocated on first use unless preset
   double *tinv_scratch() {
     if (!tinv) tinv = c->alloc<double>((size_t)(kNBS / 2) * (kNBS / 2), "inverse scratch");
     return tinv;
   }
-  // use a caller-provided workspace (no allocation later)
-  void preset(void *p, size_t bytes) {
-    ws = p;
-    ws_bytes = bytes;
+  // Digits of X (element (r, k) at X[r sr + k sk]) into buffer i.
+  OzDigits slice(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
+    const size_t need = oz_digits_bytes(R, K, S);
+    if (need > buf[i].bytes) {
+      buf[i].p = c->alloc<unsigned char>(need, "split workspace");
+      buf[i].bytes = buf[i].p ? need : 0;
+    }
+    if (!buf[i].p) return OzDigits{};
+    const OzDigits d = oz_digits_at(buf[i].p, R, K, S);
+    oz_slice(X, sr, sk, d, c->st);
+    return d;
   }
-  // make sure the digit workspace holds a product of this shape
-  bool reserve(int64_t M, int64_t N, int64_t K, bool shared) {
-    size_t need = ozaki_workspace_bytes(M, N, K, nslices, shared);
-    if (need <= ws_bytes) return true;
-    ws = c->alloc<unsigned char>(need, "split workspace");
-    ws_bytes = ws ? need : 0;
-    return ws != nullptr;
+  void mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t ra, const OzDigits &B,
+          int64_t rb, double beta, double *C, int64_t ldc, int lower) {
+    if (c->err != QML_OK || M <= 0 || N <= 0) return;
+    c->cuda_ok(oz_mm(M, N, alpha, A, ra, B, rb, beta, C, ldc, lower, c->status, c->st, reserve_sms),
+               "split-precision gemm");
   }
   void gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A,
             int64_t lda, const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
             int lower) {
     if (c->err != QML_OK || M <= 0 || N <= 0) return;
-    const bool shared = (A == B && lda == ldb && ta != tb && M == N);
-    if (!reserve(M, N, K, shared)) return;
-    c->cuda_ok(ozaki_gemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, nslices,
-                          ws, c->status, c->st, reserve_sms),
-               "split-precision gemm");
+    const OzDigits a = slice(0, A, M, K, ta ? lda : 1, ta ? 1 : lda);
+    if (A == B && lda == ldb && ta != tb && M == N) {
+      mm(M, N, alpha, a, 0, a, 0, beta, C, ldc, lower);
+      return;
+    }
+    const OzDigits b = slice(1, B, N, K, tb ? 1 : ldb, tb ? ldb : 1);
+    mm(M, N, alpha, a, 0, b, 0, beta, C, ldc, lower);
   }
 };
+// the buffers potrf_split and trsm_split need for an n x n factor and nrhs
+// right-hand sides: panel digits, block-inverse digits, right-hand-side digits
+size_t split_ws_bytes(int i, int64_t n, int64_t nrhs, int S) {
+  return oz_digits_bytes(i == 0 ? n : (i == 1 ? kNBS : (nrhs > 0 ? nrhs : 1)), kNBS, S);
+}
 
 // The float64 part of the split Cholesky for the panel of columns j .. j + jb
 // of A (its diagonal block already updated by every earlier panel), on stream
@@ -513,35 +531,40 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
     if (look && j > 0) c.cuda_ok(cudaStreamWaitEvent(c.st, e_diag, 0), "lookahead");
     double *A21 = A + (j + jb) + j * lda;
     const int64_t m2 = n - j - jb;
+    OzDigits dP;  // digits of the finished panel A21, shared by its products
     if (m2 > 0) {
       double *A22 = A + (j + jb) + (j + jb) * lda;
       const int64_t jb2 = m2 < kNBS ? m2 : kNBS;
       // panel: A21 <- A21 L_jj^-T
-      sp.gemm(0, 1, m2, jb, jb, 1.0, A21, lda, Xinv, kNBS, 0.0, A21, lda, 0);
+      dP = sp.slice(0, A21, m2, jb, 1, lda);
+      const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
+      sp.mm(m2, jb, 1.0, dP, 0, dX, 0, 0.0, A21, lda, 0);
+      dP = sp.slice(0, A21, m2, jb, 1, lda);
       if (look) {
         // the next panel's columns first: its diagonal block (lower) and the
         // rows below it; then its chain starts on the second stream
-        sp.gemm(0, 1, jb2, jb2, jb, -1.0, A21, lda, A21, lda, 1.0, A22, lda, 1);
-        if (m2 > jb2)
-          sp.gemm(0, 1, m2 - jb2, jb2, jb, -1.0, A21 + jb2, lda, A21, lda, 1.0, A22 + jb2, lda,
-                  0);
+        sp.mm(jb2, jb2, -1.0, dP, 0, dP, 0, 1.0, A22, lda, 1);
+        if (m2 > jb2) sp.mm(m2 - jb2, jb2, -1.0, dP, jb2, dP, 0, 1.0, A22 + jb2, lda, 0);
         c.cuda_ok(cudaEventRecord(e_next, c.st), "lookahead");
         c.cuda_ok(cudaStreamWaitEvent(s2, e_next, 0), "lookahead");
         panel_chain(c, sp, A, lda, j + jb, jb2, Linv64, LinvB, ldparts, dfdiag, s2, true);
         c.cuda_ok(cudaEventRecord(e_diag, s2), "lookahead");
         sp.reserve_sms = reserve;
         if (m2 > jb2)
-          sp.gemm(0, 1, m2 - jb2, m2 - jb2, jb, -1.0, A21 + jb2, lda, A21 + jb2, lda, 1.0,
-                  A22 + jb2 + jb2 * lda, lda, 1);
+          sp.mm(m2 - jb2, m2 - jb2, -1.0, dP, jb2, dP, jb2, 1.0, A22 + jb2 + jb2 * lda, lda, 1);
       } else {
-        sp.gemm(0, 1, m2, m2, jb, -1.0, A21, lda, A21, lda, 1.0, A22, lda, 1);
+        sp.mm(m2, m2, -1.0, dP, 0, dP, 0, 1.0, A22, lda, 1);
       }
     }
     if (B) {
       // forward substitution, panel j: B_j <- L_jj^-1 B_j ; B_below -= A21 B_j
-      sp.gemm(0, 0, jb, nrhs, jb, 1.0, Xinv, kNBS, B + j, ldb, 0.0, B + j, ldb, 0);
-      if (m2 > 0)
-        sp.gemm(0, 0, m2, nrhs, jb, -1.0, A21, lda, B + j, ldb, 1.0, B + j + jb, ldb, 0);
+      const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
+      OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+      sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
+      if (m2 > 0) {
+        dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+        sp.mm(m2, nrhs, -1.0, dP, 0, dB, 0, 1.0, B + j + jb, ldb, 0);
+      }
     }
     sp.reserve_sms = 0;
     if (!look && m2 > 0)
@@ -566,10 +589,15 @@ void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, con
   for (int64_t j = 0; j < n; j += kNBS) {
     const int64_t jb = (n - j) < kNBS ? (n - j) : kNBS;
     const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS;
-    sp.gemm(0, 0, jb, nrhs, jb, 1.0, Xinv, kNBS, B + j, ldb, 0.0, B + j, ldb, 0);
-    if (j + jb < n)
-      sp.gemm(0, 0, n - j - jb, nrhs, jb, -1.0, L + (j + jb) + j * lda, lda, B + j, ldb, 1.0,
-              B + j + jb, ldb, 0);
+    const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
+    OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+    sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
+    const int64_t m2 = n - j - jb;
+    if (m2 > 0) {
+      const OzDigits dP = sp.slice(0, L + (j + jb) + j * lda, m2, jb, 1, lda);
+      dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+      sp.mm(m2, nrhs, -1.0, dP, 0, dB, 0, 1.0, B + j + jb, ldb, 0);
+    }
   }
 }
 
@@ -635,7 +663,7 @@ struct qml_plan {
   double *L = nullptr, *Linv = nullptr, *X = nullptr;
   double *LinvB = nullptr;  // kNBS-block inverses (split precision)
   bool split = false;
-  int nslices = 0;
+  int S = 0;  // digits per operand of its split products
   double *F = nullptr, *b = nullptr, *Finv = nullptr, *Fm12 = nullptr;
   int *uv = nullptr;
   // native binning (Sect. 2.4): na = nspec x bins is the size of F and of
@@ -672,7 +700,7 @@ void harmonic_W_from_M(Call &c, const qml_plan *plan, double *W, double *T) {
 void plan_W(Call &c, const qml_plan *plan, double *W, double *T) {
   const Dims &d = plan->d;
   if (plan->split) {
-    Split spl{&c, plan->nslices};
+    Split spl{&c, plan->S};
     spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1);
   } else {
     launch_dgemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, c.status,
@@ -693,7 +721,7 @@ void weighted_data(Call &c, const qml_plan *plan, const double *D, int nsims, do
   if (c.err != QML_OK) return;
   launch_copy_matrix(D, d.n, U, d.n, d.n, nsims, c.st);
   if (plan->split) {
-    Split spl{&c, plan->nslices};
+    Split spl{&c, plan->S};
     trsm_split(c, spl, plan->L, d.n, d.n, plan->LinvB, U, nsims, d.n);
     spl.gemm(1, 0, d.k, nsims, d.n, 1.0, plan->X, d.n, U, d.n, 0.0, wv, d.k, 0);
   } else {
@@ -807,7 +835,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   };
   const int64_t nblocks = (d.n + kNB - 1) / kNB;
   plan->split = (prob->precision == QML_SPLIT_BF16);
-  plan->nslices = prob->nslices;
+  plan->S = oz_split_digits(prob->nslices);
   // basis: the harmonic (SMW) route costs n^3/3 + n^2 k + n k^2 + 7 k^3 / 3
   // flops, the pixel route n^3/3 + n^2 k_sig + n^2 k + n k^2 (the fixed-signal
   // terms, n^2 (k_sig - k), are common): harmonic is cheaper when 3 n^2 > 7 k^2
@@ -888,7 +916,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     return e;
   }
 
-  Split spl{&c, prob->nslices};
+  Split spl{&c, oz_split_digits(prob->nslices)};
   Split *sp_or_null = plan->split ? &spl : nullptr;
   // Signal-band pieces: the whole band for the pixel basis; for the harmonic
   // basis the fixed signal below and above the window (Eq. N_eff).  They are
@@ -1033,7 +1061,7 @@ qml_status pix_loglike(const qml_problem *prob, const double *cl_theta, const do
   double *U = c.alloc<double>((size_t)d.n * nmaps, "U");
   if (!c.make_status()) return c.finish();
   if (prob->precision == QML_SPLIT_BF16) {
-    Split spl{&c, prob->nslices};
+    Split spl{&c, oz_split_digits(prob->nslices)};
     double *LinvB = c.alloc<double>((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
     if (!LinvB) return c.finish();
     build_C_split(c, spl, sp, d, Y, C);
@@ -1119,7 +1147,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     launch_copy_lower(sp.N, d.n, LN, d.n, d.n, c.st);
     launch_copy_matrix(D, d.n, u, d.n, d.n, nm, c.st);
     if (pr->precision == QML_SPLIT_BF16) {
-      Split spl{&c, pr->nslices};
+      Split spl{&c, oz_split_digits(pr->nslices)};
       double *LinvB = c.alloc<double>((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
       if (!LinvB) return c.finish();
       potrf_split(c, spl, LN, d.n, d.n, Linv, LinvB, ldp, ms[m].lnN);
@@ -1160,19 +1188,14 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     double *K, *lamL, *z, *rr, *Linv, *LinvB, *ldp;
     double *cl, *lnK, *lnl, *chi, *ld;  // fixed slots of the captured sequence
     double *tinv;                       // block-inverse scratch (split)
-    void *ws;
-    size_t ws_bytes;
+    DigitBuf buf[3];
   };
   std::vector<Worker> wk(NS);
   const int64_t nbk = (k + kNB - 1) / kNB, nbbk = (k + kNBS - 1) / kNBS;
-  size_t wsb = 0;
-  if (any_split) {
-    wsb = ozaki_workspace_bytes(k, k, kNBS, 0, true);
-    size_t b2 = ozaki_workspace_bytes(k, kNBS, kNBS, 0, false);
-    size_t b3 = ozaki_workspace_bytes(k, maxmaps, kNBS, 0, false);
-    if (b2 > wsb) wsb = b2;
-    if (b3 > wsb) wsb = b3;
-  }
+  int Smax = 0;
+  for (int m = 0; m < nmask; ++m)
+    if (split_kt && masks[m].prob.precision == QML_SPLIT_BF16)
+      Smax = std::max(Smax, oz_split_digits(masks[m].prob.nslices));
   double *lnK = c.alloc<double>(nitems);
   for (int w = 0; w < NS; ++w) {
     wk[w].K = c.alloc<double>((size_t)k * k, "Kt");
@@ -1187,9 +1210,11 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     wk[w].lnl = c.alloc<double>(maxmaps);
     wk[w].chi = c.alloc<double>(maxmaps);
     wk[w].ld = c.alloc<double>(1);
-    wk[w].ws = any_split ? (void *)c.alloc<unsigned char>(wsb, "split workspace") : nullptr;
+    for (int b = 0; any_split && b < 3; ++b) {
+      wk[w].buf[b].bytes = split_ws_bytes(b, k, maxmaps, Smax);
+      wk[w].buf[b].p = c.alloc<unsigned char>(wk[w].buf[b].bytes, "split workspace");
+    }
     wk[w].tinv = any_split ? c.alloc<double>((size_t)(kNBS / 2) * (kNBS / 2)) : nullptr;
-    wk[w].ws_bytes = wsb;
   }
   if (c.err != QML_OK) return c.finish();
   cudaEvent_t setup_done;
@@ -1216,8 +1241,8 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     launch_form_ktilde(ms[m].M, k, d0.nc, d0.k0, d0.lmin, W.lamL, W.K, k, W.st);
     launch_lambda_t_apply(ms[m].v, k, d0.nc, d0.k0, d0.lmin, W.lamL, nm, W.z, k, W.st);
     if (split_kt && masks[m].prob.precision == QML_SPLIT_BF16) {
-      Split spl{&cw, masks[m].prob.nslices};
-      spl.preset(W.ws, W.ws_bytes);
+      Split spl{&cw, oz_split_digits(masks[m].prob.nslices)};
+      for (int b = 0; b < 3; ++b) spl.buf[b] = W.buf[b];
       spl.tinv = W.tinv;
       potrf_split(cw, spl, W.K, k, k, W.Linv, W.LinvB, W.ldp, lnKp);
       trsm_split(cw, spl, W.K, k, k, W.LinvB, W.z, nm, k);
@@ -1373,7 +1398,7 @@ qml_status qml_potrf(int64_t n, double *A, int64_t lda, double *logdet, int32_t 
   if (precision == QML_SPLIT_BF16) {
     double *LinvB = c.alloc<double>((size_t)((n + kNBS - 1) / kNBS) * kNBS * kNBS);
     if (!LinvB) return c.finish();
-    Split spl{&c, 0};
+    Split spl{&c, oz_split_digits(0)};
     potrf_split(c, spl, Ad, n, lda, Linv, LinvB, ldparts, ld);
   } else {
     potrf_blocked(c, Ad, n, lda, Linv, ldparts, ld);
@@ -1402,7 +1427,7 @@ qml_status qml_trsm(int64_t n, int64_t nrhs, const double *L, int64_t lda, doubl
     // explicit inverses of the kNBS diagonal blocks (float64), then split products
     double *LinvB = c.alloc<double>((size_t)((n + kNBS - 1) / kNBS) * kNBS * kNBS);
     if (!LinvB) return c.finish();
-    Split spl{&c, 0};
+    Split spl{&c, oz_split_digits(0)};
     double *T = spl.tinv_scratch();
     if (!T) return c.finish();
     for (int64_t j = 0; j < n; j += kNBS) {
@@ -1442,10 +1467,11 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
   if (!c.make_status()) return c.finish();
   if (precision == QML_SPLIT_BF16 && kk > 0) {  // (kk == 0: C <- beta C, no digits)
     const bool shared = (A == B && lda == ldb && transA != transB && m == nn);
-    void *ws = c.alloc<unsigned char>(ozaki_workspace_bytes(m, nn, kk, 0, shared), "split workspace");
+    const int S = oz_split_digits(0);
+    void *ws = c.alloc<unsigned char>(ozaki_workspace_bytes(m, nn, kk, S, shared), "split workspace");
     if (!ws) return c.finish();
     c.cuda_ok(ozaki_gemm(transA, transB, m, nn, kk, alpha, Ad, lda, Bd, ldb, beta, Cd, ldc, lower,
-                         0, ws, c.status, c.st),
+                         S, ws, c.status, c.st),
               "split-precision gemm");
     return c.finish();
   }

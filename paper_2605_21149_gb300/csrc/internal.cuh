@@ -200,15 +200,38 @@ void launch_batch_finish(const double *rr, const double *dnd, const double *lnN,
                          cudaStream_t st);
 
 // ---------------------------------------------------------------- ozaki --
-// Split-precision float64 GEMM (bf16 digits on tcgen05, exact FP32 chunks,
-// float64 recombination); same operand conventions as launch_dgemm.  `work`
-// must hold ozaki_workspace_bytes(...) bytes.  nslices = 0 picks the default.
-void ozaki_choose(int64_t K, int nslices, int &S, int &beta);
-size_t ozaki_workspace_bytes(int64_t M, int64_t N, int64_t K, int nslices, bool shared_operand);
-// reserve_sms: SMs the persistent kernel leaves free for other work.
+// Split-precision float64 GEMM (8-bit digits in bf16 on tcgen05, exact sums,
+// float64 output; ozaki.cu).  S: digit count, 6 (48 bits) for QML_SPLIT_BF16,
+// 7 (55 bits) for the float64-quality products of QML_FP64, 3 (24 bits);
+// oz_split_digits maps a caller's nslices (6 bits each; 0 = default).
+int oz_split_digits(int nslices);
+constexpr int kOzF64Digits = 7;
+// exponent that marks a row holding an infinity or a NaN
+constexpr int kNanExp = 1 << 24;
+// The digits of a logical matrix (R rows, K each): digit tiles, row exponents
+// and row maxima, in memory of oz_digits_bytes(R, K, S), 1024-byte aligned.
+struct OzDigits {
+  unsigned char *dig = nullptr;
+  int *e = nullptr;
+  unsigned long long *mx = nullptr;
+  int64_t R = 0, K = 0;
+  int S = 0;
+};
+size_t oz_digits_bytes(int64_t R, int64_t K, int S);
+OzDigits oz_digits_at(void *mem, int64_t R, int64_t K, int S);
+// element (r, k) at X[r sr + k sk], one of the strides 1
+void oz_slice(const double *X, int64_t sr, int64_t sk, const OzDigits &d, cudaStream_t st);
+// C (M x N) <- alpha A B^T + beta C for the rows ra .. of A and rb .. of B
+// (multiples of 128).  reserve_sms: SMs the persistent kernel leaves free.
+cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t ra,
+                  const OzDigits &B, int64_t rb, double beta_c, double *C, int64_t ldc, int lower,
+                  DevStatus *status, cudaStream_t st, int reserve_sms = 0);
+// Both steps, same operand conventions as launch_dgemm; `work` must hold
+// ozaki_workspace_bytes(...) bytes.
+size_t ozaki_workspace_bytes(int64_t M, int64_t N, int64_t K, int S, bool shared_operand);
 cudaError_t ozaki_gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
                        const double *A, int64_t lda, const double *B, int64_t ldb, double beta_c,
-                       double *C, int64_t ldc, int lower, int nslices, void *work,
-                       DevStatus *status, cudaStream_t st, int reserve_sms = 0);
+                       double *C, int64_t ldc, int lower, int S, void *work, DevStatus *status,
+                       cudaStream_t st, int reserve_sms = 0);
 
 }  // namespace qmlgb

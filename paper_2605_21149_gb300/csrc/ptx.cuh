@@ -69,6 +69,17 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
       ::"r"(dst), "l"((uint64_t)src), "r"(bytes), "r"(bar)
       : "memory");
 }
+// the same copy delivered to every CTA of the cluster named in cta_mask, at the
+// same shared-memory offset, each completing on the mbarrier at bar's offset
+// in that CTA
+__device__ __forceinline__ void bulk_load_mc(uint32_t dst, const void *src, uint32_t bytes,
+                                             uint32_t bar, uint16_t cta_mask) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
+      " [%0], [%1], %2, [%3], %4;" ::"r"(dst),
+      "l"((uint64_t)src), "r"(bytes), "r"(bar), "h"(cta_mask)
+      : "memory");
+}
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
