@@ -63,8 +63,13 @@ typedef enum {
 } qml_status;
 
 typedef enum {
-  QML_FP64 = 0,        /* every contraction in native float64 */
-  QML_SPLIT_BF16 = 1   /* large contractions as exact bf16-slice products on
+  QML_FP64 = 0,        /* float64 throughout.  Problems of order n >= 256 run
+                          their large contractions as exact products of 55-bit
+                          digits on tensor cores, recombined and rounded once
+                          to float64 (error below a float64 accumulation's);
+                          diagonal blocks, logdets and everything else, and
+                          qml_gemm / qml_potrf / qml_trsm, stay native */
+  QML_SPLIT_BF16 = 1   /* large contractions as 48-bit bf16-digit products on
                           tcgen05 tensor cores (Ozaki-style splitting),
                           recombined in float64; panels, logdets stay float64 */
 } qml_precision;
@@ -227,8 +232,8 @@ typedef struct {
  * App. C.3): ln|C| = ln|N| + ln|Kt|, d^T C^-1 d = d^T N^-1 d - |Lk^-1 L^T Y^T
  * N^-1 d|^2.  masks: HOST array of nmask descriptors (same fields and
  * multipole band).  With QML_SPLIT_BF16 masks the per-mask products are split
- * precision and each item's Kt is factored in float64 (tuning key
- * batch_split_kt = 1: split trailing updates for Kt as well).
+ * precision and each item's Kt is factored at float64 quality (as QML_FP64;
+ * tuning key batch_split_kt = 1: 48-bit trailing updates for Kt as well).
  * Item i uses mask item_mask[i] (host or device, nitems) and
  * spectra item_cl + i*6*(lmax+1).  Outputs (row-major per item, leading
  * dimension ld_out >= the largest nmaps): lnL[i*ld_out + j], chi2[...] and
@@ -396,9 +401,10 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   its 64-wide diagonal blocks and their row solves in
  *                   float64 / in float-float (about 2^-46 per operation)
  *   batch_split_kt  0 (default) / 1: with QML_SPLIT_BF16 masks,
- *                   pix_loglike_batch factors each item's inner matrix Kt in
- *                   native float64 / with split-precision trailing updates
- *                   and panel products (float64 diagonal blocks and ln|Kt|)
+ *                   pix_loglike_batch factors each item's inner matrix Kt at
+ *                   float64 quality (as QML_FP64) / with 48-bit trailing
+ *                   updates and panel products (float64 diagonal blocks and
+ *                   ln|Kt| either way)
  *   test_wait_timeout  0 (default) / 1: for testing the failure path only:
  *                   the split-precision product issues no copies and its
  *                   waits give up after 1 ms, so the call returns

@@ -388,6 +388,9 @@ struct DigitBuf {
 struct Split {
   Call *c;
   int S;  // digits per operand (oz_split_digits, kOzF64Digits)
+  // products of QML_FP64 (and of the inner SMW matrices): float64 quality,
+  // and every diagonal block in float64 whatever split_diag_df says
+  bool f64 = false;
   // SMs the split kernel leaves free (for float64 work on a second stream)
   int reserve_sms = 0;
   DigitBuf buf[3];
@@ -432,6 +435,31 @@ struct Split {
 // right-hand sides: panel digits, block-inverse digits, right-hand-side digits
 size_t split_ws_bytes(int i, int64_t n, int64_t nrhs, int S) {
   return oz_digits_bytes(i == 0 ? n : (i == 1 ? kNBS : (nrhs > 0 ? nrhs : 1)), kNBS, S);
+}
+
+// QML_FP64 at and above this order factors and multiplies with 55-bit digit
+// products (kOzF64Digits) instead of the float64 pipe, whose 1.2 TFLOP/s bound
+// every contraction (TQU Nside 16 solve: 736 ms, 46.5 with digits).  Error: on
+// the operands of C = G G^T, the trailing updates, the solves and W = X^T X at
+// TQU Nside 16, QU Nside 16 and T Nside 8 an extended-precision reference puts
+// the 55-bit products 1.6 to 50 times closer than a float64 accumulation (C:
+// 7e-18 against 3.5e-16 of the row norms); F, y, lnL of T Nside 8 come out 4 to
+// 14 times closer.  Below about 250 rows the float64 path needs fewer
+// launches: lnL 0.59 against 0.72 ms at n = 192 but Fisher 1.03 against 1.00
+// ms, both in favour of digits from n = 300 on (0.78 against 1.08, 1.30
+// against 1.34 ms).
+constexpr int64_t kF64SplitMin = 256;
+
+// The digit products of a problem's precision for an order-n factor: 0 for
+// the float64 pipe.
+int split_digits(int precision, int nslices, int64_t n) {
+  if (precision == QML_SPLIT_BF16) return oz_split_digits(nslices);
+  return n >= kF64SplitMin ? kOzF64Digits : 0;
+}
+Split make_split(Call &c, int precision, int S) {
+  Split sp{&c, S};
+  sp.f64 = precision == QML_FP64;
+  return sp;
 }
 
 // The float64 part of the split Cholesky for the panel of columns j .. j + jb
@@ -505,7 +533,7 @@ void panel_chain(Call &c, Split &sp, double *A, int64_t lda, int64_t j, int64_t 
 void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *Linv64,
                  double *LinvB, double *ldparts, double *logdet, double *B = nullptr,
                  int64_t nrhs = 0, int64_t ldb = 0) {
-  const bool dfdiag = tune_get("split_diag_df", 0) != 0;
+  const bool dfdiag = !sp.f64 && tune_get("split_diag_df", 0) != 0;
   if (!sp.tinv_scratch()) return;  // allocated on the main stream before any use
   bool look = tune_get("split_lookahead", 1) != 0 && n > kNBS;
   if (look) {
@@ -583,12 +611,14 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
   if (logdet) launch_sum_logdet(ldparts, (int)((n + kNB - 1) / kNB), logdet, c.st);
 }
 
-// B <- L^-1 B with the explicit kNBS block inverses (split products).
+// B <- L^-1 B with explicit block inverses (split products), nb = kNBS or a
+// divisor of it that 64 divides: the inverses of the nb-blocks are the diagonal
+// nb-blocks of the kNBS-block inverses.
 void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, const double *LinvB,
-                double *B, int64_t nrhs, int64_t ldb) {
-  for (int64_t j = 0; j < n; j += kNBS) {
-    const int64_t jb = (n - j) < kNBS ? (n - j) : kNBS;
-    const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS;
+                double *B, int64_t nrhs, int64_t ldb, int64_t nb = kNBS) {
+  for (int64_t j = 0; j < n; j += nb) {
+    const int64_t jb = (n - j) < nb ? (n - j) : nb;
+    const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS + (j % kNBS) * (kNBS + 1);
     const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
     OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
     sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
@@ -598,6 +628,55 @@ void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, con
       dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
       sp.mm(m2, nrhs, -1.0, dP, 0, dB, 0, 1.0, B + j + jb, ldb, 0);
     }
+  }
+}
+
+// B <- L^-T B the same way, from the last block up: B_j <- L_jj^-T B_j, then
+// B_0..j-1 -= L_j,0..j-1^T B_j.
+void trsm_split_t(Call &c, Split &sp, const double *L, int64_t n, int64_t lda,
+                  const double *LinvB, double *B, int64_t nrhs, int64_t ldb, int64_t nb = kNBS) {
+  for (int64_t b = (n + nb - 1) / nb - 1; b >= 0; --b) {
+    const int64_t j = b * nb, jb = (n - j) < nb ? (n - j) : nb;
+    const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS + (j % kNBS) * (kNBS + 1);
+    const OzDigits dX = sp.slice(1, Xinv, jb, jb, kNBS, 1);
+    OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+    sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
+    if (j > 0) {
+      const OzDigits dP = sp.slice(0, L + j, j, jb, lda, 1);
+      dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+      sp.mm(j, nrhs, -1.0, dP, 0, dB, 0, 1.0, B, ldb, 0);
+    }
+  }
+}
+
+// The SMW inner matrix Kt (order k): its Cholesky factor with what its solves
+// need, in float64 (kNB-block inverses) or with float64-quality digit products
+// (kNBS-block inverses), whichever its order asks for.
+struct InnerFactor {
+  double *L = nullptr, *Linv = nullptr, *LinvB = nullptr;
+};
+void inner_potrf(Call &c, Split &sp, const InnerFactor &K, int64_t k, double *ldparts,
+                 double *logdet) {
+  if (sp.S)
+    potrf_split(c, sp, K.L, k, k, K.Linv, K.LinvB, ldparts, logdet);
+  else
+    potrf_blocked(c, K.L, k, k, K.Linv, ldparts, logdet);
+}
+// B <- L_K^-1 B, or with both set Kt^-1 B = L_K^-T L_K^-1 B.  The harmonic
+// basis takes blocks of 128 (kInnerNB): its right-hand sides are graded along
+// the modes (sqrt(Lambda) times noise weights, two orders between T and B), and
+// digits are relative to a block column's maximum.  With 512-wide blocks small
+// entries of F lost two digits (1.2e-10 of an entry against 1.6e-12 on the
+// float64 pipe, TQU Nside 4; 1.5e-12 with 128).
+constexpr int64_t kInnerNB = 128;
+void inner_trsm(Call &c, Split &sp, const InnerFactor &K, int64_t k, double *B, int64_t nrhs,
+                int64_t ldb, bool both, int64_t nb = kNBS) {
+  if (sp.S) {
+    trsm_split(c, sp, K.L, k, k, K.LinvB, B, nrhs, ldb, nb);
+    if (both) trsm_split_t(c, sp, K.L, k, k, K.LinvB, B, nrhs, ldb, nb);
+  } else {
+    trsm_blocked(c, K.L, k, k, K.Linv, B, nrhs, ldb);
+    if (both) trsm_blocked_t(c, K.L, k, k, K.Linv, B, nrhs, ldb);
   }
 }
 
@@ -663,6 +742,7 @@ struct qml_plan {
   double *L = nullptr, *Linv = nullptr, *X = nullptr;
   double *LinvB = nullptr;  // kNBS-block inverses (split precision)
   bool split = false;
+  int precision = QML_FP64;
   int S = 0;  // digits per operand of its split products
   double *F = nullptr, *b = nullptr, *Finv = nullptr, *Fm12 = nullptr;
   int *uv = nullptr;
@@ -673,14 +753,19 @@ struct qml_plan {
   bool binned = false;
   int *bstart = nullptr, *bcount = nullptr;
   // harmonic basis (Sect. 2.3.2): L holds the factor of N (or N_eff), X holds
-  // U = L_N^-1 Y; LK the float64 factor of Kt = I + L_Lambda^T M L_Lambda with
-  // its 64-block inverses, lamL / lamLi the per-l factors of Lambda and their
+  // U = L_N^-1 Y; K the factor of Kt = I + L_Lambda^T M L_Lambda with
+  // its block inverses, lamL / lamLi the per-l factors of Lambda and their
   // inverses
   bool harmonic = false;
-  double *LK = nullptr, *LKinv = nullptr, *lamL = nullptr, *lamLi = nullptr;
+  InnerFactor K;
+  double *lamL = nullptr, *lamLi = nullptr;
 };
 
 namespace {
+
+Split inner_split(Call &c, int64_t k) {
+  return make_split(c, QML_FP64, split_digits(QML_FP64, 0, k));
+}
 
 // Harmonic basis: W (k x k) holds M = Y^T N^-1 Y on entry and W = M (I +
 // Lambda M)^-1 = L_Lambda^-T Kt^-1 L_Lambda^T M (Eq. smw_stable) on return;
@@ -688,8 +773,8 @@ namespace {
 void harmonic_W_from_M(Call &c, const qml_plan *plan, double *W, double *T) {
   const Dims &d = plan->d;
   launch_lambda_t_apply(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, d.k, T, d.k, c.st);
-  trsm_blocked(c, plan->LK, d.k, d.k, plan->LKinv, T, d.k, d.k);
-  trsm_blocked_t(c, plan->LK, d.k, d.k, plan->LKinv, T, d.k, d.k);
+  Split sk = inner_split(c, d.k);
+  inner_trsm(c, sk, plan->K, d.k, T, d.k, d.k, true, kInnerNB);
   launch_lambda_t_apply(T, d.k, d.nc, d.k0, d.lmin, plan->lamLi, d.k, W, d.k, c.st);
   launch_symmetrize_avg(W, d.k, d.k, c.st);
 }
@@ -700,7 +785,7 @@ void harmonic_W_from_M(Call &c, const qml_plan *plan, double *W, double *T) {
 void plan_W(Call &c, const qml_plan *plan, double *W, double *T) {
   const Dims &d = plan->d;
   if (plan->split) {
-    Split spl{&c, plan->S};
+    Split spl = make_split(c, plan->precision, plan->S);
     spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1);
   } else {
     launch_dgemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, c.status,
@@ -721,7 +806,7 @@ void weighted_data(Call &c, const qml_plan *plan, const double *D, int nsims, do
   if (c.err != QML_OK) return;
   launch_copy_matrix(D, d.n, U, d.n, d.n, nsims, c.st);
   if (plan->split) {
-    Split spl{&c, plan->S};
+    Split spl = make_split(c, plan->precision, plan->S);
     trsm_split(c, spl, plan->L, d.n, d.n, plan->LinvB, U, nsims, d.n);
     spl.gemm(1, 0, d.k, nsims, d.n, 1.0, plan->X, d.n, U, d.n, 0.0, wv, d.k, 0);
   } else {
@@ -731,8 +816,8 @@ void weighted_data(Call &c, const qml_plan *plan, const double *D, int nsims, do
   }
   if (plan->harmonic) {
     launch_lambda_t_apply(wv, d.k, d.nc, d.k0, d.lmin, plan->lamL, nsims, wv, d.k, c.st);
-    trsm_blocked(c, plan->LK, d.k, d.k, plan->LKinv, wv, nsims, d.k);
-    trsm_blocked_t(c, plan->LK, d.k, d.k, plan->LKinv, wv, nsims, d.k);
+    Split sk = inner_split(c, d.k);
+    inner_trsm(c, sk, plan->K, d.k, wv, nsims, d.k, true, kInnerNB);
     launch_lambda_t_apply(wv, d.k, d.nc, d.k0, d.lmin, plan->lamLi, nsims, w, d.k, c.st);
   }
 }
@@ -834,8 +919,9 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     return (double *)p;
   };
   const int64_t nblocks = (d.n + kNB - 1) / kNB;
-  plan->split = (prob->precision == QML_SPLIT_BF16);
-  plan->S = oz_split_digits(prob->nslices);
+  plan->precision = prob->precision;
+  plan->S = split_digits(prob->precision, prob->nslices, d.n);
+  plan->split = plan->S != 0;
   // basis: the harmonic (SMW) route costs n^3/3 + n^2 k + n k^2 + 7 k^3 / 3
   // flops, the pixel route n^3/3 + n^2 k_sig + n^2 k + n k^2 (the fixed-signal
   // terms, n^2 (k_sig - k), are common): harmonic is cheaper when 3 n^2 > 7 k^2
@@ -850,8 +936,9 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   if (plan->split) plan->LinvB = palloc((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
   plan->X = palloc((size_t)d.n * d.k);
   if (plan->harmonic) {
-    plan->LK = palloc((size_t)d.k * d.k);
-    plan->LKinv = palloc((size_t)((d.k + kNB - 1) / kNB) * kNB * kNB);
+    plan->K.L = palloc((size_t)d.k * d.k);
+    plan->K.Linv = palloc((size_t)((d.k + kNB - 1) / kNB) * kNB * kNB);
+    plan->K.LinvB = palloc((size_t)((d.k + kNBS - 1) / kNBS) * kNBS * kNBS);
     plan->lamL = palloc((size_t)d.nl * d.nc * d.nc);
     plan->lamLi = palloc((size_t)d.nl * d.nc * d.nc);
   }
@@ -916,7 +1003,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     return e;
   }
 
-  Split spl{&c, oz_split_digits(prob->nslices)};
+  Split spl = make_split(c, prob->precision, plan->S);
   Split *sp_or_null = plan->split ? &spl : nullptr;
   // Signal-band pieces: the whole band for the pixel basis; for the harmonic
   // basis the fixed signal below and above the window (Eq. N_eff).  They are
@@ -972,8 +1059,9 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     if (c.err == QML_OK) {
       launch_lambda_factor(sp.cl, d.lmin, d.lmax, d.nc, d.comps, plan->lamL, c.st, ldcl);
       launch_lambda_inverse(plan->lamL, d.nl, d.nc, d.lmin, plan->lamLi, c.status, c.st);
-      launch_form_ktilde(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, plan->LK, d.k, c.st);
-      potrf_blocked(c, plan->LK, d.k, d.k, plan->LKinv, ldk, nullptr);
+      launch_form_ktilde(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, plan->K.L, d.k, c.st);
+      Split sk = inner_split(c, d.k);
+      inner_potrf(c, sk, plan->K, d.k, ldk, nullptr);
       harmonic_W_from_M(c, plan, W, T);
     }
   }
@@ -1060,8 +1148,9 @@ qml_status pix_loglike(const qml_problem *prob, const double *cl_theta, const do
   double *ldparts = c.alloc<double>(nblocks);
   double *U = c.alloc<double>((size_t)d.n * nmaps, "U");
   if (!c.make_status()) return c.finish();
-  if (prob->precision == QML_SPLIT_BF16) {
-    Split spl{&c, oz_split_digits(prob->nslices)};
+  const int S = split_digits(prob->precision, prob->nslices, d.n);
+  if (S) {
+    Split spl = make_split(c, prob->precision, S);
     double *LinvB = c.alloc<double>((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
     if (!LinvB) return c.finish();
     build_C_split(c, spl, sp, d, Y, C);
@@ -1146,8 +1235,9 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     launch_ybuild(sp.y, U, d.n, c.st);
     launch_copy_lower(sp.N, d.n, LN, d.n, d.n, c.st);
     launch_copy_matrix(D, d.n, u, d.n, d.n, nm, c.st);
-    if (pr->precision == QML_SPLIT_BF16) {
-      Split spl{&c, oz_split_digits(pr->nslices)};
+    const int S = split_digits(pr->precision, pr->nslices, d.n);
+    if (S) {
+      Split spl = make_split(c, pr->precision, S);
       double *LinvB = c.alloc<double>((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
       if (!LinvB) return c.finish();
       potrf_split(c, spl, LN, d.n, d.n, Linv, LinvB, ldp, ms[m].lnN);
@@ -1175,13 +1265,19 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   // writing its results to fixed slots -- and replays it for every later item
   bool graphs = tune_get("batch_graphs", 1) != 0 && nitems > NS;
   // Split precision covers the per-mask products (L_N, U = L_N^-1 Y, M, v);
-  // the per-item inner factor Kt (the SMW inner inverse and ln|Kt|) stays in
-  // native float64 unless the tuning key batch_split_kt asks for its trailing
-  // updates and panel products in split precision too.
+  // the per-item inner factor Kt (the SMW inner inverse and ln|Kt|) stays at
+  // float64 quality (inner_split) unless the tuning key batch_split_kt asks for
+  // its trailing updates and panel products in 48 bits too.
   const bool split_kt = tune_get("batch_split_kt", 0) != 0;
-  bool any_split = false;
-  for (int m = 0; m < nmask; ++m)
-    any_split |= (split_kt && masks[m].prob.precision == QML_SPLIT_BF16);
+  auto kt_split = [&](Call &cw, int m) {
+    const qml_problem &pr = masks[m].prob;
+    return split_kt && pr.precision == QML_SPLIT_BF16
+               ? make_split(cw, pr.precision, oz_split_digits(pr.nslices))
+               : inner_split(cw, k);
+  };
+  int Smax = 0;
+  for (int m = 0; m < nmask; ++m) Smax = std::max(Smax, kt_split(c, m).S);
+  const bool any_split = Smax > 0;
   struct Worker {
     cudaStream_t st = nullptr;
     cudaEvent_t done = nullptr;
@@ -1192,10 +1288,6 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   };
   std::vector<Worker> wk(NS);
   const int64_t nbk = (k + kNB - 1) / kNB, nbbk = (k + kNBS - 1) / kNBS;
-  int Smax = 0;
-  for (int m = 0; m < nmask; ++m)
-    if (split_kt && masks[m].prob.precision == QML_SPLIT_BF16)
-      Smax = std::max(Smax, oz_split_digits(masks[m].prob.nslices));
   double *lnK = c.alloc<double>(nitems);
   for (int w = 0; w < NS; ++w) {
     wk[w].K = c.alloc<double>((size_t)k * k, "Kt");
@@ -1240,16 +1332,12 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     launch_lambda_factor(cl, d0.lmin, d0.lmax, d0.nc, d0.comps, W.lamL, W.st);
     launch_form_ktilde(ms[m].M, k, d0.nc, d0.k0, d0.lmin, W.lamL, W.K, k, W.st);
     launch_lambda_t_apply(ms[m].v, k, d0.nc, d0.k0, d0.lmin, W.lamL, nm, W.z, k, W.st);
-    if (split_kt && masks[m].prob.precision == QML_SPLIT_BF16) {
-      Split spl{&cw, oz_split_digits(masks[m].prob.nslices)};
-      for (int b = 0; b < 3; ++b) spl.buf[b] = W.buf[b];
-      spl.tinv = W.tinv;
-      potrf_split(cw, spl, W.K, k, k, W.Linv, W.LinvB, W.ldp, lnKp);
-      trsm_split(cw, spl, W.K, k, k, W.LinvB, W.z, nm, k);
-    } else {
-      potrf_blocked(cw, W.K, k, k, W.Linv, W.ldp, lnKp);
-      trsm_blocked(cw, W.K, k, k, W.Linv, W.z, nm, k);
-    }
+    Split spl = kt_split(cw, m);
+    for (int b = 0; b < 3; ++b) spl.buf[b] = W.buf[b];
+    spl.tinv = W.tinv;
+    const InnerFactor K{W.K, W.Linv, W.LinvB};
+    inner_potrf(cw, spl, K, k, W.ldp, lnKp);
+    inner_trsm(cw, spl, K, k, W.z, nm, k, false);
     launch_colnorm2(W.z, k, k, nm, W.rr, W.st);
     launch_batch_finish(W.rr, ms[m].dnd, ms[m].lnN, lnKp, nm, ol, oc, od, W.st);
   };

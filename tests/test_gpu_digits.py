@@ -1,0 +1,87 @@
+"""8-bit digit products (csrc/ozaki.cu) where they can go wrong: K beyond one
+int32 piece, digits that all agree in sign, rows with an infinity or a NaN, and
+QML_FP64 problems at the order where it changes to 55-bit digits.
+
+Bounds.  48 bits: an operand's rounding is at most 2^-49 of its row's maximum
+2^e (2 K 2^-49 over the sum), the dropped levels 8 and beyond at most 5.1 K
+2^(14-64) (levels of 5, 4, ... products of digits up to 2^7), and level 6 past
+2^24 loses no more than those: below 2^-45 K 2^(e+f) in all."""
+import numpy as np
+import pytest
+
+import parity as P
+from oracle import harmonic, qml
+from paper_2605_21149_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_21149_gb300 import api as A
+    from paper_2605_21149_gb300 import build
+    build.build()
+    return A
+
+
+def td(x):
+    return torch.as_tensor(np.asarray(x, dtype=np.float64), device="cuda").t().contiguous().t()
+
+
+@pytest.mark.parametrize("m,n,k", [(129, 131, 15361), (128, 64, 16), (1, 1, 40000)])
+def test_equal_digits_long_k(api, m, n, k):
+    """Every element (2^48 - 1) 2^-48 or the value whose digits are all 127: the
+    level sums are as large as they can be."""
+    lo = sum(127.0 * 256.0 ** i for i in range(5))
+    for v in (1.0 - 2.0 ** -48, (127.0 * 256.0 ** 5 + lo) * 2.0 ** -48):
+        A = np.full((m, k), v)
+        B = np.full((k, n), v)
+        C = api.gemm(td(A), td(B), precision=1).cpu().numpy()
+        ref = float(k) * v * v
+        e = np.frexp(v)[1]
+        assert np.abs(C - ref).max() <= k * 2.0 ** (2 * e - 45) + 2.0 ** -52 * ref
+        assert (C == C[0, 0]).all()
+
+
+def test_nonfinite_rows_poison_their_outputs_only(api):
+    rng = np.random.default_rng(3)
+    A, B = rng.normal(size=(300, 200)), rng.normal(size=(200, 150))
+    A[7, 11], A[260, 199], B[5, 149] = np.inf, np.nan, -np.inf
+    C0 = rng.normal(size=(300, 150))
+    Cd = td(C0)
+    api.gemm(td(A), td(B), Cd, alpha=-1.0, beta=1.0, precision=1)
+    C = Cd.cpu().numpy()
+    bad = np.zeros((300, 150), dtype=bool)
+    bad[[7, 260], :] = True
+    bad[:, 149] = True
+    assert np.isnan(C[bad]).all()
+    A[7, 11] = A[260, 199] = B[5, 149] = 0.0
+    ref = C0 - A @ B
+    assert np.abs(C - ref)[~bad].max() <= 1e-12 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [255, 256, 257, 511, 513])
+@pytest.mark.parametrize("basis", [0, 1])
+def test_fp64_order_where_digits_start(api, n, basis):
+    """T maps on n pixels, float64: F, b, y and lnL against the oracle, at
+    float64 rounding times the covariance's condition (about 1e4)."""
+    th, ph, _ = synth.healpix_ring_centres(8)
+    wl = synth.make_workload("T", 8, 11, True, False, 0.0, ("TT",), 7, 40 + n,
+                             geometry=(th[100:100 + n], ph[100:100 + n]))
+    Y, alm, noise, maps = P.oracle_maps(wl, 3)
+    ref = qml.qml_for(wl, Y, maps=maps)
+    prob = api.Problem.from_workload(wl, basis=basis)
+    F, plan = api.fisher(prob)
+    est = plan.estimate(td(maps))
+    plan.free()
+    assert P.rel_max(F, ref["F"]) <= 1e-11
+    assert P.rel_max(est["b"], ref["b"]) <= 1e-11
+    assert P.rel_max(est["y"], ref["y"]) <= 1e-11
+    C = qml.total_cov(Y, wl.cl_fid, wl.comps, wl.lmin, wl.lmax, wl.N())
+    lnl, chi2, ld = qml.loglike(C, maps)
+    g = api.loglike(prob, torch.as_tensor(wl.cl_fid.reshape(-1), device="cuda"), td(maps))
+    assert P.rel_max(g[0], lnl) <= 1e-12
+    assert abs(float(P.to_np(g[2])) - ld) <= 1e-12 * abs(ld)
