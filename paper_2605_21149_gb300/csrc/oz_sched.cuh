@@ -48,12 +48,13 @@ struct OzDigitsOf<7> {
   static constexpr bool kLow = true, kFrac = true;
 };
 
-// Group G of variant S (0: levels 5 and up, 1: levels 2..4).  Levels L0 ..
-// L0 + D - 1 are drained: level L0 + i after first(i) K steps of a piece and
-// every period(i) from there on (never two at one step).  They start in slots
-// 0 .. D - 1 and swap with kSpare (-1: none).  F more slots from kFixed0 on are
-// drained at the end of the piece only: level L0 + D, and (F = 2) levels L0 + D
-// + 1 and L0 + D + 2 together.
+// Group G of variant S (0: levels 5 and up, 1: levels 2..4).  Its levels are
+// its entries 0 .. NE - 1 (S = 7: levels 8 and 9 share the last entry of group
+// 0), each in one accumulator slot of the four.  The first D are drained: entry
+// i after first(i) K steps of a piece and every period(i) from there on, never
+// two at one step.  With a slot to spare (NE < 4) the entry goes on in that
+// one; otherwise it waits for its own.  The others are drained at the end of
+// the piece only.
 //
 // The longest exact chunk, |sum| <= 2^24, from |a_1| <= 2^kTop, |a_s| <= 2^7:
 //   kTop = 8: levels 2, 3: 2^16 an element (256 elements, 16 steps), level 4:
@@ -64,51 +65,52 @@ struct OzDigitsOf<7> {
 // 2^-48, 2^-47.7 K of the maxima in all, no more than the dropped level 8.
 // The first hand-overs come late because the epilogue is still writing the
 // last tile then (14 us beside 0.8 us a K step; with level 6 drained every 9
-// steps from the 4th on, a 6400 x 6400 x 512 update took 0.585 ms).
+// steps from the 4th on, a 6400 x 6400 x 512 update took 0.585 ms), and those
+// of one group are spread evenly, since each costs the epilogue about 1000
+// clocks (a K step of levels 2..4: 560).
 template <int S, int G>
 struct OzGroup {
   static constexpr bool kLowGroup = G == 0;
   static constexpr bool kWide = S == 7;
   static constexpr int L0 = kLowGroup ? 5 : 2;
   static constexpr int D = kLowGroup ? 2 : 3;
-  static constexpr int F = kLowGroup ? (kWide ? 2 : 1) : 0;
-  static constexpr int kFixed0 = kWide ? 2 : 3;
-  static constexpr int kSpare = kLowGroup ? (kWide ? -1 : 2) : 3;
+  static constexpr int NE = kLowGroup && kWide ? 4 : 3;
+  static constexpr bool kSpare = NE < 4;
   static constexpr int kDigits = kLowGroup ? S : 3;
   static constexpr int kSteps = kLowGroup ? 1 : 2;  // K steps per ring stage
   static QMLGB_HD constexpr int first(int i) {
     return kLowGroup ? (kWide ? (i == 0 ? 14 : 12) : (i == 0 ? 10 : 25))
-                     : (kWide ? (i == 0 ? 33 : (i == 1 ? 27 : 20)) : 16 - 4 * i);
+                     : (kWide ? (i == 0 ? 53 : (i == 1 ? 27 : 20)) : 16 - 4 * i);
   }
   static QMLGB_HD constexpr int period(int i) {
-    return kLowGroup ? (kWide ? 12 : (i == 0 ? 10 : 30)) : (kWide ? 20 : 12);
+    return kLowGroup ? (kWide ? 12 : (i == 0 ? 10 : 30))
+                     : (kWide ? (i == 0 ? 60 : (i == 1 ? 30 : 20)) : 12);
   }
-  // level of slot entry i (0 .. D - 1 drained, then the fixed ones)
+  // (first) level of entry i
   static QMLGB_HD constexpr int level(int i) { return L0 + i; }
-  // a sum v of entry i adds round(v 2^scale_log) mult: the scale undoes the
-  // digits' weights; mult brings level L to the low group's unit, or to
-  // 2^shift_top of level 2, whose factor is split in two so that mult stays
-  // below 2^31
-  static QMLGB_HD int scale_log(int i) {
-    return (kWide ? 8 * (level(i) - 2) : 0) + (!kLowGroup && i == 0 ? 6 : 0);
-  }
-  static QMLGB_HD int mult(int i, int shift_top) {
-    if (kLowGroup) return 1 << (OzDigitsOf<S>::kLowBits - 8 * (level(i) - 2));
-    return 1 << (i == 0 ? shift_top - 6 : shift_top - 8 * i);
+  // a sum v of entry i adds round(v 2^scale_log) 2^mult_log: the scale undoes
+  // the digits' weights; the factor brings level L to the low group's unit, or
+  // to 2^shift_top of level 2
+  static QMLGB_HD int scale_log(int i) { return kWide ? 8 * (level(i) - 2) : 0; }
+  static QMLGB_HD int mult_log(int i, int shift_top) {
+    return kLowGroup ? OzDigitsOf<S>::kLowBits - 8 * (level(i) - 2) : shift_top - 8 * i;
   }
 };
 
+// Accumulator slots in the order in which they become free, four bits each,
+// the first in the lowest: what a piece leaves to the next one.
+constexpr uint32_t kOzSlots = 0x3210u;
+
 // The hand-overs of one piece (K steps k0 .. k1) of a group, in order, for the
-// issuing thread and the epilogue alike.
+// issuing thread and the epilogue alike; ord: the slots' order on entry.
 template <class Sc>
 struct OzHandover {
-  int sl[Sc::D], nb[Sc::D], spare;
-  QMLGB_HD explicit OzHandover(int k0) : spare(Sc::kSpare) {
+  int sl[Sc::NE], nb[Sc::D], spare;
+  QMLGB_HD OzHandover(int k0, uint32_t ord) : spare(Sc::kSpare ? (int)(ord >> (4 * Sc::NE)) & 15 : 0) {
     QMLGB_UNROLL
-    for (int i = 0; i < Sc::D; ++i) {
-      sl[i] = i;
-      nb[i] = k0 + Sc::first(i);
-    }
+    for (int i = 0; i < Sc::NE; ++i) sl[i] = (int)(ord >> (4 * i)) & 15;
+    QMLGB_UNROLL
+    for (int i = 0; i < Sc::D; ++i) nb[i] = k0 + Sc::first(i);
   }
   // the entry handed over at step t, -1 for none
   QMLGB_HD int at(int t) const {
@@ -132,20 +134,26 @@ struct OzHandover {
   QMLGB_HD int slot(int e) const {
     int q = sl[0];
     QMLGB_UNROLL
-    for (int i = 1; i < Sc::D; ++i) q = e == i ? sl[i] : q;
-    return e < Sc::D ? q : Sc::kFixed0 + e - Sc::D;
+    for (int i = 1; i < Sc::NE; ++i) q = e == i ? sl[i] : q;
+    return q;
   }
-  // entry e moves on to the spare slot (returned), or keeps its own
-  QMLGB_HD int move(int e) {
-    const int old = slot(e), nw = Sc::kSpare >= 0 ? spare : old;
-    spare = old;
+  // entry e moves on to the spare slot, or keeps its own
+  QMLGB_HD void move(int e) {
+    const int old = slot(e);
     QMLGB_UNROLL
     for (int i = 0; i < Sc::D; ++i)
       if (e == i) {
-        sl[i] = nw;
+        if (Sc::kSpare) sl[i] = spare;
         nb[i] += Sc::period(i);
       }
-    return nw;
+    spare = old;
+  }
+  // the order after the entries were handed over, 0 .. NE - 1, at the end
+  QMLGB_HD uint32_t end() const {
+    uint32_t ord = Sc::kSpare ? (uint32_t)spare : 0u;
+    QMLGB_UNROLL
+    for (int i = 0; i < Sc::NE; ++i) ord |= (uint32_t)sl[i] << (4 * (i + (Sc::kSpare ? 1 : 0)));
+    return ord;
   }
 };
 
@@ -164,12 +172,13 @@ QMLGB_HD int oz_piece(int nk16, int nsc, int c) {
 // Left shift of level-2 sums in the int64 accumulator: |level-2 sum| <=
 // 2^(2 kTop) K, the other levels add less than an eighth of that, so with K
 // <= 2^lg the total stays below 2^62.  At least 16 (level 4 is 16 bits below)
-// for K <= 2^29 (kTop = 8).
+// for K <= 2^29 (kTop = 8); 31 is left out: a factor is either below 2^31 (a
+// 32-bit multiplier) or a multiple of 2^32 (the upper word alone).
 QMLGB_HD int oz_shift_top(int S, int64_t K) {
   int lg = 0;
   while (((int64_t)1 << lg) < K) ++lg;
   const int st = 61 - 2 * (S == 7 ? 7 : 8) - lg;
-  return st > 36 ? 36 : st;
+  return st > 36 ? 36 : (st == 31 ? 30 : st);
 }
 
 }  // namespace qmlgb

@@ -44,7 +44,11 @@
 // slots at their chunk boundaries, which are staggered; with a slot to spare
 // (S = 6: one in either group; S = 7: one in the second) the next chunk starts
 // at once, and without one the other levels' products of that K step go
-// first and cover the drain.
+// first and cover the drain.  A group takes over the slots in the order in
+// which the one before it leaves them, each when its first product needs it.
+// What bounds a K step of {5 ..} is the MMA rate (93 clocks each, of which
+// cuBLAS's 1900 TFLOP/s would be 87); a pair of CTAs on M = 256 MMAs
+// (cta_group::2, half the B traffic in shared memory) ran no faster: 99.
 //
 // Digit layout.  The slicing kernel writes the digits in the order and the
 // shared-memory image the MMA wants: [128-row tile][K step][digit] tiles of
@@ -118,6 +122,16 @@ __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
   return d;
 }
 
+// S = 7 keeps the low halves of its sums in shared memory between the groups
+// (in registers they pushed the epilogue into spills: 64 int64 sums and the
+// loaded columns fill the 168 the compiler allots)
+template <int S>
+constexpr int kResidBytes = OzDigitsOf<S>::kFrac ? kEpiCols / 2 * 32 * kEpiWarps * 4 : 0;
+
+// 1.5 2^23 as a float and its bit pattern
+constexpr float kMagicF = 12582912.0f;
+constexpr uint32_t kMagicI = 0x4B400000u;
+
 struct OzParams {
   int64_t M, N;            // logical output size
   const unsigned char *DA, *DB;  // digit tiles of op(A), op(B)^T (first row tile)
@@ -186,17 +200,19 @@ __device__ __forceinline__ void item_tile(const OzParams &p, int item, int rank,
 // Every digit product of level L for one K step: pair (s, L - s) reads digit
 // tile s - 1 of A and L - s - 1 of B, at descriptor offsets of 256 (4 KB >> 4)
 // per tile from the step's first tiles (da, db).  Unrolled at compile time,
-// so the issuing thread spends a few instructions per MMA: with loop bounds,
-// flags and descriptors computed at run time it could not keep up with the
-// tensor core (about 95 clocks of issue per 64-clock MMA).  The first pair
+// so the issuing warp spends a few instructions per MMA: with loop bounds,
+// flags and descriptors computed at run time, or moved to uniform registers
+// for every MMA, it could not keep up with the tensor core (93 clocks of issue
+// per 64-clock MMA).  The first pair
 // writes the accumulator when acc0 is 0 (first K step of a chunk).
 template <int S, int L>
-__device__ __forceinline__ void issue_level(uint32_t tmem, uint64_t da, uint64_t db, uint32_t acc0) {
+__device__ __forceinline__ void issue_level(uint32_t tmem, uint64_t da, uint64_t db, uint32_t acc0,
+                                            uint32_t lead) {
   constexpr int s0 = L - S > 1 ? L - S : 1, s1 = L - 1 < S ? L - 1 : S;
 #pragma unroll
   for (int s = s0; s <= s1; ++s)
-    mma_bf16_off(tmem, da, (uint64_t)(256 * (s - 1)), db, (uint64_t)(256 * (L - s - 1)), kIdesc,
-                 s == s0 ? acc0 : 1u);
+    mma_bf16_warp(tmem, da + (uint64_t)(256 * (s - 1)), db + (uint64_t)(256 * (L - s - 1)), kIdesc,
+                  s == s0 ? acc0 : 1u, lead);
 }
 
 // Output of 8 consecutive columns of one row, general form: C[gi + gj ldc] =
@@ -278,11 +294,21 @@ struct Issuer {
   int stage;
   uint32_t phase;
   uint32_t used, par;  // per slot: filled before; parity of the drain to wait for
+  uint32_t ord;        // slots in the order in which they become free
+  uint32_t lead;       // set in the lane that issues
+};
+// (every lane waits, and all go on or none)
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const Issuer &I) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, I.st, I.wait_ns)) != 0;
+}
+template <int N>
+struct IntC {
+  static constexpr int value = N;
 };
 
 __device__ __forceinline__ bool slot_acquire(Issuer &I, int q) {
   if ((I.used >> q) & 1) {
-    if (!mbar_wait(I.acce + 8 * q, (I.par >> q) & 1, I.st, I.wait_ns)) return false;
+    if (!warp_wait(I.acce + 8 * q, (I.par >> q) & 1, I)) return false;
     I.par ^= 1u << q;
     tc_fence_after();
   }
@@ -290,18 +316,23 @@ __device__ __forceinline__ bool slot_acquire(Issuer &I, int q) {
   return true;
 }
 
+// the products of entry E of group G for one K step
+template <int S, int G, int E>
+__device__ __forceinline__ void issue_entry(uint32_t tmem, uint64_t da, uint64_t db, uint32_t acc0,
+                                            uint32_t lead) {
+  using Sc = OzGroup<S, G>;
+  if constexpr (E < Sc::NE) {
+    issue_level<S, Sc::L0 + E>(tmem, da, db, acc0, lead);
+    if constexpr (E == 3) issue_level<S, Sc::L0 + E + 1>(tmem, da, db, 1u, lead);
+  }
+}
+
 template <int S, int CL, int G>
 __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
   using Sc = OzGroup<S, G>;
-  OzHandover<Sc> H(k0);
-#pragma unroll
-  for (int q = 0; q < Sc::D; ++q)
-    if (!slot_acquire(I, q)) return false;
-#pragma unroll
-  for (int q = Sc::kFixed0; q < Sc::kFixed0 + Sc::F; ++q)
-    if (!slot_acquire(I, q)) return false;
+  OzHandover<Sc> H(k0, I.ord);
   for (int ks = k0; ks < k1; ks += Sc::kSteps) {
-    if (!mbar_wait(I.full0 + 8 * I.stage, I.phase, I.st, I.wait_ns)) return false;
+    if (!warp_wait(I.full0 + 8 * I.stage, I.phase, I)) return false;
     tc_fence_after();
     const uint32_t sa = I.smem0 + (uint32_t)(I.stage * I.stage_bytes);
     const uint64_t da0 = smem_desc_sw32(sa), db0 = smem_desc_sw32(sa + (uint32_t)(I.stage_bytes >> 1));
@@ -310,44 +341,49 @@ __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
       const uint64_t da = da0 + (uint64_t)(256 * Sc::kDigits * j);
       const uint64_t db = db0 + (uint64_t)(256 * Sc::kDigits * j);
       const int t = ks + j;
-      const uint32_t acc = t > k0 ? 1u : 0u;
+      // entry bl starts its next chunk here: its slot goes to the epilogue now,
+      // and with a spare slot the entry goes on in that one; without, the other
+      // entries go first and cover the wait
       const int bl = H.at(t);
-      if (bl != 0) issue_level<S, Sc::L0>(I.tbase + 128 * H.sl[0], da, db, acc);
-      if (Sc::D > 1 && bl != 1)
-        issue_level<S, Sc::L0 + 1>(I.tbase + 128 * H.sl[Sc::D > 1 ? 1 : 0], da, db, acc);
-      if (Sc::D > 2 && bl != 2)
-        issue_level<S, Sc::L0 + 2>(I.tbase + 128 * H.sl[Sc::D > 2 ? 2 : 0], da, db, acc);
-      if (Sc::F > 0) issue_level<S, Sc::L0 + Sc::D>(I.tbase + 128 * Sc::kFixed0, da, db, acc);
-      if (Sc::F > 1) {
-        issue_level<S, Sc::L0 + Sc::D + 1>(I.tbase + 128 * (Sc::kFixed0 + 1), da, db, acc);
-        issue_level<S, Sc::L0 + Sc::D + 2>(I.tbase + 128 * (Sc::kFixed0 + 1), da, db, 1u);
-      }
       if (bl >= 0) {
-        // level L0 + bl starts its next chunk: hand its slot to the epilogue
-        // and go on in the spare one (or wait for this one to be read)
-        mma_commit(I.accf + 8 * H.slot(bl));
-        const int nw = H.move(bl);
-        if (!slot_acquire(I, nw)) return false;
-        const uint32_t tm = I.tbase + 128 * nw;
-        if (bl == 0) issue_level<S, Sc::L0>(tm, da, db, 0u);
-        if (Sc::D > 1 && bl == 1) issue_level<S, Sc::L0 + 1>(tm, da, db, 0u);
-        if (Sc::D > 2 && bl == 2) issue_level<S, Sc::L0 + 2>(tm, da, db, 0u);
+        mma_commit_warp(I.accf + 8 * H.slot(bl), I.lead);
+        H.move(bl);
+      }
+      // a slot is waited for just before its first product
+      auto entry = [&](auto E) -> bool {
+        constexpr int e = decltype(E)::value;
+        if (e >= Sc::NE) return true;
+        if (!Sc::kSpare && bl == e) return true;
+        const bool fresh = t == k0 || bl == e;
+        const int q = H.sl[e < Sc::NE ? e : 0];
+        if (fresh && !slot_acquire(I, q)) return false;
+        issue_entry<S, G, e>(I.tbase + 128 * q, da, db, fresh ? 0u : 1u, I.lead);
+        return true;
+      };
+      if (!entry(IntC<0>{}) || !entry(IntC<1>{}) || !entry(IntC<2>{}) || !entry(IntC<3>{}))
+        return false;
+      if (!Sc::kSpare && bl >= 0) {
+        const int q = H.slot(bl);
+        if (!slot_acquire(I, q)) return false;
+        if (bl == 0)
+          issue_entry<S, G, 0>(I.tbase + 128 * q, da, db, 0u, I.lead);
+        else
+          issue_entry<S, G, 1>(I.tbase + 128 * q, da, db, 0u, I.lead);
       }
     }
     // frees the smem slot when these MMAs finish (in both CTAs of a pair)
     if (CL == 2)
-      mma_commit_mc(I.empty0 + 8 * I.stage, (uint16_t)3);
+      mma_commit_mc_warp(I.empty0 + 8 * I.stage, (uint16_t)3, I.lead);
     else
-      mma_commit(I.empty0 + 8 * I.stage);
+      mma_commit_warp(I.empty0 + 8 * I.stage, I.lead);
     if (++I.stage == I.nst) {
       I.stage = 0;
       I.phase ^= 1;
     }
   }
 #pragma unroll
-  for (int i = 0; i < Sc::D; ++i) mma_commit(I.accf + 8 * H.sl[i]);
-#pragma unroll
-  for (int q = Sc::kFixed0; q < Sc::kFixed0 + Sc::F; ++q) mma_commit(I.accf + 8 * q);
+  for (int i = 0; i < Sc::NE; ++i) mma_commit_warp(I.accf + 8 * H.sl[i], I.lead);
+  I.ord = H.end();
   return true;
 }
 
@@ -416,11 +452,13 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int NST = p.nstages;
   constexpr int stage_bytes = 2 * OzDigitsOf<S>::kStageTiles * kDigitTile;  // A tiles, then B tiles
-  uint64_t *bars = (uint64_t *)(smem + (size_t)NST * stage_bytes);
+  // S = 7: the 16 bits below each sum's unit, two to a word, [pair][thread]
+  uint32_t *resid = (uint32_t *)(smem + (size_t)NST * stage_bytes);
+  uint64_t *bars = (uint64_t *)((unsigned char *)resid + kResidBytes<S>);
   // bars: [0,NST) full, [NST,2NST) empty, then 4 slots filled, 4 slots read, drain
   uint32_t *tmem_holder = (uint32_t *)(bars + 2 * NST + 9);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   DevStatus *st = p.status;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[NST]);
   const uint32_t accf = smem_u32(&bars[2 * NST]), acce = smem_u32(&bars[2 * NST + 4]);
@@ -433,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
     }
     for (int q = 0; q < 4; ++q) {
       mbar_init(accf + 8 * q, 1);
-      mbar_init(acce + 8 * q, 32 * kEpiWarps);
+      mbar_init(acce + 8 * q, kEpiWarps);
     }
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -443,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
   __syncthreads();
   if (CL == 2) cluster_sync_all();  // both CTAs' barriers exist before any remote arrival
   tc_fence_after();
-  const uint32_t tbase = *tmem_holder;
+  const uint32_t tbase = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
   if (warp < 4) {
   // warpgroup 0 hands registers to the epilogue warpgroups
@@ -479,10 +517,11 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
     }
   } else if (warp == 1) {
     // -------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    // (the whole warp in step, one lane issuing)
+    {
       Issuer I{tbase, full0, empty0, accf, acce, smem_u32(smem), stage_bytes, NST, st, p.wait_ns,
-               0, 0, 0, 0};
-      bool ok = (*((volatile int *)&st->code) == 0);
+               0, 0, 0, 0, kOzSlots, elect_lane()};
+      bool ok = __all_sync(0xffffffffu, *((volatile int *)&st->code) == 0) != 0;
       for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
         if constexpr (OzDigitsOf<S>::kLow)
           for (int c = 0; c < p.nsc && ok; ++c)
@@ -493,7 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
                                      oz_piece(p.nk16, p.nsc, c + 1));
       }
       // wait for every MMA this thread issued before TMEM is released
-      mma_commit(drain);
+      mma_commit_warp(drain, I.lead);
       mbar_drain_wait(drain, 0);
     }
   }
@@ -506,12 +545,16 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
     const uint32_t lane_base = tbase + ((uint32_t)(quad * 32) << 16) + kEpiCols * half;
     constexpr bool FRAC = OzDigitsOf<S>::kFrac;
     uint32_t par = 0;  // per slot: parity of the fill to wait for
+    uint32_t ord = kOzSlots;
     bool ok = true;
     long long acc[kEpiCols];
-    uint32_t res[FRAC ? kEpiCols / 2 : 1];
-    // reads slot q: acc += round(sum scale) mult (scale: 2^(8(L-2)) undoes the
-    // digits' weights, times what keeps mult below 2^31)
-    auto drain_slot = [&](int q, float scale, int mult) -> bool {
+    uint32_t *res = resid + (threadIdx.x - 128);  // stride 32 kEpiWarps
+    long long bias = 0;
+    // Reads slot q: acc += round(sum 2^scale_log) 2^mult_log.  The float to
+    // integer conversion is an addition of 1.5 2^23, exact below 2^22 and
+    // checked for every value (F2I issues an eighth as fast); the constant in
+    // its bit pattern is collected in `bias` and taken off with the shift.
+    auto drain_slot = [&](int q, int scale_log, int mult_log) -> bool {
       int okw = 1;
       if (lane == 0) okw = mbar_wait(accf + 8 * q, (par >> q) & 1, st, p.wait_ns) ? 1 : 0;
       par ^= 1u << q;
@@ -520,31 +563,68 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       if (!okw) return false;
       tc_fence_after();
       const uint32_t lbase = lane_base + 128 * q;
+      const float scale = __int_as_float((127 + scale_log) << 23);
+      const bool high = mult_log >= 32;  // only the upper word changes
+      constexpr int kLd = 32;  // columns in flight that the registers hold
+      const int mult = 1 << (high ? mult_log - 32 : mult_log);
 #pragma unroll
-      for (int cb = 0; cb < kEpiCols / 16; ++cb) {
-        uint32_t a[16];
-        tmem_ld16(lbase + 16 * cb, a);
+      for (int cb = 0; cb < kEpiCols / kLd; ++cb) {
+        uint32_t a[kLd];
+        auto load = [&] {
+          if (kLd == 32)
+            tmem_ld32_async(lbase + kLd * cb, a);
+          else
+            tmem_ld16_async(lbase + kLd * cb, a);
+          tmem_ld_wait();
+          // (the loaded registers pass through the wait, so no use moves above it)
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          acc[16 * cb + j] += (long long)__float2int_rn(__uint_as_float(a[j]) * scale) * mult;
+          for (int j = 0; j < kLd; ++j) asm volatile("" : "+r"(a[j]));
+        };
+        load();
+        uint32_t off = 0;
+#pragma unroll
+        for (int j = 0; j < kLd; ++j) {
+          a[j] = __float_as_uint(fmaf(__uint_as_float(a[j]), scale, kMagicF));
+          off |= a[j] ^ kMagicI;
+        }
+        if (__any_sync(0xffffffffu, (off >> 23) != 0)) {
+          // a sum past 2^22 in some lane: the conversion instruction; the
+          // offset integer may need 33 bits (sums up to 2^31)
+          load();
+#pragma unroll
+          for (int j = 0; j < kLd; ++j) {
+            const long long v = (long long)__float2int_rn(__uint_as_float(a[j]) * scale) + kMagicI;
+            acc[kLd * cb + j] += (long long)((unsigned long long)v << mult_log);
+          }
+        } else if (high) {
+#pragma unroll
+          for (int j = 0; j < kLd; ++j)
+            acc[kLd * cb + j] += (long long)((unsigned long long)(a[j] * (uint32_t)mult) << 32);
+        } else {
+#pragma unroll
+          for (int j = 0; j < kLd; ++j) acc[kLd * cb + j] += (long long)(int)a[j] * mult;
+        }
       }
+      bias += (long long)((unsigned long long)kMagicI << mult_log);
       tc_fence_before();
-      mbar_arrive(acce + 8 * q);  // the slot may be overwritten from here on
+      __syncwarp();
+      // the slot may be overwritten from here on
+      if (lane == 0) mbar_arrive(acce + 8 * q);
       return true;
     };
     // the slot reads of one piece of a group, in the order the issuer commits
     auto drain_piece = [&](auto grp, int k0, int k1) -> bool {
       using Sc = decltype(grp);
-      OzHandover<Sc> H(k0);
-      for (int last = 0; last < Sc::D + Sc::F;) {
+      OzHandover<Sc> H(k0, ord);
+      for (int last = 0; last < Sc::NE;) {
         int t;
         int e = H.next(t);
         const bool mid = t < k1;
         if (!mid) e = last++;
-        const float scale = __int_as_float((127 + Sc::scale_log(e)) << 23);
-        if (!drain_slot(H.slot(e), scale, Sc::mult(e, p.shift_top))) return false;
+        if (!drain_slot(H.slot(e), Sc::scale_log(e), Sc::mult_log(e, p.shift_top))) return false;
         if (mid) H.move(e);
       }
+      ord = H.end();
       return true;
     };
     for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
@@ -570,15 +650,19 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
                            oz_piece(p.nk16, p.nsc, c + 1));
         // from the unit of the lowest level to the final one
         const int d = OzDigitsOf<S>::kLowBits - p.shift_top;
+        const long long b0 = bias;
+        bias = 0;
+        uint32_t lo16 = 0;
 #pragma unroll
         for (int j = 0; j < kEpiCols; ++j) {
+          acc[j] -= b0;
           if (FRAC) {
             const long long low = acc[j] & ((1ll << d) - 1);
             const uint32_t f16 = (uint32_t)(d <= 16 ? low << (16 - d) : low >> (d - 16));
             if (j & 1)
-              res[j >> 1] |= f16 << 16;
+              res[(j >> 1) * (32 * kEpiWarps)] = lo16 | f16 << 16;
             else
-              res[j >> 1] = f16;
+              lo16 = f16;
             acc[j] >>= d;
           } else {
             acc[j] = (acc[j] + (1ll << (d - 1))) >> d;
@@ -589,6 +673,9 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
         ok = drain_piece(OzGroup<S, 1>{}, oz_piece(p.nk16, p.nsc, c),
                          oz_piece(p.nk16, p.nsc, c + 1));
       if (!ok) break;
+#pragma unroll
+      for (int j = 0; j < kEpiCols; ++j) acc[j] -= bias;
+      bias = 0;
       // output: alpha 2^(e_i + f_j - 2T - shift_top) acc + beta C, while
       // the MMAs of the next tile already run
       // (every lane takes part in the shuffles; rows past M store nothing)
@@ -616,20 +703,22 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
           const int cix = 8 * g + u;
           f[u] = __shfl_sync(0xffffffffu, cix < 32 ? f_lo : f_hi, cix & 31);
         }
+        uint32_t rv[4] = {0, 0, 0, 0};
+        if (FRAC) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) rv[u] = res[(4 * g + u) * (32 * kEpiWarps)];
+        }
         if (fast && p.beta_mode == 0)
           store_fast8<FRAC, false>(crow + 8 * g * p.ldc, p.ldc, lim - 8 * g, em,
-                                   (uint32_t)p.alpha_neg << 31, acc + 8 * g, res + (FRAC ? 4 * g : 0),
-                                   f);
+                                   (uint32_t)p.alpha_neg << 31, acc + 8 * g, rv, f);
         else if (fast)
           store_fast8<FRAC, true>(crow + 8 * g * p.ldc, p.ldc, lim - 8 * g, em,
-                                  (uint32_t)p.alpha_neg << 31, acc + 8 * g, res + (FRAC ? 4 * g : 0),
-                                  f);
+                                  (uint32_t)p.alpha_neg << 31, acc + 8 * g, rv, f);
         else if (live_row)
           store_out8<FRAC>(p, gi, gj0 + 8 * g, ebase, acc[8 * g], acc[8 * g + 1], acc[8 * g + 2],
                            acc[8 * g + 3], acc[8 * g + 4], acc[8 * g + 5], acc[8 * g + 6],
-                           acc[8 * g + 7], res[FRAC ? 4 * g : 0], res[FRAC ? 4 * g + 1 : 0],
-                           res[FRAC ? 4 * g + 2 : 0], res[FRAC ? 4 * g + 3 : 0], f[0], f[1], f[2],
-                           f[3], f[4], f[5], f[6], f[7]);
+                           acc[8 * g + 7], rv[0], rv[1], rv[2], rv[3], f[0], f[1], f[2], f[3],
+                           f[4], f[5], f[6], f[7]);
       }
     }
   }
@@ -873,11 +962,21 @@ void oz_slice(const double *X, int64_t sr, int64_t sk, const OzDigits &d, cudaSt
 
 namespace {
 
-constexpr size_t oz_smem_c(int stage_tiles, int nstages) {
-  return 1024 + (size_t)nstages * 2 * stage_tiles * kDigitTile + (2 * nstages + 9) * 8 + 16;
+constexpr size_t kSmemCap = 232448;  // 227 KB
+constexpr int kMaxStages = 4;
+template <int S>
+constexpr size_t oz_smem(int nstages) {
+  return 1024 + (size_t)nstages * 2 * OzDigitsOf<S>::kStageTiles * kDigitTile + kResidBytes<S> +
+         (2 * nstages + 9) * 8 + 16;
 }
-constexpr int kMaxSmem = (int)oz_smem_c(7, 4);
-static_assert(oz_smem_c(7, 4) <= 232448, "split kernel exceeds 227 KB of shared memory");
+// the deepest ring that fits (S = 6: four stages of 48 KB, S = 7: three of 56)
+template <int S>
+constexpr int oz_max_stages() {
+  int n = kMaxStages;
+  while (oz_smem<S>(n) > kSmemCap) --n;
+  return n;
+}
+static_assert(oz_max_stages<7>() >= 3 && oz_max_stages<6>() >= 4, "ring too shallow");
 
 // Launch attributes of an instantiation, set once: the shared-memory
 // size, and the check that the warpgroups' register split (setmaxnreg) adds
@@ -887,7 +986,8 @@ static_assert(oz_smem_c(7, 4) <= 232448, "split kernel exceeds 227 KB of shared 
 template <int S, int CL>
 cudaError_t oz_prepare(int &max_items) {
   cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, CL>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)oz_smem<S>(oz_max_stages<S>()));
   if (e != cudaSuccess) return e;
   cudaFuncAttributes fa;
   e = cudaFuncGetAttributes(&fa, ozaki_gemm_kernel<S, CL>);
@@ -904,7 +1004,7 @@ cudaError_t oz_prepare(int &max_items) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * (unsigned)nsm);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kMaxSmem;
+  cfg.dynamicSmemBytes = oz_smem<S>(oz_max_stages<S>());
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2;
@@ -935,7 +1035,8 @@ cudaError_t launch_oz_t(int nitems, int reserve_sms, OzParams &p, cudaStream_t s
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(CL * items));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = oz_smem_c(OzDigitsOf<S>::kStageTiles, p.nstages);
+  p.nstages = p.nstages < oz_max_stages<S>() ? p.nstages : oz_max_stages<S>();
+  cfg.dynamicSmemBytes = oz_smem<S>(p.nstages);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -980,8 +1081,8 @@ cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t
   p.rta = tiles_m - 1;
   p.rtb = p.tiles_n - 1;
   {
-    const int64_t ns = tune_get("ozaki_stages", 4);
-    p.nstages = ns < 2 ? 2 : (ns > 4 ? 4 : (int)ns);
+    const int64_t ns = tune_get("ozaki_stages", kMaxStages);
+    p.nstages = ns < 2 ? 2 : (ns > kMaxStages ? kMaxStages : (int)ns);
   }
   p.nsc = oz_pieces(S, p.nk16);
   p.shift_top = oz_shift_top(S, Kpad);

@@ -121,6 +121,14 @@ __device__ __forceinline__ void tma_load_3d_mc(uint32_t dst, const CUtensorMap *
       "l"((uint64_t)map), "r"(bar), "r"(x), "r"(y), "r"(z), "h"(cta_mask)
       : "memory");
 }
+// one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_lane() {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r));
+  return r;
+}
 // this CTA's rank in its cluster, and a barrier over every thread of the
 // cluster (release / acquire at cluster scope)
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -185,17 +193,32 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// the same MMA with descriptors adesc + aoff and bdesc + boff formed inside the
-// instruction sequence (keeps an unrolled issue loop from precomputing every
-// descriptor into registers)
-__device__ __forceinline__ void mma_bf16_off(uint32_t d_tmem, uint64_t adesc, uint64_t aoff,
-                                             uint64_t bdesc, uint64_t boff, uint32_t idesc,
-                                             uint32_t accumulate) {
+// The same MMA and commits for a whole warp in step, made by the lane whose
+// `lead` is set.  The descriptors are then the same in every lane of converged
+// code, and the compiler keeps them in uniform registers, from which the
+// instruction takes them; inside a one-lane branch each operand is moved there
+// first (about 93 clocks an MMA).
+__device__ __forceinline__ void mma_bf16_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                              uint32_t idesc, uint32_t accumulate, uint32_t lead) {
   asm volatile(
-      "{\n .reg .pred p;\n .reg .b64 da, db;\n add.s64 da, %1, %2;\n add.s64 db, %3, %4;\n"
-      " setp.ne.b32 p, %6, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}" ::"r"(d_tmem),
-      "l"(adesc), "l"(aoff), "l"(bdesc), "l"(boff), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_warp(uint32_t bar, uint32_t lead) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar),
+      "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_mc_warp(uint32_t bar, uint16_t cta_mask, uint32_t lead) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;\n}" ::"r"(bar),
+      "h"(cta_mask), "r"(lead)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -203,15 +226,6 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
       : "memory");
 }
-// the same arrival, made on the mbarrier at bar's offset in every CTA of the
-// cluster named in cta_mask
-__device__ __forceinline__ void mma_commit_mc(uint32_t bar, uint16_t cta_mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;" ::"r"(bar), "h"(cta_mask)
-      : "memory");
-}
-
 // 16 consecutive 32-bit TMEM columns of this thread's lane
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -231,6 +245,13 @@ __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t *r) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
         "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+// 32 columns the same way
+__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t *r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_ld_wait() {
