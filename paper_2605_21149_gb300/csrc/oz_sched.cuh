@@ -24,9 +24,9 @@
 namespace qmlgb {
 
 // S digits of 8 bits, the top one |a_1| <= 2^kTop, kBits = 8 (S - 1) + kTop
-// bits in all; levels 2 .. kLMax.  kLow: the levels above 4 exist.  kFrac: the
-// output keeps 16 bits below its int64 unit, and digit s carries the weight
-// 2^(-8 (s - 1)) so that two levels can share an accumulator.  kLowBits: the
+// bits in all; levels 2 .. kLMax.  kLow: the levels above 4 exist; the last two then
+// share an accumulator, for which digit s carries the weight 2^(-8 (s - 1)).
+// kFrac: the output keeps 16 bits below its int64 unit.  kLowBits: the
 // low group's unit is level 2's divided by 2^kLowBits.  kStageTiles: digit
 // tiles per operand in a ring stage (a K step of the low group, or two K steps
 // of three digits).
@@ -49,20 +49,21 @@ struct OzDigitsOf<7> {
 };
 
 // Group G of variant S (0: levels 5 and up, 1: levels 2..4).  Its levels are
-// its entries 0 .. NE - 1 (S = 7: levels 8 and 9 share the last entry of group
-// 0), each in one accumulator slot of the four.  The first D are drained: entry
-// i after first(i) K steps of a piece and every period(i) from there on, never
-// two at one step.  With a slot to spare (NE < 4) the entry goes on in that
-// one; otherwise it waits for its own.  The others are drained at the end of
-// the piece only.
+// its entries 0 .. NE - 1 (the last entry of group 0 holds its last two
+// levels), each in one accumulator slot of the four.  The first D are drained:
+// entry i after first(i) K steps of a piece and every period(i) from there on,
+// never two at one step.  With slots to spare (NE < 4) the entry goes on in the
+// one free longest; otherwise it waits for its own.  The others are drained at
+// the end of the piece only.
 //
 // The longest exact chunk, |sum| <= 2^24, from |a_1| <= 2^kTop, |a_s| <= 2^7:
 //   kTop = 8: levels 2, 3: 2^16 an element (256 elements, 16 steps), level 4:
 //             + 2^14 (204), level 5: + 2^14 (170);
 //   kTop = 7: level L: (L - 1) 2^14 (level 4: 341 elements, 5: 256, 6: 204).
-// Level 6 of the 48-bit variant runs for 30 steps: a sum past 2^24 (digits
-// that all agree in sign) then loses at most 2^2 a product at its weight of
-// 2^-48, 2^-47.7 K of the maxima in all, no more than the dropped level 8.
+// Level 6 of the 48-bit variant, with level 7, runs for 30 steps: a sum past
+// 2^24 (digits that all agree in sign) then loses at most 2^2 a product at its
+// weight of 2^-48, 2^-47.7 K of the maxima in all, no more than the dropped
+// level 8.
 // The first hand-overs come late because the epilogue is still writing the
 // last tile then (14 us beside 0.8 us a K step; with level 6 drained every 9
 // steps from the 4th on, a 6400 x 6400 x 512 update took 0.585 ms), and those
@@ -74,8 +75,9 @@ struct OzGroup {
   static constexpr bool kWide = S == 7;
   static constexpr int L0 = kLowGroup ? 5 : 2;
   static constexpr int D = kLowGroup ? 2 : 3;
-  static constexpr int NE = kLowGroup && kWide ? 4 : 3;
-  static constexpr bool kSpare = NE < 4;
+  static constexpr int NE = kLowGroup ? (kWide ? 4 : 2) : 3;
+  static constexpr int NS = 4 - NE;  // slots to spare
+  static constexpr bool kSpare = NS > 0;
   static constexpr int kDigits = kLowGroup ? S : 3;
   static constexpr int kSteps = kLowGroup ? 1 : 2;  // K steps per ring stage
   static QMLGB_HD constexpr int first(int i) {
@@ -91,7 +93,7 @@ struct OzGroup {
   // a sum v of entry i adds round(v 2^scale_log) 2^mult_log: the scale undoes
   // the digits' weights; the factor brings level L to the low group's unit, or
   // to 2^shift_top of level 2
-  static QMLGB_HD int scale_log(int i) { return kWide ? 8 * (level(i) - 2) : 0; }
+  static QMLGB_HD int scale_log(int i) { return OzDigitsOf<S>::kLow ? 8 * (level(i) - 2) : 0; }
   static QMLGB_HD int mult_log(int i, int shift_top) {
     return kLowGroup ? OzDigitsOf<S>::kLowBits - 8 * (level(i) - 2) : shift_top - 8 * i;
   }
@@ -105,8 +107,9 @@ constexpr uint32_t kOzSlots = 0x3210u;
 // issuing thread and the epilogue alike; ord: the slots' order on entry.
 template <class Sc>
 struct OzHandover {
-  int sl[Sc::NE], nb[Sc::D], spare;
-  QMLGB_HD OzHandover(int k0, uint32_t ord) : spare(Sc::kSpare ? (int)(ord >> (4 * Sc::NE)) & 15 : 0) {
+  int sl[Sc::NE], nb[Sc::D];
+  uint32_t spare;  // NS slots, the one free longest in the lowest four bits
+  QMLGB_HD OzHandover(int k0, uint32_t ord) : spare(ord >> (4 * Sc::NE)) {
     QMLGB_UNROLL
     for (int i = 0; i < Sc::NE; ++i) sl[i] = (int)(ord >> (4 * i)) & 15;
     QMLGB_UNROLL
@@ -143,16 +146,16 @@ struct OzHandover {
     QMLGB_UNROLL
     for (int i = 0; i < Sc::D; ++i)
       if (e == i) {
-        if (Sc::kSpare) sl[i] = spare;
+        if (Sc::kSpare) sl[i] = (int)(spare & 15u);
         nb[i] += Sc::period(i);
       }
-    spare = old;
+    if (Sc::kSpare) spare = (spare >> 4) | (uint32_t)old << (4 * (Sc::kSpare ? Sc::NS - 1 : 0));
   }
   // the order after the entries were handed over, 0 .. NE - 1, at the end
   QMLGB_HD uint32_t end() const {
-    uint32_t ord = Sc::kSpare ? (uint32_t)spare : 0u;
+    uint32_t ord = spare;
     QMLGB_UNROLL
-    for (int i = 0; i < Sc::NE; ++i) ord |= (uint32_t)sl[i] << (4 * (i + (Sc::kSpare ? 1 : 0)));
+    for (int i = 0; i < Sc::NE; ++i) ord |= (uint32_t)sl[i] << (4 * (i + Sc::NS));
     return ord;
   }
 };

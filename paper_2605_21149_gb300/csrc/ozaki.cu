@@ -19,9 +19,9 @@
 // up exactly in an FP32 TMEM accumulator as long as the sum stays below 2^24:
 // whatever the tensor core's order or rounding.  Levels 2..6, whose last bits
 // matter, are therefore read out ("drained") every chunk of K that cannot
-// exceed that bound (oz_sched.cuh); the levels below (7, and 8 with 9 in one
-// accumulator) carry weights of 2^-40 and less, where FP32 accumulation over
-// all of K costs less than the dropped levels, and are read once.
+// exceed that bound (oz_sched.cuh); the levels below (S = 6: 7, in level 6's
+// accumulator; S = 7: 7, and 8 with 9 in one accumulator) carry weights of 2^-40
+// and less, where FP32 rounding costs less than the dropped levels.
 // Why 8-bit digits: 6-bit digits allow chunks of 1536 elements but need 36
 // products for 48 bits; 8-bit digits need 21 and pay for it with a drain
 // every 160..512 elements, which the epilogue warps do beside the MMAs.
@@ -42,8 +42,8 @@
 // loads each digit tile the group needs once and runs all of its products.
 // TMEM holds four 128-column accumulators (slots).  Drained levels change
 // slots at their chunk boundaries, which are staggered; with a slot to spare
-// (S = 6: one in either group; S = 7: one in the second) the next chunk starts
-// at once, and without one the other levels' products of that K step go
+// (S = 6: two in the first group, one in the second; S = 7: one in the second)
+// the next chunk starts at once, and without one the other levels' products of that K step go
 // first and cover the drain.  A group takes over the slots in the order in
 // which the one before it leaves them, each when its first product needs it.
 // What bounds a K step of {5 ..} is the MMA rate (93 clocks each, of which
@@ -264,20 +264,27 @@ __device__ __noinline__ void store_out8(const OzParams &p, int64_t gi, int64_t g
 // output).  Here the conversion is integer throughout (normal_double_bits)
 // and beta = 1 costs the one addition it needs.
 // Columns 8 g .. 8 g + 7: c points at the first, lim is the number of live
-// columns from there on.
+// columns from there on; fNM: two column exponents, 16 bits each; c0 .. c7: the
+// entries of C for ADD, read by the caller a group ahead.  Not inlined: the 8
+// calls of a tile share one copy of the code (about 45 instructions an output;
+// 64 copies of it did not stay in the instruction cache).
 template <bool FRAC, bool ADD>
-__device__ __forceinline__ void store_fast8(double *c, int64_t ldc, int lim, int E0, uint32_t sflip,
-                                            const long long *av, const uint32_t *rv,
-                                            const int *fv) {
-  double cv[8];
-  if (ADD) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) cv[u] = u < lim ? c[u * ldc] : 0.0;
-  }
+__device__ __noinline__ void store_fast8(double *c, int64_t ldc, int lim, int E0, uint32_t sflip,
+                                         long long a0, long long a1, long long a2, long long a3,
+                                         long long a4, long long a5, long long a6, long long a7,
+                                         uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3,
+                                         uint32_t f01, uint32_t f23, uint32_t f45, uint32_t f67,
+                                         double c0, double c1, double c2, double c3, double c4,
+                                         double c5, double c6, double c7) {
+  const long long av[8] = {a0, a1, a2, a3, a4, a5, a6, a7};
+  const uint32_t rv[4] = {r0, r1, r2, r3};
+  const uint32_t fv[4] = {f01, f23, f45, f67};
+  const double cv[8] = {c0, c1, c2, c3, c4, c5, c6, c7};
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const uint32_t fr = FRAC ? (u & 1 ? rv[u >> 1] >> 16 : rv[u >> 1] & 0xFFFFu) : 0u;
-    const uint64_t bits = normal_double_bits<FRAC>(av[u], fr, E0 + fv[u], sflip);
+    const int f = u & 1 ? (int)fv[u >> 1] >> 16 : (int)(short)fv[u >> 1];
+    const uint64_t bits = normal_double_bits<FRAC>(av[u], fr, E0 + f, sflip);
     double v = __longlong_as_double((long long)bits);
     if (ADD) v += cv[u];
     if (u < lim) c[u * ldc] = v;
@@ -323,7 +330,8 @@ __device__ __forceinline__ void issue_entry(uint32_t tmem, uint64_t da, uint64_t
   using Sc = OzGroup<S, G>;
   if constexpr (E < Sc::NE) {
     issue_level<S, Sc::L0 + E>(tmem, da, db, acc0, lead);
-    if constexpr (E == 3) issue_level<S, Sc::L0 + E + 1>(tmem, da, db, 1u, lead);
+    if constexpr (Sc::kLowGroup && E == Sc::NE - 1)
+      issue_level<S, Sc::L0 + E + 1>(tmem, da, db, 1u, lead);
   }
 }
 
@@ -695,8 +703,19 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       int64_t lim64 = (p.lower && gi + 1 < p.N ? gi + 1 : p.N) - gj0;
       const int lim = live_row ? (int)(lim64 < 0 ? 0 : (lim64 > kEpiCols ? kEpiCols : lim64)) : 0;
       double *crow = p.C + gi + gj0 * p.ldc;
+      const bool add = fast && p.beta_mode == 1;
+      double cv[8], cn[8];
+      auto load_c = [&](int g) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          cn[u] = add && 8 * g + u < lim ? crow[(8 * g + u) * p.ldc] : 0.0;
+      };
+      load_c(0);
 #pragma unroll
       for (int g = 0; g < kEpiCols / 8; ++g) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) cv[u] = cn[u];
+        if (g + 1 < kEpiCols / 8) load_c(g + 1);  // in flight while this group is converted
         int f[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -708,17 +727,27 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
 #pragma unroll
           for (int u = 0; u < 4; ++u) rv[u] = res[(4 * g + u) * (32 * kEpiWarps)];
         }
-        if (fast && p.beta_mode == 0)
-          store_fast8<FRAC, false>(crow + 8 * g * p.ldc, p.ldc, lim - 8 * g, em,
-                                   (uint32_t)p.alpha_neg << 31, acc + 8 * g, rv, f);
-        else if (fast)
-          store_fast8<FRAC, true>(crow + 8 * g * p.ldc, p.ldc, lim - 8 * g, em,
-                                  (uint32_t)p.alpha_neg << 31, acc + 8 * g, rv, f);
-        else if (live_row)
-          store_out8<FRAC>(p, gi, gj0 + 8 * g, ebase, acc[8 * g], acc[8 * g + 1], acc[8 * g + 2],
-                           acc[8 * g + 3], acc[8 * g + 4], acc[8 * g + 5], acc[8 * g + 6],
-                           acc[8 * g + 7], rv[0], rv[1], rv[2], rv[3], f[0], f[1], f[2], f[3],
-                           f[4], f[5], f[6], f[7]);
+        const long long *av = acc + 8 * g;
+        if (fast) {
+          uint32_t fp[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) fp[u] = __byte_perm(f[2 * u], f[2 * u + 1], 0x5410);
+          if (add)
+            store_fast8<FRAC, true>(crow + 8 * g * p.ldc, p.ldc, lim - 8 * g, em,
+                                    (uint32_t)p.alpha_neg << 31, av[0], av[1], av[2], av[3], av[4],
+                                    av[5], av[6], av[7], rv[0], rv[1], rv[2], rv[3], fp[0], fp[1],
+                                    fp[2], fp[3], cv[0], cv[1], cv[2], cv[3], cv[4], cv[5], cv[6],
+                                    cv[7]);
+          else
+            store_fast8<FRAC, false>(crow + 8 * g * p.ldc, p.ldc, lim - 8 * g, em,
+                                     (uint32_t)p.alpha_neg << 31, av[0], av[1], av[2], av[3], av[4],
+                                     av[5], av[6], av[7], rv[0], rv[1], rv[2], rv[3], fp[0], fp[1],
+                                     fp[2], fp[3], 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0);
+        } else if (live_row) {
+          store_out8<FRAC>(p, gi, gj0 + 8 * g, ebase, av[0], av[1], av[2], av[3], av[4], av[5], av[6],
+                           av[7], rv[0], rv[1], rv[2], rv[3], f[0], f[1], f[2], f[3], f[4], f[5],
+                           f[6], f[7]);
+        }
       }
     }
   }
@@ -819,8 +848,8 @@ __device__ __forceinline__ long long scaled_round(double x, int sh) {
 // F = round(x 2^(bits - e)) + sum_i 2^7 2^(8 i) over the S - 1 low digits:
 // byte i of F, less 128, is the signed digit S - i, and what is above the
 // bytes is digit 1.  A byte becomes a float through the bit pattern of
-// 2^23 + byte.  Digit s carries the weight 2^(-8 (s - 1)) when two levels
-// share an accumulator (S = 7), else 1.
+// 2^23 + byte.  Digit s carries the weight 2^(-8 (s - 1)), for the two
+// levels that share an accumulator.
 template <int S>
 __global__ void __launch_bounds__(256) slice_kernel(const double *X, int64_t R, int64_t K,
                                                     int64_t sr, int64_t sk,
@@ -844,7 +873,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const double *X, int64_t R, 
 #pragma unroll
   for (int s = 0; s < S; ++s) {
     // (floats with exponents down to 2^-48: exact, and exact in bf16)
-    const float w = Dg::kFrac ? __int_as_float((127 - 8 * s) << 23) : 1.0f;
+    const float w = Dg::kLow ? __int_as_float((127 - 8 * s) << 23) : 1.0f;
     uint32_t o[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -859,7 +888,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const double *X, int64_t R, 
           const uint32_t byte = (uint32_t)(v >> (sh & 32)) >> (sh & 31) & 0xFFu;
           f[h] = __uint_as_float(0x4B000000u | byte) - 8388736.0f;  // 2^23 + 128
         }
-        if (Dg::kFrac) f[h] *= w;
+        if (Dg::kLow) f[h] *= w;
       }
       const __nv_bfloat162 b2 = __floats2bfloat162_rn(f[0], f[1]);
       o[j] = *(const uint32_t *)&b2;

@@ -45,7 +45,8 @@ static int check(int k0, int k1, uint32_t &ord_issue, uint32_t &ord_epi) {
       H.move(e);
     }
     // distinct slots, the spare one among them
-    unsigned seen = Sc::kSpare ? 1u << H.spare : 0u;
+    unsigned seen = 0;
+    for (int i = 0; i < Sc::NS; ++i) seen |= 1u << ((H.spare >> (4 * i)) & 15u);
     for (int i = 0; i < Sc::NE; ++i) seen |= 1u << H.sl[i];
     if (seen != 15u) return std::printf("FAIL slots S=%d G=%d t=%d\n", S, G, t), 1;
   }
@@ -69,8 +70,8 @@ static int check(int k0, int k1, uint32_t &ord_issue, uint32_t &ord_epi) {
       return std::printf("FAIL order S=%d G=%d %d..%d event %zu\n", S, G, k0, k1, i), 1;
     const bool drained = a[i].entry < Sc::D;
     double m = 16.0 * a[i].steps * per_element<S, G>(Sc::level(a[i].entry));
-    // the two lowest levels share the last entry of the wide variant
-    if (a[i].entry == 3)
+    // the two lowest levels share the last entry of the low group
+    if (G == 0 && a[i].entry == Sc::NE - 1)
       m += 16.0 * a[i].steps * per_element<S, G>(Sc::level(a[i].entry) + 1) / 256.0;
     // (level 6 of the 48-bit variant may pass 2^24, see oz_sched.cuh)
     const bool loose = S == 6 && Sc::level(a[i].entry) == 6;
