@@ -879,6 +879,157 @@ __global__ void vbuild_kernel(const double2 *cs, const int *rounds, int n, doubl
   for (int j = threadIdx.x; j < n; j += blockDim.x) V[row + (size_t)j * n] = vrow[j];
 }
 
+// Small matrices (padded order n <= kSmallN): every sweep in one CTA, the
+// matrix in shared memory.  The grid-wide kernel above spends 7 us a round on
+// its barrier whatever n is (n = 16: 105 rounds, 0.8 ms of a 2.6 ms analysis);
+// here a round is two block barriers around float64 issue: a thread per 2 x 2
+// block applies the round's rotations (16 float64 instructions, in place: no
+// other thread reads its entries), then one warp forms the next round's from
+// the updated entries.  Only the rotations are kept; V is built from them by
+// vbuild_kernel, one CTA a row.  Same schedule, update and stopping rule.
+constexpr int kSmallN = 62, kSmallSweeps = 30, kSmallThreads = 512;
+static_assert((kSmallN / 2) * (kSmallN / 2 + 1) / 2 <= kSmallThreads, "one thread per block");
+
+// x 2^(1022 - e) as a float, truncated (0 when tiny), from the bits of x; e: the
+// larger biased exponent of the pair, so the result is below 1
+__device__ __forceinline__ float scaled_float(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int fe = (int)((b >> 52) & 0x7FF) - e + 126;
+  const uint32_t sg = (uint32_t)(b >> 32) & 0x80000000u;
+  return __uint_as_float(fe <= 0 ? sg : sg | (uint32_t)fe << 23 | ((uint32_t)(b >> 29) & 0x7FFFFFu));
+}
+// a normal float as a double, from its bits
+__device__ __forceinline__ double widened(float f) {
+  const uint32_t b = __float_as_uint(f);
+  if ((b & 0x7F800000u) == 0) return 0.0;
+  const unsigned long long e = ((b >> 23) & 0xFFu) + 896u;
+  return __longlong_as_double((long long)((unsigned long long)(b & 0x80000000u) << 32 | e << 52 |
+                                          (unsigned long long)(b & 0x7FFFFFu) << 29));
+}
+// rotation() with eight float64 instructions: the float32 inputs and the
+// conversions by integer operations, 1 / (1 + tau^2) from a float32 quotient
+// w0 and the cubic step w0 (1 + e + e^2), e = 1 - (1 + tau^2) w0 (|e| below
+// 2^-22: an error of e^3).  Entries that are not ordinary numbers take the
+// general form.
+__device__ __forceinline__ double2 rotation_lean(double app, double aqq, double apq) {
+  const double d = aqq - app;
+  const long long bd = __double_as_longlong(d), bt = __double_as_longlong(apq);
+  const int ed = (int)((bd >> 52) & 0x7FF), et = (int)((bt >> 52) & 0x7FF) + 1;  // of 2 a_pq
+  if ((bt << 1) == 0) return make_double2(1.0, 0.0);
+  const int e = ed > et ? ed : et;
+  if (ed >= 0x7FE || et >= 0x7FE || et <= 1 || e < 2) {
+    double o[2];
+    rotation(app, aqq, apq, o);
+    return make_double2(o[0], o[1]);
+  }
+  const float ds = scaled_float(d, e), ts = scaled_float(apq, e - 1);
+  const float r = sqrtf(fmaf(ds, ds, ts * ts));
+  const float t = __fdividef(ds >= 0.0f ? ts : -ts, fabsf(ds) + r);
+  const float tau = __fdividef(t, 1.0f + sqrtf(fmaf(t, t, 1.0f)));
+  const double tv = widened(tau);
+  const double t2 = tv * tv, x = 1.0 + t2;
+  const double w0 = widened(__fdividef(1.0f, fmaf(tau, tau, 1.0f)));
+  const double er = fma(-x, w0, 1.0);
+  const double w = fma(w0, fma(er, er, er), w0);
+  return make_double2(fma(-t2, w, w), widened(2.0f * tau) * w);
+}
+
+__global__ void __launch_bounds__(kSmallThreads) jacobi_small_kernel(double *A, int n, double2 *cs,
+                                                                     int *rounds_out) {
+  __shared__ double m[kSmallN][kSmallN + 1];
+  __shared__ double2 rot[kSmallN / 2];
+  __shared__ double red[2][kSmallThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, h = n / 2;
+  for (int t = tid; t < n * n; t += kSmallThreads) m[t % n][t / n] = A[t];
+  // this thread's block: pairs bb <= a
+  int a = (int)((sqrtf(8.0f * (float)tid + 1.0f) - 1.0f) * 0.5f);
+  while ((a + 1) * (a + 2) / 2 <= tid) ++a;
+  while (a * (a + 1) / 2 > tid) --a;
+  const int bb = tid - a * (a + 1) / 2;
+  const bool mine = a < h;
+  auto at = [&](int x, int r) {  // player(x, r, n) for r < n - 1
+    int t = x - 1 + r;
+    if (t >= n - 1) t -= n - 1;
+    return x == 0 ? 0 : t + 1;
+  };
+  int g = 0;
+  double prev = 0.0;
+  __syncthreads();
+  for (int sweep = 0; sweep < kSmallSweeps; ++sweep) {
+    double off = 0.0, dia = 0.0;
+    for (int t = tid; t < n * n; t += kSmallThreads) {
+      const double v = m[t % n][t / n];
+      if (t % n == t / n)
+        dia = fma(v, v, dia);
+      else
+        off = fma(v, v, off);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      dia += __shfl_xor_sync(0xffffffffu, dia, o);
+    }
+    if (lane == 0) {
+      red[0][warp] = off;
+      red[1][warp] = dia;
+    }
+    __syncthreads();
+    double to = 0.0, td = 0.0;
+    for (int w = 0; w < kSmallThreads / 32; ++w) {
+      to += red[0][w];
+      td += red[1][w];
+    }
+    if (to <= 0x1p-104 * (td + to)) break;
+    if (sweep > 0 && to > 0.25 * prev && to <= 1e-20 * td) break;
+    prev = to;
+    for (int r = 0; r < n - 1; ++r, ++g) {
+      // the round's rotations, lane a for pair a
+      if (warp == 0 && lane < h) {
+        const int p = at(lane, r), q = at(n - 1 - lane, r);
+        const double2 c = rotation_lean(m[p][p], m[q][q], m[p][q]);
+        rot[lane] = c;
+        cs[(size_t)g * h + lane] = c;
+      }
+      __syncthreads();
+      if (mine) {
+        const int pa = at(bb, r), qa = at(n - 1 - bb, r);
+        const double2 ja = rot[bb];
+        if (a == bb) {
+          const double x00 = m[pa][pa], x01 = m[pa][qa], x11 = m[qa][qa];
+          double d0, d1;
+          rotated_diag(x00, x01, x11, ja.x, ja.y, d0, d1);
+          const double y00 = ja.x * x00 - ja.y * x01, y01 = ja.y * x00 + ja.x * x01;
+          const double y10 = ja.x * x01 - ja.y * x11, y11 = ja.y * x01 + ja.x * x11;
+          const double z = 0.5 * ((ja.x * y01 - ja.y * y11) + (ja.y * y00 + ja.x * y10));
+          m[pa][pa] = d0;
+          m[qa][qa] = d1;
+          m[pa][qa] = z;
+          m[qa][pa] = z;
+        } else {
+          const int pb = at(a, r), qb = at(n - 1 - a, r);
+          const double2 jb = rot[a];
+          const double x00 = m[pa][pb], x01 = m[pa][qb], x10 = m[qa][pb], x11 = m[qa][qb];
+          const double y00 = jb.x * x00 - jb.y * x01, y01 = jb.y * x00 + jb.x * x01;
+          const double y10 = jb.x * x10 - jb.y * x11, y11 = jb.y * x10 + jb.x * x11;
+          const double z00 = ja.x * y00 - ja.y * y10, z01 = ja.x * y01 - ja.y * y11;
+          const double z10 = ja.y * y00 + ja.x * y10, z11 = ja.y * y01 + ja.x * y11;
+          m[pa][pb] = z00;
+          m[pa][qb] = z01;
+          m[qa][pb] = z10;
+          m[qa][qb] = z11;
+          m[pb][pa] = z00;
+          m[qb][pa] = z01;
+          m[pb][qa] = z10;
+          m[qb][qa] = z11;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  for (int t = tid; t < n * n; t += kSmallThreads) A[t] = m[t % n][t / n];
+  if (tid == 0) *rounds_out = g;
+}
+
 // A <- (A + A^T) / 2 in place
 __global__ void symmetrize_kernel(double *A, int n) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)n * n;
@@ -917,6 +1068,8 @@ size_t fisher_eig_work_doubles(int na) {
     const size_t cnt = j32_rotations(n);
     total += (cnt + 1) / 2 + ((cnt + 1) / 2 & 1) + 2 * cnt + 2;
   }
+  // the one-CTA form: (c, s) pairs of every round, the round count
+  if (n <= (size_t)kSmallN) total += 2 * (size_t)kSmallSweeps * (n - 1) * (n / 2) + 2;
   return total;
 }
 
@@ -1027,6 +1180,14 @@ cudaError_t run_fisher_eig(const double *F, int na, double *work, double *Finv, 
     e = cudaLaunchCooperativeKernel((const void *)ojacobi_kernel, dim3(h), dim3(kOjThreads), args,
                                     oj_smem, st);
     if (e != cudaSuccess) return e;
+    count_launch();
+  } else if (n <= kSmallN) {
+    double2 *cs = (double2 *)(work + eig_base_doubles((size_t)n));
+    int *rounds = (int *)(cs + (size_t)kSmallSweeps * (n - 1) * h);
+    jacobi_small_kernel<<<1, kSmallThreads, 0, st>>>(A0, n, cs, rounds);
+    count_launch();
+    vbuild_kernel<<<(unsigned)n, (unsigned)((h + 31) / 32 * 32), (size_t)n * sizeof(double), st>>>(
+        cs, rounds, n, V);
     count_launch();
   } else {
     // float32 pre-rotation (tuning key eig_mixed, default on): the float64
