@@ -179,47 +179,56 @@ __global__ void fisher_select_kernel(const double *F_full, const double *t_full,
   }
 }
 
-// y for every (l, sim): one CTA, threads over the 2l+1 modes
-__global__ void quad_y_kernel(const double *w, int64_t ldw, int nc, int k0, int lmin, int nl,
-                              int nspec, const int *spec_uv, double *y) {
-  const int L = blockIdx.x, sim = blockIdx.y;
-  const int l = lmin + L;
-  const int ni = 2 * l + 1;
-  const int64_t off = (int64_t)l * l - (int64_t)lmin * lmin;
-  const double *ws = w + (int64_t)sim * ldw;
-  double acc[6] = {0, 0, 0, 0, 0, 0};  // (u, v) u <= v, row-major upper triangle
-  for (int i = threadIdx.x; i < ni; i += blockDim.x) {
-    double v[3];
-    for (int c = 0; c < nc; ++c) v[c] = ws[(int64_t)c * k0 + off + i];
+// y for every (l, sim): kQuadLanes lanes over the 2l+1 modes, the products of
+// the NC components in registers (u <= v, row-major upper triangle), added up
+// by shuffles.  Bound by float64 issue (76 clocks a warp instruction): few
+// lanes a sum, because a shuffle step costs as many additions as a pass over
+// the modes does (a CTA of 128 threads per (l, sim) with six sums whatever NC:
+// 317 us for 31 multipoles and 1000 maps of two components).
+constexpr int kQuadLanes = 4, kQuadThreads = 128;
+template <int NC>
+__global__ void __launch_bounds__(kQuadThreads) quad_y_kernel(const double *w, int64_t ldw, int k0,
+                                                              int lmin, int nl, int nsims, int nspec,
+                                                              const int *spec_uv, double *y) {
+  constexpr int NU = NC * (NC + 1) / 2;
+  const int64_t t = (int64_t)blockIdx.x * kQuadThreads + threadIdx.x;
+  const int g = (int)(t % kQuadLanes);
+  const int64_t task = t / kQuadLanes;
+  const bool on = task < (int64_t)nl * nsims;
+  const int L = on ? (int)(task % nl) : 0;
+  const int64_t sim = on ? task / nl : 0;
+  const int l = lmin + L, ni = 2 * l + 1;
+  const double *ws = w + sim * ldw + ((int64_t)l * l - (int64_t)lmin * lmin);
+  double acc[NU];
+#pragma unroll
+  for (int u = 0; u < NU; ++u) acc[u] = 0.0;
+#pragma unroll 4
+  for (int i = g; i < ni; i += kQuadLanes) {
+    double v[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) v[c] = ws[(int64_t)c * k0 + i];
     int idx = 0;
-    for (int a = 0; a < nc; ++a)
-      for (int b = a; b < nc; ++b) acc[idx++] += v[a] * v[b];
+#pragma unroll
+    for (int a = 0; a < NC; ++a)
+#pragma unroll
+      for (int b = a; b < NC; ++b, ++idx) acc[idx] = fma(v[a], v[b], acc[idx]);
   }
-  __shared__ double red[8][6];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int u = 0; u < 6; ++u) {
-    double v = acc[u];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp][u] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    double s[6];
-    for (int u = 0; u < 6; ++u) {
-      s[u] = 0.0;
-      for (int q = 0; q < nw; ++q) s[u] += red[q][u];
-    }
-    const int na = nspec * nl;
-    for (int A = 0; A < nspec; ++A) {
-      const int *uv = spec_uv + 4 * A;
-      int a = uv[0], b = uv[1];
-      if (a > b) { int t = a; a = b; b = t; }
-      int idx = a * nc - a * (a - 1) / 2 + (b - a);
-      // auto: 1/2 sum w_X^2 ; cross: 1/2 (w_X w_Y + w_Y w_X) = sum w_X w_Y
-      double val = (npairs(uv) == 1) ? 0.5 * s[idx] : s[idx];
-      y[(int64_t)A * nl + L + (int64_t)sim * na] = val;
-    }
+#pragma unroll
+  for (int u = 0; u < NU; ++u)
+#pragma unroll
+    for (int o = kQuadLanes / 2; o > 0; o >>= 1)
+      acc[u] += __shfl_down_sync(0xffffffffu, acc[u], o, kQuadLanes);
+  if (!on || g != 0) return;
+  const int64_t na = (int64_t)nspec * nl;
+  for (int A = 0; A < nspec; ++A) {
+    const int *uv = spec_uv + 4 * A;
+    const int a = uv[0] < uv[1] ? uv[0] : uv[1], b = uv[0] < uv[1] ? uv[1] : uv[0];
+    const int idx = a * NC - a * (a - 1) / 2 + (b - a);
+    double s = acc[0];
+#pragma unroll
+    for (int u = 1; u < NU; ++u) s = idx == u ? acc[u] : s;
+    // auto: 1/2 sum w_X^2 ; cross: 1/2 (w_X w_Y + w_Y w_X) = sum w_X w_Y
+    y[A * nl + L + sim * na] = npairs(uv) == 1 ? 0.5 * s : s;
   }
 }
 
@@ -267,8 +276,15 @@ void launch_fisher_select(const double *F_full, const double *t_full, const doub
 void launch_quad_y(const double *w, int64_t ldw, int nsims, int nc, int k0, int lmin, int lmax,
                    int nspec, const int *spec_uv, double *y, cudaStream_t st) {
   const int nl = lmax - lmin + 1;
-  dim3 grid(nl, nsims);
-  { quad_y_kernel<<<grid, 128, 0, st>>>(w, ldw, nc, k0, lmin, nl, nspec, spec_uv, y); count_launch(); }
+  const int64_t threads = (int64_t)nl * nsims * kQuadLanes;
+  const unsigned grid = (unsigned)((threads + kQuadThreads - 1) / kQuadThreads);
+  if (nc == 1)
+    quad_y_kernel<1><<<grid, kQuadThreads, 0, st>>>(w, ldw, k0, lmin, nl, nsims, nspec, spec_uv, y);
+  else if (nc == 2)
+    quad_y_kernel<2><<<grid, kQuadThreads, 0, st>>>(w, ldw, k0, lmin, nl, nsims, nspec, spec_uv, y);
+  else
+    quad_y_kernel<3><<<grid, kQuadThreads, 0, st>>>(w, ldw, k0, lmin, nl, nsims, nspec, spec_uv, y);
+  count_launch();
 }
 
 void launch_sub_bias(const double *y, const double *b, int na, int nsims, double *q,
