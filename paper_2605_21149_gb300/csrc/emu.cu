@@ -499,6 +499,83 @@ __global__ void predict_finish_kernel(const double *theta, int ntot, int off, in
   }
 }
 
+// What predict_finish_kernel needs of each point besides the heads, and the
+// first layer's inputs, in one pass ahead of the network: bf16 inputs into the
+// first 16 of the 64 columns of x0 (the others stay zero), the baseline q and
+// whether the point lies outside the hull.  Rows cnt .. rows - 1 are zeroed.
+// Bound by float64 issue (a division per coordinate; 76 clocks a warp
+// instruction): the coefficients are converted to float32 once a CTA instead
+// of once a point (35 us of the 73 that 2^18 points took), the Legendre values
+// sit in shared memory instead of indexed local arrays, and the sample index
+// needs no 64-bit remainder (the gather took 78 us).
+constexpr int kPrepThreads = 128;
+inline size_t prep_smem(int d, int deg, int nf) {
+  return ((size_t)d * (deg + 1) * kPrepThreads + nf) * sizeof(float) + (size_t)nf * d;
+}
+__global__ void __launch_bounds__(kPrepThreads) predict_prep_kernel(
+    const double *theta, int ntot, int off, int cnt, int rows, int d, int deg, int nf,
+    const unsigned char *midx, const double *centre, const double *half, const double *coef,
+    __nv_bfloat16 *x0, double *qout, unsigned char *outside) {
+  extern __shared__ float psm[];
+  float *leg = psm + threadIdx.x;  // value k of coordinate i: leg[(i (deg + 1) + k) kPrepThreads]
+  float *cf = psm + (size_t)d * (deg + 1) * kPrepThreads;
+  unsigned char *mi = (unsigned char *)(cf + nf);
+  for (int t = threadIdx.x; t < nf; t += kPrepThreads) cf[t] = (float)coef[t];
+  for (int t = threadIdx.x; t < nf * d; t += kPrepThreads) mi[t] = midx[t];
+  __syncthreads();
+  const double c0 = coef[0];
+  for (int b = blockIdx.x * kPrepThreads + threadIdx.x; b < rows; b += gridDim.x * kPrepThreads) {
+    __align__(16) __nv_bfloat16 xr[kIn0];
+#pragma unroll
+    for (int i = 0; i < kIn0; ++i) xr[i] = __float2bfloat16_rn(0.0f);
+    if (b < cnt) {
+      bool outs = false;
+#pragma unroll
+      for (int i = 0; i < kMaxDim; ++i) {
+        if (i >= d) break;
+        const double x = (theta[off + b + (int64_t)i * ntot] - centre[i]) / half[i];
+        outs |= (fabs(x) > kHullMargin);
+        const float xi = (float)x;
+        xr[i] = __float2bfloat16_rn(xi);
+        float *lg = leg + (size_t)i * (deg + 1) * kPrepThreads;
+        float l0 = 1.0f, l1 = xi;
+        lg[0] = l0;
+        if (deg >= 1) lg[kPrepThreads] = l1;
+        for (int k = 1; k < deg; ++k) {
+          const float l2 = ((2 * k + 1) * xi * l1 - k * l0) / (float)(k + 1);
+          lg[(k + 1) * kPrepThreads] = l2;
+          l0 = l1;
+          l1 = l2;
+        }
+      }
+      float q = 0.0f;
+      for (int j = 1; j < nf; ++j) {
+        float f = 1.0f;
+        for (int i = 0; i < d; ++i) f *= leg[(i * (deg + 1) + mi[j * d + i]) * kPrepThreads];
+        q = fmaf(cf[j], f, q);
+      }
+      qout[b] = c0 + (double)q;
+      outside[b] = outs ? 1 : 0;
+    }
+    uint4 *dst = (uint4 *)(x0 + (size_t)b * 64);
+    dst[0] = ((const uint4 *)xr)[0];
+    dst[1] = ((const uint4 *)xr)[1];
+  }
+}
+
+// predict_finish_kernel from the prepared baseline and hull flags
+__global__ void predict_combine_kernel(int off, int cnt, const double *q, const unsigned char *outside,
+                                       const double *sigma, const float *o0, const float *o1,
+                                       double thr, double *out, int *flags, double *dis) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < cnt; j += gridDim.x * blockDim.x) {
+    const double a = o0[(int64_t)j * kOut0], b = o1[(int64_t)j * kOut0];
+    out[off + j] = q[j] + *sigma * 0.5 * (a + b);
+    const double dab = *sigma * fabs(a - b);
+    if (flags) flags[off + j] = (outside[j] || dab > thr) ? 1 : 0;
+    if (dis) dis[off + j] = dab;
+  }
+}
+
 // ------------------------------------------------- tcgen05 inference layer --
 // A layer at inference, Y = X W^T + b, on tcgen05 tensor cores (kind::f16:
 // bf16 x bf16 -> fp32 in TMEM).  X is the layer's bf16 input (rows x K,
@@ -916,11 +993,16 @@ struct PredCache {
   // heads) and each head's weights (width x 64), refreshed every call
   __nv_bfloat16 *x0p = nullptr, *w0p[2] = {nullptr, nullptr};
   bool tc0 = false;
+  // baseline and hull flag of each point of a chunk (with tc0)
+  double *q = nullptr;
+  unsigned char *outside = nullptr;
   CUtensorMap mx0p, mw0p[2];
   DevStatus *dst = nullptr;
   ~PredCache() {
     if (dst) cudaFree(dst);
     if (x0p) cudaFree(x0p);
+    if (q) cudaFree(q);
+    if (outside) cudaFree(outside);
     for (auto *w : w0p)
       if (w) cudaFree(w);
   }
@@ -951,6 +1033,10 @@ PredCache *pred_cache(qml_emu *e, int rows) {
     c->tc0 = cudaMalloc(&c->x0p, (size_t)rows * 64 * sizeof(__nv_bfloat16)) == cudaSuccess &&
              cudaMalloc(&c->w0p[0], (size_t)w0 * 64 * sizeof(__nv_bfloat16)) == cudaSuccess &&
              cudaMalloc(&c->w0p[1], (size_t)w0 * 64 * sizeof(__nv_bfloat16)) == cudaSuccess &&
+             cudaMalloc(&c->q, (size_t)rows * sizeof(double)) == cudaSuccess &&
+             cudaMalloc(&c->outside, (size_t)rows) == cudaSuccess &&
+             cudaMemset(c->x0p, 0, (size_t)rows * 64 * sizeof(__nv_bfloat16)) == cudaSuccess &&
+             cudaDeviceSynchronize() == cudaSuccess &&
              make_map_bf16(&c->mx0p, c->x0p, 64, rows, 128, 64, 128) &&
              make_map_bf16(&c->mw0p[0], c->w0p[0], 64, w0, 128, 64, w0) &&
              make_map_bf16(&c->mw0p[1], c->w0p[1], 64, w0, 128, 64, w0);
@@ -987,17 +1073,37 @@ qml_status run_predict(qml_emu *e, int n, const double *th, double thr, double *
       count_launch();
     }
   }
+  const int nl = (int)e->layers.size();
+  const size_t psm = prep_smem(e->d, e->deg, e->nf);
+  const bool prep = tc0 && psm <= 48 * 1024;
   for (int off = 0; off < n; off += chunk) {
     const int cnt = std::min(chunk, n - off);
     const int Bc = (cnt + 15) / 16 * 16;
     A0.B = A1.B = Bc;
+    const int rows_tc = (Bc + 127) / 128 * 128;
+    if (tc && prep) {
+      const int blocks = (rows_tc + kPrepThreads - 1) / kPrepThreads;
+      predict_prep_kernel<<<blocks < 152 * 8 ? blocks : 152 * 8, kPrepThreads, psm, st>>>(
+          th, n, off, cnt, rows_tc, e->d, e->deg, e->nf, e->midx, e->centre, e->half, e->coef,
+          pc->x0p, pc->q, pc->outside);
+      count_launch();
+      if (forward_tc(e, 0, A0, rows_tc, mx0, mw0, &pc->mx0p, &pc->mw0p[0], dst, st) &&
+          forward_tc(e, 1, A1, rows_tc, mx1, mw1, &pc->mx0p, &pc->mw0p[1], dst, st)) {
+        predict_combine_kernel<<<grid_of(cnt), 256, 0, st>>>(off, cnt, pc->q, pc->outside, e->sigma,
+                                                             A0.Z[nl - 1], A1.Z[nl - 1], thr, od,
+                                                             fd, dis);
+        count_launch();
+        continue;
+      }
+      tc = false;  // a launch was refused: finish on the WMMA path
+      cudaGetLastError();
+    }
     gather_kernel<<<grid_of((int64_t)Bc * kIn0), 256, 0, st>>>(th + off, n, e->d, e->centre, e->half,
                                                                nullptr, Bc, cnt, 0, 1, A0.X[0], nullptr);
     count_launch();
     cudaMemcpyAsync(A1.X[0], A0.X[0], (size_t)Bc * kIn0 * sizeof(__nv_bfloat16),
                     cudaMemcpyDeviceToDevice, st);
-    const int rows_tc = (Bc + 127) / 128 * 128;
-    if (tc0) {
+    if (tc0 && tc) {
       pad_cols_kernel<<<grid_of((int64_t)Bc * 64), 256, 0, st>>>(A0.X[0], Bc, kIn0, pc->x0p, 64);
       count_launch();
     }
@@ -1013,7 +1119,6 @@ qml_status run_predict(qml_emu *e, int n, const double *th, double thr, double *
       forward(e, 0, A0, st);
       forward(e, 1, A1, st);
     }
-    const int nl = (int)e->layers.size();
     predict_finish_kernel<<<grid_of(cnt), 256, 0, st>>>(th, n, off, cnt, e->d, e->deg, e->nf,
                                                         e->midx, e->centre, e->half, e->coef,
                                                         e->sigma, A0.Z[nl - 1],
