@@ -239,7 +239,7 @@ typedef struct {
  * dimension ld_out >= the largest nmaps): lnL[i*ld_out + j], chi2[...] and
  * logdet[i]; any may be NULL.  The per-mask part (Cholesky of N, M, Y^T N^-1 d)
  * runs once; items are spread round-robin over internal worker streams
- * (tuning key batch_streams, default 4).  Errors: QML_EINVAL,
+ * (tuning key batch_streams, default 8).  Errors: QML_EINVAL,
  * QML_ENOTSPD (N not positive definite), QML_ETIMEOUT. */
 qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitems,
                              const int32_t *item_mask, const double *item_cl, int32_t ld_out,
@@ -351,7 +351,7 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   Every tile gives bit-identical results.
  *   dgemm:<ta>,<tb>,<lower>,<M>,<N>,<K>,<alias>  a measured tile (10 RM + RN,
  *                   tile 16 RM x 16 RN); unknown values are ignored
- *   batch_streams   worker streams of pix_loglike_batch (default 4, 1..16)
+ *   batch_streams   worker streams of pix_loglike_batch (default 8, 1..16)
  *   batch_graphs    1 (default) / 0: pix_loglike_batch replays each worker's
  *                   per-item kernel sequence as a captured CUDA graph
  *   ozaki_stages    4 (default) / 3 / 2: depth of the split kernel's ring of
@@ -386,7 +386,8 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   the float64 sweeps from V0^T F V0 (same stopping rule,
  *                   two float64 sweeps instead of about seven at TQU Nside
  *                   16) / float64 sweeps only.  Used for padded orders
- *                   64 .. 640; other orders take the float64 sweeps only
+ *                   64 .. 640; larger orders take the float64 sweeps only,
+ *                   smaller ones run them in one CTA
  *   eig_cluster     16 (default) / 8: CTAs in the float32 phase's cluster
  *                   (16 falls back to 8 where the part cannot launch it)
  *   split_lookahead 1 (default) / 0: the split-precision Cholesky runs the

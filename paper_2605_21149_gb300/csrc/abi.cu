@@ -1257,7 +1257,11 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   }
 
   // ---- per-item work, round-robin over worker streams
-  const int ns_max = (int)std::max<int64_t>(1, std::min<int64_t>(16, tune_get("batch_streams", 4)));
+  // (eight by default: the chain of 64-wide float64 blocks that an item's factor
+  // waits on leaves most of the GPU to other items.  256 items of k = 756: 122
+  // ms with four workers, 77 with eight or sixteen; 24 items of k = 6900: 305,
+  // 283, 281)
+  const int ns_max = (int)std::max<int64_t>(1, std::min<int64_t>(16, tune_get("batch_streams", 8)));
   const int NS = nitems < ns_max ? nitems : ns_max;
   // CUDA graphs: item 0 runs as plain launches (so that the tile autotuner
   // can time its shapes), then each (worker, mask) pair captures its per-item
