@@ -250,9 +250,9 @@ __global__ void colsum_kernel(const float *dZ, int Brows, int N, float *db) {
   db[n] = s;
 }
 
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, int64_t n, float lr,
-                            float b1, float b2, float eps, float c1, float c2,
-                            __nv_bfloat16 *ph) {
+__device__ __forceinline__ void adam_update(float *p, const float *g, float *m, float *v, int64_t n,
+                                            float lr, float b1, float b2, float eps, float c1,
+                                            float c2, __nv_bfloat16 *ph) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -264,6 +264,12 @@ __global__ void adam_kernel(float *p, const float *g, float *m, float *v, int64_
     p[i] = pi;
     ph[i] = __float2bfloat16_rn(pi);
   }
+}
+
+__global__ void adam_kernel(float *p, const float *g, float *m, float *v, int64_t n, float lr,
+                            float b1, float b2, float eps, float c1, float c2,
+                            __nv_bfloat16 *ph) {
+  adam_update(p, g, m, v, n, lr, b1, b2, eps, c1, c2, ph);
 }
 
 __global__ void to_bf16_kernel(const float *p, int64_t n, __nv_bfloat16 *ph) {
@@ -329,6 +335,184 @@ __global__ void pad_cols_kernel(const __nv_bfloat16 *src, int rows, int cols, __
     const int c = (int)(t - r * dcols);
     dst[t] = c < cols ? src[r * cols + c] : __float2bfloat16_rn(0.0f);
   }
+}
+
+// ------------------------------------------------------- training steps --
+// One optimisation step of both heads (blockIdx.y) in 2 layers + 2 launches:
+// gather, one forward launch a layer (product, bias, activation; the output
+// layer also forms the loss gradient), one backward launch a layer (weight
+// gradient, bias gradient, and the next dZ = (dZ W) gelu'), Adam.  At a batch
+// of 64 every launch is latency: a head's step took 30 launches and 230 us, its
+// products on four CTAs of 64 x 64 that load a fragment at a time.  Here a warp
+// owns one 16 x 16 tile and loads four K steps of fragments ahead.  Every
+// output is the same sum in the same order as in the separate kernels above
+// (mma.sync over ascending k; the bias gradient over ascending rows).
+struct TrainHeads {
+  const __nv_bfloat16 *X[2], *W[2];   // layer input (B x in), weights (out x in)
+  const float *bias[2];
+  float *Z[2];                        // pre-activations (B x out)
+  __nv_bfloat16 *Xn[2];               // next layer's input; null at the output
+  const float *targ[2];               // output layer: targets
+  float *dZf[2];                      // gradient of this layer's pre-activations
+  __nv_bfloat16 *dZh[2];
+  float *gW[2], *gb[2];
+  const float *Zp[2];                 // backward: pre-activations of the layer below
+  float *dZf_dn[2];                   // and their gradient
+  __nv_bfloat16 *dZh_dn[2];
+};
+constexpr int kTrWarps = 4, kTrLd = 20;  // tiles per CTA; row stride of a staged tile
+
+// acc += A B over K (a multiple of 16), fragments of four K steps in flight
+template <typename ALay, typename BLay>
+__device__ __forceinline__ void tile_product(
+    wmma::fragment<wmma::accumulator, 16, 16, 16, float> &acc, const __nv_bfloat16 *A, int lda,
+    const __nv_bfloat16 *B, int ldb, int K) {
+  constexpr bool ar = std::is_same<ALay, wmma::row_major>::value;
+  constexpr bool br = std::is_same<BLay, wmma::row_major>::value;
+  for (int k = 0; k < K; k += 64) {
+    wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, ALay> a[4];
+    wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, BLay> b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int kk = k + 16 * u;
+      if (kk < K) {
+        wmma::load_matrix_sync(a[u], ar ? A + kk : A + (int64_t)kk * lda, lda);
+        wmma::load_matrix_sync(b[u], br ? B + (int64_t)kk * ldb : B + kk, ldb);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (k + 16 * u < K) wmma::mma_sync(acc, a[u], b[u], acc);
+  }
+}
+
+__global__ void train_gather_kernel(const double *theta, int n, int d, const double *centre,
+                                    const double *half, const float *targ, int Brows, int nreal,
+                                    int64_t off0, int64_t stride0, int64_t off1, int64_t stride1,
+                                    __nv_bfloat16 *X0, __nv_bfloat16 *X1, float *t0, float *t1) {
+  const int h = blockIdx.y;
+  const int64_t off = h ? off1 : off0, stride = h ? stride1 : stride0;
+  __nv_bfloat16 *X = h ? X1 : X0;
+  float *tb = h ? t1 : t0;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < Brows * kIn0; t += gridDim.x * blockDim.x) {
+    const int b = t / kIn0, c = t % kIn0;
+    float x = 0.0f;
+    if (b < nreal && (c < d || c == 0)) {
+      const int64_t row = (off + (int64_t)b * stride) % n;
+      if (c < d) x = (float)((theta[row + (int64_t)c * n] - centre[c]) / half[c]);
+      if (c == 0) tb[b] = targ[row];
+    } else if (c == 0) {
+      tb[b] = 0.0f;
+    }
+    X[t] = __float2bfloat16_rn(x);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kTrWarps) train_fwd_kernel(TrainHeads H, int B, int N, int K,
+                                                                   int nreal) {
+  __shared__ float st[kTrWarps][16 * kTrLd];
+  const int h = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tile = blockIdx.x * kTrWarps + warp, tn = N / 16;
+  const int m0 = tile / tn * 16, n0 = tile % tn * 16;
+  if (m0 >= B) return;
+  wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc;
+  wmma::fill_fragment(acc, 0.0f);
+  tile_product<wmma::row_major, wmma::col_major>(acc, H.X[h] + (int64_t)m0 * K, K,
+                                                 H.W[h] + (int64_t)n0 * K, K, K);
+  float *s = st[warp];
+  wmma::store_matrix_sync(s, acc, kTrLd, wmma::mem_row_major);
+  __syncwarp();
+  const int r = lane >> 1, c = (lane & 1) * 8, row = m0 + r;
+  __nv_bfloat16 *xn = H.Xn[h];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int col = n0 + c + j;
+    const int64_t t = (int64_t)row * N + col;
+    const float z = s[r * kTrLd + c + j] + H.bias[h][col];
+    H.Z[h][t] = z;
+    if (xn) {
+      xn[t] = __float2bfloat16_rn(gelu_f(z));
+    } else {
+      // output layer: gradient of the mean squared error of column 0
+      float g = 0.0f;
+      if (col == 0 && row < nreal) {
+        const float e = z - H.targ[h][row];
+        g = 2.0f * e / (float)nreal;
+      }
+      H.dZf[h][t] = g;
+      H.dZh[h][t] = __float2bfloat16_rn(g);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(32 * kTrWarps) train_bwd_kernel(TrainHeads H, int B, int out, int in) {
+  __shared__ float st[kTrWarps][16 * kTrLd];
+  const int h = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tin = in / 16;
+  int tile = blockIdx.x * kTrWarps + warp;
+  // the next dZ first (the longest sums), then the weight gradient, then the
+  // bias gradient
+  if (H.dZf_dn[h]) {
+    const int cnt = B / 16 * tin;
+    if (tile < cnt) {
+      const int m0 = tile / tin * 16, n0 = tile % tin * 16;
+      wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc;
+      wmma::fill_fragment(acc, 0.0f);
+      tile_product<wmma::row_major, wmma::row_major>(acc, H.dZh[h] + (int64_t)m0 * out, out,
+                                                     H.W[h] + n0, in, out);
+      float *s = st[warp];
+      wmma::store_matrix_sync(s, acc, kTrLd, wmma::mem_row_major);
+      __syncwarp();
+      const int r = lane >> 1, c = (lane & 1) * 8;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int64_t t = (int64_t)(m0 + r) * in + n0 + c + j;
+        const float d = s[r * kTrLd + c + j] * dgelu_f(H.Zp[h][t]);
+        H.dZf_dn[h][t] = d;
+        H.dZh_dn[h][t] = __float2bfloat16_rn(d);
+      }
+      return;
+    }
+    tile -= cnt;
+  }
+  {
+    const int cnt = out / 16 * tin;
+    if (tile < cnt) {
+      const int m0 = tile / tin * 16, n0 = tile % tin * 16;
+      wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc;
+      wmma::fill_fragment(acc, 0.0f);
+      tile_product<wmma::col_major, wmma::row_major>(acc, H.dZh[h] + m0, out, H.X[h] + n0, in, B);
+      wmma::store_matrix_sync(H.gW[h] + (int64_t)m0 * in + n0, acc, in, wmma::mem_row_major);
+      return;
+    }
+    tile -= cnt;
+  }
+  const int n = 32 * tile + lane;
+  if (n < out) {
+    const float *z = H.dZf[h] + n;
+    float s = 0.0f;
+    int b = 0;
+    for (; b + 8 <= B; b += 8) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = z[(int64_t)(b + u) * out];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += v[u];
+    }
+    for (; b < B; ++b) s += z[(int64_t)b * out];
+    H.gb[h][n] = s;
+  }
+}
+
+struct AdamHeads {
+  float *p[2], *m[2], *v[2];
+  const float *g[2];
+  __nv_bfloat16 *ph[2];
+  float c1[2], c2[2];
+};
+__global__ void train_adam_kernel(AdamHeads H, int64_t n, float lr, float b1, float b2, float eps) {
+  const int h = blockIdx.y;
+  adam_update(H.p[h], H.g[h], H.m[h], H.v[h], n, lr, b1, b2, eps, H.c1[h], H.c2[h], H.ph[h]);
 }
 
 // Legendre values P_0..P_deg of each of the d coordinates (Bonnet's
@@ -960,6 +1144,87 @@ void backward(qml_emu *e, int h, Acts &A, int nreal, cudaStream_t st) {
   }
 }
 
+// The fused training steps: activations of both heads (the first head's are
+// the caller's), a second set of dZ buffers per head (a layer's backward launch
+// reads one and writes the other) and the second head's gradient.
+constexpr int kTrainFused = 512;
+struct FusedTrain {
+  Acts *A[2] = {nullptr, nullptr};
+  Acts own;
+  float *dZf[2][2] = {}, *grad[2] = {};
+  __nv_bfloat16 *dZh[2][2] = {};
+  bool make(qml_emu *e, int batch, Acts &first) {
+    if (!own.make(e, batch)) return false;
+    A[0] = &first;
+    A[1] = &own;
+    int maxw = kIn0;
+    for (auto &l : e->layers) maxw = std::max(maxw, std::max(l.first, l.second));
+    grad[0] = e->grad;
+    grad[1] = own.a<float>(e->nparam);
+    for (int h = 0; h < 2; ++h) {
+      dZf[h][0] = A[h]->dZf;
+      dZh[h][0] = A[h]->dZh;
+      dZf[h][1] = own.a<float>((size_t)batch * maxw);
+      dZh[h][1] = own.a<__nv_bfloat16>((size_t)batch * maxw);
+      if (!dZf[h][1] || !dZh[h][1]) return false;
+    }
+    return grad[1] != nullptr;
+  }
+  void forward_backward(qml_emu *e, int nreal, cudaStream_t st) {
+    const int nl = (int)e->layers.size(), B = A[0]->B;
+    auto args = [&](int l, int par) {
+      TrainHeads H{};
+      for (int h = 0; h < 2; ++h) {
+        H.X[h] = A[h]->X[l];
+        H.W[h] = e->ph[h] + e->woff[l];
+        H.bias[h] = e->p[h] + e->boff[l];
+        H.Z[h] = A[h]->Z[l];
+        H.Xn[h] = l + 1 < nl ? A[h]->X[l + 1] : nullptr;
+        H.targ[h] = A[h]->tb;
+        H.dZf[h] = dZf[h][par];
+        H.dZh[h] = dZh[h][par];
+        H.gW[h] = grad[h] + e->woff[l];
+        H.gb[h] = grad[h] + e->boff[l];
+        if (l > 0) {
+          H.Zp[h] = A[h]->Z[l - 1];
+          H.dZf_dn[h] = dZf[h][par ^ 1];
+          H.dZh_dn[h] = dZh[h][par ^ 1];
+        }
+      }
+      return H;
+    };
+    auto ctas = [](int tiles) { return dim3((unsigned)((tiles + kTrWarps - 1) / kTrWarps), 2); };
+    for (int l = 0; l < nl; ++l) {
+      const int out = e->layers[l].first, in = e->layers[l].second;
+      train_fwd_kernel<<<ctas(B / 16 * (out / 16)), 32 * kTrWarps, 0, st>>>(args(l, 0), B, out, in,
+                                                                            nreal);
+      count_launch();
+    }
+    for (int l = nl - 1, par = 0; l >= 0; --l, par ^= 1) {
+      const int out = e->layers[l].first, in = e->layers[l].second;
+      const int tiles = (l > 0 ? B / 16 * (in / 16) : 0) + out / 16 * (in / 16) + (out + 31) / 32;
+      train_bwd_kernel<<<ctas(tiles), 32 * kTrWarps, 0, st>>>(args(l, par), B, out, in);
+      count_launch();
+    }
+  }
+  void adam(qml_emu *e, float lr, float b1, float b2, float eps, const float *c1, const float *c2,
+            cudaStream_t st) {
+    AdamHeads H;
+    for (int h = 0; h < 2; ++h) {
+      H.p[h] = e->p[h];
+      H.m[h] = e->m[h];
+      H.v[h] = e->v[h];
+      H.g[h] = grad[h];
+      H.ph[h] = e->ph[h];
+      H.c1[h] = c1[h];
+      H.c2[h] = c2[h];
+    }
+    train_adam_kernel<<<dim3((unsigned)grid_of(e->nparam), 2), 256, 0, st>>>(H, e->nparam, lr, b1, b2,
+                                                                             eps);
+    count_launch();
+  }
+};
+
 bool is_dev(const void *p) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
@@ -1348,15 +1613,61 @@ qml_status emu_train(qml_emu *e, int32_t n, const double *theta, const double *l
   const int steps_per_epoch = (n + batch - 1) / batch;
   const int64_t total_steps = (int64_t)steps_per_epoch * epochs;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  for (int h = 0; h < 2; ++h) {
+  // epoch order of head h: off + j stride (mod n) with stride coprime to n
+  auto epoch_order = [&](int ep, int h, int64_t &off, int64_t &stride) {
+    const uint64_t hsh =
+        (e->seed + 1000003ull * (ep + 1) + 7919ull * (h + 1)) * 0x9E3779B97F4A7C15ull;
+    stride = (int64_t)(hsh % (uint64_t)n) | 1;
+    auto gcd = [](int64_t a, int64_t b) { while (b) { int64_t t = a % b; a = b; b = t; } return a; };
+    while (gcd(stride, n) != 1) stride += 2;
+    off = (int64_t)((hsh >> 20) % (uint64_t)n);
+  };
+  // learning rate: constant for the first 80 % of the steps (the network
+  // needs them to leave its initial plateau), then a cosine decay to 2 %
+  auto rate = [&](int64_t step) {
+    const double frac = (double)step / (double)std::max<int64_t>(1, total_steps - 1);
+    const double dec = frac < 0.8 ? 1.0
+                                   : 0.02 + 0.98 * 0.5 * (1.0 + cos(3.141592653589793 * (frac - 0.8) / 0.2));
+    return (float)(lr * dec);
+  };
+  auto corrections = [&](int h, float &c1, float &c2) {
+    e->adam_t[h] += 1;
+    c1 = 1.0f / (1.0f - powf(b1, (float)e->adam_t[h]));
+    c2 = 1.0f / (1.0f - powf(b2, (float)e->adam_t[h]));
+  };
+  // both heads in step by the fused kernels up to a batch of kTrainFused (a
+  // warp a tile, no reuse of fragments); larger ones head by head
+  const bool fused = batch <= kTrainFused;
+  FusedTrain F;
+  if (fused && !F.make(e, batch, A)) {
+    cleanup();
+    return efail(QML_ENOMEM, "emu_train: activation allocation failed");
+  }
+  if (fused) {
     int64_t step = 0;
     for (int ep = 0; ep < epochs; ++ep) {
-      // epoch order: off + j stride (mod n) with stride coprime to n
-      uint64_t hsh = (e->seed + 1000003ull * (ep + 1) + 7919ull * (h + 1)) * 0x9E3779B97F4A7C15ull;
-      int64_t stride = (int64_t)(hsh % (uint64_t)n) | 1;
-      auto gcd = [](int64_t a, int64_t b) { while (b) { int64_t t = a % b; a = b; b = t; } return a; };
-      while (gcd(stride, n) != 1) stride += 2;
-      const int64_t off = (int64_t)((hsh >> 20) % (uint64_t)n);
+      int64_t off[2], stride[2];
+      for (int h = 0; h < 2; ++h) epoch_order(ep, h, off[h], stride[h]);
+      for (int sb = 0; sb < steps_per_epoch; ++sb, ++step) {
+        const int nreal = std::min(batch, n - sb * batch);
+        train_gather_kernel<<<dim3((unsigned)((batch * kIn0 + 127) / 128), 2), 128, 0, st>>>(
+            th, n, e->d, e->centre, e->half, targ, batch, nreal,
+            off[0] + (int64_t)sb * batch * stride[0], stride[0],
+            off[1] + (int64_t)sb * batch * stride[1], stride[1], F.A[0]->X[0], F.A[1]->X[0],
+            F.A[0]->tb, F.A[1]->tb);
+        count_launch();
+        F.forward_backward(e, nreal, st);
+        float c1[2], c2[2];
+        for (int h = 0; h < 2; ++h) corrections(h, c1[h], c2[h]);
+        F.adam(e, rate(step), b1, b2, eps, c1, c2, st);
+      }
+    }
+  }
+  for (int h = 0; h < 2; ++h) {
+    int64_t step = 0;
+    for (int ep = 0; !fused && ep < epochs; ++ep) {
+      int64_t off, stride;
+      epoch_order(ep, h, off, stride);
       for (int sb = 0; sb < steps_per_epoch; ++sb, ++step) {
         const int nreal = std::min(batch, n - sb * batch);
         gather_kernel<<<grid_of((int64_t)batch * kIn0), 256, 0, st>>>(
@@ -1365,15 +1676,9 @@ qml_status emu_train(qml_emu *e, int32_t n, const double *theta, const double *l
         count_launch();
         forward(e, h, A, st);
         backward(e, h, A, nreal, st);
-        // learning rate: constant for the first 80 % of the steps (the network
-        // needs them to leave its initial plateau), then a cosine decay to 2 %
-        const double frac = (double)step / (double)std::max<int64_t>(1, total_steps - 1);
-        const double dec = frac < 0.8 ? 1.0
-                                       : 0.02 + 0.98 * 0.5 * (1.0 + cos(3.141592653589793 * (frac - 0.8) / 0.2));
-        const float lrs = (float)(lr * dec);
-        e->adam_t[h] += 1;
-        const float c1 = 1.0f / (1.0f - powf(b1, (float)e->adam_t[h]));
-        const float c2 = 1.0f / (1.0f - powf(b2, (float)e->adam_t[h]));
+        float c1, c2;
+        const float lrs = rate(step);
+        corrections(h, c1, c2);
         adam_kernel<<<grid_of(e->nparam), 256, 0, st>>>(e->p[h], e->grad, e->m[h], e->v[h],
                                                         e->nparam, lrs, b1, b2, eps, c1, c2,
                                                         e->ph[h]);
