@@ -350,7 +350,8 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   first call with a new shape synchronises its stream.
  *                   Every tile gives bit-identical results.
  *   dgemm:<ta>,<tb>,<lower>,<M>,<N>,<K>,<alias>  a measured tile (10 RM + RN,
- *                   tile 16 RM x 16 RN); unknown values are ignored
+ *                   tile 16 RM x 16 RN; 10: 16 x 16 tiles with the whole K
+ *                   range in shared memory); unknown values are ignored
  *   batch_streams   worker streams of pix_loglike_batch (default 8, 1..16)
  *   batch_graphs    1 (default) / 0: pix_loglike_batch replays each worker's
  *                   per-item kernel sequence as a captured CUDA graph

@@ -334,27 +334,23 @@ void trsm_blocked_t(Call &c, const double *L, int64_t n, int64_t lda, const doub
 // left block -R^-1 T, each one batched product over the pairs (a last pair
 // whose second block is shorter than b gets its own two products).  log2 of
 // the block count steps instead of one per block row; T (scratch) holds
-// (kNBS/2)^2 doubles.  On stream st; with fixed the float64 products skip
-// the tile autotuner (which synchronises), as work on a second stream must.
+// (kNBS/2)^2 doubles.  On stream st.
 void trinv_doubling(Call &c, const double *L, int64_t jb, int64_t lda, const double *Linv,
-                    double *X, int64_t ldx, double *T, cudaStream_t st, bool fixed) {
-  auto gemm = fixed ? launch_dgemm_fixed : launch_dgemm;
+                    double *X, int64_t ldx, double *T, cudaStream_t st) {
   launch_place_diag_inverses(Linv, jb, X, ldx, st);
   for (int64_t b = kNB; b < jb; b *= 2) {
     const int64_t full = jb / (2 * b);  // pairs with both blocks b long
-    if (full > 0) {
-      const int64_t sL = 2 * b + 2 * b * lda, sX = 2 * b + 2 * b * ldx;
-      launch_dgemm_batched(0, 0, b, b, b, 1.0, L + b, lda, sL, X, ldx, sX, 0.0, T, b, b * b,
-                           (int)full, c.status, st);
-      launch_dgemm_batched(0, 0, b, b, b, -1.0, X + b + b * ldx, ldx, sX, T, b, b * b, 0.0, X + b,
-                           ldx, sX, (int)full, c.status, st);
-    }
+    const int64_t sL = 2 * b + 2 * b * lda, sX = 2 * b + 2 * b * ldx;
+    launch_panel_gemm(0, b, b, b, 1.0, L + b, lda, sL, X, ldx, sX, 0.0, T, b, b * b, 0, 1, (int)full,
+                      c.status, st);
+    launch_panel_gemm(0, b, b, b, -1.0, X + b + b * ldx, ldx, sX, T, b, b * b, 0.0, X + b, ldx, sX, 0,
+                      2, (int)full, c.status, st);
     const int64_t r0 = full * 2 * b, b2 = jb - r0 - b;  // a last pair with a short R
     if (b2 > 0) {
-      gemm(0, 0, b2, b, b, 1.0, L + (r0 + b) + r0 * lda, lda, X + r0 + r0 * ldx, ldx, 0.0, T, b2,
-           0, c.status, st);
-      gemm(0, 0, b2, b, b2, -1.0, X + (r0 + b) + (r0 + b) * ldx, ldx, T, b2, 0.0,
-           X + (r0 + b) + r0 * ldx, ldx, 0, c.status, st);
+      launch_panel_gemm(0, b2, b, b, 1.0, L + (r0 + b) + r0 * lda, lda, 0, X + r0 + r0 * ldx, ldx, 0,
+                        0.0, T, b2, 0, 0, 1, 1, c.status, st);
+      launch_panel_gemm(0, b2, b, b2, -1.0, X + (r0 + b) + (r0 + b) * ldx, ldx, 0, T, b2, 0, 0.0,
+                        X + (r0 + b) + r0 * ldx, ldx, 0, 0, 2, 1, c.status, st);
     }
   }
 }
@@ -418,6 +414,25 @@ struct Split {
     c->cuda_ok(oz_mm(M, N, alpha, A, ra, B, rb, beta, C, ldc, lower, c->status, c->st, reserve_sms),
                "split-precision gemm");
   }
+  // A few right-hand sides (nrhs <= kSkinnyN), panel j of B <- L^-1 B: B_j <-
+  // Xinv B_j, B_below -= L21 B_j, on the float64 pipe: L is read once, where
+  // the digit products would slice it first and fill 128-column tiles.
+  void few_panel(const double *Xinv, int64_t jb, const double *L21, int64_t lda, int64_t m2,
+                 double *Bj, int64_t nrhs, int64_t ldb) {
+    const size_t need = sizeof(double) * kNBS * kSkinnyN;
+    if (need > buf[2].bytes) {
+      buf[2].p = c->alloc<unsigned char>(need, "right-hand sides");
+      buf[2].bytes = buf[2].p ? need : 0;
+    }
+    if (c->err != QML_OK) return;
+    double *X = (double *)buf[2].p;
+    launch_skinny(jb, nrhs, jb, 1.0, Xinv, kNBS, Bj, ldb, 0.0, X, jb, nullptr, 0, c->status, c->st);
+    if (m2 > 0)
+      launch_skinny(m2, nrhs, jb, -1.0, L21, lda, X, jb, 1.0, Bj + jb, ldb, Bj, ldb, c->status,
+                    c->st);
+    else
+      launch_copy_matrix(X, jb, Bj, ldb, jb, nrhs, c->st);
+  }
   void gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A,
             int64_t lda, const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
             int lower) {
@@ -473,7 +488,8 @@ Split make_split(Call &c, int precision, int S) {
 // LinvB's slot (float64, recursive doubling).  With split_diag_df the
 // 64-blocks and their row solves run in float-float instead (about 2^-46 per
 // operation; the factor goes to the inverse slot, the coefficients to S behind
-// T's panel part).  fixed: float64 products without the tile autotuner.
+// T's panel part).  fixed: the updates skip the tile autotuner (which
+// synchronises), as work on a second stream must.
 void panel_chain(Call &c, Split &sp, double *A, int64_t lda, int64_t j, int64_t jb,
                  double *Linv64, double *LinvB, double *ldparts, bool dfdiag, cudaStream_t st,
                  bool fixed) {
@@ -507,7 +523,7 @@ void panel_chain(Call &c, Split &sp, double *A, int64_t lda, int64_t j, int64_t 
   else
     launch_trtri_blocks(Ajj, lda, jb, Linv64 + (j / kNB) * kNB * kNB, c.status, st);
   trinv_doubling(c, Ajj, jb, lda, Linv64 + (j / kNB) * kNB * kNB, LinvB + (j / kNBS) * kNBS * kNBS,
-                 kNBS, T, st, fixed);
+                 kNBS, T, st);
 }
 
 // Cholesky A = L L^T (lower, in place).  Linv64: inverses of the 64-blocks
@@ -584,7 +600,9 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
         sp.mm(m2, m2, -1.0, dP, 0, dP, 0, 1.0, A22, lda, 1);
       }
     }
-    if (B) {
+    if (B && nrhs <= kSkinnyN) {
+      sp.few_panel(Xinv, jb, A21, lda, m2, B + j, nrhs, ldb);
+    } else if (B) {
       // forward substitution, panel j: B_j <- L_jj^-1 B_j ; B_below -= A21 B_j
       const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
       OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
@@ -619,6 +637,10 @@ void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, con
   for (int64_t j = 0; j < n; j += nb) {
     const int64_t jb = (n - j) < nb ? (n - j) : nb;
     const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS + (j % kNBS) * (kNBS + 1);
+    if (nrhs <= kSkinnyN) {
+      sp.few_panel(Xinv, jb, L + (j + jb) + j * lda, lda, n - j - jb, B + j, nrhs, ldb);
+      continue;
+    }
     const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
     OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
     sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
@@ -1526,7 +1548,7 @@ qml_status qml_trsm(int64_t n, int64_t nrhs, const double *L, int64_t lda, doubl
       const int64_t jb = (n - j) < kNBS ? (n - j) : kNBS;
       double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS;
       trinv_doubling(c, Ld + j + j * lda, jb, lda, Linv + (j / kNB) * kNB * kNB, Xinv, kNBS, T,
-                     c.st, false);
+                     c.st);
     }
     trsm_split(c, spl, Ld, n, lda, LinvB, Bd, nrhs, ldb);
   } else {

@@ -13,6 +13,7 @@
 
 #include <math.h>
 
+#include <mutex>
 #include <string>
 
 namespace qmlgb {
@@ -150,6 +151,124 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int64_t M, int64_t N, int64_
       if (beta != 0.0) v = fma(beta, *cp, v);
       *cp = v;
     }
+  }
+}
+
+// C_z <- alpha A_z op(B_z) + beta C_z for the small products inside a 512-wide
+// panel (K <= kPanelK): 16 x 16 tiles, one output a thread, both operands'
+// whole K range in shared memory after a single round of loads.  Bound by
+// latency and by float64 issue: at K = 64 the tiles above cover a 448-row
+// update with 56 to 105 CTAs, so that one SM works off a 2048-output tile for
+// 38 us of the 41 it took; here 406 tiles share the 152 SMs (14 us of float64
+// issue).  tri 1: B is lower triangular (terms with k < n are zero), tri 2: A
+// is (k > m); such terms are left out tile by tile, half of the work of a block
+// inverse.  Each output is the same sum in the same order as dgemm_kernel's.
+constexpr int kPanelK = 256;
+template <bool TB>
+__global__ void __launch_bounds__(256) panel_gemm_kernel(int M, int N, int K, double alpha,
+                                                         const double *A, int64_t lda,
+                                                         const double *B, int64_t ldb, double beta,
+                                                         double *C, int64_t ldc, int lower, int tri,
+                                                         const DevStatus *status, DgBatch bt) {
+  extern __shared__ double pg[];
+  if (status && *((volatile const int *)&status->code) != 0) return;
+  const int m0 = blockIdx.x * 16, n0 = blockIdx.y * 16;
+  if (lower && m0 + 15 < n0) return;  // tile strictly above the diagonal
+  A += (int64_t)blockIdx.z * bt.sA;
+  B += (int64_t)blockIdx.z * bt.sB;
+  C += (int64_t)blockIdx.z * bt.sC;
+  const int klo = tri == 1 ? (n0 < K ? n0 : K) : 0;
+  const int khi = tri == 2 ? (m0 + 16 < K ? m0 + 16 : K) : K;
+  const int kn = khi - klo;
+  double *As = pg, *Bs = pg + 17 * kn;  // [k][17]
+  const int tid = threadIdx.x, lo = tid & 15, hi = tid >> 4;
+  const bool am = m0 + lo < M, bn = n0 + (TB ? lo : hi) < N;
+  for (int k0 = 0; k0 < kn; k0 += 64) {
+    double ra[4], rb[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int ka = k0 + 16 * u + hi, kb = k0 + 16 * u + (TB ? hi : lo);
+      ra[u] = am && ka < kn ? A[m0 + lo + (int64_t)(klo + ka) * lda] : 0.0;
+      rb[u] = !(bn && kb < kn) ? 0.0
+              : TB             ? B[n0 + lo + (int64_t)(klo + kb) * ldb]
+                               : B[klo + kb + (int64_t)(n0 + hi) * ldb];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int ka = k0 + 16 * u + hi, kb = k0 + 16 * u + (TB ? hi : lo);
+      if (ka < kn) As[17 * ka + lo] = ra[u];
+      if (kb < kn) Bs[17 * kb + (TB ? lo : hi)] = rb[u];
+    }
+  }
+  __syncthreads();
+  const int gm = m0 + lo, gn = n0 + hi;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int k = 0; k < kn; ++k) acc = fma(As[17 * k + lo], Bs[17 * k + hi], acc);
+  if (gm >= M || gn >= N || (lower && gm < gn)) return;
+  double *cp = C + gm + (int64_t)gn * ldc;
+  double v = alpha * acc;
+  if (beta != 0.0) v = fma(beta, *cp, v);
+  *cp = v;
+}
+
+// A few columns: 32 rows a CTA, a lane per row, warp w the w-th eighth of K, NC
+// sums a thread; the warps' parts are added in order.  Bound by reading A once
+// (coalesced, eight loads in flight a thread); the square tiles above would
+// spend their float64 issue on columns that do not exist (N = 1: 38 us a
+// 16-row tile of K = 512).
+constexpr int kSkinnyK = 512;
+template <int NC>
+__global__ void __launch_bounds__(256) skinny_kernel(int M, int N, int K, double alpha,
+                                                     const double *A, int64_t lda, const double *B,
+                                                     int64_t ldb, double beta, double *C,
+                                                     int64_t ldc, double *Bcopy, int64_t ldbc,
+                                                     const DevStatus *status) {
+  __shared__ double b[kSkinnyK][NC], part[8][NC][32];
+  if (status && *((volatile const int *)&status->code) != 0) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int t = tid; t < K * NC; t += 256) {
+    const int k = t % K, j = t / K;
+    const double v = j < N ? B[k + j * ldb] : 0.0;
+    b[k][j] = v;
+    if (Bcopy && blockIdx.x == 0 && j < N) Bcopy[k + j * ldbc] = v;
+  }
+  __syncthreads();
+  const int row = blockIdx.x * 32 + lane;
+  const double *a = A + (row < M ? row : 0);
+  const int k1 = (warp + 1) * K / 8;
+  double acc[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) acc[j] = 0.0;
+  int k = warp * K / 8;
+  for (; k + 8 <= k1; k += 8) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = a[(int64_t)(k + u) * lda];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+      for (int j = 0; j < NC; ++j) acc[j] = fma(v[u], b[k + u][j], acc[j]);
+  }
+  for (; k < k1; ++k) {
+    const double v = a[(int64_t)k * lda];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) acc[j] = fma(v, b[k][j], acc[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < NC; ++j) part[warp][j][lane] = acc[j];
+  __syncthreads();
+  for (int t = tid; t < 32 * N; t += 256) {
+    const int r = t & 31, j = t >> 5;
+    const int64_t gm = (int64_t)blockIdx.x * 32 + r;
+    if (gm >= M) continue;
+    double s = part[0][j][r];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w][j][r];
+    double v = alpha * s;
+    double *cp = C + gm + j * ldc;
+    if (beta != 0.0) v = fma(beta, *cp, v);
+    *cp = v;
   }
 }
 
@@ -902,6 +1021,13 @@ void dgemm_dispatch(int ta, int tb, int rm, int rn, int64_t M, int64_t N, int64_
 }
 
 const int kCand[7][2] = {{4, 4}, {2, 4}, {4, 2}, {2, 2}, {1, 4}, {4, 1}, {1, 1}};
+// Tile code of panel_gemm_kernel (10 RM + RN has no RN = 0) and the products it
+// fits: A and C not transposed or aliased, K <= kPanelK, C small enough that
+// 16 x 16 tiles, which reuse an operand 16 times, are not bound by loading.
+constexpr int kPanelCode = 10;
+bool panel_fits(int ta, int64_t M, int64_t N, int64_t K, bool alias) {
+  return !ta && !alias && K >= 1 && K <= kPanelK && M * N <= 1024 * 1024;
+}
 
 // Autotuner: time every candidate tile on this shape (output into a scratch
 // matrix, beta = 0, so the caller's C is untouched) and keep the fastest.
@@ -935,6 +1061,22 @@ bool dgemm_autotune(int ta, int tb, int64_t M, int64_t N, int64_t K, const doubl
       found = i;
     }
   }
+  bool panel = false;
+  if (ok && panel_fits(ta, M, N, K, false)) {
+    float ms = 0.0f;
+    auto go = [&] {
+      launch_panel_gemm(tb, M, N, K, 1.0, A, lda, 0, B, ldb, 0, 0.0, scratch, M, 0, lower, 0, 1,
+                        status, st);
+    };
+    go();
+    cudaEventRecord(e0, st);
+    for (int r = 0; r < 3; ++r) go();
+    cudaEventRecord(e1, st);
+    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
+      ok = false;
+    else
+      panel = ms < best;
+  }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (scratch) cudaFree(scratch);
@@ -942,8 +1084,8 @@ bool dgemm_autotune(int ta, int tb, int64_t M, int64_t N, int64_t K, const doubl
     cudaGetLastError();
     return false;
   }
-  rm = kCand[found][0];
-  rn = kCand[found][1];
+  rm = panel ? kPanelCode / 10 : kCand[found][0];
+  rn = panel ? kPanelCode % 10 : kCand[found][1];
   return true;
 }
 
@@ -968,7 +1110,17 @@ void launch_dgemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, double a
                           std::to_string((aliasA ? 1 : 0) + (aliasB ? 2 : 0));
   int64_t tv;
   bool known = false;
-  if (tune_find(key, tv))
+  const bool panel = panel_fits(ta, M, N, K, aliasA || aliasB);
+  auto go_panel = [&] {
+    launch_panel_gemm(tb, M, N, K, alpha, A, lda, 0, B, ldb, 0, beta, C, ldc, 0, lower, 0, 1, status,
+                      st);
+  };
+  const bool have = tune_find(key, tv);
+  if (have && tv == kPanelCode && panel) {
+    go_panel();
+    return;
+  }
+  if (have)
     for (int i = 0; i < 7; ++i)
       known |= (tv == 10 * kCand[i][0] + kCand[i][1]);
   if (known && !(aliasA && tv % 10 != 4) && !(aliasB && tv / 10 != 4)) {
@@ -983,12 +1135,19 @@ void launch_dgemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, double a
       int rm = 4, rn = 4;
       if (dgemm_autotune(ta, tb, M, N, K, A, lda, B, ldb, lower, status, st, rm, rn)) {
         tune_put(key, 10 * rm + rn);
-        dgemm_dispatch(ta, tb, rm, rn, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, status,
+        if (10 * rm + rn == kPanelCode)
+          go_panel();
+        else
+          dgemm_dispatch(ta, tb, rm, rn, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, status,
                        st);
         return;
       }
     }
     cudaGetLastError();
+  }
+  if (panel) {
+    go_panel();
+    return;
   }
   const int64_t want = 2 * 152;
   int rm = 4, rn = 4;
@@ -1027,23 +1186,44 @@ void launch_dgemm_fixed(int ta, int tb, int64_t M, int64_t N, int64_t K, double 
   launch_dgemm_impl(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, status, st, false);
 }
 
-// count products C_z <- alpha op(A_z) op(B_z) + beta C_z, X_z = X + z sX; the
-// tile is the largest whose grid (over all products) gives every SM two CTAs
-void launch_dgemm_batched(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
-                          const double *A, int64_t lda, int64_t sA, const double *B,
-                          int64_t ldb, int64_t sB, double beta, double *C, int64_t ldc,
-                          int64_t sC, int count, const DevStatus *status, cudaStream_t st) {
+void launch_skinny(int64_t M, int64_t N, int64_t K, double alpha, const double *A, int64_t lda,
+                   const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
+                   double *Bcopy, int64_t ldbc, const DevStatus *status, cudaStream_t st) {
+  if (M <= 0 || N <= 0) return;
+  const unsigned grid = (unsigned)((M + 31) / 32);
+  if (N == 1)
+    skinny_kernel<1><<<grid, 256, 0, st>>>((int)M, 1, (int)K, alpha, A, lda, B, ldb, beta, C, ldc,
+                                           Bcopy, ldbc, status);
+  else if (N <= 4)
+    skinny_kernel<4><<<grid, 256, 0, st>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta, C,
+                                           ldc, Bcopy, ldbc, status);
+  else
+    skinny_kernel<kSkinnyN><<<grid, 256, 0, st>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb, beta,
+                                                  C, ldc, Bcopy, ldbc, status);
+  count_launch();
+}
+
+void launch_panel_gemm(int tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A,
+                       int64_t lda, int64_t sA, const double *B, int64_t ldb, int64_t sB,
+                       double beta, double *C, int64_t ldc, int64_t sC, int lower, int tri,
+                       int count, const DevStatus *status, cudaStream_t st) {
   if (M <= 0 || N <= 0 || count <= 0) return;
-  int rm = 1, rn = 1;
-  for (int i = 0; i < 7; ++i) {
-    if (dgemm_ctas(M, N, 16 * kCand[i][0], 16 * kCand[i][1], 0) * count >= 2 * 152) {
-      rm = kCand[i][0];
-      rn = kCand[i][1];
-      break;
-    }
-  }
-  dgemm_dispatch(ta, tb, rm, rn, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, 0, status, st,
-                 DgBatch{count, sA, sB, sC});
+  const size_t smem = 2 * 17 * (size_t)K * sizeof(double);
+  static std::once_flag once;
+  std::call_once(once, [] {
+    const int most = 2 * 17 * kPanelK * (int)sizeof(double);
+    cudaFuncSetAttribute(panel_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(panel_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  });
+  const dim3 grid((unsigned)((M + 15) / 16), (unsigned)((N + 15) / 16), (unsigned)count);
+  const DgBatch bt{count, sA, sB, sC};
+  if (tb)
+    panel_gemm_kernel<true><<<grid, 256, smem, st>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb,
+                                                     beta, C, ldc, lower, tri, status, bt);
+  else
+    panel_gemm_kernel<false><<<grid, 256, smem, st>>>((int)M, (int)N, (int)K, alpha, A, lda, B, ldb,
+                                                      beta, C, ldc, lower, tri, status, bt);
+  count_launch();
 }
 
 void launch_potrf_diag(double *A, int64_t lda, int64_t n, int64_t j0, double *Linv,

@@ -960,6 +960,37 @@ int grid_of(int64_t total) {
 
 }  // namespace
 
+namespace {
+// Device memory taken in one piece and handed out in 256-byte steps: an
+// emulator, a training call and an inference cache are a hundred buffers
+// between them, and allocating and freeing each took 14 of the 35 ms of a
+// two-epoch training call.
+struct Slab {
+  unsigned char *p = nullptr;
+  size_t size = 0, used = 0;
+  static size_t step(size_t bytes) { return (bytes + 255) / 256 * 256; }
+  ~Slab() {
+    if (p) cudaFree(p);
+  }
+  bool make(size_t bytes) {
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      p = nullptr;
+      return false;
+    }
+    size = bytes;
+    return true;
+  }
+  template <class T>
+  T *take(size_t count) {
+    const size_t b = step(count * sizeof(T));
+    if (!p || used + b > size) return nullptr;
+    T *q = (T *)(p + used);
+    used += b;
+    return q;
+  }
+};
+}  // namespace
+
 // ======================================================================
 struct qml_emu {
   int d = 0, width = 0, depth = 0, nheads = 2;
@@ -980,7 +1011,7 @@ struct qml_emu {
   // held-out labels, sorted by head disagreement: disagreement and the
   // running maximum of the prediction error up to it
   std::vector<double> val_dis, val_maxerr;
-  std::vector<void *> mem;
+  Slab mem;
   // buffers of emu_predict, kept between calls (freed by emu_free)
   void *pcache = nullptr;
   void (*pcache_free)(void *) = nullptr;
@@ -993,13 +1024,6 @@ qml_status efail(qml_status s, const std::string &m) {
   return s;
 }
 
-template <class T>
-T *emu_alloc(qml_emu *e, size_t count) {
-  void *p = nullptr;
-  if (cudaMalloc(&p, count * sizeof(T)) != cudaSuccess) return nullptr;
-  e->mem.push_back(p);
-  return (T *)p;
-}
 
 // activations of one batch (Brows a multiple of 16)
 struct Acts {
@@ -1009,21 +1033,21 @@ struct Acts {
   float *dZf = nullptr, *dX = nullptr, *tb = nullptr;
   __nv_bfloat16 *dZh = nullptr;
   double *partial = nullptr, *loss = nullptr;
-  std::vector<void *> mem;
-  ~Acts() {
-    for (void *p : mem) cudaFree(p);
-  }
+  Slab mem;
   template <class T>
   T *a(size_t count) {
-    void *p = nullptr;
-    if (cudaMalloc(&p, count * sizeof(T)) != cudaSuccess) return nullptr;
-    mem.push_back(p);
-    return (T *)p;
+    return mem.take<T>(count);
   }
-  bool make(const qml_emu *e, int Brows) {
+  // extra: bytes (in Slab steps) for buffers the caller takes afterwards
+  bool make(const qml_emu *e, int Brows, size_t extra = 0) {
     B = Brows;
     int maxw = kIn0;
     for (auto &l : e->layers) maxw = std::max(maxw, std::max(l.first, l.second));
+    size_t total = extra + 2 * Slab::step((size_t)B * maxw * 4) + Slab::step((size_t)B * maxw * 2) +
+                   Slab::step((size_t)B * 4) + Slab::step(256 * 8) + Slab::step(8);
+    for (auto &l : e->layers)
+      total += Slab::step((size_t)B * l.second * 2) + Slab::step((size_t)B * l.first * 4);
+    if (!mem.make(total)) return false;
     for (auto &l : e->layers) {
       X.push_back(a<__nv_bfloat16>((size_t)B * l.second));
       Z.push_back(a<float>((size_t)B * l.first));
@@ -1154,18 +1178,20 @@ struct FusedTrain {
   float *dZf[2][2] = {}, *grad[2] = {};
   __nv_bfloat16 *dZh[2][2] = {};
   bool make(qml_emu *e, int batch, Acts &first) {
-    if (!own.make(e, batch)) return false;
-    A[0] = &first;
-    A[1] = &own;
     int maxw = kIn0;
     for (auto &l : e->layers) maxw = std::max(maxw, std::max(l.first, l.second));
+    const size_t cells = (size_t)batch * maxw;
+    if (!own.make(e, batch, Slab::step(e->nparam * 4) + 2 * (Slab::step(cells * 4) + Slab::step(cells * 2))))
+      return false;
+    A[0] = &first;
+    A[1] = &own;
     grad[0] = e->grad;
     grad[1] = own.a<float>(e->nparam);
     for (int h = 0; h < 2; ++h) {
       dZf[h][0] = A[h]->dZf;
       dZh[h][0] = A[h]->dZh;
-      dZf[h][1] = own.a<float>((size_t)batch * maxw);
-      dZh[h][1] = own.a<__nv_bfloat16>((size_t)batch * maxw);
+      dZf[h][1] = own.a<float>(cells);
+      dZh[h][1] = own.a<__nv_bfloat16>(cells);
       if (!dZf[h][1] || !dZh[h][1]) return false;
     }
     return grad[1] != nullptr;
@@ -1469,17 +1495,27 @@ qml_status emu_create(int32_t ndim, const double *lo, const double *hi, int32_t 
     c[i] = 0.5 * (hi[i] + lo[i]);
     hw[i] = 0.5 * (hi[i] - lo[i]);
   }
-  e->centre = emu_alloc<double>(e, ndim);
-  e->half = emu_alloc<double>(e, ndim);
-  e->coef = emu_alloc<double>(e, kMaxFeat);
-  e->midx = emu_alloc<unsigned char>(e, kMaxFeat * kMaxDim);
-  e->sigma = emu_alloc<double>(e, 1);
-  e->grad = emu_alloc<float>(e, e->nparam);
+  {
+    const size_t np = (size_t)e->nparam;
+    const size_t total = 2 * Slab::step(ndim * 8) + Slab::step(kMaxFeat * 8) +
+                         Slab::step(kMaxFeat * kMaxDim) + Slab::step(8) + 7 * Slab::step(np * 4) +
+                         2 * Slab::step(np * 2);
+    if (!e->mem.make(total)) {
+      delete e;
+      return efail(QML_ENOMEM, "emu_create: device allocation failed");
+    }
+  }
+  e->centre = e->mem.take<double>(ndim);
+  e->half = e->mem.take<double>(ndim);
+  e->coef = e->mem.take<double>(kMaxFeat);
+  e->midx = e->mem.take<unsigned char>(kMaxFeat * kMaxDim);
+  e->sigma = e->mem.take<double>(1);
+  e->grad = e->mem.take<float>(e->nparam);
   for (int h = 0; h < 2; ++h) {
-    e->p[h] = emu_alloc<float>(e, e->nparam);
-    e->m[h] = emu_alloc<float>(e, e->nparam);
-    e->v[h] = emu_alloc<float>(e, e->nparam);
-    e->ph[h] = emu_alloc<__nv_bfloat16>(e, e->nparam);
+    e->p[h] = e->mem.take<float>(e->nparam);
+    e->m[h] = e->mem.take<float>(e->nparam);
+    e->v[h] = e->mem.take<float>(e->nparam);
+    e->ph[h] = e->mem.take<__nv_bfloat16>(e->nparam);
   }
   if (!e->centre || !e->half || !e->coef || !e->midx || !e->sigma || !e->grad || !e->p[1] ||
       !e->ph[1]) {
@@ -1519,7 +1555,6 @@ void emu_free(qml_emu *emu) {
   if (!emu) return;
   cudaDeviceSynchronize();
   if (emu->pcache && emu->pcache_free) emu->pcache_free(emu->pcache);
-  for (void *p : emu->mem) cudaFree(p);
   delete emu;
 }
 
@@ -1568,18 +1603,17 @@ qml_status emu_train(qml_emu *e, int32_t n, const double *theta, const double *l
     multi_indices(e->d, e->deg, mi);
     cudaMemcpy(e->midx, mi.data(), mi.size(), cudaMemcpyHostToDevice);
   }
-  cudaMalloc(&res, n * sizeof(double));
-  cudaMalloc(&part, 256 * sizeof(double));
-  cudaMalloc(&sumsq, sizeof(double));
-  cudaMalloc(&targ, n * sizeof(float));
-  cudaMalloc(&phi, (size_t)n * nf * sizeof(double));
-  cudaMalloc(&gram, (size_t)nf * (nf + 1) * sizeof(double));
-  keep.push_back(res);
-  keep.push_back(part);
-  keep.push_back(sumsq);
-  keep.push_back(targ);
-  keep.push_back(phi);
-  keep.push_back(gram);
+  Slab tmp;  // freed after the stream has been synchronised on every path out
+  if (tmp.make(Slab::step(n * 8) + Slab::step(256 * 8) + Slab::step(8) + Slab::step(n * 4) +
+               Slab::step((size_t)n * nf * 8) + Slab::step((size_t)nf * (nf + 1) * 8) +
+               2 * Slab::step((size_t)n_val * 8) + Slab::step((size_t)n_val * 4))) {
+    res = tmp.take<double>(n);
+    part = tmp.take<double>(256);
+    sumsq = tmp.take<double>(1);
+    targ = tmp.take<float>(n);
+    phi = tmp.take<double>((size_t)n * nf);
+    gram = tmp.take<double>((size_t)nf * (nf + 1));
+  }
   auto cleanup = [&]() {
     cudaStreamSynchronize(st);
     for (void *p : keep) cudaFree(p);
@@ -1709,12 +1743,9 @@ qml_status emu_train(qml_emu *e, int32_t n, const double *theta, const double *l
     // hull: those are always evaluated exactly and do not calibrate
     double *vd = nullptr, *vo = nullptr;
     int *vf = nullptr;
-    cudaMalloc(&vd, n_val * sizeof(double));
-    cudaMalloc(&vo, n_val * sizeof(double));
-    cudaMalloc(&vf, n_val * sizeof(int));
-    keep.push_back(vd);
-    keep.push_back(vo);
-    keep.push_back(vf);
+    vd = tmp.take<double>(n_val);
+    vo = tmp.take<double>(n_val);
+    vf = tmp.take<int>(n_val);
     const qml_status ps = (!vd || !vo || !vf)
                               ? QML_ENOMEM
                               : run_predict(e, n_val, th + (int64_t)n * e->d, INFINITY, vo, vf,

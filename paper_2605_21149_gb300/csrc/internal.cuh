@@ -65,11 +65,21 @@ void launch_dgemm_fixed(int ta, int tb, int64_t M, int64_t N, int64_t K, double 
                         const double *A, int64_t lda, const double *B, int64_t ldb, double beta,
                         double *C, int64_t ldc, int lower, const DevStatus *status,
                         cudaStream_t st);
-// strided batch: product z uses A + z sA, B + z sB, C + z sC (no aliasing)
-void launch_dgemm_batched(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
-                          const double *A, int64_t lda, int64_t sA, const double *B,
-                          int64_t ldb, int64_t sB, double beta, double *C, int64_t ldc,
-                          int64_t sC, int count, const DevStatus *status, cudaStream_t st);
+// The small products inside a 512-wide panel: C_z <- alpha A_z op(B_z) + beta
+// C_z for z < count (X_z = X + z sX), K <= 256, no aliasing; op(B) = B^T when tb.
+// tri: 1, B (not transposed) is lower triangular; 2, A is; 0, neither.  Never
+// allocates, tunes or synchronises; fit for any stream.
+void launch_panel_gemm(int tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A,
+                       int64_t lda, int64_t sA, const double *B, int64_t ldb, int64_t sB,
+                       double beta, double *C, int64_t ldc, int64_t sC, int lower, int tri,
+                       int count, const DevStatus *status, cudaStream_t st);
+
+// C (M x N) <- alpha A B + beta C for N <= kSkinnyN, K <= 512, A column-major; no
+// aliasing.  Bcopy (ld ldbc), when given, receives B.
+constexpr int kSkinnyN = 8;
+void launch_skinny(int64_t M, int64_t N, int64_t K, double alpha, const double *A, int64_t lda,
+                   const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
+                   double *Bcopy, int64_t ldbc, const DevStatus *status, cudaStream_t st);
 
 constexpr int kNB = 64;  // Cholesky / TRSM block size
 
