@@ -769,8 +769,8 @@ __global__ void predict_combine_kernel(int off, int cnt, const double *q, const 
 // 128-byte-swizzled stages of 64 columns) and then streams the tiles' X
 // through a ring of kTcRing 64-column slots; warp 1 owns the TMEM allocation
 // and issues each tile's K / 16 MMAs (M = 128, N) into one of two
-// accumulators; warps 2-9 are the epilogue (TMEM lanes 32 (w % 4) .., column
-// half (w - 2) / 4), which adds the bias and writes bf16(gelu(Y)) to Xn for a
+// accumulators; warps 2-17 are the epilogue (TMEM lanes 32 (w % 4) .., column
+// quarter (w - 2) / 4), which adds the bias and writes bf16(gelu(Y)) to Xn for a
 // hidden layer or fp32 Y to Z for the output layer.  With two accumulators a
 // tile's epilogue runs while the next tile's X arrives and is multiplied.
 // Every wait is bounded: on expiry the status takes QML_ETIMEOUT, copies and
@@ -778,7 +778,12 @@ __global__ void predict_combine_kernel(int off, int cnt, const double *q, const 
 // written.
 constexpr int kTcMaxStages = 4;  // K <= 256
 constexpr int kTcRing = 4;       // X slots of 64 columns
-constexpr int kTcThreads = 320;
+// 16 epilogue warps, four on each SM sub-partition: a GELU is a chain of two
+// special-function results and a dozen dependent multiply-adds, and with two
+// warps a sub-partition their latencies showed (86 us a hidden layer of 2^18
+// points, 50 issue slots a value for 25 instructions)
+constexpr int kTcEpiWarps = 16;
+constexpr int kTcThreads = 64 + 32 * kTcEpiWarps;
 template <int N>
 constexpr size_t tc_smem() {
   return 1024 + (size_t)kTcMaxStages * N * 128 + (size_t)kTcRing * 128 * 128 + 256;
@@ -791,7 +796,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   constexpr int kA = 128 * 128, kB = N * 128;  // bytes of one 64-column stage
   constexpr int kCols = N <= 32 ? 32 : (N <= 64 ? 64 : (N <= 128 ? 128 : 256));
-  constexpr int kEpiThreads = N > 16 ? 256 : 128;
+  constexpr int kEpiThreads = N > 16 ? 32 * kTcEpiWarps : 128;
   constexpr uint32_t kIdescN = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
                                ((uint32_t)(128 >> 4) << 24);
   unsigned char *tB = smem, *tA = smem + kTcMaxStages * kB;
@@ -872,8 +877,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   } else if (go && warp >= 2 && (N > 16 || warp < 6)) {
     // ---- epilogue
     const int quad = warp & 3;
-    const int half = N > 16 ? (warp - 2) >> 2 : 0;
-    constexpr int kW = N > 16 ? N / 2 : N;  // columns per epilogue warp
+    const int part = N > 16 ? (warp - 2) >> 2 : 0;
+    constexpr int kW = N > 16 ? N / (kTcEpiWarps / 4) : N;  // columns per epilogue warp
     uint32_t it = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
       const uint32_t bsel = it & 1u;
@@ -884,12 +889,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (!okw) break;
       tc_fence_after();
       const int row = 128 * t + quad * 32 + lane;
-      const uint32_t lb = tbase + bsel * kCols + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * kW);
+      const uint32_t lb = tbase + bsel * kCols + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * kW);
 #pragma unroll 1
       for (int cb = 0; cb < kW / 16; ++cb) {
         uint32_t a[16];
         tmem_ld16(lb + 16 * cb, a);
-        const int c0 = half * kW + 16 * cb;
+        const int c0 = part * kW + 16 * cb;
         // bias + c0 is 64-byte aligned: every layer's bias starts at a
         // multiple of 16 floats of the parameter block (widths are multiples
         // of 16), and the launch checks the block's alignment
