@@ -397,8 +397,9 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   forward substitution (not while the stream is being
  *                   captured) / everything in order on the caller's stream;
  *                   the results are bit-identical
- *   split_lookahead_sms  8 (default): SMs the split kernel leaves free for
- *                   that chain while they overlap
+ *   split_lookahead_sms  (default 24 for matrices below 10000 rows, else 8)
+ *                   SMs the split kernel leaves free for that chain while
+ *                   they overlap
  *   split_diag_df   0 (default) / 1: the split-precision Cholesky factors
  *                   its 64-wide diagonal blocks and their row solves in
  *                   float64 / in float-float (about 2^-46 per operation)

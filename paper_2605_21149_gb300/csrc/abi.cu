@@ -541,7 +541,7 @@ void panel_chain(Call &c, Split &sp, double *A, int64_t lda, int64_t j, int64_t 
 // and the rest; right after the first part, the next panel's float64 chain
 // starts on a second, high-priority stream, while the main stream runs the
 // rest of the trailing update and panel j's substitution on B with
-// split_lookahead_sms SMs (default 8) left free for the chain.  The float64
+// split_lookahead_sms SMs (default 24 below n = 10000, 8 above) left free for the chain.  The float64
 // chain (about 0.8 ms a panel at n = 5952) then hides behind split products.
 // Every output is the same product as without lookahead (the split product
 // of an element depends only on its own row and column), so the results are
@@ -566,7 +566,11 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
            cudaEventCreateWithFlags(&e_next, cudaEventDisableTiming) == cudaSuccess &&
            cudaEventCreateWithFlags(&e_diag, cudaEventDisableTiming) == cudaSuccess;
   }
-  const int reserve = look ? (int)tune_get("split_lookahead_sms", 8) : 0;
+  // The chain of a panel takes the same time whatever n is, the products beside
+  // it shrink with n: at n = 5952 the solve takes 40.3 ms (float64) and 33.5
+  // (split) with 8 SMs for the chain, 39.7 and 32.6 with 24; at n = 17152 294
+  // and 305.
+  const int reserve = look ? (int)tune_get("split_lookahead_sms", n < 10000 ? 24 : 8) : 0;
   panel_chain(c, sp, A, lda, 0, n < kNBS ? n : kNBS, Linv64, LinvB, ldparts, dfdiag, c.st, false);
   for (int64_t j = 0; j < n && c.err == QML_OK; j += kNBS) {
     const int64_t jb = (n - j) < kNBS ? (n - j) : kNBS;
