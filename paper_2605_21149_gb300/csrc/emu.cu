@@ -344,7 +344,7 @@ __global__ void pad_cols_kernel(const __nv_bfloat16 *src, int rows, int cols, __
 // gradient, bias gradient, and the next dZ = (dZ W) gelu'), Adam.  At a batch
 // of 64 every launch is latency: a head's step took 30 launches and 230 us, its
 // products on four CTAs of 64 x 64 that load a fragment at a time.  Here a warp
-// owns one 16 x 16 tile and loads four K steps of fragments ahead.  Every
+// owns one 16 x 16 tile and loads eight K steps of fragments ahead.  Every
 // output is the same sum in the same order as in the separate kernels above
 // (mma.sync over ascending k; the bias gradient over ascending rows).
 struct TrainHeads {
@@ -362,18 +362,19 @@ struct TrainHeads {
 };
 constexpr int kTrWarps = 4, kTrLd = 20;  // tiles per CTA; row stride of a staged tile
 
-// acc += A B over K (a multiple of 16), fragments of four K steps in flight
+// acc += A B over K (a multiple of 16), fragments of kTrAhead K steps in flight
+constexpr int kTrAhead = 8;
 template <typename ALay, typename BLay>
 __device__ __forceinline__ void tile_product(
     wmma::fragment<wmma::accumulator, 16, 16, 16, float> &acc, const __nv_bfloat16 *A, int lda,
     const __nv_bfloat16 *B, int ldb, int K) {
   constexpr bool ar = std::is_same<ALay, wmma::row_major>::value;
   constexpr bool br = std::is_same<BLay, wmma::row_major>::value;
-  for (int k = 0; k < K; k += 64) {
-    wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, ALay> a[4];
-    wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, BLay> b[4];
+  for (int k = 0; k < K; k += 16 * kTrAhead) {
+    wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, ALay> a[kTrAhead];
+    wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, BLay> b[kTrAhead];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kTrAhead; ++u) {
       const int kk = k + 16 * u;
       if (kk < K) {
         wmma::load_matrix_sync(a[u], ar ? A + kk : A + (int64_t)kk * lda, lda);
@@ -381,7 +382,7 @@ __device__ __forceinline__ void tile_product(
       }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < kTrAhead; ++u)
       if (k + 16 * u < K) wmma::mma_sync(acc, a[u], b[u], acc);
   }
 }
@@ -1149,12 +1150,18 @@ bool forward_tc(qml_emu *e, int h, Acts &A, int rows, const std::vector<CUtensor
 }
 
 // gradient of the mean squared error of head h over the first nreal rows
-void backward(qml_emu *e, int h, Acts &A, int nreal, cudaStream_t st) {
+// mean squared error of the output and its gradient
+void output_loss(qml_emu *e, Acts &A, int nreal, cudaStream_t st) {
   const int nl = (int)e->layers.size();
   loss_grad_kernel<<<64, 256, 0, st>>>(A.Z[nl - 1], A.tb, A.B, nreal, A.dZf, A.dZh, A.partial);
   count_launch();
   sum_partials_kernel<<<1, 32, 0, st>>>(A.partial, 64, 1.0 / nreal, A.loss);
   count_launch();
+}
+
+void backward(qml_emu *e, int h, Acts &A, int nreal, cudaStream_t st) {
+  const int nl = (int)e->layers.size();
+  output_loss(e, A, nreal, st);
   for (int l = nl - 1; l >= 0; --l) {
     const int out = e->layers[l].first, in = e->layers[l].second;
     // dW = dZ^T X: A = dZ^T (out x B) = dZ col-major (ld out), B = X (B x in) row-major
@@ -1733,8 +1740,9 @@ qml_status emu_train(qml_emu *e, int32_t n, const double *theta, const double *l
         gather_kernel<<<grid_of((int64_t)Be * kIn0), 256, 0, st>>>(th, n, e->d, e->centre, e->half,
                                                                    targ, Be, ne, 0, 1, E.X[0], E.tb);
         count_launch();
+        // (the loss alone: a backward pass over 4096 rows took 5 ms a head)
         forward(e, h, E, st);
-        backward(e, h, E, ne, st);
+        output_loss(e, E, ne, st);
         cudaMemcpyAsync(&final_loss[h], E.loss, sizeof(double), cudaMemcpyDeviceToHost, st);
         cudaStreamSynchronize(st);
       }
