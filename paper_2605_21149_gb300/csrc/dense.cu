@@ -351,6 +351,130 @@ __device__ void invert_lower_blocked(double (*a)[kLDA], double (*x)[kLDA], const
   }
 }
 
+// 1 / d for a normal d > 0 away from the range limits: a float32 quotient of the
+// mantissa r0, then the cubic step r0 (1 + e + e^2), e = 1 - d r0 (|e| below
+// 2^-22, so the result is within a rounding of 1 / d).  Three float64
+// instructions; the conversions are integer operations.
+__device__ __forceinline__ double recip_pos(double d) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const float m = __uint_as_float(0x3F800000u | (hi & 0xFFFFFu) << 3 | lo >> 29);
+  const uint32_t rb = __float_as_uint(__fdividef(1.0f, m));  // in (1/2, 1]
+  const int ex = (int)(rb >> 23) - 127 - ((int)(hi >> 20) - 1023) + 1023;
+  const double r0 = __hiloint2double((int)((uint32_t)ex << 20 | (rb & 0x7FFFFFu) >> 3),
+                                     (int)((rb & 7u) << 29));
+  const double e = fma(-d, r0, 1.0);
+  return fma(r0, fma(e, e, e), r0);
+}
+
+// Factor of the jb x jb block in a (lower triangle, in place) as L~ D L~^T, then
+// L = L~ D^(1/2); false when a pivot is not positive (the error recorded).
+// What bounds a block is float64 issue (a warp instruction holds its SM
+// sub-partition for 76 clocks), so the number of instructions on the busiest
+// sub-partition is what counts.  Without square roots a pivot costs 3 (its
+// reciprocal) + 1 + one a remaining panel column instead of about 8 + 1 + ...;
+// the 64 square roots are taken at the end, a lane each.  And the trailing
+// update is split: the next panel's eight columns at once by all warps, the
+// rest by warps 3-7 while warps 0-2 factor that panel (of 1977 instructions
+// that is close to an even share for each sub-partition).  50 us a block
+// before, with both phases in turn.
+//   w: two buffers of kNB x 9 (a panel's columns before division), dv: kNB.
+__device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *invd, int jb,
+                           int64_t j0, int *bad, DevStatus *status) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int c0 = 0, par = 0; c0 < jb; c0 += kPW, par ^= 1) {
+    const int cend = (c0 + kPW < jb) ? c0 + kPW : jb;
+    double *wp = w + par * (kNB * 9);
+    if (warp < 3) {
+      // the panel: the 8 x 8 pivot block in lanes 0-7 of each of the warps (the
+      // same operations on the same values), 24 rows below it in lanes 8-31
+      if (warp == 0 || c0 + kPW + 24 * warp < jb) {
+        const int row = lane < kPW ? c0 + lane : c0 + kPW + 24 * warp + (lane - kPW);
+        const bool live = row < jb;
+        double v[kPW], l[kPW];
+#pragma unroll
+        for (int q = 0; q < kPW; ++q) v[q] = (c0 + q < cend && live) ? a[row][c0 + q] : 0.0;
+        int fail_col = -1;
+#pragma unroll
+        for (int q = 0; q < kPW; ++q) {
+          const int c = c0 + q;
+          l[q] = 0.0;
+          if (c < cend && fail_col < 0) {
+            const double d = __shfl_sync(0xffffffffu, v[q], q);  // a_cc: lane q holds row c
+            const uint32_t hi = (uint32_t)__double2hiint(d);
+            if (hi - 0x00100000u >= 0x7FE00000u) {  // <= 0, subnormal, infinite or NaN
+              fail_col = c;
+            } else {
+              l[q] = v[q] * recip_pos(d);
+              if (warp == 0 && lane == 0) dv[c] = d;
+              double lj[kPW];
+#pragma unroll
+              for (int qj = q + 1; qj < kPW; ++qj) lj[qj] = __shfl_sync(0xffffffffu, l[q], qj);
+#pragma unroll
+              for (int qj = q + 1; qj < kPW; ++qj) v[qj] = fma(-v[q], lj[qj], v[qj]);
+            }
+          }
+        }
+        if (fail_col >= 0) {
+          if (warp == 0 && lane == 0) {
+            *bad = 1;
+            // the first error of the call is the one reported
+            if (atomicCAS(&status->code, 0, 2 /* QML_ENOTSPD */) == 0)
+              status->info = (int)(j0 + fail_col + 1);
+          }
+        } else if (live && (warp == 0 || lane >= kPW)) {
+          // (above the diagonal of the pivot block nothing is stored or read)
+#pragma unroll
+          for (int q = 0; q < kPW; ++q)
+            if (c0 + q < cend && row > c0 + q) {
+              a[row][c0 + q] = l[q];
+              wp[row * 9 + q] = v[q];
+            }
+        }
+      }
+    } else if (c0 > 0) {
+      // the previous panel's update of the columns behind this one
+      const double *wq = w + (par ^ 1) * (kNB * 9);
+      const int b0 = c0 - kPW, c1 = c0 + kPW, m = jb > c1 ? jb - c1 : 0;
+      for (int t = tid - 96; t < m * (m + 1) / 2; t += 160) {
+        int r = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+        while ((r + 1) * (r + 2) / 2 <= t) ++r;
+        while (r * (r + 1) / 2 > t) --r;
+        const int i = c1 + r, j = c1 + (t - r * (r + 1) / 2);
+        double s = a[i][j];
+#pragma unroll
+        for (int q = 0; q < kPW; ++q) s = fma(-a[i][b0 + q], wq[j * 9 + q], s);
+        a[i][j] = s;
+      }
+    }
+    __syncthreads();
+    if (*bad) return false;
+    // this panel's update of the next one's columns
+    for (int t = tid; t < kPW * (jb - cend); t += blockDim.x) {
+      const int i = cend + (t >> 3), j = cend + (t & 7);
+      if (j < jb && i >= j) {
+        double s = a[i][j];
+#pragma unroll
+        for (int q = 0; q < kPW; ++q) s = fma(-a[i][c0 + q], wp[j * 9 + q], s);
+        a[i][j] = s;
+      }
+    }
+    __syncthreads();
+  }
+  if (tid < jb) {
+    const double sq = sqrt(dv[tid]);
+    a[tid][tid] = sq;
+    invd[tid] = 1.0 / sq;
+    dv[tid] = sq;
+  }
+  __syncthreads();
+  for (int t = tid; t < jb * jb; t += blockDim.x) {
+    const int i = t % jb, j = t / jb;
+    if (i > j) a[i][j] *= dv[j];
+  }
+  __syncthreads();
+  return true;
+}
+
 // mode 1: factor and invert; mode 2: factor only, and Linv receives the
 // scaled coefficients of the row solve x L^T = b (trsm_rows_kernel) instead of
 // an inverse, Linv[c kNB + j] = L_jc / L_jj (j > c), 1 / L_cc (j = c), 0
@@ -430,7 +554,25 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_kernel(double *A, int64_t l
   }
   if (tid == 0) *bad = 0;
   __syncthreads();
+  bool in_range = true;
   if (factor) {
+    // every diagonal entry of a plain size, or not positive (found below): no
+    // pivot, at least 2^-53 of its entry if it is positive, is near the limits
+    // where a reciprocal would be
+    bool ok = true;
+    if (tid < jb) {
+      const uint32_t e = (uint32_t)__double2hiint(a[tid][tid]) >> 20;
+      ok = e - 512u < 1024u || e >= 0x7FFu;
+    }
+    in_range = __syncthreads_and(ok) != 0;
+  }
+  if (factor && in_range) {
+    if (!factor_ldl(a, dsm + kNB * kLDA, tmp, invd, jb, j0, bad, status)) return;
+    if (mode == 1) {  // the inverse starts from zeros
+      for (int t = tid; t < kNB * kLDA; t += blockDim.x) dsm[kNB * kLDA + t] = 0.0;
+      __syncthreads();
+    }
+  } else if (factor) {
     // Warps 0-2 each factor the panel's 8 x 8 pivot block in lanes 0-7 (the
     // same operations on the same values, so identical results) and carry 24
     // rows of their own below it in lanes 8-31: one row per lane, and the
@@ -532,6 +674,8 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_kernel(double *A, int64_t l
       }
       __syncthreads();
     }
+  }
+  if (factor) {
     for (int t = tid; t < jb * jb; t += blockDim.x) {
       int i = t % jb, j = t / jb;
       if (i >= j) A[i + j * lda] = a[i][j];
