@@ -579,10 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       for (int cb = 0; cb < kEpiCols / kLd; ++cb) {
         uint32_t a[kLd];
         auto load = [&] {
-          if (kLd == 32)
-            tmem_ld32_async(lbase + kLd * cb, a);
-          else
-            tmem_ld16_async(lbase + kLd * cb, a);
+          tmem_ld32_async(lbase + kLd * cb, a);
           tmem_ld_wait();
           // (the loaded registers pass through the wait, so no use moves above it)
 #pragma unroll

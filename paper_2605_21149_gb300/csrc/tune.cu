@@ -7,7 +7,8 @@
 //                    2^24 entries, K at most 4096, C not aliasing A or B, the
 //                    stream not capturing) and keep the fastest; 0: built-in
 //                    heuristic only
-//   dgemm:<ta>,<tb>,<lower>,<M>,<N>,<K>,<alias>   measured tile, 10 RM + RN
+//   dgemm:<ta>,<tb>,<lower>,<M>,<N>,<K>,<alias>   measured tile, 10 RM + RN,
+//                    or 10 for the kernel with the whole K range on chip
 //   batch_streams    worker streams of pix_loglike_batch (default 8, 1..16)
 //   ozaki_stages     4 (default) .. 2: depth of the split kernel's ring
 //   emu_tc           1 (default) / 0: emulator inference layers on tcgen05
@@ -19,8 +20,9 @@
 //                    1: in float-float (pairs of float32, about 2^-46 per
 //                    operation; faster on this part's narrow float64 pipe)
 //   batch_split_kt   0 (default): with split-precision masks the per-item
-//                    inner factor Kt of pix_loglike_batch is native float64;
-//                    1: its trailing updates and panel products are split
+//                    inner factor Kt of pix_loglike_batch is as accurate as
+//                    QML_FP64; 1: its trailing updates and panel products
+//                    have 48 bits
 //   test_wait_timeout  1: failure-path test; the split-precision kernel
 //                    issues no copies and gives up each wait after 1 ms
 //   batch_graphs     1 (default): pix_loglike_batch captures each worker's
