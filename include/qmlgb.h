@@ -239,7 +239,7 @@ typedef struct {
  * dimension ld_out >= the largest nmaps): lnL[i*ld_out + j], chi2[...] and
  * logdet[i]; any may be NULL.  The per-mask part (Cholesky of N, M, Y^T N^-1 d)
  * runs once; items are spread round-robin over internal worker streams
- * (tuning key batch_streams, default 8).  Errors: QML_EINVAL,
+ * (tuning key batch_streams).  Errors: QML_EINVAL,
  * QML_ENOTSPD (N not positive definite), QML_ETIMEOUT. */
 qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitems,
                              const int32_t *item_mask, const double *item_cl, int32_t ld_out,
@@ -352,7 +352,9 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *   dgemm:<ta>,<tb>,<lower>,<M>,<N>,<K>,<alias>  a measured tile (10 RM + RN,
  *                   tile 16 RM x 16 RN; 10: 16 x 16 tiles with the whole K
  *                   range in shared memory); unknown values are ignored
- *   batch_streams   worker streams of pix_loglike_batch (default 8, 1..16)
+ *   batch_streams   worker streams of pix_loglike_batch (1..16; default 8,
+ *                   4 from k = 10000 modes on; fewer than asked for, but at
+ *                   least 4, where their scratch does not fit)
  *   batch_graphs    1 (default) / 0: pix_loglike_batch replays each worker's
  *                   per-item kernel sequence as a captured CUDA graph
  *   ozaki_stages    4 (default) / 3 / 2: depth of the split kernel's ring of

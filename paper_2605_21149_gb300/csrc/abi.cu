@@ -97,6 +97,18 @@ struct Call {
     return (T *)p;
   }
 
+  // alloc without the error: nullptr when the device has no room
+  void *try_alloc(size_t bytes) {
+    if (err != QML_OK) return nullptr;
+    void *p = nullptr;
+    if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    bufs.push_back(p);
+    return p;
+  }
+
   // device view of an input array (copied in when it lives on the host)
   template <class T>
   const T *in(const T *p, size_t count, const char *what) {
@@ -373,6 +385,11 @@ void build_C(Call &c, const Staged &s, const Dims &d, double *Y, double *C) {
 // the panel solve and trailing update run as split-precision products with
 // K = kNBS.
 constexpr int64_t kNBS = 512;
+// Digits of at most this many columns of K exist at a time: 14 bytes an element
+// would otherwise take more than the operands of the largest problems (n = k =
+// 80000: 27 GB, not 90).  Reading and writing a tile of C takes 1 % of a piece
+// this long.
+constexpr int64_t kDigitK = 24576;
 
 // One digit buffer of the split products (oz_digits_bytes large), taken from
 // a caller's workspace or allocated on first use and grown as needed.
@@ -433,17 +450,40 @@ struct Split {
     else
       launch_copy_matrix(X, jb, Bj, ldb, jb, nrhs, c->st);
   }
+  // buffer i holds `need` bytes, if the device has the room
+  bool room(int i, size_t need) {
+    if (need <= buf[i].bytes) return true;
+    void *p = c->try_alloc(need);
+    if (p) buf[i] = DigitBuf{p, need};
+    return p != nullptr;
+  }
+  // C <- alpha op(A) op(B) + beta C, kDigitK of K at a time (one more rounding
+  // of C each).  A QML_FP64 problem that fills the device has no digits in its
+  // float64 form: it takes shorter pieces of K while the buffers do not fit,
+  // and below kNBS the float64 pipe.
   void gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A,
             int64_t lda, const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
             int lower) {
     if (c->err != QML_OK || M <= 0 || N <= 0) return;
-    const OzDigits a = slice(0, A, M, K, ta ? lda : 1, ta ? 1 : lda);
-    if (A == B && lda == ldb && ta != tb && M == N) {
-      mm(M, N, alpha, a, 0, a, 0, beta, C, ldc, lower);
-      return;
+    const bool same = A == B && lda == ldb && ta != tb && M == N;
+    int64_t kc = K < kDigitK || C == A || C == B ? K : kDigitK;  // (in place: all digits first)
+    while (f64 && !(room(0, oz_digits_bytes(M, kc, S)) &&
+                    (same || room(1, oz_digits_bytes(N, kc, S))))) {
+      if (kc <= kNBS) {
+        launch_dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, c->status, c->st);
+        return;
+      }
+      kc = (kc / 2 + 63) / 64 * 64;
     }
-    const OzDigits b = slice(1, B, N, K, tb ? 1 : ldb, tb ? ldb : 1);
-    mm(M, N, alpha, a, 0, b, 0, beta, C, ldc, lower);
+    int64_t k0 = 0;
+    do {
+      const int64_t kb = K - k0 < kc ? K - k0 : kc;
+      const OzDigits a = slice(0, A + k0 * (ta ? 1 : lda), M, kb, ta ? lda : 1, ta ? 1 : lda);
+      const OzDigits b =
+          same ? a : slice(1, B + k0 * (tb ? ldb : 1), N, kb, tb ? 1 : ldb, tb ? ldb : 1);
+      mm(M, N, alpha, a, 0, b, 0, k0 ? 1.0 : beta, C, ldc, lower);
+      k0 += kb;
+    } while (k0 < K);
   }
 };
 // the buffers potrf_split and trsm_split need for an n x n factor and nrhs
@@ -1286,9 +1326,11 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   // (eight by default: the chain of 64-wide float64 blocks that an item's factor
   // waits on leaves most of the GPU to other items.  256 items of k = 756: 122
   // ms with four workers, 77 with eight or sixteen; 24 items of k = 6900: 305,
-  // 283, 281)
-  const int ns_max = (int)std::max<int64_t>(1, std::min<int64_t>(16, tune_get("batch_streams", 8)));
-  const int NS = nitems < ns_max ? nitems : ns_max;
+  // 283, 281.  From k = 10000 on four, whose products fill the GPU and whose k x
+  // k scratch is 0.8 GB and more each)
+  const int ns_max = (int)std::max<int64_t>(
+      1, std::min<int64_t>(16, tune_get("batch_streams", k < 10000 ? 8 : 4)));
+  int NS = nitems < ns_max ? nitems : ns_max;
   // CUDA graphs: item 0 runs as plain launches (so that the tile autotuner
   // can time its shapes), then each (worker, mask) pair captures its per-item
   // sequence once -- reading the spectrum from a fixed per-worker slot and
@@ -1320,7 +1362,14 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   const int64_t nbk = (k + kNB - 1) / kNB, nbbk = (k + kNBS - 1) / kNBS;
   double *lnK = c.alloc<double>(nitems);
   for (int w = 0; w < NS; ++w) {
-    wk[w].K = c.alloc<double>((size_t)k * k, "Kt");
+    // the workers beyond four only where the device has room for their scratch
+    wk[w].K = w < 4 ? c.alloc<double>((size_t)k * k, "Kt")
+                    : (double *)c.try_alloc(sizeof(double) * k * k);
+    if (w >= 4 && !wk[w].K && c.err == QML_OK) {
+      NS = w;
+      wk.resize(NS);
+      break;
+    }
     wk[w].lamL = c.alloc<double>((size_t)d0.nl * d0.nc * d0.nc);
     wk[w].z = c.alloc<double>((size_t)k * maxmaps);
     wk[w].rr = c.alloc<double>(maxmaps);
@@ -1584,13 +1633,8 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
               "C");
   if (!c.make_status()) return c.finish();
   if (precision == QML_SPLIT_BF16 && kk > 0) {  // (kk == 0: C <- beta C, no digits)
-    const bool shared = (A == B && lda == ldb && transA != transB && m == nn);
-    const int S = oz_split_digits(0);
-    void *ws = c.alloc<unsigned char>(ozaki_workspace_bytes(m, nn, kk, S, shared), "split workspace");
-    if (!ws) return c.finish();
-    c.cuda_ok(ozaki_gemm(transA, transB, m, nn, kk, alpha, Ad, lda, Bd, ldb, beta, Cd, ldc, lower,
-                         S, ws, c.status, c.st),
-              "split-precision gemm");
+    Split spl{&c, oz_split_digits(0)};
+    spl.gemm(transA, transB, m, nn, kk, alpha, Ad, lda, Bd, ldb, beta, Cd, ldc, lower);
     return c.finish();
   }
   launch_dgemm(transA, transB, m, nn, kk, alpha, Ad, lda, Bd, ldb, beta, Cd, ldc, lower, c.status,

@@ -236,12 +236,5 @@ void oz_slice(const double *X, int64_t sr, int64_t sk, const OzDigits &d, cudaSt
 cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t ra,
                   const OzDigits &B, int64_t rb, double beta_c, double *C, int64_t ldc, int lower,
                   DevStatus *status, cudaStream_t st, int reserve_sms = 0);
-// Both steps, same operand conventions as launch_dgemm; `work` must hold
-// ozaki_workspace_bytes(...) bytes.
-size_t ozaki_workspace_bytes(int64_t M, int64_t N, int64_t K, int S, bool shared_operand);
-cudaError_t ozaki_gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
-                       const double *A, int64_t lda, const double *B, int64_t ldb, double beta_c,
-                       double *C, int64_t ldc, int lower, int S, void *work, DevStatus *status,
-                       cudaStream_t st, int reserve_sms = 0);
 
 }  // namespace qmlgb

@@ -1156,27 +1156,4 @@ cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t
   return launch_oz<7>(p.ntiles, pairs, reserve_sms, p, st);
 }
 
-size_t ozaki_workspace_bytes(int64_t M, int64_t N, int64_t K, int S, bool shared_operand) {
-  return oz_digits_bytes(M, K, S) + (shared_operand ? 0 : oz_digits_bytes(N, K, S));
-}
-
-cudaError_t ozaki_gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha,
-                       const double *A, int64_t lda, const double *B, int64_t ldb, double beta_c,
-                       double *C, int64_t ldc, int lower, int S, void *work, DevStatus *status,
-                       cudaStream_t st, int reserve_sms) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  // op(A) and op(B)^T are the same logical matrix when A == B and exactly one
-  // of them is transposed (X^T X, G G^T): slice it once
-  const bool shared = (A == B && lda == ldb && ta != tb && M == N);
-  OzDigits a = oz_digits_at(work, M, K, S), b = a;
-  // op(A)[i,k] = A[i + k lda] (ta = 0) or A[k + i lda]
-  oz_slice(A, ta ? lda : 1, ta ? 1 : lda, a, st);
-  if (!shared) {
-    // op(B) column j, entry k: B[k + j ldb] (tb = 0) or B[j + k ldb]
-    b = oz_digits_at((unsigned char *)work + oz_digits_bytes(M, K, S), N, K, S);
-    oz_slice(B, tb ? 1 : ldb, tb ? ldb : 1, b, st);
-  }
-  return oz_mm(M, N, alpha, a, 0, b, 0, beta_c, C, ldc, lower, status, st, reserve_sms);
-}
-
 }  // namespace qmlgb

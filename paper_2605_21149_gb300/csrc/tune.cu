@@ -9,7 +9,8 @@
 //                    heuristic only
 //   dgemm:<ta>,<tb>,<lower>,<M>,<N>,<K>,<alias>   measured tile, 10 RM + RN,
 //                    or 10 for the kernel with the whole K range on chip
-//   batch_streams    worker streams of pix_loglike_batch (default 8, 1..16)
+//   batch_streams    worker streams of pix_loglike_batch (1..16; default 8,
+//                    4 from k = 10000 modes on)
 //   ozaki_stages     4 (default) .. 2: depth of the split kernel's ring
 //   emu_tc           1 (default) / 0: emulator inference layers on tcgen05
 //                    / all through the WMMA product

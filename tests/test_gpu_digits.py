@@ -63,6 +63,26 @@ def test_nonfinite_rows_poison_their_outputs_only(api):
     assert np.abs(C - ref)[~bad].max() <= 1e-12 * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("m,n,k", [(130, 70, 24576), (130, 70, 24577), (33, 129, 49153)])
+def test_k_in_pieces(api, m, n, k, ta, tb):
+    """K past the digits kept at a time: each piece adds to C (bound as above, with
+    a rounding of C for each)."""
+    rng = np.random.default_rng(k + m)
+    A, B, C0 = rng.uniform(-1, 1, (m, k)), rng.uniform(-1, 1, (k, n)), rng.normal(size=(m, n))
+    Cd = td(C0)
+    api.gemm(td(A.T if ta else A), td(B.T if tb else B), Cd, transA=ta, transB=tb, alpha=-1.0,
+             beta=0.5, precision=1)
+    C = Cd.cpu().numpy()
+    bound = k * 2.0 ** -45 + 8 * 2.0 ** -52 * np.abs(C).max()
+    assert np.abs(C - (0.5 * C0 - A @ B)).max() <= bound
+    if m == 130 and ta != tb:
+        Gd = td(A.T if ta else A)
+        G = api.gemm(Gd, Gd, transA=ta, transB=tb, lower=True, precision=1).cpu().numpy()
+        ref = np.tril(A @ A.T)
+        assert np.abs(np.tril(G) - ref).max() <= k * 2.0 ** -45 + 8 * 2.0 ** -52 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("n", [255, 256, 257, 511, 513])
 @pytest.mark.parametrize("basis", [0, 1])
 def test_fp64_order_where_digits_start(api, n, basis):
