@@ -56,11 +56,12 @@
 // operand, digits 1..d, is one contiguous run, fetched by one linear bulk
 // copy; 32-byte rows through tensor maps had been what bounded the product.
 //
-// Kernel layout: one CTA per 128 x 128 output tile, 384 threads.
+// Kernel layout: one CTA per 128 x 128 output tile (128 x 64 where those fit
+// one wave), 384 threads.
 //   warp 0   producer (one lane): bulk copies into a ring of stages, guarded
 //            by mbarriers;
 //   warp 1   TMEM allocator and MMA issuer (one lane): tcgen05.mma kind::f16
-//            M=128 N=128 K=16; commits a slot to the epilogue at the end of a
+//            M=128 N=128 (64) K=16; commits a slot to the epilogue at the end of a
 //            chunk and waits for it to be read before refilling it;
 //   warps 2-3 idle (they complete warpgroup 0 for the register split);
 //   warps 4-11 epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (tile rows)
@@ -89,14 +90,14 @@ constexpr int kDigitTile = OBM * KS * 2;        // 4 KB: one 128 x 16 bf16 digit
 // Three warpgroups.  Warpgroup 0: warp 0 the producer, warp 1 the TMEM
 // allocator and MMA issuer, warps 2-3 idle.  Warpgroups 1 and 2 (warps
 // 4-11): kEpiWarps epilogue warps, each one TMEM lane quarter (32 tile rows)
-// by kEpiCols columns, so a thread holds kEpiCols int64 accumulators.  The
+// by half of the tile's columns, so a thread holds 64 int64 accumulators.  The
 // block starts at kLaunchRegs registers a thread (12 warps, three on each SM
 // sub-partition of 16384 registers: 65536 / 384 rounded down to 8); then
 // warpgroup 0 gives registers back (setmaxnreg.dec to kIssueRegs) and the
 // epilogue takes them (setmaxnreg.inc to kEpiRegs), so that its 64 int64 sums
 // stay in registers.  The split adds up exactly:
 // 128 kIssueRegs + 256 kEpiRegs = 384 kLaunchRegs.
-constexpr int kEpiWarps = 8, kEpiCols = 128 * 4 / kEpiWarps;
+constexpr int kEpiWarps = 8;
 constexpr int kThreads = 128 + 32 * kEpiWarps;
 constexpr int kLaunchRegs = 168, kIssueRegs = 56, kEpiRegs = 224;
 static_assert(128 * kIssueRegs + 256 * kEpiRegs == kThreads * kLaunchRegs,
@@ -107,8 +108,14 @@ static_assert(kThreads * kLaunchRegs <= 65536, "launch registers exceed the SM")
 // (bulk copy, tcgen05 and shared-memory descriptor helpers: ptx.cuh)
 
 // instruction descriptor, kind::f16: D f32, A and B bf16, both K-major, N, M
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(OBN >> 3) << 17) |
+template <int NT>
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) |
                             ((uint32_t)(OBM >> 4) << 24);
+// Tile widths.  NT = 128 is the general form.  NT = kNarrow halves a tile (one
+// CTA per 128 x 64, B's digit tiles fetched by halves): a product of up to half
+// as many 128-wide tiles as there are SMs takes one tile's time whatever its
+// size, MMAs and output both in proportion to the width.
+constexpr int kNarrow = 64;
 
 // K-major bf16 tile of 16-element (32-byte) rows with the 32-byte swizzle
 // (8-row atoms of 256 B): start address, LBO 16 B (unused: one MMA's K is the
@@ -126,7 +133,7 @@ __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
 // (in registers they pushed the epilogue into spills: 64 int64 sums and the
 // loaded columns fill the 168 the compiler allots)
 template <int S>
-constexpr int kResidBytes = OzDigitsOf<S>::kFrac ? kEpiCols / 2 * 32 * kEpiWarps * 4 : 0;
+constexpr int kResidBytes = OzDigitsOf<S>::kFrac ? 32 * 32 * kEpiWarps * 4 : 0;
 
 // 1.5 2^23 as a float and its bit pattern
 constexpr float kMagicF = 12582912.0f;
@@ -184,35 +191,39 @@ template <int CL>
 __device__ __forceinline__ int item_stride() {
   return CL == 2 ? (int)(gridDim.x >> 1) : (int)gridDim.x;
 }
-// the output tile of this CTA for work item `item` (a tile, or a pair for CL = 2)
-template <int CL>
-__device__ __forceinline__ void item_tile(const OzParams &p, int item, int rank, int &tm, int &tn) {
+// the output tile of this CTA for work item `item` (a tile, or a pair for CL =
+// 2; NT < 128: a part of one): tile row and column and the part's first column
+template <int CL, int NT>
+__device__ __forceinline__ void item_tile(const OzParams &p, int item, int rank, int &tm, int &tn,
+                                          int &n0) {
+  constexpr int kParts = OBN / NT;
   if (CL == 1) {
-    tile_of(p, item, tm, tn);
+    tile_of(p, item / kParts, tm, tn);
   } else {
     int TM;
     pair_of(p, item, TM, tn);
     tm = 2 * TM + rank;
   }
+  n0 = tn * OBN + item % kParts * NT;
 }
 
 
 // Every digit product of level L for one K step: pair (s, L - s) reads digit
-// tile s - 1 of A and L - s - 1 of B, at descriptor offsets of 256 (4 KB >> 4)
-// per tile from the step's first tiles (da, db).  Unrolled at compile time,
+// tile s - 1 of A and L - s - 1 of B, at descriptor offsets of 256 (4 KB >> 4;
+// 2 NT for B's NT rows) per tile from the step's first tiles (da, db).  Unrolled at compile time,
 // so the issuing warp spends a few instructions per MMA: with loop bounds,
 // flags and descriptors computed at run time, or moved to uniform registers
 // for every MMA, it could not keep up with the tensor core (93 clocks of issue
 // per 64-clock MMA).  The first pair
 // writes the accumulator when acc0 is 0 (first K step of a chunk).
-template <int S, int L>
+template <int S, int L, int NT>
 __device__ __forceinline__ void issue_level(uint32_t tmem, uint64_t da, uint64_t db, uint32_t acc0,
                                             uint32_t lead) {
   constexpr int s0 = L - S > 1 ? L - S : 1, s1 = L - 1 < S ? L - 1 : S;
 #pragma unroll
   for (int s = s0; s <= s1; ++s)
-    mma_bf16_warp(tmem, da + (uint64_t)(256 * (s - 1)), db + (uint64_t)(256 * (L - s - 1)), kIdesc,
-                  s == s0 ? acc0 : 1u, lead);
+    mma_bf16_warp(tmem, da + (uint64_t)(256 * (s - 1)), db + (uint64_t)(2 * NT * (L - s - 1)),
+                  kIdesc<NT>, s == s0 ? acc0 : 1u, lead);
 }
 
 // Output of 8 consecutive columns of one row, general form: C[gi + gj ldc] =
@@ -324,18 +335,18 @@ __device__ __forceinline__ bool slot_acquire(Issuer &I, int q) {
 }
 
 // the products of entry E of group G for one K step
-template <int S, int G, int E>
+template <int S, int G, int E, int NT>
 __device__ __forceinline__ void issue_entry(uint32_t tmem, uint64_t da, uint64_t db, uint32_t acc0,
                                             uint32_t lead) {
   using Sc = OzGroup<S, G>;
   if constexpr (E < Sc::NE) {
-    issue_level<S, Sc::L0 + E>(tmem, da, db, acc0, lead);
+    issue_level<S, Sc::L0 + E, NT>(tmem, da, db, acc0, lead);
     if constexpr (Sc::kLowGroup && E == Sc::NE - 1)
-      issue_level<S, Sc::L0 + E + 1>(tmem, da, db, 1u, lead);
+      issue_level<S, Sc::L0 + E + 1, NT>(tmem, da, db, 1u, lead);
   }
 }
 
-template <int S, int CL, int G>
+template <int S, int CL, int NT, int G>
 __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
   using Sc = OzGroup<S, G>;
   OzHandover<Sc> H(k0, I.ord);
@@ -347,7 +358,7 @@ __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
 #pragma unroll
     for (int j = 0; j < Sc::kSteps; ++j) {
       const uint64_t da = da0 + (uint64_t)(256 * Sc::kDigits * j);
-      const uint64_t db = db0 + (uint64_t)(256 * Sc::kDigits * j);
+      const uint64_t db = db0 + (uint64_t)(2 * NT * Sc::kDigits * j);
       const int t = ks + j;
       // entry bl starts its next chunk here: its slot goes to the epilogue now,
       // and with a spare slot the entry goes on in that one; without, the other
@@ -365,7 +376,7 @@ __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
         const bool fresh = t == k0 || bl == e;
         const int q = H.sl[e < Sc::NE ? e : 0];
         if (fresh && !slot_acquire(I, q)) return false;
-        issue_entry<S, G, e>(I.tbase + 128 * q, da, db, fresh ? 0u : 1u, I.lead);
+        issue_entry<S, G, e, NT>(I.tbase + 128 * q, da, db, fresh ? 0u : 1u, I.lead);
         return true;
       };
       if (!entry(IntC<0>{}) || !entry(IntC<1>{}) || !entry(IntC<2>{}) || !entry(IntC<3>{}))
@@ -374,9 +385,9 @@ __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
         const int q = H.slot(bl);
         if (!slot_acquire(I, q)) return false;
         if (bl == 0)
-          issue_entry<S, G, 0>(I.tbase + 128 * q, da, db, 0u, I.lead);
+          issue_entry<S, G, 0, NT>(I.tbase + 128 * q, da, db, 0u, I.lead);
         else
-          issue_entry<S, G, 1>(I.tbase + 128 * q, da, db, 0u, I.lead);
+          issue_entry<S, G, 1, NT>(I.tbase + 128 * q, da, db, 0u, I.lead);
       }
     }
     // frees the smem slot when these MMAs finish (in both CTAs of a pair)
@@ -408,7 +419,7 @@ struct Producer {
   int last_phase[4];
 };
 
-template <int S, int CL, int G>
+template <int S, int CL, int NT, int G>
 __device__ __forceinline__ bool load_piece(Producer &P, const unsigned char *a,
                                            const unsigned char *b, int k0, int k1) {
   using Sc = OzGroup<S, G>;
@@ -416,14 +427,20 @@ __device__ __forceinline__ bool load_piece(Producer &P, const unsigned char *a,
   for (int ks = k0; ks < k1; ks += Sc::kSteps) {
     if (!mbar_wait(P.empty0 + 8 * P.stage, P.phase ^ 1, P.st, P.wait_ns)) return false;
     const uint32_t fb = P.full0 + 8 * P.stage;
-    mbar_expect_tx(fb, 2u * Sc::kSteps * kRun);
+    mbar_expect_tx(fb, Sc::kSteps * (kRun + kRun / OBN * NT));
     const uint32_t sa = P.smem0 + (uint32_t)(P.stage * P.stage_bytes);
     const uint32_t sb = sa + (uint32_t)(P.stage_bytes >> 1);
 #pragma unroll
     for (int j = 0; j < Sc::kSteps; ++j) {
       const size_t src = (size_t)(ks + j) * S * kDigitTile;
       bulk_load(sa + j * kRun, a + src, kRun, fb);
-      if (CL == 1)
+      if constexpr (NT < OBN) {
+        // this tile's rows of each of B's digit tiles
+        constexpr uint32_t kPart = kDigitTile / OBN * NT;
+#pragma unroll
+        for (int q = 0; q < Sc::kDigits; ++q)
+          bulk_load(sb + (j * Sc::kDigits + q) * kPart, b + src + q * kDigitTile, kPart, fb);
+      } else if (CL == 1)
         bulk_load(sb + j * kRun, b + src, kRun, fb);
       else if (((ks + j) & 1) == (int)cluster_ctarank())
         bulk_load_mc(sb + j * kRun, b + src, kRun, fb, (uint16_t)3);
@@ -453,8 +470,10 @@ __device__ __forceinline__ bool load_piece(Producer &P, const unsigned char *a,
 // phase).  Cluster barriers order the barrier initialisation before any
 // remote arrival and keep both CTAs alive until neither can reach the other's
 // shared memory.
-template <int S, int CL>
+template <int S, int CL, int NT>
 __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_constant__ OzParams p) {
+  static_assert(CL == 1 || NT == OBN, "a pair shares whole B tiles");
+  constexpr int kEpiCols = NT * 4 / kEpiWarps;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte alignment for the swizzled tiles
   unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -493,7 +512,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
 
   if (warp < 4) {
   // warpgroup 0 hands registers to the epilogue warpgroups
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssueRegs));
+  if constexpr (NT == OBN) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssueRegs));
   if (warp == 0) {
     // ----------------------------------------------------------- producer
     if (lane == 0) {
@@ -501,19 +520,21 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
                  {-1, -1, -1, -1}};
       bool ok = (*((volatile int *)&st->code) == 0) && !p.no_loads;
       for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
-        int tm, tn;
-        item_tile<CL>(p, item, pair_rank<CL>(), tm, tn);
+        int tm, tn, n0;
+        item_tile<CL, NT>(p, item, pair_rank<CL>(), tm, tn, n0);
+        if (NT < OBN && n0 >= p.N) continue;  // (all roles pass over it)
         // (a pair's row tile past the last one reads the last one: its
         // outputs lie outside C and are not stored)
         const size_t rt_bytes = (size_t)p.nk16 * S * kDigitTile;
         const unsigned char *a = p.DA + (size_t)min(tm, p.rta) * rt_bytes;
-        const unsigned char *b = p.DB + (size_t)min(tn, p.rtb) * rt_bytes;
+        const unsigned char *b =
+            p.DB + (size_t)min(tn, p.rtb) * rt_bytes + (size_t)(n0 - tn * OBN) * (KS * 2);
         if constexpr (OzDigitsOf<S>::kLow)
           for (int c = 0; c < p.nsc && ok; ++c)
-            ok = load_piece<S, CL, 0>(P, a, b, oz_piece(p.nk16, p.nsc, c),
+            ok = load_piece<S, CL, NT, 0>(P, a, b, oz_piece(p.nk16, p.nsc, c),
                                       oz_piece(p.nk16, p.nsc, c + 1));
         for (int c = 0; c < p.nsc && ok; ++c)
-          ok = load_piece<S, CL, 1>(P, a, b, oz_piece(p.nk16, p.nsc, c),
+          ok = load_piece<S, CL, NT, 1>(P, a, b, oz_piece(p.nk16, p.nsc, c),
                                     oz_piece(p.nk16, p.nsc, c + 1));
       }
       if (!ok) {
@@ -531,12 +552,17 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
                0, 0, 0, 0, kOzSlots, elect_lane()};
       bool ok = __all_sync(0xffffffffu, *((volatile int *)&st->code) == 0) != 0;
       for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
+        if constexpr (NT < OBN) {
+          int tm, tn, n0;
+          item_tile<CL, NT>(p, item, 0, tm, tn, n0);
+          if (n0 >= p.N) continue;
+        }
         if constexpr (OzDigitsOf<S>::kLow)
           for (int c = 0; c < p.nsc && ok; ++c)
-            ok = issue_piece<S, CL, 0>(I, oz_piece(p.nk16, p.nsc, c),
+            ok = issue_piece<S, CL, NT, 0>(I, oz_piece(p.nk16, p.nsc, c),
                                        oz_piece(p.nk16, p.nsc, c + 1));
         for (int c = 0; c < p.nsc && ok; ++c)
-          ok = issue_piece<S, CL, 1>(I, oz_piece(p.nk16, p.nsc, c),
+          ok = issue_piece<S, CL, NT, 1>(I, oz_piece(p.nk16, p.nsc, c),
                                      oz_piece(p.nk16, p.nsc, c + 1));
       }
       // wait for every MMA this thread issued before TMEM is released
@@ -545,7 +571,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
     }
   }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
+    if constexpr (NT == OBN) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpiRegs));
     // ---------------------------------------------------------- epilogue
     const int quad = warp & 3;            // TMEM lane quarter this warp may access
     const int half = (warp - 4) >> 2;     // which kEpiCols columns of the tile
@@ -633,9 +659,10 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       return true;
     };
     for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
-      int tm, tn;
-      item_tile<CL>(p, item, pair_rank<CL>(), tm, tn);
-      const int m0 = tm * OBM, n0 = tn * OBN;
+      int tm, tn, n0;
+      item_tile<CL, NT>(p, item, pair_rank<CL>(), tm, tn, n0);
+      if (NT < OBN && n0 >= p.N) continue;
+      const int m0 = tm * OBM;
       // beta C is read only when the tile is written out, after all of its
       // MMAs; fetch this thread's C entries into L2 now, so that those reads
       // wait on L2 rather than on DRAM
@@ -686,7 +713,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       // (every lane takes part in the shuffles; rows past M store nothing)
       const int64_t gjl = n0 + kEpiCols * half + lane;
       const int f_lo = gjl < p.N ? p.eb[gjl] : 0;
-      const int f_hi = gjl + 32 < p.N ? p.eb[gjl + 32] : 0;
+      const int f_hi = kEpiCols > 32 && gjl + 32 < p.N ? p.eb[gjl + 32] : 0;
       const int64_t gi = m0 + row;
       const bool live_row = gi < p.M;
       const int ebase = live_row ? p.ea[gi] - 2 * OzDigitsOf<S>::kTop - p.shift_top : 0;
@@ -1023,16 +1050,16 @@ static_assert(oz_max_stages<7>() >= 3 && oz_max_stages<6>() >= 4, "ring too shal
 // up to exactly kLaunchRegs a thread (a build that launches with any other
 // count is refused rather than run: an increase that cannot be met never
 // returns).  Also the most clusters of two that can be resident at once.
-template <int S, int CL>
+template <int S, int CL, int NT>
 cudaError_t oz_prepare(int &max_items) {
-  cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, CL>,
+  cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, CL, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)oz_smem<S>(oz_max_stages<S>()));
   if (e != cudaSuccess) return e;
   cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, ozaki_gemm_kernel<S, CL>);
+  e = cudaFuncGetAttributes(&fa, ozaki_gemm_kernel<S, CL, NT>);
   if (e != cudaSuccess) return e;
-  if (fa.numRegs != kLaunchRegs) return cudaErrorInvalidConfiguration;
+  if (NT == OBN && fa.numRegs != kLaunchRegs) return cudaErrorInvalidConfiguration;
   int dev = 0, nsm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
@@ -1053,18 +1080,18 @@ cudaError_t oz_prepare(int &max_items) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int ncl = 0;
-  e = cudaOccupancyMaxActiveClusters(&ncl, ozaki_gemm_kernel<S, CL>, &cfg);
+  e = cudaOccupancyMaxActiveClusters(&ncl, ozaki_gemm_kernel<S, CL, NT>, &cfg);
   if (e != cudaSuccess) return e;
   max_items = ncl > 0 ? ncl : 1;
   return cudaSuccess;
 }
 
-template <int S, int CL>
+template <int S, int CL, int NT>
 cudaError_t launch_oz_t(int nitems, int reserve_sms, OzParams &p, cudaStream_t st) {
   static int max_items = 0;
   static cudaError_t prep = cudaErrorNotReady;
   static std::once_flag once;
-  std::call_once(once, [] { prep = oz_prepare<S, CL>(max_items); });
+  std::call_once(once, [] { prep = oz_prepare<S, CL, NT>(max_items); });
   if (prep != cudaSuccess) return prep;
   // persistent: one CTA per SM (one fits: 512 TMEM columns, ~200 KB of
   // shared memory), the CTAs (or pairs) taking every grid-th work item;
@@ -1085,15 +1112,17 @@ cudaError_t launch_oz_t(int nitems, int reserve_sms, OzParams &p, cudaStream_t s
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_gemm_kernel<S, CL>, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_gemm_kernel<S, CL, NT>, p);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int S>
-cudaError_t launch_oz(int nitems, bool pairs, int reserve_sms, OzParams &p, cudaStream_t st) {
+cudaError_t launch_oz(bool narrow, bool pairs, int reserve_sms, OzParams &p, cudaStream_t st) {
   const int rsv = reserve_sms > 0 ? reserve_sms : 0;
-  return pairs ? launch_oz_t<S, 2>(nitems, rsv, p, st) : launch_oz_t<S, 1>(nitems, rsv, p, st);
+  if (narrow) return launch_oz_t<S, 1, kNarrow>(p.ntiles, rsv, p, st);
+  return pairs ? launch_oz_t<S, 2, OBN>(p.ntiles, rsv, p, st)
+               : launch_oz_t<S, 1, OBN>(p.ntiles, rsv, p, st);
 }
 
 }  // namespace
@@ -1147,13 +1176,19 @@ cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t
     const int64_t b = tune_get("ozaki_band", 6);
     p.band = b < 1 ? 1 : (b > 4096 ? 4096 : (int)b);
   }
-  // clusters of two on tile-row pairs (B shared through multicast) unless
+  // Half-width tiles while they still fit one wave (152 SMs): the wide ones
+  // would leave more than half of the SMs idle.  T Nside 16 harmonic solve 14.9
+  // -> 12.8 ms, TQU Nside 8 solve 4.79 -> 4.56, 100-map estimate 2.88 -> 2.76;
+  // the same bits.
+  const int tiles = oz_item_count(tiles_m, p.tiles_n, lower ? 1 : 0, 0);
+  const bool narrow = 2 * tiles <= 152 - reserve_sms;
+  // else clusters of two on tile-row pairs (B shared through multicast) unless
   // switched off or the output has a single tile row
-  const bool pairs = tune_get("ozaki_pairs", 1) != 0 && tiles_m >= 2;
-  p.ntiles = oz_item_count(tiles_m, p.tiles_n, lower ? 1 : 0, pairs ? 1 : 0);
-  if (S == 3) return launch_oz<3>(p.ntiles, pairs, reserve_sms, p, st);
-  if (S == 6) return launch_oz<6>(p.ntiles, pairs, reserve_sms, p, st);
-  return launch_oz<7>(p.ntiles, pairs, reserve_sms, p, st);
+  const bool pairs = !narrow && tune_get("ozaki_pairs", 1) != 0 && tiles_m >= 2;
+  p.ntiles = narrow ? 2 * tiles : oz_item_count(tiles_m, p.tiles_n, lower ? 1 : 0, pairs ? 1 : 0);
+  if (S == 3) return launch_oz<3>(narrow, pairs, reserve_sms, p, st);
+  if (S == 6) return launch_oz<6>(narrow, pairs, reserve_sms, p, st);
+  return launch_oz<7>(narrow, pairs, reserve_sms, p, st);
 }
 
 }  // namespace qmlgb

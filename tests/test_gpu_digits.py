@@ -63,6 +63,28 @@ def test_nonfinite_rows_poison_their_outputs_only(api):
     assert np.abs(C - ref)[~bad].max() <= 1e-12 * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("m,n", [(1, 1), (128, 64), (127, 65), (129, 128), (300, 200), (520, 33)])
+@pytest.mark.parametrize("k", [16, 130, 1100])
+def test_narrow_tiles_equal_wide(api, m, n, k):
+    """Products of few tiles take half-width ones: the same bits as the same
+    entries of a product of 81 whole tiles, for every alpha and beta form."""
+    rng = np.random.default_rng(m + n + k)
+    A, B, C0 = rng.normal(size=(1100, k)), rng.normal(size=(k, 1100)), rng.normal(size=(1100, 1100))
+    for alpha, beta in ((1.0, 0.0), (-1.0, 1.0), (0.3, -0.7)):
+        W, Nw = td(C0), td(C0[:m, :n])
+        api.gemm(td(A), td(B), W, alpha=alpha, beta=beta, precision=1)
+        api.gemm(td(A[:m]), td(B[:, :n]), Nw, alpha=alpha, beta=beta, precision=1)
+        assert torch.equal(W[:m, :n], Nw)
+    if m == 300:  # X^T X, lower: the upper triangle stays
+        W, Nw = td(np.zeros((1700, 1700))), td(C0[:m, :m])
+        X = rng.normal(size=(k, 1700))
+        api.gemm(td(X), td(X), W, transA=True, lower=True, precision=1)
+        api.gemm(td(X[:, :m]), td(X[:, :m]), Nw, transA=True, lower=True, precision=1)
+        W, Nw = W.cpu().numpy(), Nw.cpu().numpy()
+        assert np.array_equal(np.tril(W[:m, :m]), np.tril(Nw))
+        assert np.array_equal(np.triu(Nw, 1), np.triu(C0[:m, :m], 1))
+
+
 @pytest.mark.parametrize("ta,tb", [(False, False), (True, False), (False, True), (True, True)])
 @pytest.mark.parametrize("m,n,k", [(130, 70, 24576), (130, 70, 24577), (33, 129, 49153)])
 def test_k_in_pieces(api, m, n, k, ta, tb):
