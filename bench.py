@@ -34,7 +34,7 @@ DGEMM_SYRK_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum o
                              "--set full capture of this launch")
 # the same for the split kernel (ozaki_gemm_kernel<6, 2>, clusters of two) on
 # W = X^T X at this workload; None when the kernel changes until recaptured
-OZ_SYRK_TRAFFIC = 5.69e9 + 0.17715e9
+OZ_SYRK_TRAFFIC = 3.684808e9 + 0.176423e9
 OZ_SYRK_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one capture of "
                           "the kernel alone (slicing not included), banded work order")
 UNIT = "solves/s"
