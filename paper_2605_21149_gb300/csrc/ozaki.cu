@@ -1178,7 +1178,7 @@ cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t
   }
   // Half-width tiles while they still fit one wave (152 SMs): the wide ones
   // would leave more than half of the SMs idle.  T Nside 16 harmonic solve 14.9
-  // -> 12.8 ms, TQU Nside 8 solve 4.79 -> 4.56, 100-map estimate 2.88 -> 2.76;
+  // -> 12.8 ms, TQU Nside 8 solve 4.79 -> 4.56, 1000-map estimate 2.88 -> 2.76;
   // the same bits.
   const int tiles = oz_item_count(tiles_m, p.tiles_n, lower ? 1 : 0, 0);
   const bool narrow = 2 * tiles <= 152 - reserve_sms;
