@@ -385,13 +385,14 @@ __device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *inv
   for (int c0 = 0, par = 0; c0 < jb; c0 += kPW, par ^= 1) {
     const int cend = (c0 + kPW < jb) ? c0 + kPW : jb;
     double *wp = w + par * (kNB * 9);
+    double l[kPW];  // this lane's row of the panel, divided by the pivots
     if (warp < 3) {
       // the panel: the 8 x 8 pivot block in lanes 0-7 of each of the warps (the
       // same operations on the same values), 24 rows below it in lanes 8-31
       if (warp == 0 || c0 + kPW + 24 * warp < jb) {
         const int row = lane < kPW ? c0 + lane : c0 + kPW + 24 * warp + (lane - kPW);
         const bool live = row < jb;
-        double v[kPW], l[kPW];
+        double v[kPW];
 #pragma unroll
         for (int q = 0; q < kPW; ++q) v[q] = (c0 + q < cend && live) ? a[row][c0 + q] : 0.0;
         int fail_col = -1;
@@ -422,11 +423,10 @@ __device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *inv
             if (atomicCAS(&status->code, 0, 2 /* QML_ENOTSPD */) == 0)
               status->info = (int)(j0 + fail_col + 1);
           }
-        } else if (live && (warp == 0 || lane >= kPW)) {
-          // (above the diagonal of the pivot block nothing is stored or read)
+        } else if (live && lane >= kPW) {
 #pragma unroll
           for (int q = 0; q < kPW; ++q)
-            if (c0 + q < cend && row > c0 + q) {
+            if (c0 + q < cend) {
               a[row][c0 + q] = l[q];
               wp[row * 9 + q] = v[q];
             }
@@ -452,6 +452,15 @@ __device__ bool factor_ldl(double (*a)[kLDA], double *w, double *dv, double *inv
     }
     __syncthreads();
     if (*bad) return false;
+    // The pivot block's own rows, from warp 0, only now: warps 1 and 2 load them
+    // too, at a time of their own before the barrier.  Nothing reads them
+    // before the end (the updates take the rows below), nor what lies above
+    // their diagonal.
+    if (warp == 0 && lane < kPW) {
+#pragma unroll
+      for (int q = 0; q < kPW; ++q)
+        if (c0 + lane < cend && q < lane) a[c0 + lane][c0 + q] = l[q];
+    }
     // this panel's update of the next one's columns
     for (int t = tid; t < kPW * (jb - cend); t += blockDim.x) {
       const int i = cend + (t >> 3), j = cend + (t & 7);
@@ -588,10 +597,10 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_kernel(double *A, int64_t l
     // Lane-dependent conditions are selects, so each step is one basic block.
     for (int c0 = 0; c0 < jb; c0 += kPW) {
       const int cend = (c0 + kPW < jb) ? c0 + kPW : jb;
+      double v[kPW];  // this lane's row of the panel
       if (warp == 0 || (warp < 3 && c0 + kPW + 24 * warp < jb)) {
         const int row = lane < kPW ? c0 + lane : c0 + kPW + 24 * warp + (lane - kPW);
         const bool live = row < jb;
-        double v[kPW];
 #pragma unroll
         for (int q = 0; q < kPW; ++q) v[q] = (c0 + q < cend && live) ? a[row][c0 + q] : 0.0;
         int fail_col = -1;
@@ -626,14 +635,20 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_kernel(double *A, int64_t l
             if (atomicCAS(&status->code, 0, 2 /* QML_ENOTSPD */) == 0)
               status->info = (int)(j0 + fail_col + 1);
           }
-        } else if (live && (warp == 0 || lane >= kPW)) {
+        } else if (live && lane >= kPW) {
 #pragma unroll
           for (int q = 0; q < kPW; ++q)
-            if (c0 + q < cend && row >= c0 + q) a[row][c0 + q] = v[q];
+            if (c0 + q < cend) a[row][c0 + q] = v[q];
         }
       }
       __syncthreads();
       if (*bad) return;
+      // the pivot block's own rows after the barrier, as in factor_ldl
+      if (warp == 0 && lane < kPW && c0 + lane < cend) {
+#pragma unroll
+        for (int q = 0; q < kPW; ++q)
+          if (q <= lane) a[c0 + lane][c0 + q] = v[q];
+      }
       // rank-(cend - c0) update of the trailing triangle cend <= j <= i < jb,
       // two elements per pass, each with two partial sums (a full panel takes
       // the branch-free form)
@@ -834,6 +849,7 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_df_kernel(const double *A, 
   // interleave (each step is a dependent chain of 4-cycle float32 operations).
   for (int c0 = 0; c0 < jb; c0 += kPW) {
     const int cend = (c0 + kPW < jb) ? c0 + kPW : jb;
+    dfl v[kPW];  // this lane's row of the panel
     // Warps 0-2 each factor the panel's 8 x 8 pivot block in lanes 0-7 (the
     // same operations on the same values, so identical results) and carry 24
     // rows of their own below it in lanes 8-31: no exchange between warps,
@@ -843,7 +859,7 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_df_kernel(const double *A, 
     if (warp == 0 || (warp < 3 && c0 + kPW + 24 * warp < jb)) {
       const int row = lane < kPW ? c0 + lane : c0 + kPW + 24 * warp + (lane - kPW);
       const bool live = row < jb;
-      dfl v[kPW], dg[kPW];
+      dfl dg[kPW];
 #pragma unroll
       for (int q = 0; q < kPW; ++q) {
         v[q] = (c0 + q < cend && live) ? a[row][c0 + q] : dfl{0.0f, 0.0f};
@@ -882,14 +898,20 @@ __global__ void __launch_bounds__(256, 1) potrf_diag_df_kernel(const double *A, 
           if (atomicCAS(&status->code, 0, 2 /* QML_ENOTSPD */) == 0)
             status->info = (int)(j0 + fail_col + 1);
         }
-      } else if (live && (warp == 0 || lane >= kPW)) {
+      } else if (live && lane >= kPW) {
 #pragma unroll
         for (int q = 0; q < kPW; ++q)
-          if (c0 + q < cend && row >= c0 + q) a[row][c0 + q] = v[q];
+          if (c0 + q < cend) a[row][c0 + q] = v[q];
       }
     }
     __syncthreads();
     if (bad) return;
+    // the pivot block's own rows after the barrier, as in factor_ldl
+    if (warp == 0 && lane < kPW && c0 + lane < cend) {
+#pragma unroll
+      for (int q = 0; q < kPW; ++q)
+        if (q <= lane) a[c0 + lane][c0 + q] = v[q];
+    }
     // rank-(cend - c0) update of the trailing triangle cend <= j <= i < jb,
     // two elements per pass, each with two partial sums (a full panel takes
     // the branch-free form)

@@ -178,3 +178,32 @@ def test_emu_first_layer_inputs(api, ndim, npts):
     out = (np.abs(test) > 1).any(axis=1)
     assert (fa[out] == 1).all() and (fb[out] == 1).all()
     assert np.mean(fa == fb) >= 0.99
+
+
+@pytest.mark.parametrize("form", ["ldl", "general", "float-float"])
+def test_potrf_rows_agree_between_warps(api, form):
+    """Rows 16-39 and 40-63 of a block equal in its first 16 columns: a panel's
+    rows fall to three warps, each with the pivot block factored for itself, and
+    equal rows must come out with equal bits.  'general': diagonals outside
+    the range of the fast form."""
+    g = np.random.default_rng(11)
+    B = g.normal(size=(64, 64))
+    S = B @ B.T / 64
+    S[40:, :16] = S[16:40, :16]
+    S[:16, 40:] = S[40:, :16].T
+    S += 8.0 * np.eye(64)
+    if form == "general":
+        S *= 2.0 ** -600
+    At = td(S)
+    ref = np.linalg.cholesky(S)
+    if form == "float-float":
+        api.tune_set("split_diag_df", 1)
+    try:
+        for _ in range(200):
+            W = At.clone()
+            api.potrf(W, precision=int(form == "float-float"))
+            L = W.cpu().numpy()
+            assert np.array_equal(L[16:40, :16], L[40:, :16])
+    finally:
+        api.tune_set("split_diag_df", 0)
+    assert np.abs(np.tril(L) - ref).max() <= 1e-11 * np.abs(ref).max()
