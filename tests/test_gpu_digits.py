@@ -127,3 +127,32 @@ def test_fp64_order_where_digits_start(api, n, basis):
     g = api.loglike(prob, torch.as_tensor(wl.cl_fid.reshape(-1), device="cuda"), td(maps))
     assert P.rel_max(g[0], lnl) <= 1e-12
     assert abs(float(P.to_np(g[2])) - ld) <= 1e-12 * abs(ld)
+
+
+@pytest.mark.parametrize("beta", [0.0, 1.0])
+@pytest.mark.parametrize("m,n", [(128, 64), (300, 200), (1700, 1500)])
+def test_rows_and_columns_of_any_size(api, m, n, beta):
+    """Rows and columns scaled by powers of two whose sums leave the normal range
+    one with another but not with those of the same index: a product is the
+    unscaled one times the power, down to subnormal results, 0 and infinity.
+    (128, 64) takes the half-width tiles, (1700, 1500) the whole ones."""
+    rng = np.random.default_rng(m)
+    k = 130
+    A, B = rng.uniform(0.5, 1, (m, k)), rng.uniform(0.5, 1, (k, n))
+    C0 = rng.normal(size=(m, n))
+    r, c = np.zeros(m, int), np.zeros(n, int)
+    r[3::37], r[11::41], r[20::53] = -600, 600, -530
+    c[5::29], c[14::31], c[23::43] = -600, 600, -530
+    with np.errstate(over="ignore", under="ignore"):
+        ref = beta * C0 + np.ldexp(A @ B, r[:, None] + c[None, :])
+        Cd = td(C0)
+        api.gemm(td(np.ldexp(A, r[:, None])), td(np.ldexp(B, c[None, :])), Cd, beta=beta,
+                 precision=1)
+        C = Cd.cpu().numpy()
+        inf = np.isinf(ref)
+        assert inf.any() and (C[inf] == ref[inf]).all()
+        # 48 bits: 2^-45 K against sums of at least K / 4; a rounding of C, and
+        # one in the last place of a subnormal result
+        err = np.abs(C[~inf] - ref[~inf])
+        assert (err <= 2.0 ** -43 * np.abs(ref - beta * C0)[~inf] + 2.0 ** -51 * np.abs(ref[~inf])
+                + 2.0 ** -1073).all()
