@@ -718,19 +718,15 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       const bool live_row = gi < p.M;
       const int ebase = live_row ? p.ea[gi] - 2 * OzDigitsOf<S>::kTop - p.shift_top : 0;
       const int64_t gj0 = n0 + kEpiCols * half;
-      // Every result of this warp normal or zero, for any sum: its rows' exponents
-      // and its columns' far enough inside the range in every combination (a lane
-      // holds one row and two columns, the warp stores all 32 rows against all of
-      // its columns).  Rows and columns that are not there do not count.
+      // Every result of this warp normal or zero, for any sum: each row's exponent far
+      // enough inside the range with the least and the largest of the warp's
+      // columns (a lane holds one row and two columns, the warp stores all of its
+      // rows against all of its columns).
       const int em = ebase + p.alpha_exp;
-      constexpr int kNone = 1 << 20;
-      const bool c_lo = gjl < p.N, c_hi = kEpiCols > 32 && gjl + 32 < p.N;
-      const int lowest = __reduce_min_sync(0xffffffffu, live_row ? em : kNone) +
-                         __reduce_min_sync(0xffffffffu, min(c_lo ? f_lo : kNone, c_hi ? f_hi : kNone));
-      const int highest =
-          __reduce_max_sync(0xffffffffu, live_row ? em : -kNone) +
-          __reduce_max_sync(0xffffffffu, max(c_lo ? f_lo : -kNone, c_hi ? f_hi : -kNone));
-      const bool fast = p.alpha_pow2 && p.beta_mode < 2 && lowest > -980 && highest < 940;
+      const int f_min = __reduce_min_sync(0xffffffffu, min(f_lo, f_hi));
+      const int f_max = __reduce_max_sync(0xffffffffu, max(f_lo, f_hi));
+      const bool inside = em + f_min > -980 && em + f_max < 940;
+      const bool fast = p.alpha_pow2 && p.beta_mode < 2 && __all_sync(0xffffffffu, inside);
       // live columns of this row from gj0 on
       int64_t lim64 = (p.lower && gi + 1 < p.N ? gi + 1 : p.N) - gj0;
       const int lim = live_row ? (int)(lim64 < 0 ? 0 : (lim64 > kEpiCols ? kEpiCols : lim64)) : 0;
