@@ -32,11 +32,11 @@ METRIC = "Fisher+Cl solves/s (TQU Nside16 l2-47, 100 sims)"
 DGEMM_SYRK_TRAFFIC = 8.550515e9 + 0.187149e9
 DGEMM_SYRK_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one "
                              "--set full capture of this launch")
-# the same for the split kernel (ozaki_gemm_kernel<6, 2>, clusters of two) on
+# the same for the split kernel (ozaki_gemm_kernel<6, 128>) on
 # W = X^T X at this workload; None when the kernel changes until recaptured
-OZ_SYRK_TRAFFIC = 3.684808e9 + 0.176423e9
+OZ_SYRK_TRAFFIC = 3.914475e9 + 0.179409e9
 OZ_SYRK_TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one capture of "
-                          "the kernel alone (slicing not included), banded work order")
+                          "the kernel alone (slicing not included), work order in bands of eight tile rows")
 UNIT = "solves/s"
 
 
@@ -459,7 +459,7 @@ def run_ours(args):
         torch.cuda.empty_cache()
         fp64_peak = measure_fp64_peak(torch)
         bf16_peak = peaks().get("bf16_tflops", 1900.0)
-        roof = {"kernel": "split GEMM (slicing + ozaki_gemm_kernel<6, 2>), W = X^T X lower, "
+        roof = {"kernel": "split GEMM (slicing + ozaki_gemm_kernel<6, 128>), W = X^T X lower, "
                           "k=6900, n=5952",
                 "bound": "tensor", "achieved": 21 * flops / dur_s / 1e12, "peak": bf16_peak,
                 "unit": "TFLOP/s", "frac": 21 * flops / dur_s / 1e12 / bf16_peak,

@@ -359,10 +359,6 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   per-item kernel sequence as a captured CUDA graph
  *   ozaki_stages    4 (default) / 3 / 2: depth of the split kernel's ring of
  *                   operand stages (48 or 56 KB each)
- *   ozaki_pairs     1 (default) / 0: the split kernel runs in clusters of two
- *                   CTAs on pairs of tile rows that share their B digit tiles
- *                   (loaded once from L2, multicast to both) / one CTA per
- *                   tile; the results are bit-identical
  *   emu_tc          1 (default) / 0: emulator inference runs its layers on
  *                   tcgen05 (width a multiple of 64, at most 256) / every
  *                   layer through the WMMA product
@@ -370,9 +366,9 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   the network (a multiple of 128)
  *   emu_tc0         1 (default) / 0: with emu_tc, the first layer (16
  *                   inputs, widened with zeros to 64) on tcgen05 too / WMMA
- *   ozaki_band      6 (default): row pairs per band of the split kernel's
- *                   work order (column by column inside a band; 1 = row pair
- *                   after row pair); the results are the same for any value
+ *   ozaki_band      8 (default): tile rows per band of the split kernel's
+ *                   work order (column by column inside a band; 1 = row after
+ *                   row); the results are the same for any value
  *   ozaki_prefetch_c 1 (default) / 0: with beta != 0 the split kernel
  *                   fetches each output tile's C into L2 when the tile
  *                   starts / reads it from memory when the tile is written

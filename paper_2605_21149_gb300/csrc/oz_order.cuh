@@ -3,18 +3,16 @@
 // Shared by the kernel and a host check that compiles this header with a
 // plain C++ compiler.
 //
-// One CTA per item (single form): item bid is tile (tm, tn), row by row; for
-// a lower C only the tiles with tm >= tn.  Clusters of two (pair form): item
-// idx is pair (TM, tn), tile rows 2 TM and 2 TM + 1 of tile column tn (one B
-// tile shared by both CTAs).  For a lower C only the pairs with
-// tn <= 2 TM + 1 and tn < tiles_m; a tile of a pair above the diagonal or
-// past the last tile row is computed on zeros or discarded and stores
-// nothing.  Pairs come in bands of `band` row pairs, inside a band column by
-// column and the band's row pairs within each column.  The persistent grid
-// takes the items in waves of one pair per cluster, which all stream K in
-// step, and a wave over a compact band of rows and columns reads fewer
-// distinct digit panels from DRAM than one along whole rows (about 25 panels
-// a wave instead of about 45 at k = 6900).
+// One CTA per item.  Row by row (half-width tiles, which fit one wave): item
+// bid is tile (tm, tn), for a lower C only those with tm >= tn.  In bands of
+// `band` tile rows (everything else): inside a band column by column, and the
+// band's rows within each column.  The persistent grid takes the items in
+// waves of one tile per SM, which all stream K in step, and a wave over a
+// compact band of rows and columns reads fewer distinct digit panels from DRAM
+// than one along whole rows.
+//
+// oz_pair_of and the pair count are an order of pairs of tile rows, for a lower C
+// the pairs with tn <= 2 TM + 1 and tn < tiles_m; no kernel takes it.
 #pragma once
 
 #include <math.h>
@@ -27,7 +25,7 @@
 
 namespace qmlgb {
 
-// single form: tile of item bid
+// row by row: tile of item bid
 QMLGB_HD void oz_tile_of(int lower, int tiles_n, int bid, int &tm, int &tn) {
   if (!lower) {
     tm = bid / tiles_n;
@@ -42,14 +40,35 @@ QMLGB_HD void oz_tile_of(int lower, int tiles_n, int bid, int &tm, int &tn) {
   tn = bid - r * (r + 1) / 2;
 }
 
-// pair form, lower C: pairs of column tn in the band of row pairs [t0, t1)
+// in bands: tile of item idx
+QMLGB_HD void oz_band_tile_of(int tiles_m, int tiles_n, int lower, int band, int idx, int &tm,
+                              int &tn) {
+  // the items before row r are those of the row-by-row order, so a band's
+  // items begin where its first row's do
+  int r, c;
+  oz_tile_of(lower, tiles_n, idx, r, c);
+  const int t0 = r / band * band, h = tiles_m - t0 < band ? tiles_m - t0 : band;
+  idx -= lower ? t0 * (t0 + 1) / 2 : t0 * tiles_n;
+  const int left = lower ? t0 : tiles_n;  // columns with every row of the band
+  if (idx < left * h) {
+    tn = idx / h;
+    tm = t0 + idx % h;
+    return;
+  }
+  idx -= left * h;
+  for (c = 0; idx >= h - c; ++c) idx -= h - c;
+  tn = t0 + c;
+  tm = tn + idx;
+}
+
+// pairs, lower C: pairs of column tn in the band of row pairs [t0, t1)
 QMLGB_HD int oz_band_col_count(int tn, int t0, int t1) {
   const int need = tn >= 1 ? tn / 2 : 0;  // the smallest TM with 2 TM + 1 >= tn
   const int lo = need > t0 ? need : t0;
   return t1 > lo ? t1 - lo : 0;
 }
 
-// pair form: pair (TM, tn) of item idx
+// pairs: pair (TM, tn) of item idx
 QMLGB_HD void oz_pair_of(int tiles_m, int tiles_n, int lower, int band, int idx, int &TM, int &tn) {
   const int T2 = (tiles_m + 1) / 2;
   for (int t0 = 0; t0 < T2; t0 += band) {
@@ -81,7 +100,7 @@ QMLGB_HD void oz_pair_of(int tiles_m, int tiles_n, int lower, int band, int idx,
   tn = 0;
 }
 
-// items of a launch: tiles (single form) or tile-row pairs (pair form)
+// items of a launch: tiles, or tile-row pairs
 QMLGB_HD int oz_item_count(int tiles_m, int tiles_n, int lower, int pairs) {
   if (!pairs) return lower ? tiles_m * (tiles_m + 1) / 2 : tiles_m * tiles_n;
   const int T2 = (tiles_m + 1) / 2;

@@ -46,9 +46,14 @@
 // the next chunk starts at once, and without one the other levels' products of that K step go
 // first and cover the drain.  A group takes over the slots in the order in
 // which the one before it leaves them, each when its first product needs it.
-// What bounds a K step of {5 ..} is the MMA rate (93 clocks each, of which
-// cuBLAS's 1900 TFLOP/s would be 87); a pair of CTAs on M = 256 MMAs
-// (cta_group::2, half the B traffic in shared memory) ran no faster: 99.
+// What bounds a K step is the rate at which the issuing warp hands MMAs over:
+// 71 clocks each with operands in uniform registers (93 from a one-lane branch;
+// cuBLAS's 1900 TFLOP/s would be 87 at the burst clock, 64 the tensor core's
+// own rate).  A pair of CTAs on M = 256 MMAs (cta_group::2, half the B traffic in
+// shared memory) ran no faster, 99, and clusters of two that shared B's digit
+// tiles by multicast no faster than single CTAs in bands: 16000^2 K = 512 2.56
+// against 1.86 ms, W = X^T X of 6900 x 5952 3.5-3.8 against 3.5-3.8, TQU Nside 16
+// solve (QML_FP64) 38.4 against 37.9, QU Nside 32 295.4 against 292.8.
 //
 // Digit layout.  The slicing kernel writes the digits in the order and the
 // shared-memory image the MMA wants: [128-row tile][K step][digit] tiles of
@@ -142,14 +147,13 @@ constexpr uint32_t kMagicI = 0x4B400000u;
 struct OzParams {
   int64_t M, N;            // logical output size
   const unsigned char *DA, *DB;  // digit tiles of op(A), op(B)^T (first row tile)
-  int rta, rtb;            // last row tile of each that exists (later ones read it again)
   int nk16;                // K steps of 16
   int nstages;             // ring depth
   int nsc;                 // pieces of K whose undrained sums fit an int32
   int shift_top;           // left shift of level-2 sums in the int64 accumulator
   int tiles_m, tiles_n, lower;
-  int band;                // row pairs per band of the pair order (>= 1)
-  int ntiles;              // work items (tiles, or tile pairs); the grid takes them round-robin
+  int band;                // tile rows per band of the work order (>= 1)
+  int ntiles;              // work items, taken round-robin by the grid
   double alpha, betac;
   int alpha_pow2, alpha_exp, alpha_neg;  // alpha = (-1)^neg 2^exp when alpha_pow2
   // 0: C is not read (beta = 0); 1: v + C (beta = 1); 2: fma(beta, C, v).  A
@@ -168,45 +172,18 @@ struct OzParams {
   int no_loads;
 };
 
-// the tile (single form) or tile-row pair (pair form) of a work item
-// (oz_order.cuh)
-__device__ __forceinline__ void tile_of(const OzParams &p, int bid, int &tm, int &tn) {
-  oz_tile_of(p.lower, p.tiles_n, bid, tm, tn);
-}
-__device__ __forceinline__ void pair_of(const OzParams &p, int idx, int &TM, int &tn) {
-  oz_pair_of(p.tiles_m, p.tiles_n, p.lower, p.band, idx, TM, tn);
-}
-// This CTA's rank in its pair, its first work item and the stride between
-// its items (read from special registers where used: held in registers
-// across the role loops they pushed the 56-register warpgroup into spills).
-template <int CL>
-__device__ __forceinline__ int pair_rank() {
-  return CL == 2 ? (int)cluster_ctarank() : 0;
-}
-template <int CL>
-__device__ __forceinline__ int item_first() {
-  return CL == 2 ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-}
-template <int CL>
-__device__ __forceinline__ int item_stride() {
-  return CL == 2 ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-}
-// the output tile of this CTA for work item `item` (a tile, or a pair for CL =
-// 2; NT < 128: a part of one): tile row and column and the part's first column
-template <int CL, int NT>
-__device__ __forceinline__ void item_tile(const OzParams &p, int item, int rank, int &tm, int &tn,
-                                          int &n0) {
+// The output tile of work item `item` (NT < 128: a part of one) and the part's
+// first column, which lies past the last one for some parts: every role of a
+// CTA passes over those.
+template <int NT>
+__device__ __forceinline__ void item_tile(const OzParams &p, int item, int &tm, int &tn, int &n0) {
   constexpr int kParts = OBN / NT;
-  if (CL == 1) {
-    tile_of(p, item / kParts, tm, tn);
-  } else {
-    int TM;
-    pair_of(p, item, TM, tn);
-    tm = 2 * TM + rank;
-  }
+  if (NT == OBN)
+    oz_band_tile_of(p.tiles_m, p.tiles_n, p.lower, p.band, item, tm, tn);
+  else
+    oz_tile_of(p.lower, p.tiles_n, item / kParts, tm, tn);
   n0 = tn * OBN + item % kParts * NT;
 }
-
 
 // Every digit product of level L for one K step: pair (s, L - s) reads digit
 // tile s - 1 of A and L - s - 1 of B, at descriptor offsets of 256 (4 KB >> 4;
@@ -214,7 +191,7 @@ __device__ __forceinline__ void item_tile(const OzParams &p, int item, int rank,
 // so the issuing warp spends a few instructions per MMA: with loop bounds,
 // flags and descriptors computed at run time, or moved to uniform registers
 // for every MMA, it could not keep up with the tensor core (93 clocks of issue
-// per 64-clock MMA).  The first pair
+// per 64-clock MMA; 71 as it is).  The first pair
 // writes the accumulator when acc0 is 0 (first K step of a chunk).
 template <int S, int L, int NT>
 __device__ __forceinline__ void issue_level(uint32_t tmem, uint64_t da, uint64_t db, uint32_t acc0,
@@ -346,7 +323,7 @@ __device__ __forceinline__ void issue_entry(uint32_t tmem, uint64_t da, uint64_t
   }
 }
 
-template <int S, int CL, int NT, int G>
+template <int S, int NT, int G>
 __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
   using Sc = OzGroup<S, G>;
   OzHandover<Sc> H(k0, I.ord);
@@ -390,11 +367,8 @@ __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
           issue_entry<S, G, 1, NT>(I.tbase + 128 * q, da, db, 0u, I.lead);
       }
     }
-    // frees the smem slot when these MMAs finish (in both CTAs of a pair)
-    if (CL == 2)
-      mma_commit_mc_warp(I.empty0 + 8 * I.stage, (uint16_t)3, I.lead);
-    else
-      mma_commit_warp(I.empty0 + 8 * I.stage, I.lead);
+    // frees the smem slot when these MMAs finish
+    mma_commit_warp(I.empty0 + 8 * I.stage, I.lead);
     if (++I.stage == I.nst) {
       I.stage = 0;
       I.phase ^= 1;
@@ -408,7 +382,6 @@ __device__ __forceinline__ bool issue_piece(Issuer &I, int k0, int k1) {
 
 // The producer's loads of one piece of group G: a stage holds kSteps K steps
 // of kDigits digit tiles per operand; one bulk copy per operand and K step.
-// In a pair, the CTA whose rank is the step's parity loads B for both.
 struct Producer {
   uint32_t full0, empty0, smem0;
   int stage_bytes, nst;
@@ -419,7 +392,7 @@ struct Producer {
   int last_phase[4];
 };
 
-template <int S, int CL, int NT, int G>
+template <int S, int NT, int G>
 __device__ __forceinline__ bool load_piece(Producer &P, const unsigned char *a,
                                            const unsigned char *b, int k0, int k1) {
   using Sc = OzGroup<S, G>;
@@ -440,10 +413,9 @@ __device__ __forceinline__ bool load_piece(Producer &P, const unsigned char *a,
 #pragma unroll
         for (int q = 0; q < Sc::kDigits; ++q)
           bulk_load(sb + (j * Sc::kDigits + q) * kPart, b + src + q * kDigitTile, kPart, fb);
-      } else if (CL == 1)
+      } else {
         bulk_load(sb + j * kRun, b + src, kRun, fb);
-      else if (((ks + j) & 1) == (int)cluster_ctarank())
-        bulk_load_mc(sb + j * kRun, b + src, kRun, fb, (uint16_t)3);
+      }
     }
     P.last_phase[P.stage] = (int)P.phase;
     if (++P.stage == P.nst) {
@@ -454,25 +426,13 @@ __device__ __forceinline__ bool load_piece(Producer &P, const unsigned char *a,
   return true;
 }
 
-// S: digit count (OzGroup); persistent: each CTA takes work items item_first,
-// + item_stride, ...; the producer runs on into the next tile's data and the
+// S: digit count (OzGroup); persistent: each CTA takes the work items
+// blockIdx.x, + gridDim.x, ...; the producer runs on into the next tile's data and the
 // MMAs of the next tile start as soon as the epilogue has read the
 // accumulators, while the epilogue converts and stores the finished tile from
 // its registers.
-//
-// CL = 2: clusters of two CTAs on the tile rows 2 TM, 2 TM + 1 of one tile
-// column, which need the same B digit tiles.  Each CTA loads its own A tiles
-// and the B tiles of every second K step, multicast into both CTAs' shared
-// memory at the same offsets (the stage's full barrier in each CTA expects
-// all of its bytes), so B leaves L2 once for the two tiles: a quarter less L2
-// traffic.  A stage is free again only when both CTAs' MMAs are done with it:
-// the MMA commits arrive on the empty barriers of both CTAs (two arrivals a
-// phase).  Cluster barriers order the barrier initialisation before any
-// remote arrival and keep both CTAs alive until neither can reach the other's
-// shared memory.
-template <int S, int CL, int NT>
+template <int S, int NT>
 __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_constant__ OzParams p) {
-  static_assert(CL == 1 || NT == OBN, "a pair shares whole B tiles");
   constexpr int kEpiCols = NT * 4 / kEpiWarps;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte alignment for the swizzled tiles
@@ -494,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(full0 + 8 * s, 1);
-      mbar_init(empty0 + 8 * s, CL);
+      mbar_init(empty0 + 8 * s, 1);
     }
     for (int q = 0; q < 4; ++q) {
       mbar_init(accf + 8 * q, 1);
@@ -506,7 +466,6 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
   if (warp == 1) tmem_alloc(smem_u32(tmem_holder), 512);
   tc_fence_before();
   __syncthreads();
-  if (CL == 2) cluster_sync_all();  // both CTAs' barriers exist before any remote arrival
   tc_fence_after();
   const uint32_t tbase = __shfl_sync(0xffffffffu, *tmem_holder, 0);
 
@@ -519,22 +478,20 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       Producer P{full0, empty0, smem_u32(smem), stage_bytes, NST, st, p.wait_ns, 0, 0,
                  {-1, -1, -1, -1}};
       bool ok = (*((volatile int *)&st->code) == 0) && !p.no_loads;
-      for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
+      for (int item = blockIdx.x; item < p.ntiles && ok; item += gridDim.x) {
         int tm, tn, n0;
-        item_tile<CL, NT>(p, item, pair_rank<CL>(), tm, tn, n0);
-        if (NT < OBN && n0 >= p.N) continue;  // (all roles pass over it)
-        // (a pair's row tile past the last one reads the last one: its
-        // outputs lie outside C and are not stored)
+        item_tile<NT>(p, item, tm, tn, n0);
+        if (NT < OBN && n0 >= p.N) continue;
         const size_t rt_bytes = (size_t)p.nk16 * S * kDigitTile;
-        const unsigned char *a = p.DA + (size_t)min(tm, p.rta) * rt_bytes;
+        const unsigned char *a = p.DA + (size_t)tm * rt_bytes;
         const unsigned char *b =
-            p.DB + (size_t)min(tn, p.rtb) * rt_bytes + (size_t)(n0 - tn * OBN) * (KS * 2);
+            p.DB + (size_t)tn * rt_bytes + (size_t)(n0 - tn * OBN) * (KS * 2);
         if constexpr (OzDigitsOf<S>::kLow)
           for (int c = 0; c < p.nsc && ok; ++c)
-            ok = load_piece<S, CL, NT, 0>(P, a, b, oz_piece(p.nk16, p.nsc, c),
+            ok = load_piece<S, NT, 0>(P, a, b, oz_piece(p.nk16, p.nsc, c),
                                       oz_piece(p.nk16, p.nsc, c + 1));
         for (int c = 0; c < p.nsc && ok; ++c)
-          ok = load_piece<S, CL, NT, 1>(P, a, b, oz_piece(p.nk16, p.nsc, c),
+          ok = load_piece<S, NT, 1>(P, a, b, oz_piece(p.nk16, p.nsc, c),
                                     oz_piece(p.nk16, p.nsc, c + 1));
       }
       if (!ok) {
@@ -551,18 +508,18 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       Issuer I{tbase, full0, empty0, accf, acce, smem_u32(smem), stage_bytes, NST, st, p.wait_ns,
                0, 0, 0, 0, kOzSlots, elect_lane()};
       bool ok = __all_sync(0xffffffffu, *((volatile int *)&st->code) == 0) != 0;
-      for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
+      for (int item = blockIdx.x; item < p.ntiles && ok; item += gridDim.x) {
         if constexpr (NT < OBN) {
           int tm, tn, n0;
-          item_tile<CL, NT>(p, item, 0, tm, tn, n0);
+          item_tile<NT>(p, item, tm, tn, n0);
           if (n0 >= p.N) continue;
         }
         if constexpr (OzDigitsOf<S>::kLow)
           for (int c = 0; c < p.nsc && ok; ++c)
-            ok = issue_piece<S, CL, NT, 0>(I, oz_piece(p.nk16, p.nsc, c),
+            ok = issue_piece<S, NT, 0>(I, oz_piece(p.nk16, p.nsc, c),
                                        oz_piece(p.nk16, p.nsc, c + 1));
         for (int c = 0; c < p.nsc && ok; ++c)
-          ok = issue_piece<S, CL, NT, 1>(I, oz_piece(p.nk16, p.nsc, c),
+          ok = issue_piece<S, NT, 1>(I, oz_piece(p.nk16, p.nsc, c),
                                      oz_piece(p.nk16, p.nsc, c + 1));
       }
       // wait for every MMA this thread issued before TMEM is released
@@ -658,9 +615,9 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
       ord = H.end();
       return true;
     };
-    for (int item = item_first<CL>(); item < p.ntiles && ok; item += item_stride<CL>()) {
+    for (int item = blockIdx.x; item < p.ntiles && ok; item += gridDim.x) {
       int tm, tn, n0;
-      item_tile<CL, NT>(p, item, pair_rank<CL>(), tm, tn, n0);
+      item_tile<NT>(p, item, tm, tn, n0);
       if (NT < OBN && n0 >= p.N) continue;
       const int m0 = tm * OBM;
       // beta C is read only when the tile is written out, after all of its
@@ -781,9 +738,6 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
   }
   tc_fence_before();
   __syncthreads();
-  // neither CTA of a pair leaves while the other may still write its shared
-  // memory or arrive on its barriers
-  if (CL == 2) cluster_sync_all();
   tc_fence_after();
   if (warp == 1) tmem_dealloc(tbase, 512);
 }
@@ -1053,80 +1007,44 @@ static_assert(oz_max_stages<7>() >= 3 && oz_max_stages<6>() >= 4, "ring too shal
 // size, and the check that the warpgroups' register split (setmaxnreg) adds
 // up to exactly kLaunchRegs a thread (a build that launches with any other
 // count is refused rather than run: an increase that cannot be met never
-// returns).  Also the most clusters of two that can be resident at once.
-template <int S, int CL, int NT>
-cudaError_t oz_prepare(int &max_items) {
-  cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, CL, NT>,
+// returns).  nsm: SMs of the device.
+template <int S, int NT>
+cudaError_t oz_prepare(int &nsm) {
+  cudaError_t e = cudaFuncSetAttribute(ozaki_gemm_kernel<S, NT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)oz_smem<S>(oz_max_stages<S>()));
   if (e != cudaSuccess) return e;
   cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, ozaki_gemm_kernel<S, CL, NT>);
+  e = cudaFuncGetAttributes(&fa, ozaki_gemm_kernel<S, NT>);
   if (e != cudaSuccess) return e;
   if (NT == OBN && fa.numRegs != kLaunchRegs) return cudaErrorInvalidConfiguration;
-  int dev = 0, nsm = 0;
+  int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return e;
-  if (CL == 1) {
-    max_items = nsm;
-    return cudaSuccess;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * (unsigned)nsm);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = oz_smem<S>(oz_max_stages<S>());
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int ncl = 0;
-  e = cudaOccupancyMaxActiveClusters(&ncl, ozaki_gemm_kernel<S, CL, NT>, &cfg);
-  if (e != cudaSuccess) return e;
-  max_items = ncl > 0 ? ncl : 1;
-  return cudaSuccess;
+  return cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
 }
 
-template <int S, int CL, int NT>
-cudaError_t launch_oz_t(int nitems, int reserve_sms, OzParams &p, cudaStream_t st) {
-  static int max_items = 0;
+template <int S, int NT>
+cudaError_t launch_oz_t(int reserve_sms, OzParams &p, cudaStream_t st) {
+  static int nsm = 0;
   static cudaError_t prep = cudaErrorNotReady;
   static std::once_flag once;
-  std::call_once(once, [] { prep = oz_prepare<S, CL, NT>(max_items); });
+  std::call_once(once, [] { prep = oz_prepare<S, NT>(nsm); });
   if (prep != cudaSuccess) return prep;
   // persistent: one CTA per SM (one fits: 512 TMEM columns, ~200 KB of
-  // shared memory), the CTAs (or pairs) taking every grid-th work item;
-  // reserve_sms SMs (rounded up to whole pairs) stay free for other streams
-  int cap = max_items - (reserve_sms + CL - 1) / CL;
-  if (cap < 1) cap = 1;
-  const int items = nitems < cap ? nitems : cap;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(CL * items));
-  cfg.blockDim = dim3(kThreads);
+  // shared memory), the CTAs taking every grid-th work item; reserve_sms SMs
+  // stay free for other streams
+  const int cap = nsm > reserve_sms ? nsm - reserve_sms : 1;
   p.nstages = p.nstages < oz_max_stages<S>() ? p.nstages : oz_max_stages<S>();
-  cfg.dynamicSmemBytes = oz_smem<S>(p.nstages);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, ozaki_gemm_kernel<S, CL, NT>, p);
+  ozaki_gemm_kernel<S, NT>
+      <<<(unsigned)(p.ntiles < cap ? p.ntiles : cap), kThreads, oz_smem<S>(p.nstages), st>>>(p);
   count_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return cudaGetLastError();
 }
 
 template <int S>
-cudaError_t launch_oz(bool narrow, bool pairs, int reserve_sms, OzParams &p, cudaStream_t st) {
+cudaError_t launch_oz(bool narrow, int reserve_sms, OzParams &p, cudaStream_t st) {
   const int rsv = reserve_sms > 0 ? reserve_sms : 0;
-  if (narrow) return launch_oz_t<S, 1, kNarrow>(p.ntiles, rsv, p, st);
-  return pairs ? launch_oz_t<S, 2, OBN>(p.ntiles, rsv, p, st)
-               : launch_oz_t<S, 1, OBN>(p.ntiles, rsv, p, st);
+  return narrow ? launch_oz_t<S, kNarrow>(rsv, p, st) : launch_oz_t<S, OBN>(rsv, p, st);
 }
 
 }  // namespace
@@ -1149,10 +1067,7 @@ cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t
   p.ea = A.e + ra;
   p.eb = B.e + rb;
   const int tiles_m = (int)((M + OBM - 1) / OBM);
-  p.tiles_m = tiles_m;
   p.tiles_n = (int)((N + OBN - 1) / OBN);
-  p.rta = tiles_m - 1;
-  p.rtb = p.tiles_n - 1;
   {
     const int64_t ns = tune_get("ozaki_stages", kMaxStages);
     p.nstages = ns < 2 ? 2 : (ns > kMaxStages ? kMaxStages : (int)ns);
@@ -1176,23 +1091,25 @@ cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t
   p.status = status;
   p.no_loads = tune_get("test_wait_timeout", 0) != 0 ? 1 : 0;
   p.wait_ns = p.no_loads ? 1000000ull : kWaitNs;  // 1 ms in the failure-path test
-  {
-    const int64_t b = tune_get("ozaki_band", 6);
-    p.band = b < 1 ? 1 : (b > 4096 ? 4096 : (int)b);
-  }
   // Half-width tiles while they still fit one wave (152 SMs): the wide ones
   // would leave more than half of the SMs idle.  T Nside 16 harmonic solve 14.9
   // -> 12.8 ms, TQU Nside 8 solve 4.79 -> 4.56, 1000-map estimate 2.88 -> 2.76;
   // the same bits.
   const int tiles = oz_item_count(tiles_m, p.tiles_n, lower ? 1 : 0, 0);
   const bool narrow = 2 * tiles <= 152 - reserve_sms;
-  // else clusters of two on tile-row pairs (B shared through multicast) unless
-  // switched off or the output has a single tile row
-  const bool pairs = !narrow && tune_get("ozaki_pairs", 1) != 0 && tiles_m >= 2;
-  p.ntiles = narrow ? 2 * tiles : oz_item_count(tiles_m, p.tiles_n, lower ? 1 : 0, pairs ? 1 : 0);
-  if (S == 3) return launch_oz<3>(narrow, pairs, reserve_sms, p, st);
-  if (S == 6) return launch_oz<6>(narrow, pairs, reserve_sms, p, st);
-  return launch_oz<7>(narrow, pairs, reserve_sms, p, st);
+  p.ntiles = narrow ? 2 * tiles : tiles;
+  p.tiles_m = tiles_m;
+  {
+    // bands of eight tile rows: QU Nside 32 solve 307.6 ms row by row, 292.8 in
+    // bands of 4 or 8, 294.8 of 12, 295.7 of 16 (its products re-read digits from
+    // DRAM); TQU Nside 16 solve (QML_FP64) 38.3, 37.9, 37.9, 37.9; products whose
+    // digits stay in L2 do not change
+    const int64_t b = tune_get("ozaki_band", 8);
+    p.band = b < 1 ? 1 : (b > 4096 ? 4096 : (int)b);
+  }
+  if (S == 3) return launch_oz<3>(narrow, reserve_sms, p, st);
+  if (S == 6) return launch_oz<6>(narrow, reserve_sms, p, st);
+  return launch_oz<7>(narrow, reserve_sms, p, st);
 }
 
 }  // namespace qmlgb

@@ -69,17 +69,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
       ::"r"(dst), "l"((uint64_t)src), "r"(bytes), "r"(bar)
       : "memory");
 }
-// the same copy delivered to every CTA of the cluster named in cta_mask, at the
-// same shared-memory offset, each completing on the mbarrier at bar's offset
-// in that CTA
-__device__ __forceinline__ void bulk_load_mc(uint32_t dst, const void *src, uint32_t bytes,
-                                             uint32_t bar, uint16_t cta_mask) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster"
-      " [%0], [%1], %2, [%3], %4;" ::"r"(dst),
-      "l"((uint64_t)src), "r"(bytes), "r"(bar), "h"(cta_mask)
-      : "memory");
-}
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -179,14 +168,6 @@ __device__ __forceinline__ void mma_commit_warp(uint32_t bar, uint32_t lead) {
       "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
       " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar),
       "r"(lead)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit_mc_warp(uint32_t bar, uint16_t cta_mask, uint32_t lead) {
-  asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
-      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-      " [%0], %1;\n}" ::"r"(bar),
-      "h"(cta_mask), "r"(lead)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {

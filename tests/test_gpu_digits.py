@@ -156,3 +156,26 @@ def test_rows_and_columns_of_any_size(api, m, n, beta):
         err = np.abs(C[~inf] - ref[~inf])
         assert (err <= 2.0 ** -43 * np.abs(ref - beta * C0)[~inf] + 2.0 ** -51 * np.abs(ref[~inf])
                 + 2.0 ** -1073).all()
+
+
+@pytest.mark.parametrize("m,n,lower", [(2500, 2500, True), (1300, 2300, False)])
+def test_work_order_bands_same_bits(api, m, n, lower):
+    """Tiles taken in bands of one row, of an odd few, of more rows than there are."""
+    rng = np.random.default_rng(m)
+    A = td(rng.normal(size=(m, 70)))
+    B = A if lower else td(rng.normal(size=(n, 70)))
+    outs = []
+    try:
+        for band in (1, 3, 8, 4096):
+            api.tune_set("ozaki_band", band)
+            C = td(np.ones((m, n)))
+            api.gemm(A, B, C, transB=True, alpha=-1.0, beta=1.0, lower=lower, precision=1)
+            outs.append(C)
+    finally:
+        api.tune_set("ozaki_band", 8)
+    assert all(torch.equal(outs[0], C) for C in outs[1:])
+    ref = 1.0 - (A @ B.t()).cpu().numpy()
+    got = outs[0].cpu().numpy()
+    sel = np.tril(np.ones((m, n), bool)) if lower else np.ones((m, n), bool)
+    assert np.abs(got - ref)[sel].max() <= 1e-12 * np.abs(ref).max()
+    assert (got[~sel] == 1.0).all()
