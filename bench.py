@@ -364,7 +364,7 @@ def run_ours(args):
     wl, cfg = workload_config(args.nsims)
     cfg["parallelism"] = f"replicas x{world} (no data-path collective)"
     cfg["products"] = ("QML_FP64: float64 in and out, large products by 55-bit digits "
-                       "(7 x 8 bits in bf16, exact sums), closer than a float64 accumulation")
+                       "(7 x 8 bits in bf16 below each row's maximum, exact sums)")
 
     # ---- CPU baseline (rank 0, N = 1 only): the oracle as it stands; its
     # solve is kept as the reference of the forms' relative errors

@@ -66,9 +66,15 @@ typedef enum {
   QML_FP64 = 0,        /* float64 throughout.  Problems of order n >= 256 run
                           their large contractions as exact products of 55-bit
                           digits on tensor cores, recombined and rounded once
-                          to float64 (error below a float64 accumulation's);
-                          diagonal blocks, logdets and everything else, and
-                          qml_gemm / qml_potrf / qml_trsm, stay native */
+                          to float64: K terms to within K 2^-53 max|a| max|b|,
+                          typically sqrt(K) 2^-56, the maxima over the row of
+                          one operand and the column of the other (a float64
+                          sum: K 2^-53 sum |a b|).  Products with block
+                          inverses have the pixels' scales divided out
+                          beforehand, exactly, so that the noise of the
+                          pixels may differ by any factor.  Diagonal blocks,
+                          logdets and everything else, and qml_gemm /
+                          qml_potrf / qml_trsm, stay native */
   QML_SPLIT_BF16 = 1   /* large contractions as 48-bit bf16-digit products on
                           tcgen05 tensor cores (Ozaki-style splitting),
                           recombined in float64; panels, logdets stay float64 */

@@ -398,6 +398,18 @@ struct DigitBuf {
   size_t bytes = 0;
 };
 
+// Column maxima and shifts for the products with block inverses (K <= kNBS),
+// zeroed on the call's stream.
+OzColumns make_columns(Call &c) {
+  OzColumns o;
+  unsigned char *p = c.alloc<unsigned char>(12 * kNBS + 8, "column shifts");
+  if (!p || !c.cuda_ok(cudaMemsetAsync(p, 0, 8 * kNBS + 8, c.st), "column shifts")) return o;
+  o.kmax = (unsigned long long *)p;
+  o.done = (unsigned *)(p + 8 * kNBS);
+  o.shift = (int *)(p + 8 * kNBS + 8);
+  return o;
+}
+
 struct Split {
   Call *c;
   int S;  // digits per operand (oz_split_digits, kOzF64Digits)
@@ -407,22 +419,55 @@ struct Split {
   // SMs the split kernel leaves free (for float64 work on a second stream)
   int reserve_sms = 0;
   DigitBuf buf[3];
+  OzColumns cols;  // scales of the products with block inverses
   double *tinv = nullptr;  // (kNBS/2)^2 scratch of the block-inverse doubling
   // the doubling scratch, allocated on first use unless preset
   double *tinv_scratch() {
     if (!tinv) tinv = c->alloc<double>((size_t)(kNBS / 2) * (kNBS / 2), "inverse scratch");
     return tinv;
   }
-  // Digits of X (element (r, k) at X[r sr + k sk]) into buffer i.
-  OzDigits slice(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
+  // memory for the digits of an R x K matrix in buffer i
+  OzDigits digits(int i, int64_t R, int64_t K) {
     const size_t need = oz_digits_bytes(R, K, S);
     if (need > buf[i].bytes) {
       buf[i].p = c->alloc<unsigned char>(need, "split workspace");
       buf[i].bytes = buf[i].p ? need : 0;
     }
-    if (!buf[i].p) return OzDigits{};
-    const OzDigits d = oz_digits_at(buf[i].p, R, K, S);
-    oz_slice(X, sr, sk, d, c->st);
+    return buf[i].p ? oz_digits_at(buf[i].p, R, K, S) : OzDigits{};
+  }
+  // Digits of X (element (r, k) at X[r sr + k sk]) into buffer i.
+  OzDigits slice(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
+    const OzDigits d = digits(i, R, K);
+    if (d.dig) oz_slice(X, sr, sk, d, c->st);
+    return d;
+  }
+  // The operands of a product with a block inverse: the right-hand sides (the
+  // rows of X), then the inverse.  Where the pixels of a block differ in scale by
+  // d_k, the right-hand sides' columns carry d_k and the inverse's 1 / d_k, and
+  // digits below each row's maximum lose the ratio of the d_k: with a spread of
+  // 1e4, 3.6e-14 of its row's scale on an entry of the factor and 2e-12 on a
+  // whitened map (a float64 solve: 2e-17, 1.5e-15; digits emulated on the host, n =
+  // 640, C = D R D, against extended precision).  At float64 quality both are
+  // sliced with that scale divided out by powers of two, exactly: 7e-17 and
+  // 2e-15, for a spread of 1 to 1e8.  The 48-bit form keeps plain rows.
+  OzDigits slice_rhs(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
+    const OzDigits d = digits(i, R, K);
+    if (f64 && !cols.kmax) cols = make_columns(*c);
+    if (c->err != QML_OK) return OzDigits{};
+    if (f64)
+      oz_slice_rhs(X, sr, sk, d, cols, c->st);
+    else
+      oz_slice(X, sr, sk, d, c->st);
+    return d;
+  }
+  // the inverse for the right-hand sides sliced last
+  OzDigits slice_inverse(int i, const double *X, int64_t n, int64_t sr, int64_t sk) {
+    const OzDigits d = digits(i, n, n);
+    if (c->err != QML_OK) return OzDigits{};
+    if (f64)
+      oz_slice_inverse(X, sr, sk, d, cols, c->st);
+    else
+      oz_slice(X, sr, sk, d, c->st);
     return d;
   }
   void mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t ra, const OzDigits &B,
@@ -494,15 +539,15 @@ size_t split_ws_bytes(int i, int64_t n, int64_t nrhs, int S) {
 
 // QML_FP64 at and above this order factors and multiplies with 55-bit digit
 // products (kOzF64Digits) instead of the float64 pipe, whose 1.2 TFLOP/s bound
-// every contraction (TQU Nside 16 solve: 736 ms, 46.5 with digits).  Error: on
-// the operands of C = G G^T, the trailing updates, the solves and W = X^T X at
-// TQU Nside 16, QU Nside 16 and T Nside 8 an extended-precision reference puts
-// the 55-bit products 1.6 to 50 times closer than a float64 accumulation (C:
-// 7e-18 against 3.5e-16 of the row norms); F, y, lnL of T Nside 8 come out 4 to
-// 14 times closer.  Below about 250 rows the float64 path needs fewer
-// launches: lnL 0.59 against 0.72 ms at n = 192 but Fisher 1.03 against 1.00
-// ms, both in favour of digits from n = 300 on (0.78 against 1.08, 1.30
-// against 1.34 ms).
+// every contraction (TQU Nside 16 solve: 736 ms, 46.5 with digits).  Error of a
+// product: an operand is rounded to 2^-56 of its row's power of two, so K terms
+// give at most K 2^-53 max|a| max|b| (a float64 sum: K 2^-53 sum |a b|), and
+// typically sqrt(K) 2^-56 of the maxima.  In C = G G^T, the trailing updates and W =
+// X^T X the maxima belong to the terms that matter (max_k |L_ik| <= sqrt(C_ii));
+// the products with block inverses are scaled so that they do (slice_rhs).
+// Below about 250 rows the float64 path needs fewer launches: lnL 0.59 against
+// 0.72 ms at n = 192 but Fisher 1.03 against 1.00 ms, both in favour of digits
+// from n = 300 on (0.78 against 1.08, 1.30 against 1.34 ms).
 constexpr int64_t kF64SplitMin = 256;
 
 // The digit products of a problem's precision for an order-n factor: 0 for
@@ -624,8 +669,8 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
       double *A22 = A + (j + jb) + (j + jb) * lda;
       const int64_t jb2 = m2 < kNBS ? m2 : kNBS;
       // panel: A21 <- A21 L_jj^-T
-      dP = sp.slice(0, A21, m2, jb, 1, lda);
-      const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
+      dP = sp.slice_rhs(0, A21, m2, jb, 1, lda);
+      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
       sp.mm(m2, jb, 1.0, dP, 0, dX, 0, 0.0, A21, lda, 0);
       dP = sp.slice(0, A21, m2, jb, 1, lda);
       if (look) {
@@ -648,8 +693,8 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
       sp.few_panel(Xinv, jb, A21, lda, m2, B + j, nrhs, ldb);
     } else if (B) {
       // forward substitution, panel j: B_j <- L_jj^-1 B_j ; B_below -= A21 B_j
-      const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
-      OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+      OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
+      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
       sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
       if (m2 > 0) {
         dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
@@ -685,8 +730,8 @@ void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, con
       sp.few_panel(Xinv, jb, L + (j + jb) + j * lda, lda, n - j - jb, B + j, nrhs, ldb);
       continue;
     }
-    const OzDigits dX = sp.slice(1, Xinv, jb, jb, 1, kNBS);
-    OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+    OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
+    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
     sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
     const int64_t m2 = n - j - jb;
     if (m2 > 0) {
@@ -704,8 +749,8 @@ void trsm_split_t(Call &c, Split &sp, const double *L, int64_t n, int64_t lda,
   for (int64_t b = (n + nb - 1) / nb - 1; b >= 0; --b) {
     const int64_t j = b * nb, jb = (n - j) < nb ? (n - j) : nb;
     const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS + (j % kNBS) * (kNBS + 1);
-    const OzDigits dX = sp.slice(1, Xinv, jb, jb, kNBS, 1);
-    OzDigits dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
+    OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
+    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, kNBS, 1);
     sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
     if (j > 0) {
       const OzDigits dP = sp.slice(0, L + j, j, jb, lda, 1);
@@ -730,10 +775,11 @@ void inner_potrf(Call &c, Split &sp, const InnerFactor &K, int64_t k, double *ld
 }
 // B <- L_K^-1 B, or with both set Kt^-1 B = L_K^-T L_K^-1 B.  The harmonic
 // basis takes blocks of 128 (kInnerNB): its right-hand sides are graded along
-// the modes (sqrt(Lambda) times noise weights, two orders between T and B), and
-// digits are relative to a block column's maximum.  With 512-wide blocks small
-// entries of F lost two digits (1.2e-10 of an entry against 1.6e-12 on the
-// float64 pipe, TQU Nside 4; 1.5e-12 with 128).
+// the modes (sqrt(Lambda) times noise weights, two orders between T and B), each
+// in its own way, and digits are relative to a block column's maximum.  Without
+// scaled columns (slice_rhs) 512-wide blocks lost two digits of small entries of F
+// (1.2e-10 of an entry against 1.6e-12 on the float64 pipe, TQU Nside 4; 1.5e-12
+// with 128).
 constexpr int64_t kInnerNB = 128;
 void inner_trsm(Call &c, Split &sp, const InnerFactor &K, int64_t k, double *B, int64_t nrhs,
                 int64_t ldb, bool both, int64_t nb = kNBS) {
@@ -1356,6 +1402,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     double *K, *lamL, *z, *rr, *Linv, *LinvB, *ldp;
     double *cl, *lnK, *lnl, *chi, *ld;  // fixed slots of the captured sequence
     double *tinv;                       // block-inverse scratch (split)
+    OzColumns cols;
     DigitBuf buf[3];
   };
   std::vector<Worker> wk(NS);
@@ -1386,6 +1433,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
       wk[w].buf[b].p = c.alloc<unsigned char>(wk[w].buf[b].bytes, "split workspace");
     }
     wk[w].tinv = any_split ? c.alloc<double>((size_t)(kNBS / 2) * (kNBS / 2)) : nullptr;
+    if (any_split) wk[w].cols = make_columns(c);
   }
   if (c.err != QML_OK) return c.finish();
   cudaEvent_t setup_done;
@@ -1414,6 +1462,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     Split spl = kt_split(cw, m);
     for (int b = 0; b < 3; ++b) spl.buf[b] = W.buf[b];
     spl.tinv = W.tinv;
+    spl.cols = W.cols;
     const InnerFactor K{W.K, W.Linv, W.LinvB};
     inner_potrf(cw, spl, K, k, W.ldp, lnKp);
     inner_trsm(cw, spl, K, k, W.z, nm, k, false);

@@ -231,6 +231,20 @@ size_t oz_digits_bytes(int64_t R, int64_t K, int S);
 OzDigits oz_digits_at(void *mem, int64_t R, int64_t K, int S);
 // element (r, k) at X[r sr + k sk], one of the strides 1
 void oz_slice(const double *X, int64_t sr, int64_t sk, const OzDigits &d, cudaStream_t st);
+// The two operands of a product with an inverse, B X^-T and the like, whose sizes
+// run against each other along k: the right-hand sides' columns k are brought to
+// one size by powers of two (c.shift), the inverse's by the opposite ones.  The
+// product is the same, term by term.  For d.S = kOzF64Digits and K up to the columns
+// that c has; its maxima and count are zero before each call and after it.
+struct OzColumns {
+  unsigned long long *kmax = nullptr;  // then the count and the shifts
+  unsigned *done = nullptr;
+  int *shift = nullptr;
+};
+void oz_slice_rhs(const double *X, int64_t sr, int64_t sk, const OzDigits &d, const OzColumns &c,
+                  cudaStream_t st);
+void oz_slice_inverse(const double *X, int64_t sr, int64_t sk, const OzDigits &d,
+                      const OzColumns &c, cudaStream_t st);
 // C (M x N) <- alpha A B^T + beta C for the rows ra .. of A and rb .. of B
 // (multiples of 128).  reserve_sms: SMs the persistent kernel leaves free.
 cudaError_t oz_mm(int64_t M, int64_t N, double alpha, const OzDigits &A, int64_t ra,

@@ -747,22 +747,69 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(const __grid_co
 // non-negative float64 values the integer order is the numeric order).
 // Bound by the latency of the loads: eight are in flight a thread (one at a
 // time, a 6400 x 512 panel took 17 us).
-__device__ __forceinline__ unsigned long long max_bits(double x, unsigned long long mb) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+// exponent e of a finite m > 0 in the frexp convention, m in [2^(e-1), 2^e)
+__device__ __forceinline__ int frexp_exponent(unsigned long long m) {
+  const int E = (int)(m >> 52);
+  return E ? E - 1022 : (64 - __clzll((long long)m)) - 1074;
+}
+
+// Scaled operands (kScaled): column k of the operand is taken times 2^t_k, t_k =
+// sgn shift[k] from the other operand of the product or its own (oz_slice_rhs,
+// oz_slice_inverse).  Row maxima are then kept as exponents, kKeyBias + e + t,
+// which no scaling takes out of range.  A column with shift kNoTerm has no
+// finite entry but 0 in the operand that set the shifts, so its terms are 0.
+constexpr int kNoTerm = 1 << 24, kKeyBias = 16384;
+struct Scaling {
+  const int *shift;
+  int sgn;
+};
+template <bool kScaled>
+__device__ __forceinline__ unsigned long long row_key(double x, int shift, int sgn) {
+  const unsigned long long m = abs_bits(x);
+  if (!kScaled) return m;
+  if ((m >> 52) == 0x7FF) return ~0ull;
+  if (m == 0 || shift == kNoTerm) return 0;
+  return (unsigned long long)(kKeyBias + frexp_exponent(m) + sgn * shift);
+}
+// the greatest key of x[u step], u < 8, columns k + u kstep
+template <bool kScaled>
+__device__ __forceinline__ unsigned long long row_key8(const double *x, int64_t step, Scaling sc,
+                                                       int64_t k, int kstep,
+                                                       unsigned long long mb) {
+  double v[8];
+  int t[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    v[u] = x[u * step];
+    t[u] = kScaled ? sc.shift[k + u * kstep] : 0;
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const unsigned long long b = row_key<kScaled>(v[u], t[u], sc.sgn);
+    mb = b > mb ? b : mb;
+  }
+  return mb;
+}
+template <bool kScaled>
+__device__ __forceinline__ unsigned long long row_key1(double x, Scaling sc, int64_t k,
+                                                       unsigned long long mb) {
+  const unsigned long long b = row_key<kScaled>(x, kScaled ? sc.shift[k] : 0, sc.sgn);
   return b > mb ? b : mb;
 }
-__device__ __forceinline__ unsigned long long max_bits8(const double *x, int64_t step,
-                                                        unsigned long long mb) {
-  double v[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) v[u] = x[u * step];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) mb = max_bits(v[u], mb);
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long mb) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long t = __shfl_xor_sync(0xffffffffu, mb, o);
+    mb = t > mb ? t : mb;
+  }
   return mb;
 }
 // Rows strided, k contiguous: one warp per row, lanes stride over k.
+template <bool kScaled>
 __global__ void rowmax_kcontig_kernel(const double *X, int64_t R, int64_t K, int64_t sr,
-                                      unsigned long long *bits, int Rpad) {
+                                      unsigned long long *bits, int Rpad, Scaling sc) {
   const int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= Rpad) return;
@@ -770,13 +817,10 @@ __global__ void rowmax_kcontig_kernel(const double *X, int64_t R, int64_t K, int
   if (r < R) {
     const double *x = X + r * sr;
     int64_t k = lane;
-    for (; k + 7 * 32 < K; k += 8 * 32) mb = max_bits8(x + k, 32, mb);
-    for (; k < K; k += 32) mb = max_bits(x[k], mb);
+    for (; k + 7 * 32 < K; k += 8 * 32) mb = row_key8<kScaled>(x + k, 32, sc, k, 32, mb);
+    for (; k < K; k += 32) mb = row_key1<kScaled>(x[k], sc, k, mb);
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long t = __shfl_xor_sync(0xffffffffu, mb, o);
-    mb = t > mb ? t : mb;
-  }
+  mb = warp_max(mb);
   if (lane == 0) bits[r] = mb;
 }
 
@@ -784,8 +828,9 @@ __global__ void rowmax_kcontig_kernel(const double *X, int64_t R, int64_t K, int
 // values of k; a warp reads 32 consecutive rows at one k (coalesced), the 8
 // warps take every 8th k, and the block's maximum per row joins the others
 // with atomicMax (bits zeroed beforehand).
+template <bool kScaled>
 __global__ void rowmax_rcontig_kernel(const double *X, int64_t R, int64_t K, int64_t sk,
-                                      unsigned long long *bits) {
+                                      unsigned long long *bits, Scaling sc) {
   __shared__ unsigned long long part[8][32];
   const int rl = threadIdx.x & 31, kg = threadIdx.x >> 5;
   const int64_t r = (int64_t)blockIdx.x * 32 + rl;
@@ -793,8 +838,9 @@ __global__ void rowmax_rcontig_kernel(const double *X, int64_t R, int64_t K, int
   unsigned long long mb = 0;
   if (r < R) {
     int64_t k = kc0 + kg;
-    for (; k + 7 * 8 < kc1; k += 8 * 8) mb = max_bits8(X + r + k * sk, 8 * sk, mb);
-    for (; k < kc1; k += 8) mb = max_bits(X[r + k * sk], mb);
+    for (; k + 7 * 8 < kc1; k += 8 * 8)
+      mb = row_key8<kScaled>(X + r + k * sk, 8 * sk, sc, k, 8, mb);
+    for (; k < kc1; k += 8) mb = row_key1<kScaled>(X[r + k * sk], sc, k, mb);
   }
   part[kg][rl] = mb;
   __syncthreads();
@@ -804,18 +850,89 @@ __global__ void rowmax_rcontig_kernel(const double *X, int64_t R, int64_t K, int
   }
 }
 
-// exponent e of a row maximum m (frexp convention: m < 2^e, 0 for m = 0,
-// kNanExp for an infinity or a NaN)
+// Shifts of an operand's columns: with m_k the largest finite |x_rk|, in [2^(e_k -
+// 1), 2^e_k), and e the largest e_k, shift[k] = max(0, e - e_k - 1), kNoTerm where
+// m_k = 0.  The operand's column k times 2^shift[k] against the other one's
+// times 2^-shift[k] is the same product term by term; with all columns of about
+// one size (within a factor of two) nothing is shifted.  The maxima and the count
+// of finished blocks are zero beforehand, and the last block to finish, which
+// forms the shifts, zeroes them again.  Columns run over contiguous r
+// (kRowsContig): a warp a column and kColRows rows of it; else over contiguous k: a
+// block 32 columns and kColRowsK rows.  Bound by latency: 16 (8) loads a thread.
+constexpr int kColRows = 512, kColRowsK = 64;
+template <bool kRowsContig>
+__global__ void __launch_bounds__(256) column_shift_kernel(const double *X, int64_t R, int64_t K,
+                                                           int64_t stride, OzColumns c) {
+  __shared__ unsigned long long part[8][32];
+  __shared__ int top[8];
+  __shared__ bool last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto finite_max = [](double x, unsigned long long mb) {
+    const unsigned long long b = abs_bits(x);
+    return b > mb && (b >> 52) != 0x7FF ? b : mb;
+  };
+  unsigned long long mb = 0;
+  const int64_t step = kRowsContig ? 32 : 8 * stride;
+  const int64_t k = kRowsContig ? (int64_t)blockIdx.x * 8 + warp : (int64_t)blockIdx.x * 32 + lane;
+  const int64_t chunk = kRowsContig ? kColRows : kColRowsK, ro = kRowsContig ? lane : warp;
+  const int rstep = kRowsContig ? 32 : 8;
+  const int64_t r0 = (int64_t)blockIdx.y * chunk, r1 = r0 + chunk < R ? r0 + chunk : R;
+  if (k < K) {
+    const double *x = kRowsContig ? X + k * stride : X + k;
+    int64_t r = r0 + ro;
+    const double *p = kRowsContig ? x + r : x + r * stride;
+    for (; r + 7 * rstep < r1; r += 8 * rstep, p += 8 * step) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = p[u * step];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) mb = finite_max(v[u], mb);
+    }
+    for (; r < r1; r += rstep, p += step) mb = finite_max(*p, mb);
+  }
+  if (kRowsContig) {
+    mb = warp_max(mb);
+    if (lane == 0 && mb) atomicMax(&c.kmax[k], mb);
+  } else {
+    part[warp][lane] = mb;
+    __syncthreads();
+    if (warp == 0) {
+      for (int q = 1; q < 8; ++q) mb = part[q][lane] > mb ? part[q][lane] : mb;
+      if (mb) atomicMax(&c.kmax[k], mb);
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(c.done, 1u) + 1 == gridDim.x * gridDim.y;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  volatile unsigned long long *km = c.kmax;
+  int e = -kNoTerm;
+  for (int64_t q = tid; q < K; q += 256) {
+    const unsigned long long m = km[q];
+    if (m) e = max(e, frexp_exponent(m));
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) top[warp] = e;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 8; ++q) e = max(e, top[q]);
+  for (int64_t q = tid; q < K; q += 256) {
+    const unsigned long long m = km[q];
+    c.shift[q] = m ? max(0, e - frexp_exponent(m) - 1) : kNoTerm;
+    km[q] = 0;
+  }
+  if (tid == 0) *c.done = 0;
+}
+
+// exponent e of a row from its maximum (frexp convention: every |x| < 2^e, 0 for
+// a row of zeros, kNanExp for one with an infinity or a NaN)
+template <bool kScaled>
 __device__ __forceinline__ int exponent_of(unsigned long long m) {
   if (m == 0) return 0;
-  const int E = (int)(m >> 52);
-  if (E == 0x7FF) return kNanExp;
-  if (E == 0) {  // subnormal maximum
-    int ex = 0;
-    frexp(__longlong_as_double((long long)m), &ex);
-    return ex;
-  }
-  return E - 1022;  // m = 1.f 2^(E-1023) = (1.f / 2) 2^(E-1022)
+  if (kScaled) return m == ~0ull ? kNanExp : (int)m - kKeyBias;
+  return (m >> 52) == 0x7FF ? kNanExp : frexp_exponent(m);
 }
 
 // x 2^sh rounded to an integer (halves away from zero) by integer operations
@@ -829,7 +946,7 @@ __device__ __forceinline__ long long scaled_round(double x, int sh) {
   const int t = (bexp != 0 ? bexp : 1) - 1075 + sh;
   unsigned long long q;
   if (t >= 0)
-    q = m << t;
+    q = m << (t & 63);  // (t above 55 for a zero only)
   else
     q = t < -54 ? 0 : (m + (1ull << (-t - 1))) >> -t;
   return bits < 0 ? -(long long)q : (long long)q;
@@ -846,15 +963,15 @@ __device__ __forceinline__ long long scaled_round(double x, int sh) {
 // bytes is digit 1.  A byte becomes a float through the bit pattern of
 // 2^23 + byte.  Digit s carries the weight 2^(-8 (s - 1)), for the two
 // levels that share an accumulator.
-template <int S>
+template <int S, bool kScaled>
 __global__ void __launch_bounds__(256) slice_kernel(const double *X, int64_t R, int64_t K,
                                                     int64_t sr, int64_t sk,
                                                     const unsigned long long *mx, int *e,
-                                                    unsigned char *D) {
+                                                    unsigned char *D, Scaling sc) {
   using Dg = OzDigitsOf<S>;
   const int rl = threadIdx.x >> 1, ch = threadIdx.x & 1;
   const int64_t r = (int64_t)blockIdx.y * OBM + rl, k0 = (int64_t)blockIdx.x * KS + 8 * ch;
-  const int er = r < R ? exponent_of(mx[r]) : 0;
+  const int er = r < R ? exponent_of<kScaled>(mx[r]) : 0;
   if (blockIdx.x == 0 && ch == 0) e[r] = er;
   double x[8];
 #pragma unroll
@@ -863,7 +980,15 @@ __global__ void __launch_bounds__(256) slice_kernel(const double *X, int64_t R, 
   unsigned long long F[8];
   constexpr unsigned long long kBias = 0x8080808080808080ull >> (64 - 8 * (S - 1));
 #pragma unroll
-  for (int j = 0; j < 8; ++j) F[j] = (unsigned long long)scaled_round(x[j], Dg::kBits - er) + kBias;
+  for (int j = 0; j < 8; ++j) {
+    int t = 0;
+    if (kScaled && k0 + j < K) {
+      t = sc.shift[k0 + j];
+      if (t == kNoTerm) x[j] = 0.0;
+      t *= sc.sgn;
+    }
+    F[j] = (unsigned long long)scaled_round(x[j], Dg::kBits - er + t) + kBias;
+  }
   unsigned char *dst = D + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * S * kDigitTile + rl * 32 +
                        ((ch ^ ((rl >> 2) & 1)) << 4);
 #pragma unroll
@@ -936,22 +1061,6 @@ bool make_map_bf16(CUtensorMap *map, const void *base, int64_t inner, int64_t ro
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// row maxima of one operand (element (r, k) at X[r sr + k sk], one of the
-// strides 1) into bits[0 .. Rpad), padding rows 0
-void launch_rowmax(const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk,
-                   unsigned long long *bits, int64_t Rpad, cudaStream_t st) {
-  if (sr == 1) {
-    cudaMemsetAsync(bits, 0, (size_t)Rpad * sizeof(unsigned long long), st);
-    dim3 g((unsigned)((Rpad + 31) / 32), (unsigned)((K + 255) / 256));
-    rowmax_rcontig_kernel<<<g, 256, 0, st>>>(X, R, K, sk, bits);
-  } else {
-    rowmax_kcontig_kernel<<<(unsigned)((Rpad + 7) / 8), 256, 0, st>>>(X, R, K, sr, bits,
-                                                                      (int)Rpad);
-  }
-  count_launch();
-}
-
-
 int oz_split_digits(int nslices) { return nslices <= 0 ? 6 : (nslices <= 4 ? 3 : (nslices <= 8 ? 6 : 7)); }
 
 size_t oz_digits_bytes(int64_t R, int64_t K, int S) {
@@ -972,17 +1081,56 @@ OzDigits oz_digits_at(void *mem, int64_t R, int64_t K, int S) {
   return d;
 }
 
-void oz_slice(const double *X, int64_t sr, int64_t sk, const OzDigits &d, cudaStream_t st) {
+namespace {
+template <bool kScaled>
+void slice_rows(const double *X, int64_t sr, int64_t sk, const OzDigits &d, Scaling sc,
+                cudaStream_t st) {
   const int64_t Rpad = rup(d.R, OBM), Kpad = rup(d.K, OBK);
-  launch_rowmax(X, d.R, d.K, sr, sk, d.mx, Rpad, st);
-  dim3 g((unsigned)(Kpad / KS), (unsigned)(Rpad / OBM));
-  if (d.S == 3)
-    slice_kernel<3><<<g, 256, 0, st>>>(X, d.R, d.K, sr, sk, d.mx, d.e, d.dig);
-  else if (d.S == 6)
-    slice_kernel<6><<<g, 256, 0, st>>>(X, d.R, d.K, sr, sk, d.mx, d.e, d.dig);
-  else
-    slice_kernel<7><<<g, 256, 0, st>>>(X, d.R, d.K, sr, sk, d.mx, d.e, d.dig);
+  if (sr == 1) {
+    cudaMemsetAsync(d.mx, 0, (size_t)Rpad * sizeof(unsigned long long), st);
+    dim3 g((unsigned)((Rpad + 31) / 32), (unsigned)((d.K + 255) / 256));
+    rowmax_rcontig_kernel<kScaled><<<g, 256, 0, st>>>(X, d.R, d.K, sk, d.mx, sc);
+  } else {
+    rowmax_kcontig_kernel<kScaled>
+        <<<(unsigned)((Rpad + 7) / 8), 256, 0, st>>>(X, d.R, d.K, sr, d.mx, (int)Rpad, sc);
+  }
   count_launch();
+  dim3 g((unsigned)(Kpad / KS), (unsigned)(Rpad / OBM));
+  auto go = [&](auto kernel) {
+    kernel<<<g, 256, 0, st>>>(X, d.R, d.K, sr, sk, d.mx, d.e, d.dig, sc);
+  };
+  if constexpr (kScaled)
+    go(slice_kernel<kOzF64Digits, true>);
+  else if (d.S == 3)
+    go(slice_kernel<3, false>);
+  else if (d.S == 6)
+    go(slice_kernel<6, false>);
+  else
+    go(slice_kernel<7, false>);
+  count_launch();
+}
+}  // namespace
+
+void oz_slice(const double *X, int64_t sr, int64_t sk, const OzDigits &d, cudaStream_t st) {
+  slice_rows<false>(X, sr, sk, d, Scaling{nullptr, 0}, st);
+}
+
+void oz_slice_rhs(const double *X, int64_t sr, int64_t sk, const OzDigits &d, const OzColumns &c,
+                  cudaStream_t st) {
+  if (sr == 1) {
+    dim3 g((unsigned)((d.K + 7) / 8), (unsigned)((d.R + kColRows - 1) / kColRows));
+    column_shift_kernel<true><<<g, 256, 0, st>>>(X, d.R, d.K, sk, c);
+  } else {
+    dim3 g((unsigned)((d.K + 31) / 32), (unsigned)((d.R + kColRowsK - 1) / kColRowsK));
+    column_shift_kernel<false><<<g, 256, 0, st>>>(X, d.R, d.K, sr, c);
+  }
+  count_launch();
+  slice_rows<true>(X, sr, sk, d, Scaling{c.shift, 1}, st);
+}
+
+void oz_slice_inverse(const double *X, int64_t sr, int64_t sk, const OzDigits &d,
+                      const OzColumns &c, cudaStream_t st) {
+  slice_rows<true>(X, sr, sk, d, Scaling{c.shift, -1}, st);
 }
 
 namespace {
