@@ -12,6 +12,7 @@
 #include <cstring>
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace qmlgb;
@@ -97,9 +98,13 @@ struct Call {
     return (T *)p;
   }
 
-  // alloc without the error: nullptr when the device has no room
+  // alloc without the error: nullptr when the device has no room (tuning key
+  // test_room: requests above so many bytes find none, so that what a call does
+  // without this memory can be tested on a device that has it)
   void *try_alloc(size_t bytes) {
     if (err != QML_OK) return nullptr;
+    const int64_t room = tune_get("test_room", 0);
+    if (room > 0 && bytes > (size_t)room) return nullptr;
     void *p = nullptr;
     if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
       cudaGetLastError();
@@ -398,11 +403,11 @@ struct DigitBuf {
   size_t bytes = 0;
 };
 
-// Column maxima and shifts for the products with block inverses (K <= kNBS),
-// zeroed on the call's stream.
-OzColumns make_columns(Call &c) {
+// Column maxima and shifts for the products with block inverses (K <= kNBS) in
+// kColumnBytes at p (null: none), zeroed on the call's stream.
+constexpr size_t kColumnBytes = 12 * kNBS + 8;
+OzColumns make_columns(Call &c, unsigned char *p) {
   OzColumns o;
-  unsigned char *p = c.alloc<unsigned char>(12 * kNBS + 8, "column shifts");
   if (!p || !c.cuda_ok(cudaMemsetAsync(p, 0, 8 * kNBS + 8, c.st), "column shifts")) return o;
   o.kmax = (unsigned long long *)p;
   o.done = (unsigned *)(p + 8 * kNBS);
@@ -452,7 +457,8 @@ struct Split {
   // 2e-15, for a spread of 1 to 1e8.  The 48-bit form keeps plain rows.
   OzDigits slice_rhs(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
     const OzDigits d = digits(i, R, K);
-    if (f64 && !cols.kmax) cols = make_columns(*c);
+    if (f64 && !cols.kmax)
+      cols = make_columns(*c, c->alloc<unsigned char>(kColumnBytes, "column shifts"));
     if (c->err != QML_OK) return OzDigits{};
     if (f64)
       oz_slice_rhs(X, sr, sk, d, cols, c->st);
@@ -1377,11 +1383,6 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   const int ns_max = (int)std::max<int64_t>(
       1, std::min<int64_t>(16, tune_get("batch_streams", k < 10000 ? 8 : 4)));
   int NS = nitems < ns_max ? nitems : ns_max;
-  // CUDA graphs: item 0 runs as plain launches (so that the tile autotuner
-  // can time its shapes), then each (worker, mask) pair captures its per-item
-  // sequence once -- reading the spectrum from a fixed per-worker slot and
-  // writing its results to fixed slots -- and replays it for every later item
-  bool graphs = tune_get("batch_graphs", 1) != 0 && nitems > NS;
   // Split precision covers the per-mask products (L_N, U = L_N^-1 Y, M, v);
   // the per-item inner factor Kt (the SMW inner inverse and ln|Kt|) stays at
   // float64 quality (inner_split) unless the tuning key batch_split_kt asks for
@@ -1399,42 +1400,65 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   struct Worker {
     cudaStream_t st = nullptr;
     cudaEvent_t done = nullptr;
-    double *K, *lamL, *z, *rr, *Linv, *LinvB, *ldp;
+    double *K, *lamL, *z, *rr, *Linv, *LinvB = nullptr, *ldp;
     double *cl, *lnK, *lnl, *chi, *ld;  // fixed slots of the captured sequence
-    double *tinv;                       // block-inverse scratch (split)
+    double *tinv = nullptr;             // block-inverse scratch (split)
     OzColumns cols;
     DigitBuf buf[3];
   };
   std::vector<Worker> wk(NS);
   const int64_t nbk = (k + kNB - 1) / kNB, nbbk = (k + kNBS - 1) / kNBS;
   double *lnK = c.alloc<double>(nitems);
+  // a worker's scratch, laid out in one piece at p (null: its size only)
+  auto place = [&](Worker &W, unsigned char *p) {
+    size_t used = 0;
+    auto take = [&](auto *&q, size_t count) {
+      q = p ? (std::remove_reference_t<decltype(q)>)(p + used) : nullptr;
+      used += (count * sizeof(*q) + 1023) / 1024 * 1024;
+    };
+    take(W.K, (size_t)k * k);
+    take(W.lamL, (size_t)d0.nl * d0.nc * d0.nc);
+    take(W.z, (size_t)k * maxmaps);
+    take(W.rr, maxmaps);
+    take(W.Linv, (size_t)nbk * kNB * kNB);
+    take(W.ldp, nbk);
+    take(W.cl, 6 * L);
+    take(W.lnK, 1);
+    take(W.lnl, maxmaps);
+    take(W.chi, maxmaps);
+    take(W.ld, 1);
+    if (any_split) {
+      take(W.LinvB, (size_t)nbbk * kNBS * kNBS);
+      take(W.tinv, (size_t)(kNBS / 2) * (kNBS / 2));
+      for (int b = 0; b < 3; ++b) {
+        W.buf[b].bytes = split_ws_bytes(b, k, maxmaps, Smax);
+        unsigned char *q;
+        take(q, W.buf[b].bytes);
+        W.buf[b].p = q;
+      }
+      unsigned char *q;
+      take(q, kColumnBytes);
+      W.cols = make_columns(c, q);
+    }
+    return used;
+  };
+  // the workers beyond four only where the device has room for all of their scratch
   for (int w = 0; w < NS; ++w) {
-    // the workers beyond four only where the device has room for their scratch
-    wk[w].K = w < 4 ? c.alloc<double>((size_t)k * k, "Kt")
-                    : (double *)c.try_alloc(sizeof(double) * k * k);
-    if (w >= 4 && !wk[w].K && c.err == QML_OK) {
+    const size_t need = place(wk[w], nullptr);
+    unsigned char *p = w < 4 ? c.alloc<unsigned char>(need, "worker scratch")
+                             : (unsigned char *)c.try_alloc(need);
+    if (w >= 4 && !p && c.err == QML_OK) {
       NS = w;
       wk.resize(NS);
       break;
     }
-    wk[w].lamL = c.alloc<double>((size_t)d0.nl * d0.nc * d0.nc);
-    wk[w].z = c.alloc<double>((size_t)k * maxmaps);
-    wk[w].rr = c.alloc<double>(maxmaps);
-    wk[w].Linv = c.alloc<double>((size_t)nbk * kNB * kNB);
-    wk[w].LinvB = any_split ? c.alloc<double>((size_t)nbbk * kNBS * kNBS) : nullptr;
-    wk[w].ldp = c.alloc<double>(nbk);
-    wk[w].cl = c.alloc<double>(6 * L);
-    wk[w].lnK = c.alloc<double>(1);
-    wk[w].lnl = c.alloc<double>(maxmaps);
-    wk[w].chi = c.alloc<double>(maxmaps);
-    wk[w].ld = c.alloc<double>(1);
-    for (int b = 0; any_split && b < 3; ++b) {
-      wk[w].buf[b].bytes = split_ws_bytes(b, k, maxmaps, Smax);
-      wk[w].buf[b].p = c.alloc<unsigned char>(wk[w].buf[b].bytes, "split workspace");
-    }
-    wk[w].tinv = any_split ? c.alloc<double>((size_t)(kNBS / 2) * (kNBS / 2)) : nullptr;
-    if (any_split) wk[w].cols = make_columns(c);
+    place(wk[w], p);
   }
+  // CUDA graphs: item 0 runs as plain launches (so that the tile autotuner
+  // can time its shapes), then each (worker, mask) pair captures its per-item
+  // sequence once -- reading the spectrum from a fixed per-worker slot and
+  // writing its results to fixed slots -- and replays it for every later item
+  bool graphs = tune_get("batch_graphs", 1) != 0 && nitems > NS;
   if (c.err != QML_OK) return c.finish();
   cudaEvent_t setup_done;
   if (!c.cuda_ok(cudaEventCreateWithFlags(&setup_done, cudaEventDisableTiming), "event"))

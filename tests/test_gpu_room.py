@@ -1,0 +1,57 @@
+"""Memory that a call can do without: the tuning key test_room makes it count as
+not available, and the call gives the same answer without it."""
+import numpy as np
+import pytest
+
+import parity as P
+from paper_2605_21149_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_21149_gb300 import api as A
+    from paper_2605_21149_gb300 import build
+    build.build()
+    return A
+
+
+def td(x):
+    return torch.as_tensor(np.asarray(x, dtype=np.float64), device="cuda").t().contiguous().t()
+
+
+def with_room(api, nbytes, fn):
+    api.tune_set("test_room", nbytes)
+    try:
+        return fn()
+    finally:
+        api.tune_set("test_room", 0)
+
+
+@pytest.mark.parametrize("graphs", [0, 1])
+@pytest.mark.parametrize("items", [5, 20])
+def test_scan_without_more_workers(api, items, graphs):
+    """Eight workers, or the four that are always there: an item's result does not
+    depend on its worker.  (2.5 MB: an extra worker's inner matrix would fit, the
+    rest of its scratch would not.)"""
+    masks, taus, rs = synth.batch_workload(nside=8, lmax=12, rank=30, ngrid=5)
+    wls = masks[:2]
+    probs = []
+    for j, wl in enumerate(wls):
+        probs.append((api.Problem.from_workload(wl, precision=1),
+                      td(P.oracle_maps(wl, 2, seed_purpose=20 + j)[3])))
+    cl = torch.as_tensor(synth.batch_item_spectra(12, taus[:items], rs[:items]), device="cuda")
+    im = np.arange(items) % 2
+    run = lambda: [P.to_np(v) for v in api.loglike_batch(probs, im, cl)]
+    api.tune_set("batch_graphs", graphs)
+    try:
+        full = run()
+        for nbytes in (1, 2_500_000):
+            part = with_room(api, nbytes, run)
+            assert all(np.array_equal(a, b) for a, b in zip(full, part))
+    finally:
+        api.tune_set("batch_graphs", 1)
