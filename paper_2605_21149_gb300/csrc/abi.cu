@@ -114,6 +114,15 @@ struct Call {
     return p;
   }
 
+  // give a buffer of this call back before its end (after the work on it that
+  // the stream already has)
+  void release(void *p) {
+    const auto it = std::find(bufs.begin(), bufs.end(), p);
+    if (it == bufs.end()) return;
+    bufs.erase(it);
+    cudaFreeAsync(p, st);
+  }
+
   // device view of an input array (copied in when it lives on the host)
   template <class T>
   const T *in(const T *p, size_t count, const char *what) {
@@ -431,10 +440,19 @@ struct Split {
     if (!tinv) tinv = c->alloc<double>((size_t)(kNBS / 2) * (kNBS / 2), "inverse scratch");
     return tinv;
   }
+  // Give the digit buffers back: they are as large as the matrices, and what the
+  // call allocates next may need the room.
+  void release() {
+    for (auto &b : buf) {
+      c->release(b.p);
+      b = DigitBuf{};
+    }
+  }
   // memory for the digits of an R x K matrix in buffer i
   OzDigits digits(int i, int64_t R, int64_t K) {
     const size_t need = oz_digits_bytes(R, K, S);
     if (need > buf[i].bytes) {
+      c->release(buf[i].p);
       buf[i].p = c->alloc<unsigned char>(need, "split workspace");
       buf[i].bytes = buf[i].p ? need : 0;
     }
@@ -489,6 +507,7 @@ struct Split {
                  double *Bj, int64_t nrhs, int64_t ldb) {
     const size_t need = sizeof(double) * kNBS * kSkinnyN;
     if (need > buf[2].bytes) {
+      c->release(buf[2].p);
       buf[2].p = c->alloc<unsigned char>(need, "right-hand sides");
       buf[2].bytes = buf[2].p ? need : 0;
     }
@@ -504,9 +523,10 @@ struct Split {
   // buffer i holds `need` bytes, if the device has the room
   bool room(int i, size_t need) {
     if (need <= buf[i].bytes) return true;
-    void *p = c->try_alloc(need);
-    if (p) buf[i] = DigitBuf{p, need};
-    return p != nullptr;
+    c->release(buf[i].p);
+    buf[i].p = c->try_alloc(need);
+    buf[i].bytes = buf[i].p ? need : 0;
+    return buf[i].p != nullptr;
   }
   // C <- alpha op(A) op(B) + beta C, kDigitK of K at a time (one more rounding
   // of C each).  A QML_FP64 problem that fills the device has no digits in its
@@ -893,6 +913,7 @@ void harmonic_W_from_M(Call &c, const qml_plan *plan, double *W, double *T) {
   launch_lambda_t_apply(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, d.k, T, d.k, c.st);
   Split sk = inner_split(c, d.k);
   inner_trsm(c, sk, plan->K, d.k, T, d.k, d.k, true, kInnerNB);
+  sk.release();
   launch_lambda_t_apply(T, d.k, d.nc, d.k0, d.lmin, plan->lamLi, d.k, W, d.k, c.st);
   launch_symmetrize_avg(W, d.k, d.k, c.st);
 }
@@ -905,6 +926,7 @@ void plan_W(Call &c, const qml_plan *plan, double *W, double *T) {
   if (plan->split) {
     Split spl = make_split(c, plan->precision, plan->S);
     spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1);
+    spl.release();
   } else {
     launch_dgemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, c.status,
                  c.st);
@@ -927,6 +949,7 @@ void weighted_data(Call &c, const qml_plan *plan, const double *D, int nsims, do
     Split spl = make_split(c, plan->precision, plan->S);
     trsm_split(c, spl, plan->L, d.n, d.n, plan->LinvB, U, nsims, d.n);
     spl.gemm(1, 0, d.k, nsims, d.n, 1.0, plan->X, d.n, U, d.n, 0.0, wv, d.k, 0);
+    spl.release();
   } else {
     trsm_blocked(c, plan->L, d.n, d.n, plan->Linv, U, nsims, d.n);
     launch_dgemm(1, 0, d.k, nsims, d.n, 1.0, plan->X, d.n, U, d.n, 0.0, wv, d.k, 0, c.status,
@@ -936,6 +959,7 @@ void weighted_data(Call &c, const qml_plan *plan, const double *D, int nsims, do
     launch_lambda_t_apply(wv, d.k, d.nc, d.k0, d.lmin, plan->lamL, nsims, wv, d.k, c.st);
     Split sk = inner_split(c, d.k);
     inner_trsm(c, sk, plan->K, d.k, wv, nsims, d.k, true, kInnerNB);
+    sk.release();
     launch_lambda_t_apply(wv, d.k, d.nc, d.k0, d.lmin, plan->lamLi, nsims, w, d.k, c.st);
   }
 }
@@ -1169,6 +1193,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
                    c.status, c.st);
     }
     launch_symmetrize_lower(W, d.k, d.k, c.st);
+    spl.release();
     // Kt = I + L_Lambda^T M L_Lambda, factored in float64 (the SMW inner
     // matrix); then W = L_Lambda^-T Kt^-1 L_Lambda^T M = M (I + Lambda M)^-1
     // (Eq. smw_stable) by two triangular solves and two per-(l, m) mixes
@@ -1180,6 +1205,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
       launch_form_ktilde(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, plan->K.L, d.k, c.st);
       Split sk = inner_split(c, d.k);
       inner_potrf(c, sk, plan->K, d.k, ldk, nullptr);
+      sk.release();
       harmonic_W_from_M(c, plan, W, T);
     }
   }
@@ -1363,6 +1389,8 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
       trsm_split(c, spl, LN, d.n, d.n, LinvB, u, nm, d.n);
       spl.gemm(1, 0, k, k, d.n, 1.0, U, d.n, U, d.n, 0.0, ms[m].M, k, 1);
       spl.gemm(1, 0, k, nm, d.n, 1.0, U, d.n, u, d.n, 0.0, ms[m].v, k, 0);
+      spl.release();
+      c.release(LinvB);
     } else {
       potrf_blocked(c, LN, d.n, d.n, Linv, ldp, ms[m].lnN);
       trsm_blocked(c, LN, d.n, d.n, Linv, U, k, d.n);

@@ -1,5 +1,7 @@
 """Memory that a call can do without: the tuning key test_room makes it count as
 not available, and the call gives the same answer without it."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -55,3 +57,35 @@ def test_scan_without_more_workers(api, items, graphs):
             assert all(np.array_equal(a, b) for a, b in zip(full, part))
     finally:
         api.tune_set("batch_graphs", 1)
+
+
+def peak_pool_bytes(fn):
+    """Highest use of the device's default memory pool while fn runs, above what was
+    in use before."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, v = ctypes.c_void_p(), ctypes.c_uint64(0)
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    used_now, used_high = 7, 8  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH
+    torch.cuda.synchronize()
+    assert cu.cuMemPoolSetAttribute(pool, used_high, ctypes.byref(v)) == 0
+    assert cu.cuMemPoolGetAttribute(pool, used_now, ctypes.byref(v)) == 0
+    before = v.value
+    fn()
+    torch.cuda.synchronize()
+    assert cu.cuMemPoolGetAttribute(pool, used_high, ctypes.byref(v)) == 0
+    return v.value - before
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_scan_masks_share_digit_buffers(api, precision):
+    """Each further mask of a scan adds its own matrices and no digits."""
+    masks, taus, rs = synth.batch_workload(nside=8, lmax=12, rank=30, ngrid=4)
+    wl = masks[0]
+    prob = api.Problem.from_workload(wl, precision=precision)
+    maps = td(P.oracle_maps(wl, 2, seed_purpose=20)[3])
+    cl = torch.as_tensor(synth.batch_item_spectra(12, taus[:4], rs[:4]), device="cuda")
+    n, k = prob.n, prob.k
+    one, four = (peak_pool_bytes(lambda: api.loglike_batch([(prob, maps)] * nm, np.arange(4) % nm, cl))
+                 for nm in (1, 4))
+    own = 8 * (n * k + n * n + 64 * (n + 64) + k * k + 3 * n + 3 * k) + (1 << 20)
+    assert four - one <= 3 * own
