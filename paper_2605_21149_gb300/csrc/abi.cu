@@ -99,19 +99,29 @@ struct Call {
   }
 
   // alloc without the error: nullptr when the device has no room (tuning key
-  // test_room: requests above so many bytes find none, so that what a call does
-  // without this memory can be tested on a device that has it)
-  void *try_alloc(size_t bytes) {
+  // test_digit_room, or `key`: requests above so many bytes find none, so that what a
+  // call does without this memory can be tested on a device that has it)
+  void *try_alloc(size_t bytes, const char *key = "test_digit_room") {
+    void *p = try_malloc(bytes, key);
+    if (p) bufs.push_back(p);
+    return p;
+  }
+  // the same for a buffer that the caller owns
+  void *try_malloc(size_t bytes, const char *key = "test_digit_room") {
     if (err != QML_OK) return nullptr;
-    const int64_t room = tune_get("test_room", 0);
+    const int64_t room = tune_get(key, 0);
     if (room > 0 && bytes > (size_t)room) return nullptr;
     void *p = nullptr;
-    if (cudaMallocAsync(&p, bytes, st) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    bufs.push_back(p);
-    return p;
+    if (cudaMallocAsync(&p, bytes, st) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+  }
+  // whether what was tried leaves room for the small buffers that the call still
+  // takes and cannot do without
+  bool slack_left() {
+    void *p = try_malloc(32 << 20);
+    if (p) cudaFreeAsync(p, st);
+    return p != nullptr;
   }
 
   // give a buffer of this call back before its end (after the work on it that
@@ -424,6 +434,14 @@ OzColumns make_columns(Call &c, unsigned char *p) {
   return o;
 }
 
+// the buffers potrf_split and trsm_split need for an n x n factor and nrhs
+// right-hand sides: panel digits, block-inverse digits, right-hand-side digits
+size_t split_ws_bytes(int i, int64_t n, int64_t nrhs, int S) {
+  return oz_digits_bytes(i == 0 ? n : (i == 1 ? kNBS : (nrhs > 0 ? nrhs : 1)), kNBS, S);
+}
+// doubles of the kNBS-block inverses of an order-n factor
+size_t linvb_count(int64_t n) { return (size_t)((n + kNBS - 1) / kNBS) * kNBS * kNBS; }
+
 struct Split {
   Call *c;
   int S;  // digits per operand (oz_split_digits, kOzF64Digits)
@@ -433,11 +451,12 @@ struct Split {
   // SMs the split kernel leaves free (for float64 work on a second stream)
   int reserve_sms = 0;
   DigitBuf buf[3];
+  static constexpr size_t kTinvBytes = sizeof(double) * (kNBS / 2) * (kNBS / 2);
   OzColumns cols;  // scales of the products with block inverses
   double *tinv = nullptr;  // (kNBS/2)^2 scratch of the block-inverse doubling
   // the doubling scratch, allocated on first use unless preset
   double *tinv_scratch() {
-    if (!tinv) tinv = c->alloc<double>((size_t)(kNBS / 2) * (kNBS / 2), "inverse scratch");
+    if (!tinv) tinv = (double *)c->alloc<unsigned char>(kTinvBytes, "inverse scratch");
     return tinv;
   }
   // Give the digit buffers back: they are as large as the matrices, and what the
@@ -528,6 +547,33 @@ struct Split {
     buf[i].bytes = buf[i].p ? need : 0;
     return buf[i].p != nullptr;
   }
+  // Memory for the kNBS-block inverses of an order-n factor, for the call; null at
+  // float64 quality when there is no room, as below.
+  double *block_inverses(int64_t n) {
+    if (!f64) return c->alloc<double>(linvb_count(n));
+    return (double *)c->try_alloc(sizeof(double) * linvb_count(n));
+  }
+  // The buffers that potrf_split (factor) or a trsm_split of an n x n factor with
+  // nrhs right-hand sides takes, all at once.  At float64 quality the float64 pipe
+  // needs none of them, so that a device without the room is no error: false,
+  // and the caller takes the *_blocked form.  (The split precision has no other
+  // form: true, and a buffer that does not fit fails the call.)
+  bool ready(int64_t n, int64_t nrhs, bool factor) {
+    if (!f64 || c->err != QML_OK) return true;
+    bool ok = room(2, split_ws_bytes(2, n, nrhs, S));
+    if (factor || nrhs > kSkinnyN)
+      ok = ok && room(0, split_ws_bytes(0, n, nrhs, S)) && room(1, split_ws_bytes(1, n, nrhs, S));
+    if (ok && !cols.kmax) {
+      unsigned char *p = (unsigned char *)c->try_alloc(kColumnBytes);
+      if (p) cols = make_columns(*c, p);
+      ok = cols.kmax != nullptr;
+    }
+    if (ok && factor && !tinv) tinv = (double *)c->try_alloc(kTinvBytes);
+    if (factor) ok = ok && tinv;
+    ok = ok && c->slack_left();
+    if (!ok) release();
+    return ok || c->err != QML_OK;
+  }
   // C <- alpha op(A) op(B) + beta C, kDigitK of K at a time (one more rounding
   // of C each).  A QML_FP64 problem that fills the device has no digits in its
   // float64 form: it takes shorter pieces of K while the buffers do not fit,
@@ -539,11 +585,13 @@ struct Split {
     const bool same = A == B && lda == ldb && ta != tb && M == N;
     int64_t kc = K < kDigitK || C == A || C == B ? K : kDigitK;  // (in place: all digits first)
     while (f64 && !(room(0, oz_digits_bytes(M, kc, S)) &&
-                    (same || room(1, oz_digits_bytes(N, kc, S))))) {
+                    (same || room(1, oz_digits_bytes(N, kc, S))) && c->slack_left())) {
       if (kc <= kNBS) {
+        release();
         launch_dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, c->status, c->st);
         return;
       }
+      release();  // (one of the two may have taken the room of both)
       kc = (kc / 2 + 63) / 64 * 64;
     }
     int64_t k0 = 0;
@@ -557,12 +605,6 @@ struct Split {
     } while (k0 < K);
   }
 };
-// the buffers potrf_split and trsm_split need for an n x n factor and nrhs
-// right-hand sides: panel digits, block-inverse digits, right-hand-side digits
-size_t split_ws_bytes(int i, int64_t n, int64_t nrhs, int S) {
-  return oz_digits_bytes(i == 0 ? n : (i == 1 ? kNBS : (nrhs > 0 ? nrhs : 1)), kNBS, S);
-}
-
 // QML_FP64 at and above this order factors and multiplies with 55-bit digit
 // products (kOzF64Digits) instead of the float64 pipe, whose 1.2 TFLOP/s bound
 // every contraction (TQU Nside 16 solve: 736 ms, 46.5 with digits).  Error of a
@@ -791,6 +833,7 @@ void trsm_split_t(Call &c, Split &sp, const double *L, int64_t n, int64_t lda,
 // (kNBS-block inverses), whichever its order asks for.
 struct InnerFactor {
   double *L = nullptr, *Linv = nullptr, *LinvB = nullptr;
+  int S = 0;  // its digits (0: float64 blocks, no LinvB)
 };
 void inner_potrf(Call &c, Split &sp, const InnerFactor &K, int64_t k, double *ldparts,
                  double *logdet) {
@@ -901,8 +944,12 @@ struct qml_plan {
 
 namespace {
 
-Split inner_split(Call &c, int64_t k) {
-  return make_split(c, QML_FP64, split_digits(QML_FP64, 0, k));
+// the products with a factor in this form; without the room for nrhs right-hand
+// sides' digits its float64 blocks, which every factor has
+Split inner_split(Call &c, const InnerFactor &K, int64_t k, int64_t nrhs) {
+  Split sk = make_split(c, QML_FP64, K.S);
+  if (K.S && !sk.ready(k, nrhs, false)) sk.S = 0;
+  return sk;
 }
 
 // Harmonic basis: W (k x k) holds M = Y^T N^-1 Y on entry and W = M (I +
@@ -911,7 +958,7 @@ Split inner_split(Call &c, int64_t k) {
 void harmonic_W_from_M(Call &c, const qml_plan *plan, double *W, double *T) {
   const Dims &d = plan->d;
   launch_lambda_t_apply(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, d.k, T, d.k, c.st);
-  Split sk = inner_split(c, d.k);
+  Split sk = inner_split(c, plan->K, d.k, d.k);
   inner_trsm(c, sk, plan->K, d.k, T, d.k, d.k, true, kInnerNB);
   sk.release();
   launch_lambda_t_apply(T, d.k, d.nc, d.k0, d.lmin, plan->lamLi, d.k, W, d.k, c.st);
@@ -945,19 +992,21 @@ void weighted_data(Call &c, const qml_plan *plan, const double *D, int nsims, do
   double *wv = plan->harmonic ? c.alloc<double>((size_t)d.k * nsims, "v") : w;
   if (c.err != QML_OK) return;
   launch_copy_matrix(D, d.n, U, d.n, d.n, nsims, c.st);
-  if (plan->split) {
-    Split spl = make_split(c, plan->precision, plan->S);
+  Split spl = make_split(c, plan->precision, plan->S);
+  if (plan->split && spl.ready(d.n, nsims, false))
     trsm_split(c, spl, plan->L, d.n, d.n, plan->LinvB, U, nsims, d.n);
+  else
+    trsm_blocked(c, plan->L, d.n, d.n, plan->Linv, U, nsims, d.n);
+  if (plan->split) {
     spl.gemm(1, 0, d.k, nsims, d.n, 1.0, plan->X, d.n, U, d.n, 0.0, wv, d.k, 0);
     spl.release();
   } else {
-    trsm_blocked(c, plan->L, d.n, d.n, plan->Linv, U, nsims, d.n);
     launch_dgemm(1, 0, d.k, nsims, d.n, 1.0, plan->X, d.n, U, d.n, 0.0, wv, d.k, 0, c.status,
                  c.st);
   }
   if (plan->harmonic) {
     launch_lambda_t_apply(wv, d.k, d.nc, d.k0, d.lmin, plan->lamL, nsims, wv, d.k, c.st);
-    Split sk = inner_split(c, d.k);
+    Split sk = inner_split(c, plan->K, d.k, nsims);
     inner_trsm(c, sk, plan->K, d.k, wv, nsims, d.k, true, kInnerNB);
     sk.release();
     launch_lambda_t_apply(wv, d.k, d.nc, d.k0, d.lmin, plan->lamLi, nsims, w, d.k, c.st);
@@ -1075,12 +1124,10 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   const int ldcl = d.lsig1 + 1;
   plan->L = palloc((size_t)d.n * d.n);
   plan->Linv = palloc((size_t)nblocks * kNB * kNB);
-  if (plan->split) plan->LinvB = palloc((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
   plan->X = palloc((size_t)d.n * d.k);
   if (plan->harmonic) {
     plan->K.L = palloc((size_t)d.k * d.k);
     plan->K.Linv = palloc((size_t)((d.k + kNB - 1) / kNB) * kNB * kNB);
-    plan->K.LinvB = palloc((size_t)((d.k + kNBS - 1) / kNBS) * kNBS * kNBS);
     plan->lamL = palloc((size_t)d.nl * d.nc * d.nc);
     plan->lamLi = palloc((size_t)d.nl * d.nc * d.nc);
   }
@@ -1153,12 +1200,44 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   auto scratch_for = [&](int kb) -> double * {
     return kb <= d.k ? plan->X : c.alloc<double>((size_t)d.n * kb, "signal-band Y");
   };
+  double *T = plan->harmonic ? c.alloc<double>((size_t)d.k * d.k, "SMW product") : nullptr;
+  double *ldk = plan->harmonic ? c.alloc<double>((d.k + kNB - 1) / kNB) : nullptr;
+  double *Yb[2] = {nullptr, nullptr};
+  if (!plan->harmonic)
+    Yb[0] = scratch_for(d.nc * band_k0(d.lsig0, d.lsig1));
+  else if (d.lsig0 < d.lmin)
+    Yb[0] = scratch_for(d.nc * band_k0(d.lsig0, d.lmin - 1));
+  if (plan->harmonic && d.lsig1 > d.lmax)
+    Yb[1] = scratch_for(d.nc * band_k0(d.lmax + 1, d.lsig1));
+  if (c.err != QML_OK) {
+    qml_status e = c.finish();
+    qml_plan_free(plan);
+    return e;
+  }
+  // The kNBS-block inverses of an order-n factor, which digit solves need and
+  // the float64 pipe does not: QML_FP64 takes the latter where they, or the
+  // digits (Split::ready), do not fit.  All that the call cannot do without is
+  // allocated before.
+  auto block_inverses = [&](int64_t n, bool optional) -> double * {
+    if (!optional) return palloc(linvb_count(n));
+    void *p = c.try_malloc(sizeof(double) * linvb_count(n));
+    if (p) plan->mem.push_back(p);
+    return (double *)p;
+  };
+  auto ready_plan = [&] {
+    if (!plan->split) return;
+    spl.release();
+    plan->LinvB = block_inverses(d.n, spl.f64);
+    plan->split = plan->LinvB && spl.ready(d.n, d.k, true);
+    if (!plan->split) plan->S = 0;
+  };
   launch_copy_lower(sp.N, d.n, plan->L, d.n, d.n, c.st);
   if (!plan->harmonic) {
     // C = Y_sig Lambda Y_sig^T + N ; L L^T = C ; X = L^-1 Y_win ; W = X^T X
     add_band_signal(c, sp_or_null, sp, d, d.lsig0, d.lsig1, ldcl,
-                    scratch_for(d.nc * band_k0(d.lsig0, d.lsig1)), plan->L);
+                    Yb[0], plan->L);
     launch_ybuild(sp.y, plan->X, d.n, c.st);  // X no longer holds the band signal
+    ready_plan();
     if (plan->split) {
       // factor and X = L^-1 Y in one panel loop (the forward substitution
       // runs beside the next panel's float64 chain)
@@ -1176,12 +1255,13 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     // N_eff = N + fixed signal outside the window ; L_N L_N^T = N_eff
     if (d.lsig0 < d.lmin)
       add_band_signal(c, sp_or_null, sp, d, d.lsig0, d.lmin - 1, ldcl,
-                      scratch_for(d.nc * band_k0(d.lsig0, d.lmin - 1)), plan->L);
+                      Yb[0], plan->L);
     if (d.lsig1 > d.lmax)
       add_band_signal(c, sp_or_null, sp, d, d.lmax + 1, d.lsig1, ldcl,
-                      scratch_for(d.nc * band_k0(d.lmax + 1, d.lsig1)), plan->L);
+                      Yb[1], plan->L);
     // U = L_N^-1 Y_win ; M = U^T U (the noise-weighted Gramian Y^T N^-1 Y)
     launch_ybuild(sp.y, plan->X, d.n, c.st);
+    ready_plan();
     if (plan->split) {
       potrf_split(c, spl, plan->L, d.n, d.n, plan->Linv, plan->LinvB, ldparts, nullptr, plan->X,
                   d.k, d.n);
@@ -1197,13 +1277,16 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     // Kt = I + L_Lambda^T M L_Lambda, factored in float64 (the SMW inner
     // matrix); then W = L_Lambda^-T Kt^-1 L_Lambda^T M = M (I + Lambda M)^-1
     // (Eq. smw_stable) by two triangular solves and two per-(l, m) mixes
-    double *T = c.alloc<double>((size_t)d.k * d.k, "SMW product");
-    double *ldk = c.alloc<double>((size_t)((d.k + kNB - 1) / kNB));
     if (c.err == QML_OK) {
       launch_lambda_factor(sp.cl, d.lmin, d.lmax, d.nc, d.comps, plan->lamL, c.st, ldcl);
       launch_lambda_inverse(plan->lamL, d.nl, d.nc, d.lmin, plan->lamLi, c.status, c.st);
       launch_form_ktilde(W, d.k, d.nc, d.k0, d.lmin, plan->lamL, plan->K.L, d.k, c.st);
-      Split sk = inner_split(c, d.k);
+      Split sk = make_split(c, QML_FP64, split_digits(QML_FP64, 0, d.k));
+      if (sk.S) {
+        plan->K.LinvB = block_inverses(d.k, true);
+        if (!plan->K.LinvB || !sk.ready(d.k, 0, true)) sk.S = 0;
+      }
+      plan->K.S = sk.S;
       inner_potrf(c, sk, plan->K, d.k, ldk, nullptr);
       sk.release();
       harmonic_W_from_M(c, plan, W, T);
@@ -1293,17 +1376,20 @@ qml_status pix_loglike(const qml_problem *prob, const double *cl_theta, const do
   double *U = c.alloc<double>((size_t)d.n * nmaps, "U");
   if (!c.make_status()) return c.finish();
   const int S = split_digits(prob->precision, prob->nslices, d.n);
+  Split spl = make_split(c, prob->precision, S);
+  double *LinvB = nullptr;
   if (S) {
-    Split spl = make_split(c, prob->precision, S);
-    double *LinvB = c.alloc<double>((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
-    if (!LinvB) return c.finish();
     build_C_split(c, spl, sp, d, Y, C);
-    launch_copy_matrix(D, d.n, U, d.n, d.n, nmaps, c.st);
-    potrf_split(c, spl, C, d.n, d.n, Linv, LinvB, ldparts, o_ld, U, nmaps, d.n);
+    spl.release();
+    LinvB = spl.block_inverses(d.n);
   } else {
     build_C(c, sp, d, Y, C);
+  }
+  launch_copy_matrix(D, d.n, U, d.n, d.n, nmaps, c.st);
+  if (LinvB && spl.ready(d.n, nmaps, true)) {
+    potrf_split(c, spl, C, d.n, d.n, Linv, LinvB, ldparts, o_ld, U, nmaps, d.n);
+  } else {
     potrf_blocked(c, C, d.n, d.n, Linv, ldparts, o_ld);
-    launch_copy_matrix(D, d.n, U, d.n, d.n, nmaps, c.st);
     trsm_blocked(c, C, d.n, d.n, Linv, U, nmaps, d.n);
   }
   launch_colnorm2(U, d.n, d.n, nmaps, o_chi, c.st);
@@ -1380,21 +1466,23 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     launch_copy_lower(sp.N, d.n, LN, d.n, d.n, c.st);
     launch_copy_matrix(D, d.n, u, d.n, d.n, nm, c.st);
     const int S = split_digits(pr->precision, pr->nslices, d.n);
-    if (S) {
-      Split spl = make_split(c, pr->precision, S);
-      double *LinvB = c.alloc<double>((size_t)((d.n + kNBS - 1) / kNBS) * kNBS * kNBS);
-      if (!LinvB) return c.finish();
+    Split spl = make_split(c, pr->precision, S);
+    double *LinvB = S ? spl.block_inverses(d.n) : nullptr;
+    if (LinvB && spl.ready(d.n, std::max(k, nm), true)) {
       potrf_split(c, spl, LN, d.n, d.n, Linv, LinvB, ldp, ms[m].lnN);
       trsm_split(c, spl, LN, d.n, d.n, LinvB, U, k, d.n);
       trsm_split(c, spl, LN, d.n, d.n, LinvB, u, nm, d.n);
-      spl.gemm(1, 0, k, k, d.n, 1.0, U, d.n, U, d.n, 0.0, ms[m].M, k, 1);
-      spl.gemm(1, 0, k, nm, d.n, 1.0, U, d.n, u, d.n, 0.0, ms[m].v, k, 0);
-      spl.release();
-      c.release(LinvB);
     } else {
       potrf_blocked(c, LN, d.n, d.n, Linv, ldp, ms[m].lnN);
       trsm_blocked(c, LN, d.n, d.n, Linv, U, k, d.n);
       trsm_blocked(c, LN, d.n, d.n, Linv, u, nm, d.n);
+    }
+    c.release(LinvB);
+    if (S) {
+      spl.gemm(1, 0, k, k, d.n, 1.0, U, d.n, U, d.n, 0.0, ms[m].M, k, 1);
+      spl.gemm(1, 0, k, nm, d.n, 1.0, U, d.n, u, d.n, 0.0, ms[m].v, k, 0);
+      spl.release();
+    } else {
       launch_dgemm(1, 0, k, k, d.n, 1.0, U, d.n, U, d.n, 0.0, ms[m].M, k, 1, c.status, c.st);
       launch_dgemm(1, 0, k, nm, d.n, 1.0, U, d.n, u, d.n, 0.0, ms[m].v, k, 0, c.status, c.st);
     }
@@ -1416,15 +1504,20 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   // float64 quality (inner_split) unless the tuning key batch_split_kt asks for
   // its trailing updates and panel products in 48 bits too.
   const bool split_kt = tune_get("batch_split_kt", 0) != 0;
+  auto kt_48 = [&](int m) { return split_kt && masks[m].prob.precision == QML_SPLIT_BF16; };
+  // digits of the inner factors: of the 48-bit ones, which have no other form, and of
+  // those at float64 quality, which take the float64 pipe without (Sk = 0)
+  int S48 = 0, Sk = 0;
+  for (int m = 0; m < nmask; ++m) {
+    if (kt_48(m))
+      S48 = std::max(S48, oz_split_digits(masks[m].prob.nslices));
+    else
+      Sk = split_digits(QML_FP64, 0, k);
+  }
   auto kt_split = [&](Call &cw, int m) {
-    const qml_problem &pr = masks[m].prob;
-    return split_kt && pr.precision == QML_SPLIT_BF16
-               ? make_split(cw, pr.precision, oz_split_digits(pr.nslices))
-               : inner_split(cw, k);
+    return kt_48(m) ? make_split(cw, QML_SPLIT_BF16, oz_split_digits(masks[m].prob.nslices))
+                    : make_split(cw, QML_FP64, Sk);
   };
-  int Smax = 0;
-  for (int m = 0; m < nmask; ++m) Smax = std::max(Smax, kt_split(c, m).S);
-  const bool any_split = Smax > 0;
   struct Worker {
     cudaStream_t st = nullptr;
     cudaEvent_t done = nullptr;
@@ -1435,52 +1528,70 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     DigitBuf buf[3];
   };
   std::vector<Worker> wk(NS);
-  const int64_t nbk = (k + kNB - 1) / kNB, nbbk = (k + kNBS - 1) / kNBS;
+  const int64_t nbk = (k + kNB - 1) / kNB;
   double *lnK = c.alloc<double>(nitems);
-  // a worker's scratch, laid out in one piece at p (null: its size only)
+  // a worker's scratch, and what its digit products need besides, each laid out in
+  // one piece at p (null: its size only)
+  auto take = [](auto *&q, size_t count, unsigned char *p, size_t &used) {
+    q = p ? (std::remove_reference_t<decltype(q)>)(p + used) : nullptr;
+    used += (count * sizeof(*q) + 1023) / 1024 * 1024;
+  };
   auto place = [&](Worker &W, unsigned char *p) {
     size_t used = 0;
-    auto take = [&](auto *&q, size_t count) {
-      q = p ? (std::remove_reference_t<decltype(q)>)(p + used) : nullptr;
-      used += (count * sizeof(*q) + 1023) / 1024 * 1024;
-    };
-    take(W.K, (size_t)k * k);
-    take(W.lamL, (size_t)d0.nl * d0.nc * d0.nc);
-    take(W.z, (size_t)k * maxmaps);
-    take(W.rr, maxmaps);
-    take(W.Linv, (size_t)nbk * kNB * kNB);
-    take(W.ldp, nbk);
-    take(W.cl, 6 * L);
-    take(W.lnK, 1);
-    take(W.lnl, maxmaps);
-    take(W.chi, maxmaps);
-    take(W.ld, 1);
-    if (any_split) {
-      take(W.LinvB, (size_t)nbbk * kNBS * kNBS);
-      take(W.tinv, (size_t)(kNBS / 2) * (kNBS / 2));
-      for (int b = 0; b < 3; ++b) {
-        W.buf[b].bytes = split_ws_bytes(b, k, maxmaps, Smax);
-        unsigned char *q;
-        take(q, W.buf[b].bytes);
-        W.buf[b].p = q;
-      }
-      unsigned char *q;
-      take(q, kColumnBytes);
-      W.cols = make_columns(c, q);
-    }
+    take(W.K, (size_t)k * k, p, used);
+    take(W.lamL, (size_t)d0.nl * d0.nc * d0.nc, p, used);
+    take(W.z, (size_t)k * maxmaps, p, used);
+    take(W.rr, maxmaps, p, used);
+    take(W.Linv, (size_t)nbk * kNB * kNB, p, used);
+    take(W.ldp, nbk, p, used);
+    take(W.cl, 6 * L, p, used);
+    take(W.lnK, 1, p, used);
+    take(W.lnl, maxmaps, p, used);
+    take(W.chi, maxmaps, p, used);
+    take(W.ld, 1, p, used);
     return used;
   };
-  // the workers beyond four only where the device has room for all of their scratch
-  for (int w = 0; w < NS; ++w) {
-    const size_t need = place(wk[w], nullptr);
-    unsigned char *p = w < 4 ? c.alloc<unsigned char>(need, "worker scratch")
-                             : (unsigned char *)c.try_alloc(need);
-    if (w >= 4 && !p && c.err == QML_OK) {
+  auto place_digits = [&](Worker &W, int S, unsigned char *p) {
+    size_t used = 0;
+    take(W.LinvB, linvb_count(k), p, used);
+    take(W.tinv, Split::kTinvBytes / sizeof(double), p, used);
+    unsigned char *q;
+    for (int b = 0; b < 3; ++b) {
+      take(q, split_ws_bytes(b, k, maxmaps, S), p, used);
+      W.buf[b] = DigitBuf{q, split_ws_bytes(b, k, maxmaps, S)};
+    }
+    take(q, kColumnBytes, p, used);
+    W.cols = make_columns(c, q);
+    return used;
+  };
+  const int sure = NS < 4 ? NS : 4;  // workers that the call cannot do without
+  for (int w = 0; w < sure; ++w)
+    place(wk[w], c.alloc<unsigned char>(place(wk[w], nullptr), "worker scratch"));
+  std::vector<void *> dig(NS, nullptr);
+  for (int w = 0; w < sure && (S48 || Sk); ++w) {
+    const size_t need = place_digits(wk[w], std::max(S48, Sk), nullptr);
+    dig[w] = S48 ? c.alloc<unsigned char>(need, "split workspace") : c.try_alloc(need);
+    if (!S48 && (!dig[w] || !c.slack_left())) {
+      for (int v = 0; v <= w; ++v) c.release(dig[v]);
+      Sk = 0;
+      break;
+    }
+    place_digits(wk[w], std::max(S48, Sk), (unsigned char *)dig[w]);
+  }
+  // the others only where the device has room for all of their scratch
+  const int Smax = std::max(S48, Sk);
+  for (int w = sure; w < NS; ++w) {
+    void *p = c.try_alloc(place(wk[w], nullptr), "test_room");
+    if (Smax && p) dig[w] = c.try_alloc(place_digits(wk[w], Smax, nullptr), "test_room");
+    if (!p || (Smax && !dig[w]) || !c.slack_left()) {
+      c.release(p);
+      c.release(dig[w]);
       NS = w;
       wk.resize(NS);
       break;
     }
-    place(wk[w], p);
+    place(wk[w], (unsigned char *)p);
+    if (Smax) place_digits(wk[w], Smax, (unsigned char *)dig[w]);
   }
   // CUDA graphs: item 0 runs as plain launches (so that the tile autotuner
   // can time its shapes), then each (worker, mask) pair captures its per-item

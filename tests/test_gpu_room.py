@@ -1,11 +1,13 @@
-"""Memory that a call can do without: the tuning key test_room makes it count as
-not available, and the call gives the same answer without it."""
+"""Memory that a call can do without: the tuning keys test_room (scan workers beyond
+four) and test_digit_room make it count as not available, and the call gives the
+same answer without it."""
 import ctypes
 
 import numpy as np
 import pytest
 
 import parity as P
+from oracle import qml
 from paper_2605_21149_gb300 import synth
 
 torch = pytest.importorskip("torch")
@@ -26,12 +28,16 @@ def td(x):
     return torch.as_tensor(np.asarray(x, dtype=np.float64), device="cuda").t().contiguous().t()
 
 
-def with_room(api, nbytes, fn):
-    api.tune_set("test_room", nbytes)
+def with_room(api, nbytes, fn, key="test_room"):
+    api.tune_set(key, nbytes)
     try:
         return fn()
     finally:
-        api.tune_set("test_room", 0)
+        api.tune_set(key, 0)
+
+
+def with_digit_room(api, nbytes, fn):
+    return with_room(api, nbytes, fn, "test_digit_room")
 
 
 @pytest.mark.parametrize("graphs", [0, 1])
@@ -89,3 +95,38 @@ def test_scan_masks_share_digit_buffers(api, precision):
                  for nm in (1, 4))
     own = 8 * (n * k + n * n + 64 * (n + 64) + k * k + 3 * n + 3 * k) + (1 << 20)
     assert four - one <= 3 * own
+
+
+@pytest.mark.parametrize("nbytes", [1, 2_200_000, 40_000_000])
+@pytest.mark.parametrize("basis", [0, 1])
+def test_fp64_without_room_for_digits(api, basis, nbytes):
+    """QML_FP64 on a device without room for digits (or for some of them): the
+    float64 pipe, in every call that would use them, with plans of either kind."""
+    th, ph, _ = synth.healpix_ring_centres(16)
+    wl = synth.make_workload("T", 16, 17, True, False, 0.0, ("TT",), 7, 9,
+                             geometry=(th[300:900], ph[300:900]))
+    Y, _, _, maps = P.oracle_maps(wl, 11)
+    ref = qml.qml_for(wl, Y, maps=maps)
+    rl, rc, rd = qml.loglike(qml.total_cov(Y, wl.cl_fid, wl.comps, wl.lmin, wl.lmax, wl.N()), maps)
+    prob = api.Problem.from_workload(wl, basis=basis)
+    cl = torch.as_tensor(wl.cl_fid.reshape(-1), device="cuda")
+    d = td(maps)
+    Ff, full = api.fisher(prob)
+    Fs, small = with_digit_room(api, nbytes, lambda: api.fisher(prob))
+    for F in (Ff, Fs):
+        assert P.rel_max(F, ref["F"]) <= P.TOL
+    for plan in (full, small):
+        for room in (0, nbytes):
+            est = with_digit_room(api, room, lambda: plan.estimate(d))
+            assert P.rel_max(est["y"], ref["y"]) <= P.TOL
+    x = with_digit_room(api, nbytes, lambda: api.cross(full, small, d, d))
+    assert P.rel_max(x["q"], ref["y"]) <= P.TOL and P.rel_max(x["Wx"], ref["F"]) <= P.TOL
+    full.free()
+    small.free()
+    lnl, chi2, ld = (P.to_np(v) for v in with_digit_room(api, nbytes, lambda: api.loglike(prob, cl, d)))
+    assert np.abs(lnl - rl).max() <= P.TOL * np.abs(rl).max()
+    assert np.abs(chi2 - rc).max() <= P.TOL * rc.max()
+    lnl, chi2, ld = (P.to_np(v) for v in with_digit_room(
+        api, nbytes, lambda: api.loglike_batch([(prob, d)], np.zeros(6, int), cl.repeat(6, 1))))
+    assert np.abs(chi2 - rc).max() <= P.TOL * rc.max()
+    assert np.abs(ld - rd).max() <= P.TOL * abs(rd)
