@@ -1198,8 +1198,11 @@ const int kCand[7][2] = {{4, 4}, {2, 4}, {4, 2}, {2, 2}, {1, 4}, {4, 1}, {1, 1}}
 // fits: A and C not transposed or aliased, K <= kPanelK, C small enough that
 // 16 x 16 tiles, which reuse an operand 16 times, are not bound by loading.
 constexpr int kPanelCode = 10;
+// A tile of 16 rn columns puts N / (16 rn) CTAs along the grid's second dimension,
+// which a launch limits to 65535.
+bool grid_fits(int64_t N, int rn) { return (N + 16 * rn - 1) / (16 * rn) <= 65535; }
 bool panel_fits(int ta, int64_t M, int64_t N, int64_t K, bool alias) {
-  return !ta && !alias && K >= 1 && K <= kPanelK && M * N <= 1024 * 1024;
+  return !ta && !alias && K >= 1 && K <= kPanelK && M * N <= 1024 * 1024 && grid_fits(N, 1);
 }
 
 // Autotuner: time every candidate tile on this shape (output into a scratch
@@ -1218,6 +1221,7 @@ bool dgemm_autotune(int ta, int tb, int64_t M, int64_t N, int64_t K, const doubl
   int found = -1;
   for (int i = 0; ok && i < 7; ++i) {
     const int r1 = kCand[i][0], r2 = kCand[i][1];
+    if (!grid_fits(N, r2)) continue;
     dgemm_dispatch(ta, tb, r1, r2, M, N, K, 1.0, A, lda, B, ldb, 0.0, scratch, M, lower, status, st);
     cudaEventRecord(e0, st);
     for (int r = 0; r < 3; ++r)
@@ -1225,7 +1229,9 @@ bool dgemm_autotune(int ta, int tb, int64_t M, int64_t N, int64_t K, const doubl
                      st);
     cudaEventRecord(e1, st);
     float ms = 0.0f;
-    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
+    // (a launch that was refused takes no time)
+    if (cudaGetLastError() != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+        cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
       ok = false;
       break;
     }
@@ -1245,7 +1251,8 @@ bool dgemm_autotune(int ta, int tb, int64_t M, int64_t N, int64_t K, const doubl
     cudaEventRecord(e0, st);
     for (int r = 0; r < 3; ++r) go();
     cudaEventRecord(e1, st);
-    if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
+    if (cudaGetLastError() != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+        cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
       ok = false;
     else
       panel = ms < best;
@@ -1295,14 +1302,15 @@ void launch_dgemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, double a
   }
   if (have)
     for (int i = 0; i < 7; ++i)
-      known |= (tv == 10 * kCand[i][0] + kCand[i][1]);
+      known |= (tv == 10 * kCand[i][0] + kCand[i][1] && grid_fits(N, kCand[i][1]));
   if (known && !(aliasA && tv % 10 != 4) && !(aliasB && tv / 10 != 4)) {
     dgemm_dispatch(ta, tb, (int)(tv / 10), (int)(tv % 10), M, N, K, alpha, A, lda, B, ldb, beta,
                    C, ldc, lower, status, st);
     return;
   }
   if (may_tune && !aliasA && !aliasB && M * N <= (1 << 24) && K <= 4096 &&
-      tune_get("dgemm_autotune", 1)) {
+      tune_get("dgemm_autotune", 1) && cudaPeekAtLastError() == cudaSuccess) {
+    // (an error that is pending stays for the call to report)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
       int rm = 4, rn = 4;
@@ -1329,6 +1337,7 @@ void launch_dgemm_impl(int ta, int tb, int64_t M, int64_t N, int64_t K, double a
     const int r1 = kCand[i][0], r2 = kCand[i][1];
     if (aliasA && r2 != 4) continue;
     if (aliasB && r1 != 4) continue;
+    if (!grid_fits(N, r2)) continue;
     const int64_t n = dgemm_ctas(M, N, 16 * r1, 16 * r2, lower);
     if (n >= want) {  // candidates run from the largest tile down
       rm = r1;

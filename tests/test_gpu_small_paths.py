@@ -207,3 +207,24 @@ def test_potrf_rows_agree_between_warps(api, form):
     finally:
         api.tune_set("split_diag_df", 0)
     assert np.abs(np.tril(L) - ref).max() <= 1e-11 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("transB", [False, True])
+@pytest.mark.parametrize("m,n", [(1, 1048560), (1, 1048561), (1, 1048576), (3, 1048577)])
+def test_gemm_more_columns_than_a_grid(api, m, n, transB):
+    """16-wide tiles would put more CTAs along the columns than a launch takes: the
+    autotuner, the built-in choice, and a tuning table that names them (codes 10 and
+    11)."""
+    g = np.random.default_rng(n)
+    A, B = g.normal(size=(m, 3)), g.normal(size=(3, n))
+    ref = A @ B
+    bound = 8 * 2.0 ** -53 * (np.abs(A) @ np.abs(B))
+    Bd = td(B.T) if transB else td(B)
+    key = f"dgemm:0,{int(transB)},0,{m},{n},3,0"
+    try:
+        for text in ("dgemm_autotune 0\n", "dgemm_autotune 1\n", key + " 10\n", key + " 11\n"):
+            api.tune_load(text)
+            C = api.gemm(td(A), Bd, transB=transB).cpu().numpy()
+            assert (np.abs(C - ref) <= bound).all()
+    finally:
+        api.tune_set("dgemm_autotune", 1)
