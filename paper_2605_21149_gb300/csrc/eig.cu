@@ -908,8 +908,8 @@ __device__ __forceinline__ double widened(float f) {
 }
 // rotation() with eight float64 instructions: the float32 inputs and the
 // conversions by integer operations, 1 / (1 + tau^2) from a float32 quotient
-// w0 and the cubic step w0 (1 + e + e^2), e = 1 - (1 + tau^2) w0 (|e| below
-// 2^-22: an error of e^3).  Entries that are not ordinary numbers take the
+// w0 and one step of the third-order Newton series, w0 (1 + e + e^2) with e = 1 -
+// (1 + tau^2) w0 (|e| below 2^-21: an error of e^3 < 2^-63).  Entries that are not ordinary numbers take the
 // general form.
 __device__ __forceinline__ double2 rotation_lean(double app, double aqq, double apq) {
   const double d = aqq - app;

@@ -228,3 +228,22 @@ def test_gemm_more_columns_than_a_grid(api, m, n, transB):
             assert (np.abs(C - ref) <= bound).all()
     finally:
         api.tune_set("dgemm_autotune", 1)
+
+
+def test_potrf_column_by_reciprocal(api):
+    """First column of a block, L_i0 = (a_i0 (1 / d)) sqrt(d), for pivots d of many
+    mantissas and exponents: four roundings, each at most 0.51 units."""
+    g = np.random.default_rng(17)
+    for e in (-500, -40, -1, 0, 1, 30, 500):
+        for d in np.ldexp(np.concatenate([[0.5, np.nextafter(1.0, 0.0), 0.75],
+                                          g.uniform(0.5, 1.0, size=37)]), e):
+            A = np.diag(np.full(64, 64.0 * d))
+            A[0, 0] = d
+            A[1:, 0] = d * g.uniform(-1.0, 1.0, size=63)
+            W = td(A)
+            api.potrf(W)
+            L = W.cpu().numpy()[:, 0].astype(np.longdouble)
+            dl = np.longdouble(d)
+            ref = A[:, 0].astype(np.longdouble) / np.sqrt(dl)
+            assert (np.abs(L - ref)[1:] <= 4 * 0.51 * 2.0 ** -52 * np.abs(ref)[1:]).all()
+            assert abs(L[0] - np.sqrt(dl)) <= 0.51 * 2.0 ** -52 * np.sqrt(dl)
