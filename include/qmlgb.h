@@ -59,7 +59,7 @@ typedef enum {
   QML_ENOTSPD = 2,    /* a Cholesky pivot was <= 0: matrix not positive definite */
   QML_ENOMEM = 3,     /* device workspace allocation failed */
   QML_ECUDA = 4,      /* a CUDA runtime call failed */
-  QML_ETIMEOUT = 5    /* a device-side wait exceeded its iteration budget */
+  QML_ETIMEOUT = 5    /* a device-side wait exceeded its time budget */
 } qml_status;
 
 typedef enum {
@@ -126,7 +126,8 @@ typedef struct {
 typedef enum {
   QML_BASIS_PIXEL = 0,     /* C = Y Lambda Y^T + N factored by Cholesky; W = X^T X */
   QML_BASIS_HARMONIC = 1,  /* SMW: M = Y^T N^-1 Y, the inner matrix Kt = I + L^T M L
-                              (Lambda = L L^T per (l, m)) factored in float64, and
+                              (Lambda = L L^T per (l, m)) factored at float64
+                              quality (as QML_FP64), and
                               W = L^-T Kt^-1 L^T M, the subtraction-free form of
                               M - M K^-1 M (App. C.3); needs the fiducial Lambda
                               positive definite at every window multipole */
@@ -176,7 +177,9 @@ qml_status qml_synthesize(const qml_problem *prob, const double *alm, const doub
  * eig_onesided, eig_mixed, eig_cluster).  Errors: QML_ENOTSPD if C is not
  * positive definite (info = the failing column) or F has an eigenvalue <= 0
  * (info = -1); QML_EINVAL for bad bin edges, a bad signal band, or (harmonic
- * basis) a fiducial block that is not positive definite. */
+ * basis) a fiducial block that is not positive definite; QML_ETIMEOUT as for
+ * every call with digit products (either precision; QML_FP64 from 256 rows or
+ * modes on): qml_fisher, qml_estimate, qml_cross, pix_loglike. */
 qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan, void *stream);
 
 /* Quadratic estimates for nsims maps (n x nsims) against a plan from
@@ -413,8 +416,8 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   updates and panel products (float64 diagonal blocks and
  *                   ln|Kt| either way)
  *   test_wait_timeout  0 (default) / 1: for testing the failure path only:
- *                   the split-precision product issues no copies and its
- *                   waits give up after 1 ms, so the call returns
+ *                   the digit products (of either precision) issue no copies
+ *                   and their waits give up after 1 ms, so the call returns
  *                   QML_ETIMEOUT (no fault; the context stays usable)
  *   test_room, test_digit_room  0 (default): for testing only: memory that a
  *                   call can do without (scan workers beyond four; digits of

@@ -179,3 +179,54 @@ def test_work_order_bands_same_bits(api, m, n, lower):
     sel = np.tril(np.ones((m, n), bool)) if lower else np.ones((m, n), bool)
     assert np.abs(got - ref)[sel].max() <= 1e-12 * np.abs(ref).max()
     assert (got[~sel] == 1.0).all()
+
+
+@pytest.mark.parametrize("nslices,bits", [(1, 24), (4, 24), (5, 48), (9, 55), (10, 55)])
+def test_nslices_forms(api, nslices, bits):
+    """Every digit count that nslices asks for, through a Fisher matrix and estimates.
+    A product's error is about sqrt(K) 2^-bits of its row's and column's maxima; C
+    passes it on with its condition number (and the float64 parts add 1e-11)."""
+    th, ph, _ = synth.healpix_ring_centres(8)
+    n = 560
+    wl = synth.make_workload("T", 8, 11, True, False, 0.0, ("TT",), 7, 50,
+                             geometry=(th[100:100 + n], ph[100:100 + n]))
+    Y, alm, noise, maps = P.oracle_maps(wl, 10)
+    ref = qml.qml_for(wl, Y, maps=maps)
+    cond = np.linalg.cond(qml.total_cov(Y, wl.cl_fid, wl.comps, wl.lmin, wl.lmax, wl.N()))
+    tol = 4 * cond * np.sqrt(n) * 2.0 ** -bits + 1e-11
+    prob = api.Problem.from_workload(wl, precision=1, nslices=nslices)
+    F, plan = api.fisher(prob)
+    est = plan.estimate(td(maps))
+    plan.free()
+    assert P.rel_max(F, ref["F"]) <= tol
+    assert P.rel_max(est["y"], ref["y"]) <= tol
+
+
+@pytest.mark.parametrize("call", ["fisher", "estimate", "loglike", "cross", "batch"])
+def test_fp64_calls_report_a_timeout(api, call):
+    """QML_FP64 calls with digit products report a wait that runs out as the split
+    ones do, and run normally afterwards."""
+    th, ph, _ = synth.healpix_ring_centres(8)
+    wl = synth.make_workload("T", 8, 9, True, False, 0.0, ("TT",), 7, 51,
+                             geometry=(th[100:700], ph[100:700]))
+    maps = td(P.oracle_maps(wl, 10)[3])
+    prob = api.Problem.from_workload(wl)
+    cl = torch.as_tensor(wl.cl_fid.reshape(-1), device="cuda")
+    F0, plan = api.fisher(prob)
+    run = {"fisher": lambda: api.fisher(prob, keep_plan=False),
+           "estimate": lambda: plan.estimate(maps),
+           "loglike": lambda: api.loglike(prob, cl, maps),
+           "cross": lambda: api.cross(plan, plan, maps, maps),
+           "batch": lambda: api.loglike_batch([(prob, maps)], np.zeros(2, int), cl.repeat(2, 1))}
+    api.tune_set("test_wait_timeout", 1)
+    try:
+        with pytest.raises(api.QMLError) as ei:
+            run[call]()
+    finally:
+        api.tune_set("test_wait_timeout", 0)
+    assert ei.value.status == 5, str(ei.value)
+    run[call]()
+    plan.free()
+    F1, p1 = api.fisher(prob)
+    p1.free()
+    assert torch.equal(F0, F1)
