@@ -420,9 +420,9 @@ qml_status qml_gemm(int32_t transA, int32_t transB, int64_t m, int64_t nn, int64
  *                   and their waits give up after 1 ms, so the call returns
  *                   QML_ETIMEOUT (no fault; the context stays usable)
  *   test_room, test_digit_room  0 (default): for testing only: memory that a
- *                   call can do without (scan workers beyond four; digits of
- *                   QML_FP64 products and solves, which then run on the
- *                   float64 pipe) counts as not available above this many
+ *                   call can do without (scan workers beyond four, the fused
+ *                   training steps; digits of QML_FP64 products and solves,
+ *                   which then run on the float64 pipe) counts as not available above this many
  *                   bytes a request
  * qml_tune_set / qml_tune_get: one entry (key without white space; get
  * returns QML_EINVAL when absent).  qml_tune_table writes the table as text,

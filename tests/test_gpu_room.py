@@ -130,3 +130,21 @@ def test_fp64_without_room_for_digits(api, basis, nbytes):
         api, nbytes, lambda: api.loglike_batch([(prob, d)], np.zeros(6, int), cl.repeat(6, 1))))
     assert np.abs(chi2 - rc).max() <= P.TOL * rc.max()
     assert np.abs(ld - rd).max() <= P.TOL * abs(rd)
+
+
+@pytest.mark.parametrize("width,depth,n,batch", [(64, 2, 300, 64), (256, 4, 1000, 512), (16, 1, 50, 16)])
+def test_training_without_second_activations(api, width, depth, n, batch):
+    """Both heads in fused steps, or head by head without the memory for them."""
+    g = np.random.default_rng(n)
+    th = g.uniform(-1, 1, size=(n, 3))
+    y = -(th ** 2).sum(axis=1) + np.sin(5 * th[:, 0]) * th[:, 1]
+
+    def train():
+        emu = api.Emulator(-np.ones(3), np.ones(3), width=width, depth=depth, seed=3)
+        loss = emu.train(th, y, epochs=3, batch=batch, lr=1e-3)
+        out = [emu.params(h) for h in (0, 1)]
+        emu.free()
+        return np.array(loss), *out
+
+    full, part = train(), with_room(api, 1, train)
+    assert all(np.array_equal(a, b) for a, b in zip(full, part))
