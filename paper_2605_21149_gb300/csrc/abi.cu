@@ -720,9 +720,11 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
            cudaEventCreateWithFlags(&e_diag, cudaEventDisableTiming) == cudaSuccess;
   }
   // The chain of a panel takes the same time whatever n is, the products beside
-  // it shrink with n: at n = 5952 the solve takes 40.3 ms (float64) and 33.5
-  // (split) with 8 SMs for the chain, 39.7 and 32.6 with 24; at n = 17152 294
-  // and 305.
+  // it shrink with n.  Fisher matrices with 8, 16 and 24 SMs for the chain, float64 |
+  // split: n = 4000 11.2, 11.2, 11.0 | 10.2, 10.1, 10.0 ms; 6000 22.5, 22.1, 21.9 |
+  // 19.4, 19.1, 18.8; 8000 32.9, 32.3, 32.3 | 27.5, 26.6, 26.1; 10000 53.0, 53.1,
+  // 53.6 | 40.6, 39.6, 39.5; 12000 71.1, 71.6, 72.5 | 52.6, 51.6, 51.9; n = 17152
+  // (split, with estimate) 294 with 8, 305 with 24.
   const int reserve = look ? (int)tune_get("split_lookahead_sms", n < 10000 ? 24 : 8) : 0;
   panel_chain(c, sp, A, lda, 0, n < kNBS ? n : kNBS, Linv64, LinvB, ldparts, dfdiag, c.st, false);
   for (int64_t j = 0; j < n && c.err == QML_OK; j += kNBS) {
@@ -1492,10 +1494,11 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
 
   // ---- per-item work, round-robin over worker streams
   // (eight by default: the chain of 64-wide float64 blocks that an item's factor
-  // waits on leaves most of the GPU to other items.  256 items of k = 756: 122
-  // ms with four workers, 77 with eight or sixteen; 24 items of k = 6900: 305,
-  // 283, 281.  From k = 10000 on four, whose products fill the GPU and whose k x
-  // k scratch is 0.8 GB and more each)
+  // waits on leaves most of the GPU to other items.  With four, eight and sixteen
+  // workers: 256 items of k = 756 122, 77 and 77 ms; 64 of k = 2871 113, 88, 89; 32
+  // of k = 5031 127, 110, 112; 16 of k = 8100 154, 146, 150; of k = 10080 237, 226,
+  // 229; of k = 12276 365, 352, 353.  From k = 10000 on four: 5 % and less are not
+  // worth 0.8 GB and more of k x k scratch a worker)
   const int ns_max = (int)std::max<int64_t>(
       1, std::min<int64_t>(16, tune_get("batch_streams", k < 10000 ? 8 : 4)));
   int NS = nitems < ns_max ? nitems : ns_max;
@@ -1628,6 +1631,8 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     spl.cols = W.cols;
     const InnerFactor K{W.K, W.Linv, W.LinvB};
     inner_potrf(cw, spl, K, k, W.ldp, lnKp);
+    // (512-wide blocks also for more than kSkinnyN maps: chi^2 sums over all modes,
+    // so that its small entries need not keep all their digits as F's do)
     inner_trsm(cw, spl, K, k, W.z, nm, k, false);
     launch_colnorm2(W.z, k, k, nm, W.rr, W.st);
     launch_batch_finish(W.rr, ms[m].dnd, ms[m].lnN, lnKp, nm, ol, oc, od, W.st);

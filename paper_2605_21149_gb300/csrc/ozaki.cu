@@ -65,7 +65,7 @@
 // one wave), 384 threads.
 //   warp 0   producer (one lane): bulk copies into a ring of stages, guarded
 //            by mbarriers;
-//   warp 1   TMEM allocator and MMA issuer (one lane): tcgen05.mma kind::f16
+//   warp 1   TMEM allocator and MMA issuer (in step, one lane issuing): tcgen05.mma kind::f16
 //            M=128 N=128 (64) K=16; commits a slot to the epilogue at the end of a
 //            chunk and waits for it to be read before refilling it;
 //   warps 2-3 idle (they complete warpgroup 0 for the register split);

@@ -12,6 +12,7 @@
 //   batch_streams    worker streams of pix_loglike_batch (1..16; default 8,
 //                    4 from k = 10000 modes on)
 //   ozaki_stages     4 (default) .. 2: depth of the split kernel's ring
+//   ozaki_band       8 (default): tile rows per band of its work order
 //   emu_tc           1 (default) / 0: emulator inference layers on tcgen05
 //                    / all through the WMMA product
 //   emu_tc0          1 (default) / 0: with emu_tc, the first layer too (its
@@ -24,8 +25,10 @@
 //                    inner factor Kt of pix_loglike_batch is as accurate as
 //                    QML_FP64; 1: its trailing updates and panel products
 //                    have 48 bits
-//   test_wait_timeout  1: failure-path test; the split-precision kernel
-//                    issues no copies and gives up each wait after 1 ms
+//   test_wait_timeout  1: failure-path test; the digit products issue no
+//                    copies and give up each wait after 1 ms
+//   test_room, test_digit_room  bytes above which memory that a call can do
+//                    without counts as not available (tests)
 //   batch_graphs     1 (default): pix_loglike_batch captures each worker's
 //                    per-item sequence once per mask as a CUDA graph and
 //                    replays it; 0: plain launches
