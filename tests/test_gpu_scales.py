@@ -122,3 +122,46 @@ def test_batch_uneven_noise(api, nmaps):
         assert np.abs(chi2[i, :nmaps] - rc).max() <= 1e-10 * rc.max()
         assert np.abs(chi2[i, :nmaps] - rc).max() <= 1e-10 * np.abs(rc).min()
         assert abs(ld[i] - rd) <= 1e-10 * abs(rd)
+
+
+@pytest.mark.parametrize("n", [300, 700])
+def test_maps_with_zeros_and_nonfinite_pixels(api, n):
+    """Pixels that are 0 in every map, a map of zeros, and maps with an infinity or a
+    NaN, which spoil their own results and no others."""
+    g = np.random.default_rng(n)
+    S = correlated(n, g)
+    x = np.linalg.cholesky(S) @ g.normal(size=(n, 14))
+    x[5:n:7] = 0.0
+    x[:, 3] = 0.0
+    wl = t_workload(n, 6, 3)
+    wl.cl_fid[:] = 0.0
+    wl.N = lambda: S
+    prob = api.Problem.from_workload(wl)
+    cl = torch.zeros(6 * (wl.lmax + 1), dtype=torch.float64, device="cuda")
+    ref = (np.linalg.solve(np.linalg.cholesky(S), x) ** 2).sum(axis=0)
+    bad = x.copy()
+    bad[n // 3, 8], bad[n - 2, 11], bad[0, 12] = np.nan, np.inf, -np.inf
+    for m in (x, bad):
+        lnl, chi2, ld = (P.to_np(v) for v in api.loglike(prob, cl, td(m)))
+        ok = np.isfinite(m).all(axis=0)
+        assert np.abs(chi2 - ref)[ok].max() <= 1e-12 * ref.max()
+        assert chi2[3] == 0.0 and not np.isfinite(chi2[~ok]).any()
+    chi2 = P.to_np(api.loglike(prob, cl, td(0.0 * x))[1])
+    assert (chi2 == 0.0).all()
+
+
+@pytest.mark.parametrize("n", [100, 300, 700])
+def test_pixels_over_most_of_the_exponent_range(api, n):
+    """Standard deviations between 2^-480 and 2^480 (covariances to 2^+-960)."""
+    g = np.random.default_rng(n)
+    S = correlated(n, g)
+    x = np.linalg.cholesky(S) @ g.normal(size=(n, 10))
+    e = g.integers(-480, 481, size=n)
+    wl = t_workload(n, 6, 3)
+    wl.cl_fid[:] = 0.0
+    wl.N = lambda: np.ldexp(S, e[:, None] + e[None, :])
+    lnl, chi2, ld = (P.to_np(v) for v in api.loglike(
+        api.Problem.from_workload(wl), torch.zeros(6 * (wl.lmax + 1), dtype=torch.float64,
+                                                   device="cuda"), td(np.ldexp(x, e[:, None]))))
+    ref = (np.linalg.solve(np.linalg.cholesky(S), x) ** 2).sum(axis=0)
+    assert np.abs(chi2 - ref).max() <= 1e-12 * ref.max()
