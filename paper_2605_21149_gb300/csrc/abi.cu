@@ -448,6 +448,15 @@ struct Split {
   // products of QML_FP64 (and of the inner SMW matrices): float64 quality,
   // and every diagonal block in float64 whatever split_diag_df says
   bool f64 = false;
+  // Where the pixels of one field end and those of the next begin, when the right-
+  // hand sides are modes of either (0: nowhere).  A mode of one field is 0, or small
+  // through a cross-spectrum, on the other's pixels; with noise that differs
+  // between the fields a row of a product then has terms whose sizes no scaling
+  // of k brings together, so that at float64 quality K is cut here.  T noise 1e4
+  // times that of Q and U, TQU Nside 8: entries of F to 3e-9 and of y to 4e-9 in one
+  // piece, 7e-12 and 9e-12 cut, as on the float64 pipe.  TQU Nside 16 solve 38.5 ->
+  // 39.2 ms, Nside 8 4.69 -> 4.73.
+  int64_t cut = 0;
   // SMs the split kernel leaves free (for float64 work on a second stream)
   int reserve_sms = 0;
   DigitBuf buf[3];
@@ -503,9 +512,9 @@ struct Split {
       oz_slice(X, sr, sk, d, c->st);
     return d;
   }
-  // the inverse for the right-hand sides sliced last
-  OzDigits slice_inverse(int i, const double *X, int64_t n, int64_t sr, int64_t sk) {
-    const OzDigits d = digits(i, n, n);
+  // the inverse (R x K) for the right-hand sides sliced last
+  OzDigits slice_inverse(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
+    const OzDigits d = digits(i, R, K);
     if (c->err != QML_OK) return OzDigits{};
     if (f64)
       oz_slice_inverse(X, sr, sk, d, cols, c->st);
@@ -518,6 +527,39 @@ struct Split {
     if (c->err != QML_OK || M <= 0 || N <= 0) return;
     c->cuda_ok(oz_mm(M, N, alpha, A, ra, B, rb, beta, C, ldc, lower, c->status, c->st, reserve_sms),
                "split-precision gemm");
+  }
+  // columns of the block j .. j + jb before the cut, 0 when it has none or no others
+  int64_t before_cut(int64_t j, int64_t jb) const {
+    return f64 && cut > j && cut < j + jb ? cut - j : 0;
+  }
+  // Panel j of B <- L^-1 B: B_j <- Xinv B_j (jb rows, nrhs columns).
+  void solve_block(const double *Xinv, int64_t j, int64_t jb, double *Bj, int64_t nrhs, int64_t ldb) {
+    const int64_t t = before_cut(j, jb), u = jb - t;
+    if (t > 0) {
+      // B_2 <- X_22 B_2 + X_21 B_1, then B_1 <- X_11 B_1
+      OzDigits dB = slice_rhs(2, Bj + t, nrhs, u, ldb, 1);
+      mm(u, nrhs, 1.0, slice_inverse(1, Xinv + t * (kNBS + 1), u, u, 1, kNBS), 0, dB, 0, 0.0, Bj + t,
+         ldb, 0);
+      dB = slice_rhs(2, Bj, nrhs, t, ldb, 1);
+      mm(u, nrhs, 1.0, slice_inverse(1, Xinv + t, u, t, 1, kNBS), 0, dB, 0, 1.0, Bj + t, ldb, 0);
+      mm(t, nrhs, 1.0, slice_inverse(1, Xinv, t, t, 1, kNBS), 0, dB, 0, 0.0, Bj, ldb, 0);
+      return;
+    }
+    const OzDigits dB = slice_rhs(2, Bj, nrhs, jb, ldb, 1);
+    mm(jb, nrhs, 1.0, slice_inverse(1, Xinv, jb, jb, 1, kNBS), 0, dB, 0, 0.0, Bj, ldb, 0);
+  }
+  // ... and B_below -= L21 B_j (m2 rows); dP: the digits of L21 in buffer 0, if there
+  void update_below(const OzDigits &dP, const double *L21, int64_t lda, int64_t m2, int64_t j,
+                    int64_t jb, double *Bj, int64_t nrhs, int64_t ldb) {
+    if (m2 <= 0) return;
+    const int64_t t = before_cut(j, jb);
+    for (int64_t k0 = 0; k0 < jb;) {
+      const int64_t kb = k0 < t ? t : jb - k0;
+      const OzDigits dL = dP.dig && kb == jb ? dP : slice(0, L21 + k0 * lda, m2, kb, 1, lda);
+      const OzDigits dB = slice(2, Bj + k0, nrhs, kb, ldb, 1);
+      mm(m2, nrhs, -1.0, dL, 0, dB, 0, 1.0, Bj + jb, ldb, 0);
+      k0 += kb;
+    }
   }
   // A few right-hand sides (nrhs <= kSkinnyN), panel j of B <- L^-1 B: B_j <-
   // Xinv B_j, B_below -= L21 B_j, on the float64 pipe: L is read once, where
@@ -577,10 +619,10 @@ struct Split {
   // C <- alpha op(A) op(B) + beta C, kDigitK of K at a time (one more rounding
   // of C each).  A QML_FP64 problem that fills the device has no digits in its
   // float64 form: it takes shorter pieces of K while the buffers do not fit,
-  // and below kNBS the float64 pipe.
+  // and below kNBS the float64 pipe.  kcut: K in two pieces there (0: no).
   void gemm(int ta, int tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A,
             int64_t lda, const double *B, int64_t ldb, double beta, double *C, int64_t ldc,
-            int lower) {
+            int lower, int64_t kcut = 0) {
     if (c->err != QML_OK || M <= 0 || N <= 0) return;
     const bool same = A == B && lda == ldb && ta != tb && M == N;
     int64_t kc = K < kDigitK || C == A || C == B ? K : kDigitK;  // (in place: all digits first)
@@ -596,7 +638,7 @@ struct Split {
     }
     int64_t k0 = 0;
     do {
-      const int64_t kb = K - k0 < kc ? K - k0 : kc;
+      const int64_t kend = k0 < kcut ? kcut : K, kb = kend - k0 < kc ? kend - k0 : kc;
       const OzDigits a = slice(0, A + k0 * (ta ? 1 : lda), M, kb, ta ? lda : 1, ta ? 1 : lda);
       const OzDigits b =
           same ? a : slice(1, B + k0 * (tb ? ldb : 1), N, kb, tb ? 1 : ldb, tb ? ldb : 1);
@@ -628,6 +670,10 @@ Split make_split(Call &c, int precision, int S) {
   Split sp{&c, S};
   sp.f64 = precision == QML_FP64;
   return sp;
+}
+// Split::cut of a problem's pixel rows: T | Q, U (float64 quality only)
+int64_t field_cut(const Split &sp, const Dims &d) {
+  return sp.f64 && d.nT < d.n ? d.nT : 0;
 }
 
 // The float64 part of the split Cholesky for the panel of columns j .. j + jb
@@ -740,7 +786,7 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
       const int64_t jb2 = m2 < kNBS ? m2 : kNBS;
       // panel: A21 <- A21 L_jj^-T
       dP = sp.slice_rhs(0, A21, m2, jb, 1, lda);
-      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
+      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, jb, 1, kNBS);
       sp.mm(m2, jb, 1.0, dP, 0, dX, 0, 0.0, A21, lda, 0);
       dP = sp.slice(0, A21, m2, jb, 1, lda);
       if (look) {
@@ -763,13 +809,8 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
       sp.few_panel(Xinv, jb, A21, lda, m2, B + j, nrhs, ldb);
     } else if (B) {
       // forward substitution, panel j: B_j <- L_jj^-1 B_j ; B_below -= A21 B_j
-      OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
-      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
-      sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
-      if (m2 > 0) {
-        dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
-        sp.mm(m2, nrhs, -1.0, dP, 0, dB, 0, 1.0, B + j + jb, ldb, 0);
-      }
+      sp.solve_block(Xinv, j, jb, B + j, nrhs, ldb);
+      sp.update_below(dP, A21, lda, m2, j, jb, B + j, nrhs, ldb);
     }
     sp.reserve_sms = 0;
     if (!look && m2 > 0)
@@ -800,15 +841,8 @@ void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, con
       sp.few_panel(Xinv, jb, L + (j + jb) + j * lda, lda, n - j - jb, B + j, nrhs, ldb);
       continue;
     }
-    OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
-    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
-    sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
-    const int64_t m2 = n - j - jb;
-    if (m2 > 0) {
-      const OzDigits dP = sp.slice(0, L + (j + jb) + j * lda, m2, jb, 1, lda);
-      dB = sp.slice(2, B + j, nrhs, jb, ldb, 1);
-      sp.mm(m2, nrhs, -1.0, dP, 0, dB, 0, 1.0, B + j + jb, ldb, 0);
-    }
+    sp.solve_block(Xinv, j, jb, B + j, nrhs, ldb);
+    sp.update_below(OzDigits{}, L + (j + jb) + j * lda, lda, n - j - jb, j, jb, B + j, nrhs, ldb);
   }
 }
 
@@ -820,7 +854,7 @@ void trsm_split_t(Call &c, Split &sp, const double *L, int64_t n, int64_t lda,
     const int64_t j = b * nb, jb = (n - j) < nb ? (n - j) : nb;
     const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS + (j % kNBS) * (kNBS + 1);
     OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
-    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, kNBS, 1);
+    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, jb, kNBS, 1);
     sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
     if (j > 0) {
       const OzDigits dP = sp.slice(0, L + j, j, jb, lda, 1);
@@ -974,7 +1008,7 @@ void plan_W(Call &c, const qml_plan *plan, double *W, double *T) {
   const Dims &d = plan->d;
   if (plan->split) {
     Split spl = make_split(c, plan->precision, plan->S);
-    spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1);
+    spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, field_cut(spl, d));
     spl.release();
   } else {
     launch_dgemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, c.status,
@@ -1195,6 +1229,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   }
 
   Split spl = make_split(c, prob->precision, plan->S);
+  spl.cut = field_cut(spl, d);
   Split *sp_or_null = plan->split ? &spl : nullptr;
   // Signal-band pieces: the whole band for the pixel basis; for the harmonic
   // basis the fixed signal below and above the window (Eq. N_eff).  They are
@@ -1245,7 +1280,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
       // runs beside the next panel's float64 chain)
       potrf_split(c, spl, plan->L, d.n, d.n, plan->Linv, plan->LinvB, ldparts, nullptr, plan->X,
                   d.k, d.n);
-      spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1);
+      spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, spl.cut);
     } else {
       potrf_blocked(c, plan->L, d.n, d.n, plan->Linv, ldparts, nullptr);
       trsm_blocked(c, plan->L, d.n, d.n, plan->Linv, plan->X, d.k, d.n);
@@ -1267,7 +1302,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
     if (plan->split) {
       potrf_split(c, spl, plan->L, d.n, d.n, plan->Linv, plan->LinvB, ldparts, nullptr, plan->X,
                   d.k, d.n);
-      spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1);
+      spl.gemm(1, 0, d.k, d.k, d.n, 1.0, plan->X, d.n, plan->X, d.n, 0.0, W, d.k, 1, spl.cut);
     } else {
       potrf_blocked(c, plan->L, d.n, d.n, plan->Linv, ldparts, nullptr);
       trsm_blocked(c, plan->L, d.n, d.n, plan->Linv, plan->X, d.k, d.n);
@@ -1469,6 +1504,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     launch_copy_matrix(D, d.n, u, d.n, d.n, nm, c.st);
     const int S = split_digits(pr->precision, pr->nslices, d.n);
     Split spl = make_split(c, pr->precision, S);
+    spl.cut = field_cut(spl, d);
     double *LinvB = S ? spl.block_inverses(d.n) : nullptr;
     if (LinvB && spl.ready(d.n, std::max(k, nm), true)) {
       potrf_split(c, spl, LN, d.n, d.n, Linv, LinvB, ldp, ms[m].lnN);
@@ -1481,7 +1517,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
     }
     c.release(LinvB);
     if (S) {
-      spl.gemm(1, 0, k, k, d.n, 1.0, U, d.n, U, d.n, 0.0, ms[m].M, k, 1);
+      spl.gemm(1, 0, k, k, d.n, 1.0, U, d.n, U, d.n, 0.0, ms[m].M, k, 1, spl.cut);
       spl.gemm(1, 0, k, nm, d.n, 1.0, U, d.n, u, d.n, 0.0, ms[m].v, k, 0);
       spl.release();
     } else {

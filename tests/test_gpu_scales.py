@@ -165,3 +165,27 @@ def test_pixels_over_most_of_the_exponent_range(api, n):
                                                    device="cuda"), td(np.ldexp(x, e[:, None]))))
     ref = (np.linalg.solve(np.linalg.cholesky(S), x) ** 2).sum(axis=0)
     assert np.abs(chi2 - ref).max() <= 1e-12 * ref.max()
+
+
+@pytest.mark.parametrize("tnoise", [1.0, 1e4, 1e6])
+def test_fields_of_different_noise(api, tnoise):
+    """TQU with T noise far above that of Q and U, in a block that holds pixels of
+    both: entries of F down to 1e-6 of their diagonal's, one by one (TOL of each: on
+    the float64 pipe 7e-12)."""
+    wl = synth.workload(1, "small")
+    assert len(wl.theta_T) % 512 != 0
+    N = wl.N()
+    s = np.ones(len(N))
+    s[:len(wl.theta_T)] = tnoise
+    N = N * s[:, None] * s[None, :]
+    wl.N = lambda: N
+    Y, _, _, maps = P.oracle_maps(wl, 12)
+    ref = qml.qml_for(wl, Y, maps=maps)
+    F, plan = api.fisher(api.Problem.from_workload(wl))
+    est = plan.estimate(td(maps))
+    plan.free()
+    F, Fr = P.to_np(F), ref["F"]
+    big = np.abs(Fr) >= 1e-6 * np.sqrt(np.outer(np.diag(Fr), np.diag(Fr)))
+    assert (np.abs(F - Fr) / np.abs(Fr))[big].max() <= P.TOL
+    for a in range(len(Fr)):
+        assert P.rel_max(est["y"][a], ref["y"][a]) <= P.TOL
