@@ -116,10 +116,13 @@ struct Call {
     cudaGetLastError();
     return nullptr;
   }
-  // whether what was tried leaves room for the small buffers that the call still
-  // takes and cannot do without
-  bool slack_left() {
-    void *p = try_malloc(32 << 20);
+  // whether `bytes` of memory that were tried leave room for the small buffers that
+  // the call still takes and cannot do without (not asked for less than kSlack: an
+  // allocation is 2 us of a small call)
+  static constexpr size_t kSlack = 32 << 20;
+  bool slack_left(size_t bytes) {
+    if (bytes < kSlack) return true;
+    void *p = try_malloc(kSlack);
     if (p) cudaFreeAsync(p, st);
     return p != nullptr;
   }
@@ -476,6 +479,10 @@ struct Split {
       b = DigitBuf{};
     }
   }
+  // the same where they are large: a small call keeps them for its next stage
+  void release_large() {
+    if (buf[0].bytes + buf[1].bytes + buf[2].bytes >= 2 * Call::kSlack) release();
+  }
   // memory for the digits of an R x K matrix in buffer i
   OzDigits digits(int i, int64_t R, int64_t K) {
     const size_t need = oz_digits_bytes(R, K, S);
@@ -512,9 +519,9 @@ struct Split {
       oz_slice(X, sr, sk, d, c->st);
     return d;
   }
-  // the inverse (R x K) for the right-hand sides sliced last
-  OzDigits slice_inverse(int i, const double *X, int64_t R, int64_t K, int64_t sr, int64_t sk) {
-    const OzDigits d = digits(i, R, K);
+  // the inverse for the right-hand sides sliced last
+  OzDigits slice_inverse(int i, const double *X, int64_t n, int64_t sr, int64_t sk) {
+    const OzDigits d = digits(i, n, n);
     if (c->err != QML_OK) return OzDigits{};
     if (f64)
       oz_slice_inverse(X, sr, sk, d, cols, c->st);
@@ -528,37 +535,25 @@ struct Split {
     c->cuda_ok(oz_mm(M, N, alpha, A, ra, B, rb, beta, C, ldc, lower, c->status, c->st, reserve_sms),
                "split-precision gemm");
   }
-  // columns of the block j .. j + jb before the cut, 0 when it has none or no others
-  int64_t before_cut(int64_t j, int64_t jb) const {
-    return f64 && cut > j && cut < j + jb ? cut - j : 0;
-  }
-  // Panel j of B <- L^-1 B: B_j <- Xinv B_j (jb rows, nrhs columns).
-  void solve_block(const double *Xinv, int64_t j, int64_t jb, double *Bj, int64_t nrhs, int64_t ldb) {
-    const int64_t t = before_cut(j, jb), u = jb - t;
-    if (t > 0) {
-      // B_2 <- X_22 B_2 + X_21 B_1, then B_1 <- X_11 B_1
-      OzDigits dB = slice_rhs(2, Bj + t, nrhs, u, ldb, 1);
-      mm(u, nrhs, 1.0, slice_inverse(1, Xinv + t * (kNBS + 1), u, u, 1, kNBS), 0, dB, 0, 0.0, Bj + t,
+  // Panel j of B <- L^-1 B (jb columns of L from row and column j on, Ljj at its
+  // corner, m rows from there to the last): B_j <- Xinv B_j, B_below -= L_below B_j; a
+  // panel that the cut lies in as two of its own.  dP: the digits of the rows below
+  // the panel, in buffer 0, if they are there.
+  void forward_panel(const double *Ljj, int64_t lda, int64_t m, const double *Xinv, int64_t j,
+                     int64_t jb, const OzDigits &dP, double *Bj, int64_t nrhs, int64_t ldb) {
+    for (int64_t i = 0; i < jb;) {
+      const int64_t ib = f64 && cut > j + i && cut < j + jb ? cut - (j + i) : jb - i;
+      OzDigits dB = slice_rhs(2, Bj + i, nrhs, ib, ldb, 1);
+      mm(ib, nrhs, 1.0, slice_inverse(1, Xinv + i * (kNBS + 1), ib, 1, kNBS), 0, dB, 0, 0.0, Bj + i,
          ldb, 0);
-      dB = slice_rhs(2, Bj, nrhs, t, ldb, 1);
-      mm(u, nrhs, 1.0, slice_inverse(1, Xinv + t, u, t, 1, kNBS), 0, dB, 0, 1.0, Bj + t, ldb, 0);
-      mm(t, nrhs, 1.0, slice_inverse(1, Xinv, t, t, 1, kNBS), 0, dB, 0, 0.0, Bj, ldb, 0);
-      return;
-    }
-    const OzDigits dB = slice_rhs(2, Bj, nrhs, jb, ldb, 1);
-    mm(jb, nrhs, 1.0, slice_inverse(1, Xinv, jb, jb, 1, kNBS), 0, dB, 0, 0.0, Bj, ldb, 0);
-  }
-  // ... and B_below -= L21 B_j (m2 rows); dP: the digits of L21 in buffer 0, if there
-  void update_below(const OzDigits &dP, const double *L21, int64_t lda, int64_t m2, int64_t j,
-                    int64_t jb, double *Bj, int64_t nrhs, int64_t ldb) {
-    if (m2 <= 0) return;
-    const int64_t t = before_cut(j, jb);
-    for (int64_t k0 = 0; k0 < jb;) {
-      const int64_t kb = k0 < t ? t : jb - k0;
-      const OzDigits dL = dP.dig && kb == jb ? dP : slice(0, L21 + k0 * lda, m2, kb, 1, lda);
-      const OzDigits dB = slice(2, Bj + k0, nrhs, kb, ldb, 1);
-      mm(m2, nrhs, -1.0, dL, 0, dB, 0, 1.0, Bj + jb, ldb, 0);
-      k0 += kb;
+      const int64_t m2 = m - i - ib;
+      if (m2 > 0) {
+        const OzDigits dL =
+            dP.dig && ib == jb ? dP : slice(0, Ljj + (i + ib) + i * lda, m2, ib, 1, lda);
+        dB = slice(2, Bj + i, nrhs, ib, ldb, 1);
+        mm(m2, nrhs, -1.0, dL, 0, dB, 0, 1.0, Bj + i + ib, ldb, 0);
+      }
+      i += ib;
     }
   }
   // A few right-hand sides (nrhs <= kSkinnyN), panel j of B <- L^-1 B: B_j <-
@@ -602,17 +597,23 @@ struct Split {
   // form: true, and a buffer that does not fit fails the call.)
   bool ready(int64_t n, int64_t nrhs, bool factor) {
     if (!f64 || c->err != QML_OK) return true;
-    bool ok = room(2, split_ws_bytes(2, n, nrhs, S));
-    if (factor || nrhs > kSkinnyN)
-      ok = ok && room(0, split_ws_bytes(0, n, nrhs, S)) && room(1, split_ws_bytes(1, n, nrhs, S));
-    if (ok && !cols.kmax) {
-      unsigned char *p = (unsigned char *)c->try_alloc(kColumnBytes);
-      if (p) cols = make_columns(*c, p);
-      ok = cols.kmax != nullptr;
+    const int need = factor || nrhs > kSkinnyN ? 0 : 2;  // buffers 0 .. 2, or 2 alone
+    size_t total = 0;
+    bool ok = true;
+    for (int i = 2; i >= need && ok; --i) {
+      const size_t bytes = split_ws_bytes(i, n, nrhs, S);
+      total += bytes;
+      ok = room(i, bytes);
     }
-    if (ok && factor && !tinv) tinv = (double *)c->try_alloc(kTinvBytes);
-    if (factor) ok = ok && tinv;
-    ok = ok && c->slack_left();
+    if (ok && !cols.kmax) {
+      unsigned char *p = (unsigned char *)c->try_alloc(kTinvBytes + kColumnBytes);
+      ok = p != nullptr;
+      if (p) {
+        tinv = (double *)p;
+        cols = make_columns(*c, p + kTinvBytes);
+      }
+    }
+    ok = ok && c->slack_left(total);
     if (!ok) release();
     return ok || c->err != QML_OK;
   }
@@ -627,7 +628,8 @@ struct Split {
     const bool same = A == B && lda == ldb && ta != tb && M == N;
     int64_t kc = K < kDigitK || C == A || C == B ? K : kDigitK;  // (in place: all digits first)
     while (f64 && !(room(0, oz_digits_bytes(M, kc, S)) &&
-                    (same || room(1, oz_digits_bytes(N, kc, S))) && c->slack_left())) {
+                    (same || room(1, oz_digits_bytes(N, kc, S))) &&
+                    c->slack_left(buf[0].bytes + buf[1].bytes))) {
       if (kc <= kNBS) {
         release();
         launch_dgemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, lower, c->status, c->st);
@@ -786,7 +788,7 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
       const int64_t jb2 = m2 < kNBS ? m2 : kNBS;
       // panel: A21 <- A21 L_jj^-T
       dP = sp.slice_rhs(0, A21, m2, jb, 1, lda);
-      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, jb, 1, kNBS);
+      const OzDigits dX = sp.slice_inverse(1, Xinv, jb, 1, kNBS);
       sp.mm(m2, jb, 1.0, dP, 0, dX, 0, 0.0, A21, lda, 0);
       dP = sp.slice(0, A21, m2, jb, 1, lda);
       if (look) {
@@ -809,8 +811,7 @@ void potrf_split(Call &c, Split &sp, double *A, int64_t n, int64_t lda, double *
       sp.few_panel(Xinv, jb, A21, lda, m2, B + j, nrhs, ldb);
     } else if (B) {
       // forward substitution, panel j: B_j <- L_jj^-1 B_j ; B_below -= A21 B_j
-      sp.solve_block(Xinv, j, jb, B + j, nrhs, ldb);
-      sp.update_below(dP, A21, lda, m2, j, jb, B + j, nrhs, ldb);
+      sp.forward_panel(A + j + j * lda, lda, n - j, Xinv, j, jb, dP, B + j, nrhs, ldb);
     }
     sp.reserve_sms = 0;
     if (!look && m2 > 0)
@@ -841,8 +842,7 @@ void trsm_split(Call &c, Split &sp, const double *L, int64_t n, int64_t lda, con
       sp.few_panel(Xinv, jb, L + (j + jb) + j * lda, lda, n - j - jb, B + j, nrhs, ldb);
       continue;
     }
-    sp.solve_block(Xinv, j, jb, B + j, nrhs, ldb);
-    sp.update_below(OzDigits{}, L + (j + jb) + j * lda, lda, n - j - jb, j, jb, B + j, nrhs, ldb);
+    sp.forward_panel(L + j + j * lda, lda, n - j, Xinv, j, jb, OzDigits{}, B + j, nrhs, ldb);
   }
 }
 
@@ -854,7 +854,7 @@ void trsm_split_t(Call &c, Split &sp, const double *L, int64_t n, int64_t lda,
     const int64_t j = b * nb, jb = (n - j) < nb ? (n - j) : nb;
     const double *Xinv = LinvB + (j / kNBS) * kNBS * kNBS + (j % kNBS) * (kNBS + 1);
     OzDigits dB = sp.slice_rhs(2, B + j, nrhs, jb, ldb, 1);
-    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, jb, kNBS, 1);
+    const OzDigits dX = sp.slice_inverse(1, Xinv, jb, kNBS, 1);
     sp.mm(jb, nrhs, 1.0, dX, 0, dB, 0, 0.0, B + j, ldb, 0);
     if (j > 0) {
       const OzDigits dP = sp.slice(0, L + j, j, jb, lda, 1);
@@ -1263,7 +1263,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   };
   auto ready_plan = [&] {
     if (!plan->split) return;
-    spl.release();
+    spl.release_large();
     plan->LinvB = block_inverses(d.n, spl.f64);
     plan->split = plan->LinvB && spl.ready(d.n, d.k, true);
     if (!plan->split) plan->S = 0;
@@ -1417,7 +1417,7 @@ qml_status pix_loglike(const qml_problem *prob, const double *cl_theta, const do
   double *LinvB = nullptr;
   if (S) {
     build_C_split(c, spl, sp, d, Y, C);
-    spl.release();
+    spl.release_large();
     LinvB = spl.block_inverses(d.n);
   } else {
     build_C(c, sp, d, Y, C);
@@ -1610,7 +1610,7 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   for (int w = 0; w < sure && (S48 || Sk); ++w) {
     const size_t need = place_digits(wk[w], std::max(S48, Sk), nullptr);
     dig[w] = S48 ? c.alloc<unsigned char>(need, "split workspace") : c.try_alloc(need);
-    if (!S48 && (!dig[w] || !c.slack_left())) {
+    if (!S48 && (!dig[w] || !c.slack_left(need))) {
       for (int v = 0; v <= w; ++v) c.release(dig[v]);
       Sk = 0;
       break;
@@ -1620,9 +1620,11 @@ qml_status pix_loglike_batch(const lnl_mask *masks, int32_t nmask, int32_t nitem
   // the others only where the device has room for all of their scratch
   const int Smax = std::max(S48, Sk);
   for (int w = sure; w < NS; ++w) {
-    void *p = c.try_alloc(place(wk[w], nullptr), "test_room");
-    if (Smax && p) dig[w] = c.try_alloc(place_digits(wk[w], Smax, nullptr), "test_room");
-    if (!p || (Smax && !dig[w]) || !c.slack_left()) {
+    const size_t base = place(wk[w], nullptr);
+    const size_t more = Smax ? place_digits(wk[w], Smax, nullptr) : 0;
+    void *p = c.try_alloc(base, "test_room");
+    if (Smax && p) dig[w] = c.try_alloc(more, "test_room");
+    if (!p || (Smax && !dig[w]) || !c.slack_left(base + more)) {
       c.release(p);
       c.release(dig[w]);
       NS = w;
