@@ -463,6 +463,7 @@ struct Split {
   // SMs the split kernel leaves free (for float64 work on a second stream)
   int reserve_sms = 0;
   DigitBuf buf[3];
+  void *block = nullptr;  // what ready took: buffers, scales and doubling scratch
   static constexpr size_t kTinvBytes = sizeof(double) * (kNBS / 2) * (kNBS / 2);
   OzColumns cols;  // scales of the products with block inverses
   double *tinv = nullptr;  // (kNBS/2)^2 scratch of the block-inverse doubling
@@ -478,10 +479,11 @@ struct Split {
       c->release(b.p);
       b = DigitBuf{};
     }
-  }
-  // the same where they are large: a small call keeps them for its next stage
-  void release_large() {
-    if (buf[0].bytes + buf[1].bytes + buf[2].bytes >= 2 * Call::kSlack) release();
+    if (!block) return;
+    c->release(block);
+    block = nullptr;
+    tinv = nullptr;
+    cols = OzColumns{};
   }
   // memory for the digits of an R x K matrix in buffer i
   OzDigits digits(int i, int64_t R, int64_t K) {
@@ -595,27 +597,31 @@ struct Split {
   // needs none of them, so that a device without the room is no error: false,
   // and the caller takes the *_blocked form.  (The split precision has no other
   // form: true, and a buffer that does not fit fails the call.)
+  // One allocation: they come before the first launch of a small call, 2-4 us each.
   bool ready(int64_t n, int64_t nrhs, bool factor) {
     if (!f64 || c->err != QML_OK) return true;
-    const int need = factor || nrhs > kSkinnyN ? 0 : 2;  // buffers 0 .. 2, or 2 alone
-    size_t total = 0;
-    bool ok = true;
-    for (int i = 2; i >= need && ok; --i) {
-      const size_t bytes = split_ws_bytes(i, n, nrhs, S);
-      total += bytes;
-      ok = room(i, bytes);
+    release();
+    const int first = factor || nrhs > kSkinnyN ? 0 : 2;  // buffers 0 .. 2, or 2 alone
+    const size_t scratch = cols.kmax ? 0 : (kTinvBytes + kColumnBytes + 1023) / 1024 * 1024;
+    // (no buffer begins where the block does: one that grows is given back by its
+    // pointer, which must not name the block)
+    size_t total = 1024 + scratch;
+    for (int i = first; i < 3; ++i) total += split_ws_bytes(i, n, nrhs, S);
+    block = c->try_alloc(total);
+    if (!block || !c->slack_left(total)) {
+      release();
+      return c->err != QML_OK;
     }
-    if (ok && !cols.kmax) {
-      unsigned char *p = (unsigned char *)c->try_alloc(kTinvBytes + kColumnBytes);
-      ok = p != nullptr;
-      if (p) {
-        tinv = (double *)p;
-        cols = make_columns(*c, p + kTinvBytes);
-      }
+    unsigned char *p = (unsigned char *)block + 1024;
+    for (int i = first; i < 3; ++i) {
+      buf[i] = DigitBuf{p, split_ws_bytes(i, n, nrhs, S)};
+      p += buf[i].bytes;
     }
-    ok = ok && c->slack_left(total);
-    if (!ok) release();
-    return ok || c->err != QML_OK;
+    if (scratch) {
+      tinv = (double *)p;
+      cols = make_columns(*c, p + kTinvBytes);
+    }
+    return true;
   }
   // C <- alpha op(A) op(B) + beta C, kDigitK of K at a time (one more rounding
   // of C each).  A QML_FP64 problem that fills the device has no digits in its
@@ -1263,7 +1269,7 @@ qml_status qml_fisher(const qml_problem *prob, double *F, qml_plan **plan_out, v
   };
   auto ready_plan = [&] {
     if (!plan->split) return;
-    spl.release_large();
+    spl.release();
     plan->LinvB = block_inverses(d.n, spl.f64);
     plan->split = plan->LinvB && spl.ready(d.n, d.k, true);
     if (!plan->split) plan->S = 0;
@@ -1417,7 +1423,7 @@ qml_status pix_loglike(const qml_problem *prob, const double *cl_theta, const do
   double *LinvB = nullptr;
   if (S) {
     build_C_split(c, spl, sp, d, Y, C);
-    spl.release_large();
+    spl.release();
     LinvB = spl.block_inverses(d.n);
   } else {
     build_C(c, sp, d, Y, C);
